@@ -395,6 +395,28 @@ def test_select_keys_constant_and_narrow_rows(T, B):
     np.testing.assert_array_equal(gp.k_idx[0, :, :B].cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("mode", ["cosine", "dot"])
+@pytest.mark.parametrize("T,n_kv", [(513, 3), (8193, 8), (16385, 8), (16385, 33), (20011, 73), (32768, 14), (32769, 15)])
+def test_select_keys_every_cluster_width(T, n_kv, mode):
+    """Rows cut into 1 / 2 / 4 / 8 CTAs (by length and number of rows): a spread row, rows whose threshold falls into a
+    bin of more rows than are ranked against each other (equal and nearly equal scores, with the cut inside a CTA and
+    at a CTA's edge), scores outside [-1, 1] and rows of two values.  Integer parity with the oracle."""
+    B = T // 7 + 1
+    r = np.random.default_rng(T + n_kv)
+    s = (0.25 + 0.03 * r.normal(size=(n_kv, T))).astype(np.float32)
+    s[0, :] = np.float32(0.3) + r.integers(0, 40, T).astype(np.float32) * np.float32(2.0 ** -24)
+    s[1, :] = (s[1] > np.quantile(s[1], 0.95)).astype(np.float32)         # the cut lies among the zeros
+    s[2, :] *= 40.0                                                       # far outside the cosine range
+    gp = scores_only_problem(T, B, n_kv)
+    gp.p.score_mode = {"cosine": api.SCORE_COSINE, "dot": api.SCORE_DOT}[mode]
+    gp.scores[0] = torch.from_numpy(s).cuda()
+    api.quoka_select_keys(gp.p, gp.scores, gp.k_idx, gp.k_cnt, gp.ws)
+    torch.cuda.synchronize()
+    want = O.select_keys(s.astype(np.float64), B)
+    np.testing.assert_array_equal(gp.k_idx[0, :, :B].cpu().numpy(), want)
+    assert int(gp.k_cnt[0]) == B
+
+
 # ---------------------------------------------------------------- full-size configurations
 def test_llama8b_32k_full_size():
     w = synth.WORKLOADS["llama8b_32k"]
