@@ -67,7 +67,7 @@ typedef enum { QUOKA_BF16 = 0, QUOKA_F32 = 1 } quoka_dtype;
 
 /* Which kernels serve the contraction steps (scoring, attention). */
 typedef enum {
-  QUOKA_IMPL_AUTO = 0,   /* tcgen05 tensor-core kernels for bf16, scalar kernels for f32 */
+  QUOKA_IMPL_AUTO = 0,   /* tcgen05 tensor-core kernels for bf16, tiled fp32 kernels for f32 */
   QUOKA_IMPL_SIMT = 1,   /* scalar fp32 kernels (any dtype); the on-device cross-check */
   QUOKA_IMPL_TENSOR = 2  /* tcgen05 kernels; QUOKA_ERR_UNSUPPORTED if dtype is f32 */
 } quoka_impl;

@@ -1,5 +1,5 @@
 // Scalar fp32 attention over [selected cached rows | the chunk's own causal rows] (Algorithm 2's
-// attention line; Eq. 1 / Eq. 2).  Serves the f32 dtype and cross-checks the tensor-core kernel.
+// attention line; Eq. 1 / Eq. 2): the on-device cross-check of the other kernels (QUOKA_IMPL_SIMT, both data types).
 // One warp per (sequence, query head, chunk row); the 32 lanes split head_dim; keys are visited one
 // by one with a running maximum, running denominator and running output (online softmax, fp32).
 // The two running sums are compensated (Kahan): once a dominant key is in them, thousands of weights below half

@@ -191,12 +191,16 @@ cudaError_t launch_aggregate_queries(const DevParams& P, int dtype, const void* 
                                      cudaStream_t st, bool chained = false);
 cudaError_t launch_score_keys_simt(const DevParams& P, int dtype, const void* qbar, const void* k, float* scores,
                                    cudaStream_t st);
+cudaError_t launch_score_keys_f32(const DevParams& P, const float* qbar, const float* k, float* scores, cudaStream_t st,
+                                  bool chained);
 cudaError_t launch_key_norms(const DevParams& P, int dtype, const void* k, float* k_inv_norm, int all_rows,
                              cudaStream_t st);
 cudaError_t launch_select_keys(const DevParams& P, const float* scores, int32_t* k_idx, int32_t* k_cnt,
                                cudaStream_t st, bool chained = false);
 cudaError_t launch_attn_simt(const DevParams& P, int dtype, const void* q, const void* k, const void* v,
                              const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st);
+cudaError_t launch_attn_f32(const DevParams& P, const float* q, const float* k, const float* v, const int32_t* k_idx,
+                            const int32_t* k_cnt, float* out, float* lse, cudaStream_t st, bool chained);
 
 // Generation phase (chunk of one query): matrix-vector scoring and a gather attention kernel.
 bool decode_path_applies(const DevParams& P);

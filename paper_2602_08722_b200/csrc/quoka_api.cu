@@ -170,6 +170,10 @@ static quoka_status run_score_keys(const quoka_params* p, const DevParams& P, co
   }
   if (use_tensor(p) && score_keys_tc_supported(p)) return launch_score_keys_tc(p, P, qbar, k, scores, st, chained);
   if (p->impl == QUOKA_IMPL_TENSOR) return QUOKA_ERR_UNSUPPORTED;
+  if (p->impl == QUOKA_IMPL_AUTO && p->dtype == QUOKA_F32) {
+    QUOKA_TRY_CUDA(launch_score_keys_f32(P, static_cast<const float*>(qbar), static_cast<const float*>(k), scores, st, chained));
+    return QUOKA_OK;
+  }
   QUOKA_TRY_CUDA(launch_score_keys_simt(P, p->dtype, qbar, k, scores, st));
   return QUOKA_OK;
 }
@@ -184,6 +188,11 @@ static quoka_status run_attn(const quoka_params* p, const DevParams& P, const vo
   if (use_tensor(p) && attn_tc_supported(p))
     return launch_attn_tc(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection);
   if (p->impl == QUOKA_IMPL_TENSOR) return QUOKA_ERR_UNSUPPORTED;
+  if (p->impl == QUOKA_IMPL_AUTO && p->dtype == QUOKA_F32) {
+    QUOKA_TRY_CUDA(launch_attn_f32(P, static_cast<const float*>(q), static_cast<const float*>(k), static_cast<const float*>(v),
+                                   k_idx, k_cnt, static_cast<float*>(out), lse, st, after_selection));
+    return QUOKA_OK;
+  }
   QUOKA_TRY_CUDA(launch_attn_simt(P, p->dtype, q, k, v, k_idx, k_cnt, out, lse, st));
   return QUOKA_OK;
 }

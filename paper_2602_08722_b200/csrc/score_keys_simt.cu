@@ -1,9 +1,13 @@
-// Scalar fp32 scoring kernel (Algorithm 1: S = Qbar K^T on normalised keys, max over queries).
-// Serves the f32 dtype and is the on-device cross-check of the tensor-core kernel.
-// One CTA = 128 cached keys of one (sequence, KV head); one thread = one key.  The key tile is
+// fp32 scoring kernels (Algorithm 1: S = Qbar K^T on normalised keys, max over queries).
+//
+// score_keys_f32_kernel serves the f32 dtype: 64 keys per CTA against all retained queries, 4 x J products per thread.
+// What bounds it: the FMA pipes on large problems; on small ones the latency of one tile, hence 64 keys per CTA (8192
+// keys fill 128 SMs).  4096 rows of 2 KV heads against 32 queries: 20.6 -> 7.5 us (a thread per key, 64 CTAs, before).
+//
+// score_keys_simt_kernel is the on-device cross-check of the others (impl = QUOKA_IMPL_SIMT, both dtypes): one CTA = 128 cached keys of one (sequence, KV head); one thread = one key.  The key tile is
 // staged in shared memory as fp32 (padded rows), Qbar streams through shared memory 32 queries at a
 // time, each thread keeps 32 running dot products and folds them into its running maximum.
-#include "common.cuh"
+#include "f32_tiles.cuh"
 
 namespace quoka {
 
@@ -74,6 +78,84 @@ __global__ void __launch_bounds__(kScoreTile) score_keys_simt_kernel(DevParams P
     else val = agg / fmaxf(sqrtf(nn), kNormEps);
     scores[((int64_t)s * P.n_kv + kv) * P.max_ctx + t0 + tid] = val;
   }
+}
+
+template <int D, int J>
+__global__ void __launch_bounds__(kF32Threads) score_keys_f32_kernel(DevParams P, const float* __restrict__ qbar,
+                                                                     const float* __restrict__ k,
+                                                                     float* __restrict__ scores) {
+  constexpr int LD = f32_pitch<D>(), W = D / 4, kQ = 16 * J;
+  extern __shared__ __align__(16) float smf[];
+  float* ks = smf;                                   // [64][LD]
+  float* qs = ks + kF32Tile * LD;                    // [kQ][LD]
+  grid_launch_dependents();
+  const int s = blockIdx.z, kv = blockIdx.y, t0 = blockIdx.x * kF32Tile;
+  const int T = __ldg(P.ctx_len + s);
+  if (t0 >= T) { grid_dependency_wait(); return; }
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, N = P.n_sel;
+  for (int e = tid; e < kF32Tile * W; e += kF32Threads) {
+    const int r = e / W, c = e % W;
+    ptx::cp_async_16(ptx::smem_u32(ks + r * LD + 4 * c), k + kv_row_offset(P, s, kv, min(t0 + r, T - 1)) + 4 * c, true);
+  }
+  grid_dependency_wait();                            // Q-bar comes from the kernel before
+  const float* qb = qbar + ((long long)s * P.n_kv + kv) * (long long)N * D;
+  float best[4], total[4], nn[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { best[i] = -INFINITY; total[i] = 0.f; nn[i] = 0.f; }
+  for (int j0 = 0; j0 < N; j0 += kQ) {
+    for (int e = tid; e < kQ * W; e += kF32Threads) {
+      const int r = e / W, c = e % W;
+      ptx::cp_async_16(ptx::smem_u32(qs + r * LD + 4 * c), qb + (long long)min(j0 + r, N - 1) * D + 4 * c, true);
+    }
+    ptx::cp_async_wait_all();
+    __syncthreads();
+    float acc[4][J];
+    f32_dot_tile<D, J>(ks, qs, ty, tx, acc);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < J; ++j)
+        if (j0 + tx + 16 * j < N) { best[i] = fmaxf(best[i], acc[i][j]); total[i] += acc[i][j]; }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int g = 0; g < D / 64; ++g) {
+      const float4 x = *reinterpret_cast<const float4*>(ks + (4 * ty + i) * LD + 64 * g + 4 * tx);
+      nn[i] = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, nn[i]))));
+    }
+    nn[i] = half_warp_sum(nn[i]);
+    const float agg = P.agg_mean ? half_warp_sum(total[i]) / (float)N : half_warp_max(best[i]);
+    const int t = t0 + 4 * ty + i;
+    if (tx == 0 && t < T) {
+      float val;
+      if (P.score_dot) val = agg;
+      else if (P.k_inv_norm) val = agg * __ldg(P.k_inv_norm + kv_norm_index(P, s, kv, t));
+      else val = agg / fmaxf(sqrtf(nn[i]), kNormEps);
+      scores[((long long)s * P.n_kv + kv) * P.max_ctx + t] = val;
+    }
+  }
+}
+
+cudaError_t launch_score_keys_f32(const DevParams& P, const float* qbar, const float* k, float* scores, cudaStream_t st,
+                                  bool chained) {
+  if (P.max_ctx <= 0) return cudaSuccess;
+  const dim3 grid((P.max_ctx + kF32Tile - 1) / kF32Tile, P.n_kv, P.batch), block(kF32Threads);
+  cudaError_t e;
+#define QUOKA_SCORE_F32(D_, J_)                                                                                           \
+  do {                                                                                                                    \
+    const size_t smem = (size_t)(kF32Tile + 16 * (J_)) * f32_pitch<D_>() * sizeof(float);                                 \
+    e = cudaFuncSetAttribute(score_keys_f32_kernel<D_, J_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);      \
+    if (e != cudaSuccess) return e;                                                                                       \
+    e = launch_kernel("score_keys_f32", score_keys_f32_kernel<D_, J_>, grid, block, smem, st, 1, chained, P, qbar, k, scores); \
+  } while (0)
+  if (P.n_sel <= 32) { if (P.d == 128) QUOKA_SCORE_F32(128, 2); else QUOKA_SCORE_F32(64, 2); }
+  else { if (P.d == 128) QUOKA_SCORE_F32(128, 4); else QUOKA_SCORE_F32(64, 4); }
+#undef QUOKA_SCORE_F32
+  if (e != cudaSuccess) return e;
+  count_launch();
+  return cudaGetLastError();
 }
 
 // Inverse norms of cache rows (one warp per row): rows [T_s, T_s + C) of every (sequence, KV head), or all of

@@ -395,6 +395,26 @@ def test_select_keys_constant_and_narrow_rows(T, B):
     np.testing.assert_array_equal(gp.k_idx[0, :, :B].cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("T,C,B,n_q,n_kv,d,n_retain", [
+    (63, 2, 40, 4, 2, 128, 1),          # fewer keys than a tile, two query rows
+    (129, 63, 128, 2, 1, 64, 16),       # the last tile of the list holds one key
+    (2000, 65, 700, 3, 3, 128, 33),     # parts of unequal length, a row block of one row, 33 retained queries
+    (1500, 640, 64, 32, 8, 64, 32),     # more row blocks than SMs: one part
+])
+def test_f32_tiles_at_their_edges(T, C, B, n_q, n_kv, d, n_retain, paged):
+    """The f32 kernels at the edges of their 64 x 64 tiles and of the parts a row block's keys are cut into."""
+    gp = problem(970 + T, n_q=n_q, n_kv=n_kv, d=d, T=T, C=C, dtype="f32", n_retain=n_retain, kv_budget=B, paged=paged)
+    gp.run_staged()
+    check_chain(gp)
+    q, k, v, _ = gp.oracle_inputs(0)
+    api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, gp.lse, gp.ws)
+    torch.cuda.synchronize()
+    dense, lse = O.dense_chunk_attention(q, k, v, T)
+    check_attention(f64(gp.out[0]), dense, "f32")
+    assert np.abs(f64(gp.lse[0]) - lse).max() <= 2e-3
+
+
 @pytest.mark.parametrize("mode", ["cosine", "dot"])
 @pytest.mark.parametrize("T,n_kv", [(513, 3), (8193, 8), (16385, 8), (16385, 33), (20011, 73), (32768, 14), (32769, 15)])
 def test_select_keys_every_cluster_width(T, n_kv, mode):
