@@ -204,7 +204,6 @@ cudaError_t launch_attn_f32(const DevParams& P, const float* q, const float* k, 
 
 // Generation phase (chunk of one query): matrix-vector scoring and a gather attention kernel.
 bool decode_path_applies(const DevParams& P);
-bool decode_attn_fits(const DevParams& P, bool with_list);
 cudaError_t launch_score_keys_gemv(const DevParams& P, int dtype, const void* qbar, const void* k, float* scores,
                                    cudaStream_t st, bool chained);
 cudaError_t launch_decode_attn(const DevParams& P, int dtype, const void* q, const void* k, const void* v,

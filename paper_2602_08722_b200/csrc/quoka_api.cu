@@ -181,7 +181,7 @@ static quoka_status run_score_keys(const quoka_params* p, const DevParams& P, co
 static quoka_status run_attn(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                              const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                              bool after_selection = false) {
-  if (p->impl == QUOKA_IMPL_AUTO && P.chunk == 1 && decode_attn_fits(P, k_idx != nullptr)) {
+  if (p->impl == QUOKA_IMPL_AUTO && P.chunk == 1) {
     QUOKA_TRY_CUDA(launch_decode_attn(P, p->dtype, q, k, v, k_idx, k_cnt, out, lse, st, after_selection));
     return QUOKA_OK;
   }

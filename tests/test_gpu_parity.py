@@ -395,6 +395,28 @@ def test_select_keys_constant_and_narrow_rows(T, B):
     np.testing.assert_array_equal(gp.k_idx[0, :, :B].cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("d,dtype", [(128, "bf16"), (64, "bf16"), (128, "f32"), (64, "f32")])
+@pytest.mark.parametrize("n_q,n_kv,T,B", [
+    (4, 4, 1, 5),              # one cached row, a head per KV group
+    (4, 2, 64, 63),            # 64 keys with the query's own: exactly one trip of one CTA
+    (6, 2, 400, 127),          # groups of 3: a CTA of 4 heads with one unused; 128 keys
+    (10, 2, 3000, 600),        # groups of 5: two CTAs per group; 8 parts, several trips
+    (32, 2, 9000, 8300),       # groups of 16, a list beyond 8192 rows
+])
+def test_decode_attention_parts_and_groups(n_q, n_kv, T, B, d, dtype):
+    """The generation step's attention at the edges of its parts, trips and head groups, with a list and without."""
+    gp = problem(980 + T, batch=2, n_q=n_q, n_kv=n_kv, d=d, T=[T, max(1, T // 3)], C=1, dtype=dtype, n_retain=4, kv_budget=B)
+    gp.run_staged()
+    check_chain(gp)
+    api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, gp.lse, gp.ws)
+    torch.cuda.synchronize()
+    for s in range(2):
+        q, k, v, T_s = gp.oracle_inputs(s)
+        dense, lse = O.dense_chunk_attention(q, k, v, T_s)
+        check_attention(f64(gp.out[s]), dense, dtype)
+        assert np.abs(f64(gp.lse[s]) - lse).max() <= 2e-3
+
+
 @pytest.mark.parametrize("paged", [False, True])
 @pytest.mark.parametrize("T,C,B,n_q,n_kv,d,n_retain", [
     (63, 2, 40, 4, 2, 128, 1),          # fewer keys than a tile, two query rows
