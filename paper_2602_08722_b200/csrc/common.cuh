@@ -148,7 +148,8 @@ __device__ __forceinline__ float warp_sum(float x) {
 // returns once that grid has completed and its writes are visible; without the launch attribute it returns at
 // once).  A kernel lets the one after it start early with grid_launch_dependents(), which every CTA executes at
 // its start; the dependent grid is launched when all of them have, so it never holds resources that this
-// grid's own CTAs still need.
+// grid's own CTAs still need.  The first kernel of a call is launched this way too, whatever is before it on the stream;
+// it waits before anything else and lets the second one start only after that.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -186,7 +187,8 @@ inline cudaError_t launch_kernel(const char* name, void (*kernel)(KArgs...), dim
 
 // ---- launch functions implemented in the .cu files (host side) -------------------------------
 // `chained`: the kernel before it on the stream is the one of the same fused call whose output it reads (see above).
-cudaError_t launch_rank_queries(const DevParams& P, int dtype, const void* q, int32_t* q_idx, cudaStream_t st);
+cudaError_t launch_rank_queries(const DevParams& P, int dtype, const void* q, int32_t* q_idx, cudaStream_t st,
+                                bool chained = false);
 cudaError_t launch_aggregate_queries(const DevParams& P, int dtype, const void* q, int32_t* q_idx, void* qbar,
                                      cudaStream_t st, bool chained = false);
 cudaError_t launch_score_keys_simt(const DevParams& P, int dtype, const void* qbar, const void* k, float* scores,
@@ -204,13 +206,14 @@ cudaError_t launch_attn_f32(const DevParams& P, const float* q, const float* k, 
 
 // Generation phase (chunk of one query): matrix-vector scoring and a gather attention kernel.
 bool decode_path_applies(const DevParams& P);
-cudaError_t launch_score_keys_gemv(const DevParams& P, int dtype, const void* qbar, const void* k, float* scores,
-                                   cudaStream_t st, bool chained);
+// (q != nullptr: Q-bar is formed from the queries in the kernel, `qbar` is not read)
+cudaError_t launch_score_keys_gemv(const DevParams& P, int dtype, const void* q, const void* qbar, const void* k,
+                                   float* scores, cudaStream_t st, bool chained);
 cudaError_t launch_decode_attn(const DevParams& P, int dtype, const void* q, const void* k, const void* v,
                                const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                                bool chained);
 cudaError_t launch_append_kv(const DevParams& P, int dtype, const void* k_new, const void* v_new, void* k_cache,
-                             void* v_cache, cudaStream_t st);
+                             void* v_cache, float* k_inv_norm, cudaStream_t st);
 
 // Host checks shared by the fused entry points (everything but the workspace); nothing is enqueued before they pass.
 quoka_status check_prefill_args(const quoka_params* p, const void* q, const void* k_cache, const void* v_cache,

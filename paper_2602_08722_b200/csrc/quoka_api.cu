@@ -153,10 +153,11 @@ static bool use_tensor(const quoka_params* p) {
     if (e_ != cudaSuccess) return QUOKA_ERR_CUDA;     \
   } while (0)
 
+// early: launched before what is before it on the stream has completed (the first kernel waits for that itself)
 static quoka_status run_select_queries(const quoka_params* p, const DevParams& P, const void* q, int32_t* q_idx,
-                                       void* qbar, cudaStream_t st) {
-  QUOKA_TRY_CUDA(launch_rank_queries(P, p->dtype, q, q_idx, st));
-  QUOKA_TRY_CUDA(launch_aggregate_queries(P, p->dtype, q, q_idx, qbar, st, /*chained=*/true));
+                                       void* qbar, cudaStream_t st, bool early = false) {
+  QUOKA_TRY_CUDA(launch_rank_queries(P, p->dtype, q, q_idx, st, early));
+  QUOKA_TRY_CUDA(launch_aggregate_queries(P, p->dtype, q, q_idx, qbar, st, early || P.chunk > P.n_retain));
   return QUOKA_OK;
 }
 
@@ -165,7 +166,7 @@ static quoka_status run_score_keys(const quoka_params* p, const DevParams& P, co
                                    float* scores, cudaStream_t st, bool chained = false) {
   if (p->max_ctx_len == 0) return QUOKA_OK;
   if (p->impl == QUOKA_IMPL_AUTO && decode_path_applies(P)) {       // one query: a matrix-vector product
-    QUOKA_TRY_CUDA(launch_score_keys_gemv(P, p->dtype, qbar, k, scores, st, chained));
+    QUOKA_TRY_CUDA(launch_score_keys_gemv(P, p->dtype, nullptr, qbar, k, scores, st, chained));
     return QUOKA_OK;
   }
   if (use_tensor(p) && score_keys_tc_supported(p)) return launch_score_keys_tc(p, P, qbar, k, scores, st, chained);
@@ -243,8 +244,12 @@ quoka_status prefill_chunk_impl(const quoka_params* p, const void* q, const void
   // kernel and the attention kernel on the stream
   if (w.attn_counters) QUOKA_TRY_CUDA(cudaMemsetAsync(w.attn_counters, 0, attn_split_counter_bytes(p), cs));
   if (p->max_ctx_len > 0) {
-    if ((st = run_select_queries(p, P, q, w.q_idx, w.qbar, cs)) != QUOKA_OK) return st;
-    if ((st = run_score_keys(p, P, w.qbar, k_cache, w.scores, cs, /*chained=*/true)) != QUOKA_OK) return st;
+    if (p->impl == QUOKA_IMPL_AUTO && decode_path_applies(P)) {       // one query: the scoring kernel forms Q-bar itself
+      QUOKA_TRY_CUDA(launch_score_keys_gemv(P, p->dtype, q, nullptr, k_cache, w.scores, cs, /*chained=*/true));
+    } else {
+      if ((st = run_select_queries(p, P, q, w.q_idx, w.qbar, cs, /*early=*/true)) != QUOKA_OK) return st;
+      if ((st = run_score_keys(p, P, w.qbar, k_cache, w.scores, cs, /*chained=*/true)) != QUOKA_OK) return st;
+    }
   }
   // with an empty cache the selection kernel only writes k_cnt = 0 and the -1 padding
   QUOKA_TRY_CUDA(launch_select_keys(P, w.scores, k_idx, k_cnt, cs, /*chained=*/p->max_ctx_len > 0));
@@ -440,8 +445,7 @@ quoka_status quoka_append_kv(const quoka_params* p, const void* k_new, const voi
   if ((st = check_ws(p, ws, ws_bytes)) != QUOKA_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   const DevParams P = make_dev(p, ws);
-  QUOKA_TRY_CUDA(launch_append_kv(P, p->dtype, k_new, v_new, k_cache, v_cache, cs));
-  if (k_inv_norm) QUOKA_TRY_CUDA(launch_key_norms(P, p->dtype, k_cache, k_inv_norm, 0, cs));
+  QUOKA_TRY_CUDA(launch_append_kv(P, p->dtype, k_new, v_new, k_cache, v_cache, k_inv_norm, cs));
   return QUOKA_OK;
 }
 

@@ -19,6 +19,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "qbar.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -55,6 +56,9 @@ template <typename T, int D, int CL>
 __global__ void __launch_bounds__(kRankThreads, 2) rank_queries_kernel(DevParams P, const T* __restrict__ q,
                                                                      int32_t* __restrict__ q_idx, int rpc, int n_sort,
                                                                      int staged, int m_peer) {
+  // The first kernel of a fused call is launched early as well (its launch runs under the tail of whatever is before it on
+  // the stream); nothing is read or written, and no later kernel of the call starts, before that has completed.
+  grid_dependency_wait();
   grid_launch_dependents();                 // the aggregation kernel may become resident; it waits for this grid itself
   constexpr int LG = D / 8;                 // lanes per row, 8 elements each
   constexpr int RPI = kRankThreads / LG;    // rows per iteration
@@ -307,11 +311,12 @@ template <typename T, int D>
 __global__ void __launch_bounds__(256) aggregate_queries_kernel(DevParams P, const T* __restrict__ q,
                                                                  int32_t* __restrict__ q_idx,
                                                                  T* __restrict__ qbar) {
-  grid_launch_dependents();
-  grid_dependency_wait();                   // the ranks come from the kernel before
   // a chunk no longer than the number of retained queries keeps every query, in position order (Alg. 1's `if`):
   // no ranking kernel runs then, and this kernel writes the identity ranks itself
   const bool identity = P.chunk <= P.n_retain;
+  if (!identity) grid_launch_dependents();
+  grid_dependency_wait();                   // the ranks come from the kernel before
+  if (identity) grid_launch_dependents();   // the call's first kernel: nothing of it starts before the inputs are there
   constexpr int NE = D / 32;
   const int N = P.n_sel;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -322,53 +327,17 @@ __global__ void __launch_bounds__(256) aggregate_queries_kernel(DevParams P, con
   const int kv = (int)((warp / N) % P.n_kv);
   const int s = (int)(warp / ((int64_t)N * P.n_kv));
   float acc[NE];
-#pragma unroll
-  for (int i = 0; i < NE; ++i) acc[i] = 0.f;
-  for (int g0 = 0; g0 < P.group; g0 += 32) {
-    // the group's ranks in one load, then the rows four at a time so their loads overlap
-    const int gl = g0 + lane;
-    int r_lane = j;
-    if (gl < P.group) {
-      int32_t* slot = q_idx + ((int64_t)s * P.n_q + kv * P.group + gl) * N + j;
-      if (identity) *slot = j; else r_lane = __ldcg(slot);
-    }
-    const int g_end = min(32, P.group - g0);
-    for (int g4 = 0; g4 < g_end; g4 += 4) {
-      float x[4][NE];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int g = g4 + u;
-        const int r = __shfl_sync(0xFFFFFFFFu, r_lane, g & 31);
-        if (g < g_end) {
-          const int h = kv * P.group + g0 + g;
-          load_vec<T, NE>(q + (int64_t)s * P.q_sb + (int64_t)h * P.q_sh + (int64_t)r * P.q_st + lane * NE, x[u]);
-        } else {
-#pragma unroll
-          for (int i = 0; i < NE; ++i) x[u][i] = 0.f;
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        float nn = 0.f;
-#pragma unroll
-        for (int i = 0; i < NE; ++i) nn += x[u][i] * x[u][i];
-        nn = warp_sum(nn);
-        const float norm = P.score_dot ? 1.f : fmaxf(sqrtf(nn), kNormEps);
-        if (g4 + u < g_end) {
-#pragma unroll
-          for (int i = 0; i < NE; ++i) acc[i] += x[u][i] / norm;
-        }
-      }
-    }
-  }
-  const float inv_g = 1.f / (float)P.group;
-#pragma unroll
-  for (int i = 0; i < NE; ++i) acc[i] *= inv_g;
+  mean_normalised_query<T, NE>(P, q, s, kv, lane, [&](int g) {
+    int32_t* slot = q_idx + ((int64_t)s * P.n_q + kv * P.group + g) * N + j;
+    if (!identity) return (int)__ldcg(slot);
+    *slot = j;
+    return j;
+  }, acc);
   store_vec<T, NE>(qbar + warp * D + lane * NE, acc);
 }
 
 template <typename T, int D, int CL>
-static cudaError_t launch_rank_t(const DevParams& P, const void* q, int32_t* q_idx, cudaStream_t st) {
+static cudaError_t launch_rank_t(const DevParams& P, const void* q, int32_t* q_idx, cudaStream_t st, bool chained) {
   constexpr int LG = D / 8, RPI = kRankThreads / LG;
   int rpc = (P.chunk + CL - 1) / CL;
   int n_sort = 32;
@@ -381,24 +350,24 @@ static cudaError_t launch_rank_t(const DevParams& P, const void* q, int32_t* q_i
   const size_t smem = fixed + (staged ? row_bytes : 0);
   cudaError_t e = cudaFuncSetAttribute(rank_queries_kernel<T, D, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_kernel("rank_queries", rank_queries_kernel<T, D, CL>, dim3(P.batch * P.n_q * CL), dim3(kRankThreads), smem, st, CL, false, P,
+  return launch_kernel("rank_queries", rank_queries_kernel<T, D, CL>, dim3(P.batch * P.n_q * CL), dim3(kRankThreads), smem, st, CL, chained, P,
                        (const T*)q, q_idx, rpc, n_sort, staged, m_peer);
 }
 
 // A cluster per (sequence, head), sized so that a CTA's slice is about 256 rows: shorter slices only multiply the
 // per-CTA costs (four cluster barriers, the sort, the merge).
 template <typename T, int D>
-static cudaError_t launch_rank_d(const DevParams& P, const void* q, int32_t* q_idx, cudaStream_t st) {
-  if (P.chunk <= 512) return launch_rank_t<T, D, 2>(P, q, q_idx, st);
-  if (P.chunk <= 1024) return launch_rank_t<T, D, 4>(P, q, q_idx, st);
-  return launch_rank_t<T, D, kRankCluster>(P, q, q_idx, st);
+static cudaError_t launch_rank_d(const DevParams& P, const void* q, int32_t* q_idx, cudaStream_t st, bool chained) {
+  if (P.chunk <= 512) return launch_rank_t<T, D, 2>(P, q, q_idx, st, chained);
+  if (P.chunk <= 1024) return launch_rank_t<T, D, 4>(P, q, q_idx, st, chained);
+  return launch_rank_t<T, D, kRankCluster>(P, q, q_idx, st, chained);
 }
 
-cudaError_t launch_rank_queries(const DevParams& P, int dtype, const void* q, int32_t* q_idx, cudaStream_t st) {
+cudaError_t launch_rank_queries(const DevParams& P, int dtype, const void* q, int32_t* q_idx, cudaStream_t st, bool chained) {
   if (P.chunk <= P.n_retain) return cudaSuccess;      // every query is kept: the aggregation kernel writes the ranks
   cudaError_t e;
-  if (dtype == QUOKA_BF16) e = P.d == 128 ? launch_rank_d<__nv_bfloat16, 128>(P, q, q_idx, st) : launch_rank_d<__nv_bfloat16, 64>(P, q, q_idx, st);
-  else e = P.d == 128 ? launch_rank_d<float, 128>(P, q, q_idx, st) : launch_rank_d<float, 64>(P, q, q_idx, st);
+  if (dtype == QUOKA_BF16) e = P.d == 128 ? launch_rank_d<__nv_bfloat16, 128>(P, q, q_idx, st, chained) : launch_rank_d<__nv_bfloat16, 64>(P, q, q_idx, st, chained);
+  else e = P.d == 128 ? launch_rank_d<float, 128>(P, q, q_idx, st, chained) : launch_rank_d<float, 64>(P, q, q_idx, st, chained);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -417,6 +417,23 @@ def test_decode_attention_parts_and_groups(n_q, n_kv, T, B, d, dtype):
         assert np.abs(f64(gp.lse[s]) - lse).max() <= 2e-3
 
 
+@pytest.mark.parametrize("cached_norms,paged", [(False, False), (True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("d,dtype,group", [(128, "bf16", 4), (64, "bf16", 3), (128, "f32", 1), (64, "f32", 40)])
+@pytest.mark.parametrize("T", [[1, 8, 15, 17], [0, 31, 0, 33], [3000, 63, 0, 1], [65] * 35])
+def test_decode_scoring_units(T, d, dtype, group, cached_norms, paged):
+    """The generation step's scoring kernel: lengths around its units of 8 to 32 rows, empty sequences between others,
+    more than 32 sequences; and the fused call, which forms Q-bar inside it, against the staged calls."""
+    gp = problem(990 + d, batch=len(T), n_q=2 * group, n_kv=2, d=d, T=T, C=1, dtype=dtype, n_retain=4, kv_budget=12,
+                 paged=paged, cached_norms=cached_norms)
+    gp.run_staged()
+    check_chain(gp)
+    want_out, want_idx = gp.out.clone(), gp.k_idx.clone()
+    gp.out.zero_()
+    api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, gp.k_idx, gp.k_cnt, gp.ws)
+    torch.cuda.synchronize()
+    assert torch.equal(gp.out, want_out) and torch.equal(gp.k_idx, want_idx)
+
+
 @pytest.mark.parametrize("paged", [False, True])
 @pytest.mark.parametrize("T,C,B,n_q,n_kv,d,n_retain", [
     (63, 2, 40, 4, 2, 128, 1),          # fewer keys than a tile, two query rows
