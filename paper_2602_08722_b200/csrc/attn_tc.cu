@@ -52,8 +52,8 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WaitCtx wc{&abort_flag, P.status};
   // grid = (heads, row blocks, batch): heads vary fastest so the CTAs resident together share a KV head's
-  // rows in L2, and the row blocks run heaviest (most causal tiles) first, lightest last
-  const int s = blockIdx.z, h = blockIdx.x, kv = h / P.group;
+  // rows in L2, and the row blocks run heaviest (most causal tiles) first, lightest last, the sequences longest first
+  const int s = longest_first(P, blockIdx.z), h = blockIdx.x, kv = h / P.group;
   // (SPLIT: grid.y = row blocks times the parts a row block's key tiles are cut into)
   const int n_parts = SPLIT ? P.attn_parts : 1;
   const int n_rb = gridDim.y / n_parts;
@@ -388,6 +388,8 @@ int attn_split_parts_for_launch(const quoka_params* p, const DevParams& P, bool 
   if (!P.attn_partials) return 1;
   return attn_split_parts(p, ((sparse ? P.budget_cap : P.max_ctx) + kKeyTile - 1) / kKeyTile + 1);
 }
+
+bool attn_below_a_wave(const quoka_params* p) { return attn_jobs(p) < device_sm_count(); }
 
 bool attn_tc_supported(const quoka_params* p) {
   if (p->dtype != QUOKA_BF16) return false;

@@ -58,7 +58,7 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WaitCtx wc{&abort_flag, P.status};
   const uint32_t rank = cluster_cta_rank();                   // 0: issues the MMAs; the pair is heads (2j, 2j + 1)
-  const int s = blockIdx.z, h = blockIdx.x, kv = h / P.group;
+  const int s = longest_first(P, blockIdx.z), h = blockIdx.x, kv = h / P.group;
   // grid.y = row blocks (heaviest first), times the parts a row block's key tiles are cut into (SPLIT)
   const int n_parts = SPLIT ? P.attn_parts : 1;
   const int n_rb = gridDim.y / n_parts;

@@ -37,6 +37,7 @@ struct DevParams {
   // split attention (small grids): room for the parts' partial results and their arrival counters, or null
   float* attn_partials;
   int32_t* attn_counters;
+  int n_attn_counters;
   int attn_parts;   // parts per row block of the launch at hand (set by the launcher), 1 = no split
 };
 
@@ -189,6 +190,7 @@ inline cudaError_t launch_kernel(const char* name, void (*kernel)(KArgs...), dim
 // `chained`: the kernel before it on the stream is the one of the same fused call whose output it reads (see above).
 cudaError_t launch_rank_queries(const DevParams& P, int dtype, const void* q, int32_t* q_idx, cudaStream_t st,
                                 bool chained = false);
+// (with split-attention scratch in P it also clears the arrival counters, for the attention kernel of the same call)
 cudaError_t launch_aggregate_queries(const DevParams& P, int dtype, const void* q, int32_t* q_idx, void* qbar,
                                      cudaStream_t st, bool chained = false);
 cudaError_t launch_score_keys_simt(const DevParams& P, int dtype, const void* qbar, const void* k, float* scores,

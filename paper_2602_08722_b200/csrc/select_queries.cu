@@ -317,6 +317,10 @@ __global__ void __launch_bounds__(256) aggregate_queries_kernel(DevParams P, con
   if (!identity) grid_launch_dependents();
   grid_dependency_wait();                   // the ranks come from the kernel before
   if (identity) grid_launch_dependents();   // the call's first kernel: nothing of it starts before the inputs are there
+  if (P.attn_counters) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    for (int e = i; e < P.n_attn_counters; e += step) P.attn_counters[e] = 0;
+  }
   constexpr int NE = D / 32;
   const int N = P.n_sel;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;

@@ -11,6 +11,8 @@ quoka_status launch_score_keys_tc(const quoka_params* p, const DevParams& P, con
                                   float* scores, cudaStream_t st, bool chained);
 
 bool attn_tc_supported(const quoka_params* p);
+// Whether the attention grid (256 chunk rows of a head per CTA) has fewer CTAs than the GPU has SMs.
+bool attn_below_a_wave(const quoka_params* p);
 quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                             const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                             bool after_selection);
