@@ -120,10 +120,12 @@ quoka_status quoka_kv_budget_cap(const quoka_params* p, int32_t* cap);
  * once after allocating; the rest is scratch whose contents mean nothing between
  * calls.  Two calls that share a workspace must not overlap on the GPU.
  * For problems whose attention grid is smaller than the GPU (few heads, a short
- * chunk) the size includes room for the partial results of the split attention
- * kernel (each row block's keys are cut into up to 8 parts, one CTA each, and added
- * up in part order: results are reproducible from run to run, and differ from the
- * unsplit kernel's in the last bits only). */
+ * chunk) or leaves much of its last wave empty, the size includes room for the
+ * partial results of the split attention kernel, at most 128 MiB of them on large
+ * grids (the keys of the lightest row blocks, or of all, are cut into up to 8 parts,
+ * one CTA each, and added up in part order: results are reproducible from run to
+ * run, and differ from the unsplit kernel's in the last bits only).
+ */
 quoka_status quoka_workspace_size(const quoka_params* p, size_t* bytes);
 
 /* Alg. 1, "Query Sub-selection", then the normalisation and the mean over the G

@@ -56,8 +56,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
   const int s = longest_first(P, blockIdx.z), h = blockIdx.x, kv = h / P.group;
   // (SPLIT: grid.y = row blocks times the parts a row block's key tiles are cut into)
   const int n_parts = SPLIT ? P.attn_parts : 1;
-  const int n_rb = gridDim.y / n_parts;
-  const int rb = n_rb - 1 - blockIdx.y / n_parts;
+  const int rb = (SPLIT ? P.attn_split_rb : P.attn_row_blocks) - 1 - blockIdx.y / n_parts;
   const int r0 = rb * 2 * kQTile;
   AttnGeom g = make_geom<SPARSE>(P, s, r0);
   // SPLIT: this CTA walks the tiles [t_lo, t_hi) of the row block's sequence only and leaves, per row, a partial
@@ -65,7 +64,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
   // nothing of the walk starts before the selection has ended.
   int t_lo = 0;
   if (SPLIT) {
-    if (SPARSE) resolve(g, k_cnt, s);
+    if (SPARSE) { if (P.attn_after_whole) learn_count(g, k_cnt, s); else resolve(g, k_cnt, s); }
     const int part = blockIdx.y % n_parts;
     t_lo = (int)(((long long)part * g.n_known) / n_parts);
     g.n_known = (int)(((long long)(part + 1) * g.n_known) / n_parts);
@@ -87,6 +86,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (!SPARSE && !SPLIT) grid_launch_dependents();
 
   if (warp < 8) {
     // ================================================================== softmax + epilogue
@@ -125,7 +125,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     } else {
       const bool have = ok && active_x && mbar_wait(&o_full[x], 0, wc);
       if (have) tc_fence_after();
-      attn_split_epilogue<D>(P, (s * P.n_q + h) * n_rb + rb, blockIdx.y % n_parts, n_parts, x, quarter, lane, row_in_tile, row, have,
+      attn_split_epilogue<D>(P, (s * P.n_q + h) * P.attn_split_rb + rb, blockIdx.y % n_parts, n_parts, x, quarter, lane, row_in_tile, row, have,
                              o_addr, m_run, l_run, s, h, out, lse);
     }
   } else if (warp < 8 + kLoaderWarps) {
@@ -325,7 +325,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
         mma_commit(&kv_empty[k_slot]);
       }
       for (int t = t_lo; ok; ++t) {
-        if (t + 1 == g.n_known && !g.resolved) resolve(g, k_cnt, s);
+        if (t + 1 == g.n_known && !g.resolved) { resolve(g, k_cnt, s); grid_launch_dependents(); }
         const bool more = t + 1 < g.n_known;
         v_slot = acquire();
         if (ok && more) k_slot = acquire();
@@ -348,6 +348,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
       }
     }
   }
+  if (SPLIT && attn_last_cta()) grid_dependency_wait();       // this grid's end is the whole row blocks' end too
   tc_fence_before();
   __syncthreads();
   if (warp == kMmaWarp) tmem_dealloc(tmem_base, 512);
@@ -358,35 +359,100 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
 // every CTA walks its whole key sequence; cutting each row block's tiles into parts, one CTA each, fills it.
 // The number of parts minimises  waves(parts) * (tiles / parts + 6):  a part costs about six tiles' time of
 // start-up, partial results and merge (the model fits the measured times of 1 to 5 parts on grids of 32 to 288 CTAs
-// within 3 %), parts keep at least six tiles, and a split has to promise 3 % to be taken.  Grids of a wave or more
-// stay whole: their sparse jobs are too short to gain, and the partial results of long dense ones would take
-// hundreds of megabytes.
-static long long attn_jobs(const quoka_params* p) {
-  return (long long)p->n_q_heads * ((p->chunk_len + 2 * kQTile - 1) / (2 * kQTile)) * p->batch;
-}
-int attn_split_parts(const quoka_params* p, int tiles) {
-  if (p->dtype != QUOKA_BF16) return 1;
-  const long long jobs = attn_jobs(p), sms = device_sm_count();
-  if (sms <= 0 || jobs >= sms) return 1;
-  const double t = tiles + (p->chunk_len + 2 * kQTile - 1) / (2 * kQTile);   // plus the chunk's own tiles, on average
-  int best = 1;
-  double best_cost = t;
-  for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
-    const long long waves = (jobs * parts + sms - 1) / sms;
-    const double cost = (double)waves * (t / parts + 6.0);
-    if (cost < 0.97 * best_cost) { best = parts; best_cost = cost; }
+// within 3 %), parts keep at least six tiles, and a split has to promise 3 % to be taken.
+// A grid of q full waves and a rest has its lightest row blocks, as many as the rest, cut instead: the whole ones then
+// end after about q waves and the parts level the end.  The model is the total work over the SMs plus a third of a part
+// for the uneven end, against q + 1 waves of average jobs; list-scheduling simulations agree with it within 4 %.  Dense
+// calls take 3 % promised, sparse ones 7 % and equal lengths (their parts run a quarter slower per tile than whole row
+// blocks, and a batch's budgets differ): 32 heads, without / with parts: 1536 queries at 64K, a quarter listed 508 / 420 us,
+// 4096 at 128K 1039 / 990, 3072 at 32K, half listed 789 / 746; 40 heads, 1536 at 32K, promised 4 %: 290 / 309; dense 1536 at
+// 32K 920 / 692, 2048 at 32K 942 / 908, 4096 at 128K 7412 / 6689.
+// Partial results above 128 MB are not written: such jobs have waves enough.
+static long long attn_row_blocks(const quoka_params* p) { return (p->chunk_len + 2 * kQTile - 1) / (2 * kQTile); }
+static long long attn_jobs(const quoka_params* p) { return p->n_q_heads * attn_row_blocks(p) * p->batch; }
+static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
+  constexpr double kPartCost = 6.0;
+  AttnPlan plan;
+  if (p->dtype != QUOKA_BF16 || p->impl == QUOKA_IMPL_SIMT || p->chunk_len <= 1) return plan;
+  const long long n_rb = attn_row_blocks(p), per_rb = (long long)p->n_q_heads * p->batch, jobs = per_rb * n_rb;
+  const long long sms = device_sm_count();
+  if (sms <= 0) return plan;
+  if (jobs < sms) {
+    const double t = tiles + n_rb;                                          // plus the chunk's own tiles, on average
+    double best = t;
+    for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
+      const long long waves = (jobs * parts + sms - 1) / sms;
+      const double cost = (double)waves * (t / parts + kPartCost);
+      if (cost < 0.97 * best) { plan.split_rb = (int)n_rb; plan.parts = parts; best = cost; }
+    }
+    return plan;
   }
-  return best;
+  const long long q = jobs / sms, rest = jobs % sms;
+  if (rest == 0 || (sparse && p->batch > 1)) return plan;
+  const long long split = (rest + per_rb - 1) / per_rb;                      // row blocks to cut; block r has 2 r + 2 own tiles
+  const double t_all = tiles + 2 + n_rb, t_whole = tiles + 2 + split + n_rb, t_split = tiles + 2 + split;
+  double best = (sparse ? 0.93 : 0.97) * (double)(q + 1) * t_all;
+  for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
+    const double t_part = t_split / parts + kPartCost;
+    const double cost = ((double)(jobs - split * per_rb) * t_whole + (double)(split * per_rb * parts) * t_part) / (double)sms + 0.3 * t_part;
+    AttnPlan cand;
+    cand.split_rb = (int)split; cand.parts = parts;
+    if (cost < best && attn_split_partial_bytes(p, cand) <= ((size_t)128 << 20)) { best = cost; plan = cand; }
+  }
+  return plan;
 }
-size_t attn_split_partial_bytes(const quoka_params* p, int parts) {
-  return parts <= 1 ? 0 : (size_t)attn_jobs(p) * parts * 2 * kSplitTileFloats * sizeof(float);
+AttnPlan attn_plan_sparse(const quoka_params* p, int budget_cap) { return attn_plan(p, (budget_cap + kKeyTile - 1) / kKeyTile + 1, true); }
+AttnPlan attn_plan_dense(const quoka_params* p) { return attn_plan(p, (p->max_ctx_len + kKeyTile - 1) / kKeyTile + 1, false); }
+static size_t attn_split_jobs(const quoka_params* p, const AttnPlan& plan) { return (size_t)p->n_q_heads * p->batch * plan.split_rb; }
+size_t attn_split_partial_bytes(const quoka_params* p, const AttnPlan& plan) {
+  return attn_split_jobs(p, plan) * plan.parts * 2 * kSplitTileFloats * sizeof(float);
 }
-size_t attn_split_counter_bytes(const quoka_params* p) { return (size_t)attn_jobs(p) * 8 * sizeof(int32_t); }
-// Parts of the launch at hand: `tiles` = key tiles of the longest row block the call can meet (the list or the
-// cache, plus the chunk's own).  Without room for the partial results (the no-allocation entry point) nothing splits.
-int attn_split_parts_for_launch(const quoka_params* p, const DevParams& P, bool sparse) {
-  if (!P.attn_partials) return 1;
-  return attn_split_parts(p, ((sparse ? P.budget_cap : P.max_ctx) + kKeyTile - 1) / kKeyTile + 1);
+size_t attn_split_counter_bytes(const quoka_params* p, const AttnPlan& plan) { return attn_split_jobs(p, plan) * 8 * sizeof(int32_t); }
+
+// The launches of an attention call: the whole row blocks, then the ones in parts.
+//
+// Programmatic stream serialisation, (1) inside the fused call: the first launch may start while the kernel before it on
+// the stream (the key selection, which signals early and writes none of this kernel's other inputs) still runs; it touches
+// the selection's outputs only after its own griddepcontrol.wait.  A stand-alone call keeps the ordinary stream order:
+// whatever ran before it may have written q, k or v.  (2) The parts always: their CTAs take the SMs that the whole row
+// blocks' last wave leaves idle.  The whole row blocks let them start once every CTA has begun (dense) or has learnt the
+// list length (sparse: the selection is complete by then, so the parts need not wait for it), and the parts' last CTA
+// waits for the whole row blocks before it ends.
+quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const AttnPlan& plan, AttnKernel (*pick)(bool, bool),
+                              const char* name, int cluster, size_t smem, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
+                              const CUtensorMap& tm_v, const void* k, const void* v, const int32_t* k_idx, const int32_t* k_cnt,
+                              void* out, float* lse, cudaStream_t st, bool after_selection) {
+  const bool sparse = k_idx != nullptr, split = plan.split_rb > 0 && P.attn_partials;
+  DevParams PP = P;
+  PP.attn_row_blocks = (int)attn_row_blocks(p);
+  PP.attn_split_rb = split ? plan.split_rb : 0;
+  PP.attn_parts = split ? plan.parts : 1;
+  const int whole = PP.attn_row_blocks - PP.attn_split_rb;
+  PP.attn_after_whole = whole > 0 ? 1 : 0;
+  if (split && !after_selection &&          // (the fused call clears the counters in an earlier kernel)
+      cudaMemsetAsync(P.attn_counters, 0, attn_split_counter_bytes(p, plan), st) != cudaSuccess)
+    return QUOKA_ERR_CUDA;
+  for (int parts = whole > 0 ? 0 : 1; parts <= (split ? 1 : 0); ++parts) {
+    AttnKernel kernel = pick(sparse, parts != 0);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return QUOKA_ERR_CUDA;
+    const bool early = parts && whole > 0 ? true : sparse && after_selection;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(P.n_q, parts ? PP.attn_split_rb * PP.attn_parts : whole, P.batch);   // (pairs: n_q is even)
+    cfg.blockDim = dim3(kAttnThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = early ? 1 : 0;
+    log_launch(name, cfg.gridDim, cfg.blockDim, smem, cluster, early);
+    if (cudaLaunchKernelEx(&cfg, kernel, PP, tm_q, tm_k, tm_v, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, k_idx, k_cnt,
+                           (__nv_bfloat16*)out, lse) != cudaSuccess)
+      return QUOKA_ERR_CUDA;
+    count_launch();
+  }
+  return cudaGetLastError() == cudaSuccess ? QUOKA_OK : QUOKA_ERR_CUDA;
 }
 
 bool attn_below_a_wave(const quoka_params* p) { return attn_jobs(p) < device_sm_count(); }
@@ -399,10 +465,16 @@ bool attn_tc_supported(const quoka_params* p) {
   return true;
 }
 
+template <int HALVES>
+static AttnKernel pick_attn_tc(bool sparse, bool parts) {
+  if (parts) return sparse ? attn_tc_kernel<HALVES, true, true> : attn_tc_kernel<HALVES, false, true>;
+  return sparse ? attn_tc_kernel<HALVES, true, false> : attn_tc_kernel<HALVES, false, false>;
+}
+
 quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                             const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
-                            bool after_selection) {
-  if (attn_tc_pair_applies(P)) return launch_attn_tc_pair(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection);
+                            bool after_selection, const AttnPlan& plan) {
+  if (attn_tc_pair_applies(P)) return launch_attn_tc_pair(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection, plan);
   CUtensorMap tm_q;
   {
     const uint64_t dims[4] = {(uint64_t)P.d, (uint64_t)P.chunk, (uint64_t)P.n_q, (uint64_t)P.batch};
@@ -415,49 +487,7 @@ quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P, const voi
   const int halves = P.d / 64;
   const size_t tile = (size_t)halves * 128 * 128;
   const size_t smem = 1024 + (2 + kSlots) * tile + 512;
-  const bool sparse = k_idx != nullptr;
-  const int parts = attn_split_parts_for_launch(p, P, sparse);
-  DevParams PP = P;
-  PP.attn_parts = parts;
-  dim3 grid(P.n_q, (P.chunk + 2 * kQTile - 1) / (2 * kQTile) * parts, P.batch);
-  if (parts > 1 && !after_selection &&          // (the fused call clears the counters before its first kernel)
-      cudaMemsetAsync(P.attn_counters, 0, attn_split_counter_bytes(p), st) != cudaSuccess)
-    return QUOKA_ERR_CUDA;
-  log_launch(sparse ? "attn_tc<sparse>" : "attn_tc<dense>", grid, dim3(kAttnThreads), smem, 1, sparse && after_selection);
-  cudaError_t e = cudaSuccess;
-  // Inside the fused call the sparse kernel is launched with programmatic stream serialisation: it may start
-  // while the kernel before it on the stream (the key selection, which signals early and writes none of this
-  // kernel's other inputs) still runs; it touches the selection's outputs only after its own
-  // griddepcontrol.wait.  A stand-alone call keeps the ordinary stream order: whatever ran before it may have
-  // written q, k or v.
-#define QUOKA_ATTN_TC(H, S, X)                                                                                   \
-  do {                                                                                                           \
-    e = cudaFuncSetAttribute(attn_tc_kernel<H, S, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   \
-    if (e != cudaSuccess) return QUOKA_ERR_CUDA;                                                                 \
-    cudaLaunchConfig_t cfg = {};                                                                                 \
-    cfg.gridDim = grid;                                                                                          \
-    cfg.blockDim = dim3(kAttnThreads);                                                                           \
-    cfg.dynamicSmemBytes = smem;                                                                                 \
-    cfg.stream = st;                                                                                             \
-    cudaLaunchAttribute attr[1];                                                                                 \
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;                                             \
-    attr[0].val.programmaticStreamSerializationAllowed = 1;                                                      \
-    cfg.attrs = attr;                                                                                            \
-    cfg.numAttrs = ((S) && after_selection) ? 1 : 0;                                                                                \
-    e = cudaLaunchKernelEx(&cfg, attn_tc_kernel<H, S, X>, PP, tm_q, tm_k, tm_v, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, \
-                           k_idx, k_cnt, (__nv_bfloat16*)out, lse);                                              \
-    if (e != cudaSuccess) return QUOKA_ERR_CUDA;                                                                 \
-  } while (0)
-  if (parts > 1) {
-    if (halves == 2) { if (sparse) QUOKA_ATTN_TC(2, true, true); else QUOKA_ATTN_TC(2, false, true); }
-    else { if (sparse) QUOKA_ATTN_TC(1, true, true); else QUOKA_ATTN_TC(1, false, true); }
-  } else {
-    if (halves == 2) { if (sparse) QUOKA_ATTN_TC(2, true, false); else QUOKA_ATTN_TC(2, false, false); }
-    else { if (sparse) QUOKA_ATTN_TC(1, true, false); else QUOKA_ATTN_TC(1, false, false); }
-  }
-#undef QUOKA_ATTN_TC
-  count_launch();
-  return cudaGetLastError() == cudaSuccess ? QUOKA_OK : QUOKA_ERR_CUDA;
+  return launch_attn_plan(p, P, plan, halves == 2 ? pick_attn_tc<2> : pick_attn_tc<1>, "attn_tc", /*cluster=*/1, smem, tm_q, tm_k, tm_v, k, v, k_idx, k_cnt, out, lse, st, after_selection);
 }
 
 }  // namespace quoka

@@ -61,8 +61,7 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
   const int s = longest_first(P, blockIdx.z), h = blockIdx.x, kv = h / P.group;
   // grid.y = row blocks (heaviest first), times the parts a row block's key tiles are cut into (SPLIT)
   const int n_parts = SPLIT ? P.attn_parts : 1;
-  const int n_rb = gridDim.y / n_parts;
-  const int rb = n_rb - 1 - blockIdx.y / n_parts;
+  const int rb = (SPLIT ? P.attn_split_rb : P.attn_row_blocks) - 1 - blockIdx.y / n_parts;
   const int r0 = rb * 2 * kQTile;
   AttnGeom g = make_geom<SPARSE>(P, s, r0);
   // SPLIT: this CTA walks the tiles [t_lo, t_hi) of the row block's sequence only and leaves, per row, a partial
@@ -70,7 +69,7 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
   // length has to be known before the range is, so nothing of the walk starts before the selection has ended.
   int t_lo = 0;
   if (SPLIT) {
-    if (SPARSE) resolve(g, k_cnt, s);
+    if (SPARSE) { if (P.attn_after_whole) learn_count(g, k_cnt, s); else resolve(g, k_cnt, s); }
     const int part = blockIdx.y % n_parts;
     t_lo = (int)(((long long)part * g.n_known) / n_parts);
     g.n_known = (int)(((long long)(part + 1) * g.n_known) / n_parts);
@@ -97,6 +96,7 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
   cluster_sync_all();                                         // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  if (!SPARSE && !SPLIT) grid_launch_dependents();
 
   if (warp < 8) {
     // ================================================================== softmax + epilogue
@@ -137,7 +137,7 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
     } else {
       const bool have = ok && active_x && mbar_wait(&o_full[x], 0, wc);
       if (have) tc_fence_after();
-      attn_split_epilogue<D>(P, (s * P.n_q + h) * n_rb + rb, blockIdx.y % n_parts, n_parts, x, quarter, lane, row_in_tile, row, have,
+      attn_split_epilogue<D>(P, (s * P.n_q + h) * P.attn_split_rb + rb, blockIdx.y % n_parts, n_parts, x, quarter, lane, row_in_tile, row, have,
                              o_addr, m_run, l_run, s, h, out, lse);
     }
   } else if (warp < 8 + kPairLoaderWarps) {
@@ -293,6 +293,7 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
         if (tile == g.n_known) {
           if (g.resolved) break;
           resolve(g, k_cnt, s);
+          grid_launch_dependents();
           if (tile == g.n_known) break;
         }
 #pragma unroll 1
@@ -365,7 +366,7 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
           mma_pair_commit(&kv_empty[k_slot]);
         }
         for (int t = t_lo; ok; ++t) {
-          if (t + 1 == g.n_known && !g.resolved) resolve(g, k_cnt, s);
+          if (t + 1 == g.n_known && !g.resolved) { resolve(g, k_cnt, s); grid_launch_dependents(); }
           const bool more = t + 1 < g.n_known;
           v_slot = acquire();
           if (ok && more) k_slot = acquire();
@@ -389,6 +390,7 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
       }
     }
   }
+  if (SPLIT && attn_last_cta()) grid_dependency_wait();       // this grid's end is the whole row blocks' end too
   tc_fence_before();
   cluster_sync_all();                                         // the other CTA's MMAs no longer read this CTA
   if (warp == kMmaWarp) tmem_dealloc_pair(tmem_base, 512);
@@ -399,7 +401,7 @@ bool attn_tc_pair_applies(const DevParams& P) { return P.d == 128 && P.group % 2
 
 quoka_status launch_attn_tc_pair(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                                  const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
-                                 bool after_selection) {
+                                 bool after_selection, const AttnPlan& plan) {
   CUtensorMap tm_q;
   {
     const uint64_t dims[4] = {(uint64_t)P.d, (uint64_t)P.chunk, (uint64_t)P.n_q, (uint64_t)P.batch};
@@ -410,41 +412,11 @@ quoka_status launch_attn_tc_pair(const quoka_params* p, const DevParams& P, cons
   CUtensorMap tm_k, tm_v;
   if (!encode_kv_tensor_map(&tm_k, p, k, 64) || !encode_kv_tensor_map(&tm_v, p, v, 64)) return QUOKA_ERR_CUDA;
   const size_t smem = 1024 + 2 * kPairQTileBytes + (size_t)kPairSlots * kPairSlotBytes + 512;
-  const bool sparse = k_idx != nullptr;
-  const int parts = attn_split_parts_for_launch(p, P, sparse);
-  DevParams PP = P;
-  PP.attn_parts = parts;
-  dim3 grid(P.n_q, (P.chunk + 2 * kQTile - 1) / (2 * kQTile) * parts, P.batch);   // n_q is even: clusters of (2, 1, 1)
-  if (parts > 1 && !after_selection &&          // (the fused call clears the counters before its first kernel)
-      cudaMemsetAsync(P.attn_counters, 0, attn_split_counter_bytes(p), st) != cudaSuccess)
-    return QUOKA_ERR_CUDA;
-  log_launch(sparse ? "attn_tc_pair<sparse>" : "attn_tc_pair<dense>", grid, dim3(kAttnThreads), smem, 2,
-             sparse && after_selection);
-  cudaError_t e = cudaSuccess;
-  // Programmatic stream serialisation inside the fused call only, as for the one-CTA kernel.
-#define QUOKA_ATTN_PAIR(S, X)                                                                                      \
-  do {                                                                                                            \
-    e = cudaFuncSetAttribute(attn_tc_pair_kernel<S, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);  \
-    if (e != cudaSuccess) return QUOKA_ERR_CUDA;                                                                  \
-    cudaLaunchConfig_t cfg = {};                                                                                  \
-    cfg.gridDim = grid;                                                                                           \
-    cfg.blockDim = dim3(kAttnThreads);                                                                            \
-    cfg.dynamicSmemBytes = smem;                                                                                  \
-    cfg.stream = st;                                                                                              \
-    cudaLaunchAttribute attr[1];                                                                                  \
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;                                              \
-    attr[0].val.programmaticStreamSerializationAllowed = 1;                                                       \
-    cfg.attrs = attr;                                                                                             \
-    cfg.numAttrs = ((S) && after_selection) ? 1 : 0;                                                              \
-    e = cudaLaunchKernelEx(&cfg, attn_tc_pair_kernel<S, X>, PP, tm_q, tm_k, tm_v, (const __nv_bfloat16*)k,        \
-                           (const __nv_bfloat16*)v, k_idx, k_cnt, (__nv_bfloat16*)out, lse);                      \
-    if (e != cudaSuccess) return QUOKA_ERR_CUDA;                                                                  \
-  } while (0)
-  if (parts > 1) { if (sparse) QUOKA_ATTN_PAIR(true, true); else QUOKA_ATTN_PAIR(false, true); }
-  else { if (sparse) QUOKA_ATTN_PAIR(true, false); else QUOKA_ATTN_PAIR(false, false); }
-#undef QUOKA_ATTN_PAIR
-  count_launch();
-  return cudaGetLastError() == cudaSuccess ? QUOKA_OK : QUOKA_ERR_CUDA;
+  const auto pick = [](bool sparse, bool parts) -> AttnKernel {
+    if (parts) return sparse ? attn_tc_pair_kernel<true, true> : attn_tc_pair_kernel<false, true>;
+    return sparse ? attn_tc_pair_kernel<true, false> : attn_tc_pair_kernel<false, false>;
+  };
+  return launch_attn_plan(p, P, plan, pick, "attn_tc_pair", /*cluster=*/2, smem, tm_q, tm_k, tm_v, k, v, k_idx, k_cnt, out, lse, st, after_selection);
 }
 
 }  // namespace quoka

@@ -22,6 +22,14 @@ constexpr int kSlots = 5;
 // write of the whole accumulator row on the softmax -> PV chain) still ran often enough to cost 1-2 % of the kernel.
 constexpr float kRescaleThreshold = 32.0f;   // log2 units
 
+// Any of the tensor-core attention kernels.
+typedef void (*AttnKernel)(DevParams, const CUtensorMap, const CUtensorMap, const CUtensorMap, const __nv_bfloat16*,
+                           const __nv_bfloat16*, const int32_t*, const int32_t*, __nv_bfloat16*, float*);
+quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const AttnPlan& plan, AttnKernel (*pick)(bool, bool),
+                              const char* name, int cluster, size_t smem, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
+                              const CUtensorMap& tm_v, const void* k, const void* v, const int32_t* k_idx, const int32_t* k_cnt,
+                              void* out, float* lse, cudaStream_t st, bool after_selection);
+
 bool encode_kv_tensor_map(CUtensorMap* out, const quoka_params* p, const void* cache, uint32_t box_rows);
 
 __device__ __forceinline__ float ex2(float x) {
@@ -100,6 +108,16 @@ __device__ __forceinline__ void resolve(AttnGeom& g, const int32_t* k_cnt, int s
   g.cnt = __ldcg(k_cnt + s);
   g.n_known = g.n_chunk + (g.cnt + kKeyTile - 1) / kKeyTile;
   g.resolved = true;
+}
+
+// The same where the selection is known to be complete.
+__device__ __forceinline__ void learn_count(AttnGeom& g, const int32_t* k_cnt, int s) {
+  g.cnt = __ldcg(k_cnt + s);
+  g.n_known = g.n_chunk + (g.cnt + kKeyTile - 1) / kKeyTile;
+  g.resolved = true;
+}
+__device__ __forceinline__ bool attn_last_cta() {
+  return blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1;
 }
 
 // Rows of tile t: from the selected list (`from_list`, rows list[base .. base + count)), or the consecutive cache

@@ -38,7 +38,9 @@ struct DevParams {
   float* attn_partials;
   int32_t* attn_counters;
   int n_attn_counters;
-  int attn_parts;   // parts per row block of the launch at hand (set by the launcher), 1 = no split
+  // plan of the attention call at hand (set by the launcher): the row blocks [0, attn_split_rb) of every head are cut
+  // into attn_parts parts each, in a launch of their own after the one of the heavier row blocks above them, if any
+  int attn_row_blocks, attn_split_rb, attn_parts, attn_after_whole;
 };
 
 // B_s of one sequence: min(B_SA, T) or floor(frac*T + 0.5) in double.

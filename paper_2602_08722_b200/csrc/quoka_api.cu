@@ -35,12 +35,18 @@ static int budget_cap_of(const quoka_params* p) {
   return cap < 1 ? 1 : cap;
 }
 
-// Parts the attention kernels may cut a row block into for this problem (the larger of the sparse and the dense call's).
-static int attn_parts_bound(const quoka_params* p) {
-  if (p->impl == QUOKA_IMPL_SIMT || p->chunk_len <= 1) return 1;
-  const int cap = budget_cap_of(p);
-  const int sparse = attn_split_parts(p, (cap + 127) / 128 + 1), dense = attn_split_parts(p, (p->max_ctx_len + 127) / 128 + 1);
-  return sparse > dense ? sparse : dense;
+// The two plans an attention call of this problem may follow, and the scratch that serves either.
+struct AttnScratch { AttnPlan sparse, dense; size_t counters = 0, partials = 0; };
+static AttnScratch attn_scratch(const quoka_params* p) {
+  AttnScratch a;
+  a.sparse = attn_plan_sparse(p, budget_cap_of(p));
+  a.dense = attn_plan_dense(p);
+  for (const AttnPlan& plan : {a.sparse, a.dense}) {
+    const size_t c = attn_split_counter_bytes(p, plan), b = attn_split_partial_bytes(p, plan);
+    a.counters = c > a.counters ? c : a.counters;
+    a.partials = b > a.partials ? b : a.partials;
+  }
+  return a;
 }
 
 // with_split = false: the layout without the split-attention scratch (every call still works, small grids unsplit)
@@ -62,11 +68,13 @@ static Workspace carve(const quoka_params* p, void* ws, bool with_split = true) 
   w.scores = reinterpret_cast<float*>(take((size_t)p->batch * p->n_kv_heads * (size_t)(p->max_ctx_len > 0 ? p->max_ctx_len : 1) * 4));
   w.k_idx = reinterpret_cast<int32_t*>(take((size_t)p->batch * p->n_kv_heads * cap * 4));
   w.k_cnt = reinterpret_cast<int32_t*>(take((size_t)p->batch * 4));
-  const int parts = with_split ? attn_parts_bound(p) : 1;
-  if (parts > 1) {
-    w.attn_counters = reinterpret_cast<int32_t*>(take(attn_split_counter_bytes(p)));
-    w.n_attn_counters = (int)(attn_split_counter_bytes(p) / sizeof(int32_t));
-    w.attn_partials = reinterpret_cast<float*>(take(attn_split_partial_bytes(p, parts)));
+  if (with_split) {
+    const AttnScratch a = attn_scratch(p);
+    if (a.counters > 0) {
+      w.attn_counters = reinterpret_cast<int32_t*>(take(a.counters));
+      w.attn_partials = reinterpret_cast<float*>(take(a.partials));
+      w.n_attn_counters = (int)(a.counters / sizeof(int32_t));
+    }
   }
   w.total = off;
   return w;
@@ -120,7 +128,7 @@ static quoka_status check_ws(const quoka_params* p, void* ws, size_t ws_bytes, b
 
 size_t workspace_bytes(const quoka_params* p, bool with_split) { return carve(p, nullptr, with_split).total; }
 
-static DevParams make_dev(const quoka_params* p, void* ws, bool with_split = true) {
+static DevParams make_dev(const quoka_params* p, void* ws, const Workspace& w) {
   DevParams P{};
   P.batch = p->batch; P.n_q = p->n_q_heads; P.n_kv = p->n_kv_heads; P.group = p->n_q_heads / p->n_kv_heads;
   P.d = p->head_dim; P.chunk = p->chunk_len; P.n_retain = p->n_retain;
@@ -138,10 +146,11 @@ static DevParams make_dev(const quoka_params* p, void* ws, bool with_split = tru
   P.agg_mean = p->query_agg == QUOKA_AGG_MEAN ? 1 : 0;
   P.k_inv_norm = p->k_inv_norm;
   P.kv_rows = p->kv_rows;
-  const Workspace w = carve(p, ws, with_split);
-  P.attn_partials = w.attn_partials; P.attn_counters = w.attn_counters; P.n_attn_counters = w.n_attn_counters; P.attn_parts = 1;
+  P.attn_partials = w.attn_partials; P.attn_counters = w.attn_counters; P.n_attn_counters = w.n_attn_counters;
+  P.attn_row_blocks = 0; P.attn_split_rb = 0; P.attn_parts = 1; P.attn_after_whole = 0;
   return P;
 }
+static DevParams make_dev(const quoka_params* p, void* ws) { return make_dev(p, ws, carve(p, ws)); }
 
 static bool use_tensor(const quoka_params* p) {
   if (p->impl == QUOKA_IMPL_SIMT) return false;
@@ -183,13 +192,14 @@ static quoka_status run_score_keys(const quoka_params* p, const DevParams& P, co
 
 static quoka_status run_attn(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                              const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
-                             bool after_selection = false) {
+                             bool after_selection = false, const AttnPlan* plan = nullptr) {
   if (p->impl == QUOKA_IMPL_AUTO && P.chunk == 1) {
     QUOKA_TRY_CUDA(launch_decode_attn(P, p->dtype, q, k, v, k_idx, k_cnt, out, lse, st, after_selection));
     return QUOKA_OK;
   }
   if (use_tensor(p) && attn_tc_supported(p))
-    return launch_attn_tc(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection);
+    return launch_attn_tc(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection,
+                          plan ? *plan : (k_idx ? attn_plan_sparse(p, P.budget_cap) : attn_plan_dense(p)));
   if (p->impl == QUOKA_IMPL_TENSOR) return QUOKA_ERR_UNSUPPORTED;
   if (p->impl == QUOKA_IMPL_AUTO && p->dtype == QUOKA_F32) {
     QUOKA_TRY_CUDA(launch_attn_f32(P, static_cast<const float*>(q), static_cast<const float*>(k), static_cast<const float*>(v),
@@ -229,19 +239,12 @@ static HostPipe* host_pipe_for_current_device() {
   return hp.ok ? &hp : nullptr;
 }
 
-// The fused loop body.  with_split = false keeps to the workspace layout without the split-attention scratch (the
-// built-in array of the no-allocation entry point has no room for it).
-quoka_status prefill_chunk_impl(const quoka_params* p, const void* q, const void* k_cache, const void* v_cache, void* out,
-                                int32_t* k_idx_out, int32_t* k_cnt_out, void* ws, size_t ws_bytes, void* stream,
-                                bool with_split) {
-  quoka_status st = check_prefill_args(p, q, k_cache, v_cache, out);
-  if (st != QUOKA_OK) return st;
-  if ((st = check_ws(p, ws, ws_bytes, with_split)) != QUOKA_OK) return st;
-  cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  DevParams P = make_dev(p, ws, with_split);
-  Workspace w = carve(p, ws, with_split);
-  int32_t* k_idx = k_idx_out ? k_idx_out : w.k_idx;
-  int32_t* k_cnt = k_cnt_out ? k_cnt_out : w.k_cnt;
+// The fused loop body on checked arguments: P and w for the problem at hand, the attention by `plan` (no split without
+// scratch in P).
+static quoka_status run_prefill(const quoka_params* p, const DevParams& P, const Workspace& w, const AttnPlan& plan,
+                                const void* q, const void* k_cache, const void* v_cache, void* out, int32_t* k_idx,
+                                int32_t* k_cnt, cudaStream_t cs) {
+  quoka_status st;
   if (p->max_ctx_len > 0) {
     if (p->impl == QUOKA_IMPL_AUTO && decode_path_applies(P)) {       // one query: the scoring kernel forms Q-bar itself
       QUOKA_TRY_CUDA(launch_score_keys_gemv(P, p->dtype, q, nullptr, k_cache, w.scores, cs, /*chained=*/true));
@@ -253,12 +256,25 @@ quoka_status prefill_chunk_impl(const quoka_params* p, const void* q, const void
       if ((st = run_select_queries(p, P, q, w.q_idx, w.qbar, cs, early)) != QUOKA_OK) return st;
       if ((st = run_score_keys(p, P, w.qbar, k_cache, w.scores, cs, /*chained=*/true)) != QUOKA_OK) return st;
     }
-  } else if (w.attn_counters) {
-    QUOKA_TRY_CUDA(cudaMemsetAsync(w.attn_counters, 0, attn_split_counter_bytes(p), cs));
+  } else if (P.attn_counters) {
+    QUOKA_TRY_CUDA(cudaMemsetAsync(P.attn_counters, 0, P.n_attn_counters * sizeof(int32_t), cs));
   }
   // with an empty cache the selection kernel only writes k_cnt = 0 and the -1 padding
   QUOKA_TRY_CUDA(launch_select_keys(P, w.scores, k_idx, k_cnt, cs, /*chained=*/p->max_ctx_len > 0));
-  return run_attn(p, P, q, k_cache, v_cache, k_idx, k_cnt, out, nullptr, cs, /*after_selection=*/true);
+  return run_attn(p, P, q, k_cache, v_cache, k_idx, k_cnt, out, nullptr, cs, /*after_selection=*/true, &plan);
+}
+
+// with_split = false keeps to the workspace layout without the split-attention scratch (the built-in array of the
+// no-allocation entry point has no room for it).
+quoka_status prefill_chunk_impl(const quoka_params* p, const void* q, const void* k_cache, const void* v_cache, void* out,
+                                int32_t* k_idx_out, int32_t* k_cnt_out, void* ws, size_t ws_bytes, void* stream,
+                                bool with_split) {
+  quoka_status st = check_prefill_args(p, q, k_cache, v_cache, out);
+  if (st != QUOKA_OK) return st;
+  if ((st = check_ws(p, ws, ws_bytes, with_split)) != QUOKA_OK) return st;
+  const Workspace w = carve(p, ws, with_split);
+  return run_prefill(p, make_dev(p, ws, w), w, attn_plan_sparse(p, budget_cap_of(p)), q, k_cache, v_cache, out,
+                     k_idx_out ? k_idx_out : w.k_idx, k_cnt_out ? k_cnt_out : w.k_cnt, static_cast<cudaStream_t>(stream));
 }
 
 }  // namespace quoka
@@ -398,12 +414,13 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
                              (size_t)n_kv * G * head_bytes, p->batch, cudaMemcpyDeviceToHost, on);
   };
   // A large chunk is cut into slices of whole KV groups (the selection and the attention of a KV group need nothing
-  // of another group): slice i + 1 comes in and slice i - 1 goes out while slice i is computed.  Only for problems
-  // the attention kernels would not split (a slice must give the same bits as the whole), without a cache of key
-  // norms (indexed by the whole problem's head count), and when the side streams exist.
+  // of another group): slice i + 1 comes in and slice i - 1 goes out while slice i is computed.  Every slice's attention
+  // follows the whole problem's plan, so that it gives the same bits as the whole.  Not for grids below a wave, without
+  // a cache of key norms (indexed by the whole problem's head count), and when the side streams exist.
   int slices = 1;
   const size_t q_bytes = (size_t)p->batch * p->n_q_heads * head_bytes;
-  if (!p->k_inv_norm && attn_parts_bound(p) == 1 && q_bytes >= ((size_t)8 << 20)) {
+  const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p));
+  if (!p->k_inv_norm && !attn_below_a_wave(p) && q_bytes >= ((size_t)8 << 20)) {
     if (p->n_kv_heads % 4 == 0) slices = 4;
     else if (p->n_kv_heads % 2 == 0) slices = 2;
   }
@@ -415,10 +432,15 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
     QUOKA_TRY_CUDA(copy_out(0, p->n_kv_heads, cs));
     return QUOKA_OK;
   }
+  if ((st = check_prefill_args(p, q_dev, k_cache, v_cache, out_dev)) != QUOKA_OK) return st;
   const int kv_per = p->n_kv_heads / slices;
   quoka_params sub = *p;
   sub.n_kv_heads = kv_per;
   sub.n_q_heads = kv_per * G;
+  // (a slice's intermediates end below the whole problem's split-attention scratch)
+  const Workspace whole = carve(p, ws), w = carve(&sub, ws, /*with_split=*/false);
+  DevParams P = make_dev(&sub, ws, w);
+  P.attn_partials = whole.attn_partials; P.attn_counters = whole.attn_counters; P.n_attn_counters = whole.n_attn_counters;
   QUOKA_TRY_CUDA(cudaEventRecord(hp->fork, cs));
   QUOKA_TRY_CUDA(cudaStreamWaitEvent(hp->h2d, hp->fork, 0));
   for (int i = 0; i < slices; ++i) {
@@ -426,11 +448,10 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
     QUOKA_TRY_CUDA(copy_in(kv0, kv_per, hp->h2d));
     QUOKA_TRY_CUDA(cudaEventRecord(hp->in[i], hp->h2d));
     QUOKA_TRY_CUDA(cudaStreamWaitEvent(cs, hp->in[i], 0));
-    st = prefill_chunk_impl(&sub, static_cast<char*>(q_dev) + (size_t)kv0 * G * head_bytes,
-                            static_cast<char*>(k_cache) + (size_t)kv0 * p->kv_stride_h * es,
-                            static_cast<char*>(v_cache) + (size_t)kv0 * p->kv_stride_h * es,
-                            static_cast<char*>(out_dev) + (size_t)kv0 * G * head_bytes, nullptr, nullptr, ws, ws_bytes,
-                            stream, /*with_split=*/false);
+    st = run_prefill(&sub, P, w, plan, static_cast<char*>(q_dev) + (size_t)kv0 * G * head_bytes,
+                     static_cast<char*>(k_cache) + (size_t)kv0 * p->kv_stride_h * es,
+                     static_cast<char*>(v_cache) + (size_t)kv0 * p->kv_stride_h * es,
+                     static_cast<char*>(out_dev) + (size_t)kv0 * G * head_bytes, w.k_idx, w.k_cnt, cs);
     if (st != QUOKA_OK) return st;
     QUOKA_TRY_CUDA(cudaEventRecord(hp->done[i], cs));
     QUOKA_TRY_CUDA(cudaStreamWaitEvent(hp->d2h, hp->done[i], 0));

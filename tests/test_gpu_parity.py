@@ -434,6 +434,34 @@ def test_decode_scoring_units(T, d, dtype, group, cached_norms, paged):
     assert torch.equal(gp.out, want_out) and torch.equal(gp.k_idx, want_idx)
 
 
+@pytest.mark.parametrize("n_q,n_kv,d,C,T,B", [
+    (32, 8, 128, 1300, 9000, 5000),     # pairs, 6 row blocks: the lightest in parts after the whole ones, ragged last block
+    (24, 8, 64, 1800, 7000, 6000),      # one-CTA kernel, 8 row blocks
+    (32, 8, 128, 1281, 6000, 6000),     # the budget covers the cache: the list is the identity
+])
+def test_attention_with_its_lightest_row_blocks_in_parts(n_q, n_kv, d, C, T, B):
+    """Grids of a full wave and a rest: whole row blocks and parts in one call, sparse (staged and fused) and dense, twice
+    over the same workspace (the arrival counters go back to zero), every row against the oracle for two KV groups."""
+    gp = problem(1000 + C, n_q=n_q, n_kv=n_kv, d=d, T=T, C=C, n_retain=32, kv_budget=B)
+    assert n_q * -(-C // 256) > 148 and n_q * -(-C // 256) % 148
+    gp.run_staged()
+    check_chain(gp, attn_rows=200)
+    staged = gp.out.clone()
+    for _ in range(2):
+        gp.out.zero_()
+        api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+        torch.cuda.synchronize()
+        assert torch.equal(gp.out, staged)
+    q, k, v, _ = gp.oracle_inputs(0)
+    for _ in range(2):
+        gp.out.zero_()
+        api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, gp.lse, gp.ws)
+        torch.cuda.synchronize()
+        heads, rows = stratified_rows(n_q, C, 200, 5)
+        want = O.sparse_attention_rows(q, k, v, T, [np.arange(T)] * n_kv, heads, rows)
+        check_attention(f64(gp.out[0])[heads, rows], want, "bf16")
+
+
 @pytest.mark.parametrize("paged", [False, True])
 @pytest.mark.parametrize("T,C,B,n_q,n_kv,d,n_retain", [
     (63, 2, 40, 4, 2, 128, 1),          # fewer keys than a tile, two query rows
