@@ -216,6 +216,13 @@ cudaError_t launch_score_keys_gemv(const DevParams& P, int dtype, const void* q,
 cudaError_t launch_decode_attn(const DevParams& P, int dtype, const void* q, const void* k, const void* v,
                                const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                                bool chained);
+// Selection and attention in one launch, where the problem's rows of scores are few; and the staged call's attention on
+// those problems, with the same sums.
+bool decode_select_attn_applies(const DevParams& P);
+cudaError_t launch_decode_select_attn(const DevParams& P, int dtype, const void* q, const void* k, const void* v,
+                                      const float* scores, int32_t* k_idx, int32_t* k_cnt, void* out, cudaStream_t st);
+cudaError_t launch_decode_listed_attn(const DevParams& P, int dtype, const void* q, const void* k, const void* v,
+                                      const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st);
 cudaError_t launch_append_kv(const DevParams& P, int dtype, const void* k_new, const void* v_new, void* k_cache,
                              void* v_cache, float* k_inv_norm, cudaStream_t st);
 

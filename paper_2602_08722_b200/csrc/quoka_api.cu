@@ -194,7 +194,11 @@ static quoka_status run_attn(const quoka_params* p, const DevParams& P, const vo
                              const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                              bool after_selection = false, const AttnPlan* plan = nullptr) {
   if (p->impl == QUOKA_IMPL_AUTO && P.chunk == 1) {
-    QUOKA_TRY_CUDA(launch_decode_attn(P, p->dtype, q, k, v, k_idx, k_cnt, out, lse, st, after_selection));
+    // (a fused call that gets here does not have the one-launch form: run_prefill would have taken it)
+    if (k_idx && !after_selection && decode_path_applies(P) && decode_select_attn_applies(P))
+      QUOKA_TRY_CUDA(launch_decode_listed_attn(P, p->dtype, q, k, v, k_idx, k_cnt, out, lse, st));
+    else
+      QUOKA_TRY_CUDA(launch_decode_attn(P, p->dtype, q, k, v, k_idx, k_cnt, out, lse, st, after_selection));
     return QUOKA_OK;
   }
   if (use_tensor(p) && attn_tc_supported(p))
@@ -248,6 +252,11 @@ static quoka_status run_prefill(const quoka_params* p, const DevParams& P, const
   if (p->max_ctx_len > 0) {
     if (p->impl == QUOKA_IMPL_AUTO && decode_path_applies(P)) {       // one query: the scoring kernel forms Q-bar itself
       QUOKA_TRY_CUDA(launch_score_keys_gemv(P, p->dtype, q, nullptr, k_cache, w.scores, cs, /*chained=*/true));
+      if (decode_select_attn_applies(P)) {
+        QUOKA_TRY_CUDA(launch_decode_select_attn(P, p->dtype, q, k_cache, v_cache, w.scores, k_idx == w.k_idx ? nullptr : k_idx,
+                                                 k_cnt == w.k_cnt ? nullptr : k_cnt, out, cs));
+        return QUOKA_OK;
+      }
     } else {
       // The aggregation kernel also sets the split attention's arrival counters to zero.  The early launch of the first
       // kernel is for calls whose launches count; where the attention fills the GPU it gains nothing (2048 queries at 32K:

@@ -417,6 +417,44 @@ def test_decode_attention_parts_and_groups(n_q, n_kv, T, B, d, dtype):
         assert np.abs(f64(gp.lse[s]) - lse).max() <= 2e-3
 
 
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("T,max_ctx,B,n_q,n_kv,d,dtype", [
+    ([2049], 2049, 64, 8, 2, 128, "bf16"),        # just beyond the two-launch form: 258 positions per CTA
+    ([0, 5, 4096], 4096, 200, 6, 2, 64, "f32"),   # an empty cache, a budget that covers one, exactly 512 positions per CTA
+    ([4097, 300], 9000, 299, 8, 4, 128, "f32"),   # two items per thread, the second CTA's last rows alone
+    ([33000], 33000, 3000, 5, 1, 64, "bf16"),     # beyond eight items per thread; two head blocks per group
+    ([40000], 70000, 8448, 3, 3, 128, "bf16"),    # as many listed rows as a CTA can keep
+])
+def test_decode_select_and_attend_in_one_launch(T, max_ctx, B, n_q, n_kv, d, dtype, paged):
+    """The generation step's selection + attention kernel: its list and its output against the staged calls (same bits),
+    those against the oracle; then with every listed row in the first CTAs' parts of the cache, at equal scores."""
+    inp = synth.make_chunk_inputs(1010 + d, len(T), n_q, n_kv, d, T, 1, dtype, capacity=max_ctx + 1)
+    if paged:
+        inp = synth.to_paged(inp, 3)
+        extra = -(-(max_ctx + 1) // 64) - inp.block_table.shape[1]
+        inp.block_table = torch.nn.functional.pad(inp.block_table, (0, max(extra, 0)), value=-1)
+    gp = GpuProblem(inp, 4, kv_budget=B, paged=paged, max_ctx_len=max_ctx)
+    for _ in range(2):
+        gp.run_staged()
+        check_chain(gp)
+        want_out, want_idx, want_cnt = gp.out.clone(), gp.k_idx.clone(), gp.k_cnt.clone()
+        gp.out.zero_(); gp.k_idx.fill_(-9); gp.k_cnt.fill_(-9)
+        api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, gp.k_idx, gp.k_cnt, gp.ws)
+        torch.cuda.synchronize()
+        assert torch.equal(gp.out, want_out) and torch.equal(gp.k_idx, want_idx) and torch.equal(gp.k_cnt, want_cnt)
+        gp.out.zero_()
+        api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)      # no list asked for
+        torch.cuda.synchronize()
+        assert torch.equal(gp.out, want_out) and api.quoka_last_device_status(gp.ws) == 0
+        if paged:
+            break
+        n = min(t for t in T if t > 0)
+        n = min(n, B + 30)                          # equal keys along the group's queries: the cut lies among them
+        toward = gp.q.view(len(T), n_kv, n_q // n_kv, d).float().mean(2)[:, :, None] + 0.5 * gp.k[:, :, :1].float()
+        gp.k[:, :, :n] = toward.to(gp.k.dtype)      # (cosine well below 1: Q-bar's own rounding may exceed it by 2^-8)
+        inp.k = gp.k.cpu()
+
+
 @pytest.mark.parametrize("cached_norms,paged", [(False, False), (True, False), (False, True), (True, True)])
 @pytest.mark.parametrize("d,dtype,group", [(128, "bf16", 4), (64, "bf16", 3), (128, "f32", 1), (64, "f32", 40)])
 @pytest.mark.parametrize("T", [[1, 8, 15, 17], [0, 31, 0, 33], [3000, 63, 0, 1], [65] * 35])
