@@ -197,7 +197,7 @@ quoka_status quoka_prefill_chunk(const quoka_params* p, const void* q, const voi
  * ([b][n_Q][C][d] dense), all on `stream`.  ctx_len_host is a HOST copy of T_s.
  * Paged caches are not supported here (QUOKA_ERR_UNSUPPORTED).  q_dev / out_dev
  * must be dense [b][n_Q][C][d] and p's q/o strides must describe them.
- * A chunk of 8 MiB of queries or more is cut into 2 or 4 slices of whole KV
+ * A chunk of 8 MiB of queries or more is cut into 2 or 3 slices of whole KV
  * groups, and slice i+1 is copied in and slice i-1 copied out on two streams of
  * the library's own (made on first use, one set per device) while slice i is
  * computed on `stream`; the result is the same bits as the unsliced call's.

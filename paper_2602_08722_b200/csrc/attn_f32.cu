@@ -240,7 +240,7 @@ cudaError_t launch_attn_f32(const DevParams& P, const float* q, const float* k, 
   int parts = (int)(sms / jobs);
   parts = parts > 8 ? 8 : parts;
   parts = parts > tiles / 2 ? tiles / 2 : parts;
-  if (parts < 1) parts = 1;
+  if (parts < 1 || P.attn_one_part) parts = 1;
   const dim3 grid((unsigned)(P.n_q * parts), (unsigned)rb, (unsigned)P.batch), block(kF32Threads);
   cudaError_t e;
 #define QUOKA_ATTN_F32(D_)                                                                                                \

@@ -147,7 +147,7 @@ static DevParams make_dev(const quoka_params* p, void* ws, const Workspace& w) {
   P.k_inv_norm = p->k_inv_norm;
   P.kv_rows = p->kv_rows;
   P.attn_partials = w.attn_partials; P.attn_counters = w.attn_counters; P.n_attn_counters = w.n_attn_counters;
-  P.attn_row_blocks = 0; P.attn_split_rb = 0; P.attn_parts = 1; P.attn_after_whole = 0;
+  P.attn_one_part = 0; P.attn_row_blocks = 0; P.attn_split_rb = 0; P.attn_parts = 1; P.attn_after_whole = 0;
   return P;
 }
 static DevParams make_dev(const quoka_params* p, void* ws) { return make_dev(p, ws, carve(p, ws)); }
@@ -216,9 +216,10 @@ static quoka_status run_attn(const quoka_params* p, const DevParams& P, const vo
 
 // Two side streams and the events that tie them to the caller's stream, made once per device: the host-buffer entry
 // point brings the next slice of a chunk in and takes the previous one out while the current one is computed.
+constexpr int kHostSlices = 3;
 struct HostPipe {
   cudaStream_t h2d = nullptr, d2h = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr, in[4] = {}, done[4] = {};
+  cudaEvent_t fork = nullptr, join = nullptr, in[kHostSlices] = {}, done[kHostSlices] = {};
   bool ok = false, tried = false;
 };
 static HostPipe* host_pipe_for_current_device() {
@@ -235,7 +236,7 @@ static HostPipe* host_pipe_for_current_device() {
                 cudaStreamCreateWithFlags(&hp.d2h, cudaStreamNonBlocking) == cudaSuccess &&
                 cudaEventCreateWithFlags(&hp.fork, cudaEventDisableTiming) == cudaSuccess &&
                 cudaEventCreateWithFlags(&hp.join, cudaEventDisableTiming) == cudaSuccess;
-    for (int i = 0; i < 4 && good; ++i)
+    for (int i = 0; i < kHostSlices && good; ++i)
       good = cudaEventCreateWithFlags(&hp.in[i], cudaEventDisableTiming) == cudaSuccess &&
              cudaEventCreateWithFlags(&hp.done[i], cudaEventDisableTiming) == cudaSuccess;
     hp.ok = good;
@@ -399,20 +400,23 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
   // both sides, the sequences are `pitch` apart.
   const int G = p->n_q_heads / p->n_kv_heads;
   const size_t head_bytes = (size_t)C * d * es;
-  auto copy_in = [&](int kv0, int n_kv, cudaStream_t on) -> cudaError_t {
-    cudaError_t e = cudaMemcpy2DAsync(static_cast<char*>(q_dev) + (size_t)kv0 * G * head_bytes, (size_t)p->q_stride_b * es,
-                                      static_cast<const char*>(q_host) + (size_t)kv0 * G * head_bytes,
-                                      (size_t)p->n_q_heads * head_bytes, (size_t)n_kv * G * head_bytes, p->batch,
-                                      cudaMemcpyHostToDevice, on);
+  auto copy_in_q = [&](int kv0, int n_kv, cudaStream_t on) -> cudaError_t {
+    return cudaMemcpy2DAsync(static_cast<char*>(q_dev) + (size_t)kv0 * G * head_bytes, (size_t)p->q_stride_b * es,
+                             static_cast<const char*>(q_host) + (size_t)kv0 * G * head_bytes,
+                             (size_t)p->n_q_heads * head_bytes, (size_t)n_kv * G * head_bytes, p->batch,
+                             cudaMemcpyHostToDevice, on);
+  };
+  auto copy_in_kv = [&](cudaStream_t on) -> cudaError_t {
+    cudaError_t e = cudaSuccess;
     for (int s = 0; s < p->batch && e == cudaSuccess; ++s) {
-      const size_t dst_off = ((size_t)s * p->kv_stride_b + (size_t)kv0 * p->kv_stride_h + (size_t)ctx_len_host[s] * p->kv_stride_t) * es;
-      const size_t src_off = ((size_t)s * p->n_kv_heads + kv0) * head_bytes;
+      const size_t dst_off = ((size_t)s * p->kv_stride_b + (size_t)ctx_len_host[s] * p->kv_stride_t) * es;
+      const size_t src_off = (size_t)s * p->n_kv_heads * head_bytes;
       e = cudaMemcpy2DAsync(static_cast<char*>(k_cache) + dst_off, (size_t)p->kv_stride_h * es,
-                            static_cast<const char*>(k_new_host) + src_off, head_bytes, head_bytes, n_kv,
+                            static_cast<const char*>(k_new_host) + src_off, head_bytes, head_bytes, p->n_kv_heads,
                             cudaMemcpyHostToDevice, on);
       if (e == cudaSuccess)
         e = cudaMemcpy2DAsync(static_cast<char*>(v_cache) + dst_off, (size_t)p->kv_stride_h * es,
-                              static_cast<const char*>(v_new_host) + src_off, head_bytes, head_bytes, n_kv,
+                              static_cast<const char*>(v_new_host) + src_off, head_bytes, head_bytes, p->n_kv_heads,
                               cudaMemcpyHostToDevice, on);
     }
     return e;
@@ -423,40 +427,48 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
                              (size_t)n_kv * G * head_bytes, p->batch, cudaMemcpyDeviceToHost, on);
   };
   // A large chunk is cut into slices of whole KV groups (the selection and the attention of a KV group need nothing
-  // of another group): slice i + 1 comes in and slice i - 1 goes out while slice i is computed.  Every slice's attention
-  // follows the whole problem's plan, so that it gives the same bits as the whole.  Not for grids below a wave, without
-  // a cache of key norms (indexed by the whole problem's head count), and when the side streams exist.
-  int slices = 1;
+  // of another group): the next slice's queries come in and the last one's output goes out while a slice is computed.
+  // Every slice's attention follows the whole problem's plan, so that it gives the same bits as the whole.  Not for grids
+  // below a wave, without a cache of key norms (indexed by the whole problem's head count), and when the side streams exist.
+  // What bounds it: the host link, and on it the number of copies: one that starts while the other direction is busy costs
+  // about 17 us.  So all keys and values first, then the queries in three pieces, the first the smallest.  32 query / 8 KV
+  // heads, 2048 queries at 32K (25.2 MB in: 500 us alone, 16.8 MB out): slices of 2, 3 and 3 KV groups 745 us, of 2 / 2 / 2 / 2
+  // 811, of 4 / 4 791; queries, keys and values of four equal slices one after another 805.
+  int n_slices = 1, slice[kHostSlices] = {p->n_kv_heads, 0, 0};
   const size_t q_bytes = (size_t)p->batch * p->n_q_heads * head_bytes;
   const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p));
-  if (!p->k_inv_norm && !attn_below_a_wave(p) && q_bytes >= ((size_t)8 << 20)) {
-    if (p->n_kv_heads % 4 == 0) slices = 4;
-    else if (p->n_kv_heads % 2 == 0) slices = 2;
+  if (!p->k_inv_norm && !attn_below_a_wave(p) && q_bytes >= ((size_t)8 << 20) && p->n_kv_heads > 1) {
+    slice[0] = p->n_kv_heads / 4 > 0 ? p->n_kv_heads / 4 : 1;
+    slice[1] = p->n_kv_heads == 2 ? 1 : (p->n_kv_heads - slice[0]) / 2;
+    slice[2] = p->n_kv_heads - slice[0] - slice[1];
+    n_slices = slice[2] > 0 ? 3 : 2;
   }
-  HostPipe* hp = slices > 1 ? host_pipe_for_current_device() : nullptr;
+  HostPipe* hp = n_slices > 1 ? host_pipe_for_current_device() : nullptr;
   if (!hp) {
-    QUOKA_TRY_CUDA(copy_in(0, p->n_kv_heads, cs));
+    QUOKA_TRY_CUDA(copy_in_q(0, p->n_kv_heads, cs));
+    QUOKA_TRY_CUDA(copy_in_kv(cs));
     st = quoka_prefill_chunk(p, q_dev, k_cache, v_cache, out_dev, nullptr, nullptr, ws, ws_bytes, stream);
     if (st != QUOKA_OK) return st;
     QUOKA_TRY_CUDA(copy_out(0, p->n_kv_heads, cs));
     return QUOKA_OK;
   }
   if ((st = check_prefill_args(p, q_dev, k_cache, v_cache, out_dev)) != QUOKA_OK) return st;
-  const int kv_per = p->n_kv_heads / slices;
-  quoka_params sub = *p;
-  sub.n_kv_heads = kv_per;
-  sub.n_q_heads = kv_per * G;
-  // (a slice's intermediates end below the whole problem's split-attention scratch)
-  const Workspace whole = carve(p, ws), w = carve(&sub, ws, /*with_split=*/false);
-  DevParams P = make_dev(&sub, ws, w);
-  P.attn_partials = whole.attn_partials; P.attn_counters = whole.attn_counters; P.n_attn_counters = whole.n_attn_counters;
+  const Workspace whole = carve(p, ws);
   QUOKA_TRY_CUDA(cudaEventRecord(hp->fork, cs));
   QUOKA_TRY_CUDA(cudaStreamWaitEvent(hp->h2d, hp->fork, 0));
-  for (int i = 0; i < slices; ++i) {
-    const int kv0 = i * kv_per;
-    QUOKA_TRY_CUDA(copy_in(kv0, kv_per, hp->h2d));
+  QUOKA_TRY_CUDA(copy_in_kv(hp->h2d));
+  for (int i = 0, kv0 = 0; i < n_slices; kv0 += slice[i++]) {
+    QUOKA_TRY_CUDA(copy_in_q(kv0, slice[i], hp->h2d));
     QUOKA_TRY_CUDA(cudaEventRecord(hp->in[i], hp->h2d));
     QUOKA_TRY_CUDA(cudaStreamWaitEvent(cs, hp->in[i], 0));
+    quoka_params sub = *p;
+    sub.n_kv_heads = slice[i];
+    sub.n_q_heads = slice[i] * G;
+    // (a slice's intermediates end below the whole problem's split-attention scratch)
+    const Workspace w = carve(&sub, ws, /*with_split=*/false);
+    DevParams P = make_dev(&sub, ws, w);
+    P.attn_partials = whole.attn_partials; P.attn_counters = whole.attn_counters; P.n_attn_counters = whole.n_attn_counters;
+    P.attn_one_part = 1;
     st = run_prefill(&sub, P, w, plan, static_cast<char*>(q_dev) + (size_t)kv0 * G * head_bytes,
                      static_cast<char*>(k_cache) + (size_t)kv0 * p->kv_stride_h * es,
                      static_cast<char*>(v_cache) + (size_t)kv0 * p->kv_stride_h * es,
@@ -464,7 +476,7 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
     if (st != QUOKA_OK) return st;
     QUOKA_TRY_CUDA(cudaEventRecord(hp->done[i], cs));
     QUOKA_TRY_CUDA(cudaStreamWaitEvent(hp->d2h, hp->done[i], 0));
-    QUOKA_TRY_CUDA(copy_out(kv0, kv_per, hp->d2h));
+    QUOKA_TRY_CUDA(copy_out(kv0, slice[i], hp->d2h));
   }
   QUOKA_TRY_CUDA(cudaEventRecord(hp->join, hp->d2h));
   QUOKA_TRY_CUDA(cudaStreamWaitEvent(cs, hp->join, 0));

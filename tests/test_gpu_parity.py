@@ -278,6 +278,24 @@ def test_host_buffer_entry_point_matches_device_entry_point(shape):
     assert torch.equal(out_host, want.cpu())
 
 
+@pytest.mark.parametrize("dtype,n_q,n_kv,C", [
+    ("f32", 32, 8, 2048), ("bf16", 32, 16, 1300), ("bf16", 30, 5, 1536), ("bf16", 16, 2, 2560), ("bf16", 24, 1, 2048)])
+def test_host_buffer_slices_give_the_whole_calls_bits(dtype, n_q, n_kv, C):
+    """Slices of 1 to 6 KV groups, grids with row blocks in parts among them, and a single KV head (unsliced)."""
+    T = 1500
+    gp = problem(14, n_q=n_q, n_kv=n_kv, T=T, C=C, n_retain=32, kv_budget=1100, dtype=dtype)
+    api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+    torch.cuda.synchronize()
+    want, want_k = gp.out.cpu(), gp.k.clone()
+    host = [x.contiguous().pin_memory() for x in (gp.inp.q, gp.inp.k[:, :, T:T + C], gp.inp.v[:, :, T:T + C])]
+    out_host = torch.zeros_like(host[0]).pin_memory()
+    gp.k[:, :, T:] = 0
+    gp.v[:, :, T:] = 0
+    api.quoka_prefill_chunk_host(gp.p, gp.inp.ctx_len.clone(), *host, out_host, torch.zeros_like(gp.q), gp.k, gp.v, gp.out, gp.ws)
+    torch.cuda.synchronize()
+    assert torch.equal(out_host, want) and torch.equal(gp.k, want_k)
+
+
 def test_host_buffer_entry_point_replayed_from_a_cuda_graph():
     # the sliced call forks to the library's two copy streams and joins again: captured as one graph and replayed
     shape = dict(n_q=32, n_kv=8, T=3000, C=2048, n_retain=64, kv_budget=700)
