@@ -21,6 +21,7 @@
 // 384 threads and no register re-balancing between roles: every thread may use 168 registers
 // (with 512 threads and setmaxnreg the compiler still scheduled the softmax for 128 registers,
 // which halved its speed).
+#include <algorithm>
 #include "attn_tiles.cuh"
 
 namespace quoka {
@@ -360,6 +361,14 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
 // The number of parts minimises  waves(parts) * (tiles / parts + 6):  a part costs about six tiles' time of
 // start-up, partial results and merge (the model fits the measured times of 1 to 5 parts on grids of 32 to 288 CTAs
 // within 3 %), parts keep at least six tiles, and a split has to promise 3 % to be taken.
+// The pair kernel's parts merge in a cluster of 2 * parts CTAs where all of a grid's clusters are resident at once: the
+// device holds 33, 22 or 15 of 4, 6 or 8 CTAs of this shared memory, the limits leave one or two free (a second wave costs
+// more than any split gives: 16 clusters of eight took 38 us where the 14 that fit take 30).  A part then costs about one
+// tile on top of the walk against parts through memory, and four and a half against a whole row block (a sparse part's step
+// is slower than a whole row block's).  Sparse attention, whole or parts through memory / clusters: 32 heads, 128 queries
+// over 2396 listed rows 32.8 / 24.5 us, over 1024 22.0 / 17.2; 256 over 3600 42.9 / 38.0; 512 over 1966 41.6 / 36.4; 8 heads,
+// 256 queries over 1024 25.3 / 19.6, over 2048 35.7 / 23.9.  Below the line: 8 heads, 256 over 512 18.5 / 19.4; 32 heads,
+// 512 queries over 1024 in a whole prefill call 58.0 / 59.2.  Dense, 8 heads, 256 over 4096 37.0 / 30.4.
 // A grid of q full waves and a rest has its lightest row blocks, as many as the rest, cut instead: the whole ones then
 // end after about q waves and the parts level the end.  The model is the total work over the SMs plus a third of a part
 // for the uneven end, against q + 1 waves of average jobs; list-scheduling simulations agree with it within 4 %.  Dense
@@ -383,7 +392,17 @@ static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
     for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
       const long long waves = (jobs * parts + sms - 1) / sms;
       const double cost = (double)waves * (t / parts + kPartCost);
-      if (cost < 0.97 * best) { plan.split_rb = (int)n_rb; plan.parts = parts; best = cost; }
+      if (cost < 0.97 * best) { plan.split_rb = (int)n_rb; plan.parts = parts; plan.in_cluster = false; best = cost; }
+    }
+    // the pair kernel's, in clusters
+    const int group = p->n_q_heads / p->n_kv_heads;
+    if (p->head_dim == 128 && group % 2 == 0) {
+      for (int parts = 2; parts <= 4 && parts <= tiles / 2; ++parts) {
+        const double cost = t / parts + 1.0, limit = std::min(0.95 * best, 0.97 * t - 4.5);
+        if (jobs / 2 <= (parts == 2 ? 32 : parts == 3 ? 20 : 14) && cost < limit) {
+          plan.split_rb = (int)n_rb; plan.parts = parts; plan.in_cluster = true; best = cost / 0.95;
+        }
+      }
     }
     return plan;
   }
@@ -405,9 +424,9 @@ AttnPlan attn_plan_sparse(const quoka_params* p, int budget_cap) { return attn_p
 AttnPlan attn_plan_dense(const quoka_params* p) { return attn_plan(p, (p->max_ctx_len + kKeyTile - 1) / kKeyTile + 1, false); }
 static size_t attn_split_jobs(const quoka_params* p, const AttnPlan& plan) { return (size_t)p->n_q_heads * p->batch * plan.split_rb; }
 size_t attn_split_partial_bytes(const quoka_params* p, const AttnPlan& plan) {
-  return attn_split_jobs(p, plan) * plan.parts * 2 * kSplitTileFloats * sizeof(float);
+  return plan.in_cluster ? 0 : attn_split_jobs(p, plan) * plan.parts * 2 * kSplitTileFloats * sizeof(float);
 }
-size_t attn_split_counter_bytes(const quoka_params* p, const AttnPlan& plan) { return attn_split_jobs(p, plan) * 8 * sizeof(int32_t); }
+size_t attn_split_counter_bytes(const quoka_params* p, const AttnPlan& plan) { return plan.in_cluster ? 0 : attn_split_jobs(p, plan) * 8 * sizeof(int32_t); }
 
 // The launches of an attention call: the whole row blocks, then the ones in parts.
 //
@@ -418,22 +437,22 @@ size_t attn_split_counter_bytes(const quoka_params* p, const AttnPlan& plan) { r
 // blocks' last wave leaves idle.  The whole row blocks let them start once every CTA has begun (dense) or has learnt the
 // list length (sparse: the selection is complete by then, so the parts need not wait for it), and the parts' last CTA
 // waits for the whole row blocks before it ends.
-quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const AttnPlan& plan, AttnKernel (*pick)(bool, bool),
+quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const AttnPlan& plan, AttnKernel (*pick)(bool, bool, bool),
                               const char* name, int cluster, size_t smem, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                               const CUtensorMap& tm_v, const void* k, const void* v, const int32_t* k_idx, const int32_t* k_cnt,
                               void* out, float* lse, cudaStream_t st, bool after_selection) {
-  const bool sparse = k_idx != nullptr, split = plan.split_rb > 0 && P.attn_partials;
+  const bool sparse = k_idx != nullptr, split = plan.split_rb > 0 && (P.attn_partials || plan.in_cluster);
   DevParams PP = P;
   PP.attn_row_blocks = (int)attn_row_blocks(p);
   PP.attn_split_rb = split ? plan.split_rb : 0;
   PP.attn_parts = split ? plan.parts : 1;
   const int whole = PP.attn_row_blocks - PP.attn_split_rb;
   PP.attn_after_whole = whole > 0 ? 1 : 0;
-  if (split && !after_selection &&          // (the fused call clears the counters in an earlier kernel)
+  if (split && !plan.in_cluster && !after_selection &&          // (the fused call clears the counters in an earlier kernel)
       cudaMemsetAsync(P.attn_counters, 0, attn_split_counter_bytes(p, plan), st) != cudaSuccess)
     return QUOKA_ERR_CUDA;
   for (int parts = whole > 0 ? 0 : 1; parts <= (split ? 1 : 0); ++parts) {
-    AttnKernel kernel = pick(sparse, parts != 0);
+    AttnKernel kernel = pick(sparse, parts != 0, plan.in_cluster);
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return QUOKA_ERR_CUDA;
     const bool early = parts && whole > 0 ? true : sparse && after_selection;
     cudaLaunchConfig_t cfg = {};
@@ -441,11 +460,18 @@ quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const A
     cfg.blockDim = dim3(kAttnThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = early ? 1 : 0;
+    if (early) {
+      attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (parts && plan.in_cluster) {           // (the other kernels' clusters are part of the kernel)
+      attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+      attr[cfg.numAttrs].val.clusterDim.x = (unsigned)cluster;
+      attr[cfg.numAttrs].val.clusterDim.y = (unsigned)PP.attn_parts;
+      attr[cfg.numAttrs++].val.clusterDim.z = 1;
+    }
     log_launch(name, cfg.gridDim, cfg.blockDim, smem, cluster, early);
     if (cudaLaunchKernelEx(&cfg, kernel, PP, tm_q, tm_k, tm_v, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, k_idx, k_cnt,
                            (__nv_bfloat16*)out, lse) != cudaSuccess)
@@ -466,7 +492,7 @@ bool attn_tc_supported(const quoka_params* p) {
 }
 
 template <int HALVES>
-static AttnKernel pick_attn_tc(bool sparse, bool parts) {
+static AttnKernel pick_attn_tc(bool sparse, bool parts, bool) {
   if (parts) return sparse ? attn_tc_kernel<HALVES, true, true> : attn_tc_kernel<HALVES, false, true>;
   return sparse ? attn_tc_kernel<HALVES, true, false> : attn_tc_kernel<HALVES, false, false>;
 }

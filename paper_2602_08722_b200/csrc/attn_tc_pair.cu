@@ -31,12 +31,15 @@ constexpr int kPairLoaderWarps = 3;
 constexpr uint32_t kPairSlotBytes = 16384;
 constexpr uint32_t kPairQTileBytes = 32768;
 
-template <bool SPARSE, bool SPLIT>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kAttnThreads, 1)
-attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                    const __grid_constant__ CUtensorMap tm_v, const __nv_bfloat16* __restrict__ kc,
-                    const __nv_bfloat16* __restrict__ vc, const int32_t* __restrict__ k_idx,
-                    const int32_t* __restrict__ k_cnt, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
+enum { kWhole = 0, kParts = 1, kPartsCluster = 2 };     // a row block per pair; parts merged through memory / in a cluster
+
+template <bool SPARSE, int MODE>
+__device__ __forceinline__ void
+attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
+                  const __nv_bfloat16* __restrict__ kc, const __nv_bfloat16* __restrict__ vc,
+                  const int32_t* __restrict__ k_idx, const int32_t* __restrict__ k_cnt, __nv_bfloat16* __restrict__ out,
+                  float* __restrict__ lse) {
+  constexpr bool SPLIT = MODE != kWhole;
   constexpr int D = 128;
   constexpr uint32_t S_COL[2] = {0, 128}, O_COL[2] = {256, 384};
   extern __shared__ unsigned char smem_raw[];
@@ -53,27 +56,21 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
   uint64_t* q_full = o_full + 2;                  // this CTA's Q tiles (TMA)
   uint64_t* peer_q = q_full + 1;                  // first CTA only: the second CTA's Q tiles have landed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(peer_q + 1);
+  float* part_ml = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(bars) + 512);   // [2][m | l][128], kPartsCluster
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WaitCtx wc{&abort_flag, P.status};
-  const uint32_t rank = cluster_cta_rank();                   // 0: issues the MMAs; the pair is heads (2j, 2j + 1)
+  const uint32_t cta = cluster_cta_rank();
+  const uint32_t rank = MODE == kPartsCluster ? cta & 1u : cta;   // 0: issues the MMAs; the pair is heads (2j, 2j + 1)
+  const uint32_t first = MODE == kPartsCluster ? cta & ~1u : 0u;  // the pair's first CTA
   const int s = longest_first(P, blockIdx.z), h = blockIdx.x, kv = h / P.group;
   // grid.y = row blocks (heaviest first), times the parts a row block's key tiles are cut into (SPLIT)
   const int n_parts = SPLIT ? P.attn_parts : 1;
   const int rb = (SPLIT ? P.attn_split_rb : P.attn_row_blocks) - 1 - blockIdx.y / n_parts;
   const int r0 = rb * 2 * kQTile;
   AttnGeom g = make_geom<SPARSE>(P, s, r0);
-  // SPLIT: this CTA walks the tiles [t_lo, t_hi) of the row block's sequence only and leaves, per row, a partial
-  // result (reference point, sum, un-normalised output); the part that finishes last adds the parts up.  The list
-  // length has to be known before the range is, so nothing of the walk starts before the selection has ended.
   int t_lo = 0;
-  if (SPLIT) {
-    if (SPARSE) { if (P.attn_after_whole) learn_count(g, k_cnt, s); else resolve(g, k_cnt, s); }
-    const int part = blockIdx.y % n_parts;
-    t_lo = (int)(((long long)part * g.n_known) / n_parts);
-    g.n_known = (int)(((long long)(part + 1) * g.n_known) / n_parts);
-  }
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -96,6 +93,24 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
   cluster_sync_all();                                         // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  const uint16_t both = MODE == kPartsCluster ? (uint16_t)(3u << first) : (uint16_t)3;   // this pair in the cluster
+  const auto load_q = [&]() {
+    mbar_arrive_expect_tx(q_full, 2 * kPairQTileBytes);
+    for (int x = 0; x < 2; ++x)
+      for (int hh = 0; hh < 2; ++hh)
+        tma_load_4d(q_smem + x * kPairQTileBytes + hh * 16384, &tm_q, q_full, hh * 64, r0 + x * kQTile, h, s);
+  };
+  // SPLIT: this CTA walks the tiles [t_lo, t_hi) of the row block's sequence only and leaves, per row, a partial
+  // result (reference point, sum, un-normalised output); the part that finishes last adds the parts up.  The list
+  // length has to be known before the range is, so nothing of the walk starts before the selection has ended.
+  if (SPLIT) {
+    if (warp == kMmaWarp && lane == 0) load_q();
+    if (SPARSE) { if (P.attn_after_whole) learn_count(g, k_cnt, s); else resolve(g, k_cnt, s); }
+    const int part = blockIdx.y % n_parts;
+    t_lo = (int)(((long long)part * g.n_known) / n_parts);
+    g.n_known = (int)(((long long)(part + 1) * g.n_known) / n_parts);
+  }
+
   if (!SPARSE && !SPLIT) grid_launch_dependents();
 
   if (warp < 8) {
@@ -107,8 +122,8 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
     const uint32_t s_addr = lane_addr + S_COL[x], o_addr = lane_addr + O_COL[x];
     const float scale_log2 = P.scale * 1.4426950408889634f;
-    const uint32_t p_bar0 = map_to_cta(smem_u32(&p_full[2 * x]), 0);   // the first CTA's barriers
-    const uint32_t p_bar1 = map_to_cta(smem_u32(&p_full[2 * x + 1]), 0);
+    const uint32_t p_bar0 = map_to_cta(smem_u32(&p_full[2 * x]), first);   // the first CTA's barriers
+    const uint32_t p_bar1 = map_to_cta(smem_u32(&p_full[2 * x + 1]), first);
     float m_run = -INFINITY, l_run = 0.f;
     uint32_t phase = 0;
     bool ok = true;
@@ -134,6 +149,13 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
         tc_fence_after();
         attn_store_row<D>(P, o_addr, m_run, l_run, s, h, row, out, lse);
       }
+    } else if constexpr (MODE == kPartsCluster) {
+      // every product of the CTA has been formed when both are final: the ring and the Q tiles are free
+      const bool other = x ? max(g.skip_a, t_lo) < g.n_known : g.active_b && t_lo < g.n_known;
+      bool have = ok && active_x && mbar_wait(&o_full[x], 0, wc);
+      if (have && other) have = mbar_wait(&o_full[x ^ 1], 0, wc);
+      if (have) tc_fence_after();
+      attn_part_to_smem<D>(smem, part_ml, x, row_in_tile, have, o_addr, m_run, l_run);
     } else {
       const bool have = ok && active_x && mbar_wait(&o_full[x], 0, wc);
       if (have) tc_fence_after();
@@ -278,15 +300,12 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
     cp_async_wait_all();                                      // nothing of this thread is in flight at exit
   } else if (lane == 0) {
     // ================================================================== warp 11, one thread
-    mbar_arrive_expect_tx(q_full, 2 * kPairQTileBytes);
-    for (int x = 0; x < 2; ++x)
-      for (int hh = 0; hh < 2; ++hh)
-        tma_load_4d(q_smem + x * kPairQTileBytes + hh * 16384, &tm_q, q_full, hh * 64, r0 + x * kQTile, h, s);
+    if (!SPLIT) load_q();
     bool ok = mbar_wait(q_full, 0, wc);
     if (rank != 0) {
       // ---------------------------------------------------------------- second CTA: forward "full" to the first
-      if (ok) mbar_arrive_cluster(map_to_cta(smem_u32(peer_q), 0));
-      const uint32_t peer_full0 = map_to_cta(smem_u32(peer_full), 0);
+      if (ok) mbar_arrive_cluster(map_to_cta(smem_u32(peer_q), first));
+      const uint32_t peer_full0 = map_to_cta(smem_u32(peer_full), first);
       int slot = 0;
       uint32_t phase = 0;
       for (int tile = t_lo; ok; ++tile) {
@@ -339,7 +358,7 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
             const uint64_t offb = (uint64_t)((hh * 8192 + kk * 32) >> 4);    // K: halves of 64 rows
             mma_pair_ss(tmem_base + S_COL[x], da + offa, db + offb, idesc_qk, (hh | kk) ? 1u : 0u);
           }
-        mma_pair_commit(&s_full[x]);
+        mma_pair_commit(both, &s_full[x]);
       };
       auto issue_pv = [&](int x, int vs, bool first) {
         const uint64_t dv = desc_kv + (uint64_t)((uint32_t)vs * (kPairSlotBytes >> 4));
@@ -363,7 +382,7 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
         if (ok) {
           if (part(0, t_lo)) issue_qk(0, k_slot);
           if (part(1, t_lo)) issue_qk(1, k_slot);
-          mma_pair_commit(&kv_empty[k_slot]);
+          mma_pair_commit(both, &kv_empty[k_slot]);
         }
         for (int t = t_lo; ok; ++t) {
           if (t + 1 == g.n_known && !g.resolved) { resolve(g, k_cnt, s); grid_launch_dependents(); }
@@ -374,26 +393,44 @@ attn_tc_pair_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const
           if (part(0, t)) {
             issue_pv(0, v_slot, t == max(g.skip_a, t_lo));
             if (!ok) break;
-            if (!more) mma_pair_commit(&o_full[0]);
+            if (!more) mma_pair_commit(both, &o_full[0]);
           }
           if (more && part(0, t + 1)) issue_qk(0, k_slot);
           if (part(1, t)) {
             issue_pv(1, v_slot, t == t_lo);
             if (!ok) break;
-            if (!more) mma_pair_commit(&o_full[1]);
+            if (!more) mma_pair_commit(both, &o_full[1]);
           }
-          mma_pair_commit(&kv_empty[v_slot]);
+          mma_pair_commit(both, &kv_empty[v_slot]);
           if (!more) break;
           if (part(1, t + 1)) issue_qk(1, k_slot);
-          mma_pair_commit(&kv_empty[k_slot]);
+          mma_pair_commit(both, &kv_empty[k_slot]);
         }
       }
     }
   }
   if (SPLIT && attn_last_cta()) grid_dependency_wait();       // this grid's end is the whole row blocks' end too
   tc_fence_before();
+  if constexpr (MODE == kPartsCluster) {
+    cluster_sync_all();                                       // every part's result is in its shared memory
+    if (warp < 8) attn_merge_cluster<D>(P, smem, part_ml, warp, lane, 2, (int)rank, n_parts, blockIdx.y % n_parts, r0, s, h, out, lse);
+  }
   cluster_sync_all();                                         // the other CTA's MMAs no longer read this CTA
   if (warp == kMmaWarp) tmem_dealloc_pair(tmem_base, 512);
+}
+
+#define QUOKA_PAIR_PARAMS                                                                                               \
+  DevParams P, const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,                      \
+      const __grid_constant__ CUtensorMap tm_v, const __nv_bfloat16 *__restrict__ kc, const __nv_bfloat16 *__restrict__ vc, \
+      const int32_t *__restrict__ k_idx, const int32_t *__restrict__ k_cnt, __nv_bfloat16 *__restrict__ out, float *__restrict__ lse
+template <bool SPARSE, bool SPLIT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kAttnThreads, 1) attn_tc_pair_kernel(QUOKA_PAIR_PARAMS) {
+  attn_tc_pair_body<SPARSE, SPLIT ? kParts : kWhole>(P, tm_q, tm_k, tm_v, kc, vc, k_idx, k_cnt, out, lse);
+}
+// clusters of (2, parts): the pairs of a row block's parts
+template <bool SPARSE>
+__global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_pair_cluster_kernel(QUOKA_PAIR_PARAMS) {
+  attn_tc_pair_body<SPARSE, kPartsCluster>(P, tm_q, tm_k, tm_v, kc, vc, k_idx, k_cnt, out, lse);
 }
 
 // ---------------------------------------------------------------------------------------------- host
@@ -411,8 +448,9 @@ quoka_status launch_attn_tc_pair(const quoka_params* p, const DevParams& P, cons
   }
   CUtensorMap tm_k, tm_v;
   if (!encode_kv_tensor_map(&tm_k, p, k, 64) || !encode_kv_tensor_map(&tm_v, p, v, 64)) return QUOKA_ERR_CUDA;
-  const size_t smem = 1024 + 2 * kPairQTileBytes + (size_t)kPairSlots * kPairSlotBytes + 512;
-  const auto pick = [](bool sparse, bool parts) -> AttnKernel {
+  const size_t smem = 1024 + 2 * kPairQTileBytes + (size_t)kPairSlots * kPairSlotBytes + 512 + (plan.in_cluster ? 2048 : 0);
+  const auto pick = [](bool sparse, bool parts, bool in_cluster) -> AttnKernel {
+    if (parts && in_cluster) return sparse ? attn_tc_pair_cluster_kernel<true> : attn_tc_pair_cluster_kernel<false>;
     if (parts) return sparse ? attn_tc_pair_kernel<true, true> : attn_tc_pair_kernel<false, true>;
     return sparse ? attn_tc_pair_kernel<true, false> : attn_tc_pair_kernel<false, false>;
   };

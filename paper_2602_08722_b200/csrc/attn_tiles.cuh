@@ -25,7 +25,7 @@ constexpr float kRescaleThreshold = 32.0f;   // log2 units
 // Any of the tensor-core attention kernels.
 typedef void (*AttnKernel)(DevParams, const CUtensorMap, const CUtensorMap, const CUtensorMap, const __nv_bfloat16*,
                            const __nv_bfloat16*, const int32_t*, const int32_t*, __nv_bfloat16*, float*);
-quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const AttnPlan& plan, AttnKernel (*pick)(bool, bool),
+quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const AttnPlan& plan, AttnKernel (*pick)(bool, bool, bool),
                               const char* name, int cluster, size_t smem, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                               const CUtensorMap& tm_v, const void* k, const void* v, const int32_t* k_idx, const int32_t* k_cnt,
                               void* out, float* lse, cudaStream_t st, bool after_selection);
@@ -388,6 +388,101 @@ __device__ __forceinline__ void attn_split_epilogue(const DevParams& P, int job,
       }
     }
     if (store && lse) lse[((long long)s * P.n_q + h) * P.chunk + row] = (M + log2f(l)) * 0.6931471805599453f;
+  }
+}
+
+// The same with the parts of a row block in one cluster: every part leaves its result in its own shared memory, and after a
+// cluster barrier each adds up an equal share of the rows, in part order, reading the others through distributed shared
+// memory.  The merge is bound by the latency of those reads, so a warp issues the reads of four rows of every part before it
+// uses any.  Against results through global memory, an arrival counter and a merge by the last part to arrive (five
+// dependent L2 round trips) it is about 6 us shorter; `attn_plan` has the times.
+constexpr int kPartPitch = 132;                  // floats per row: 16 bytes off a multiple of the banks
+
+// A softmax thread's row of O, its m and l.  Nothing of the CTA may still read the shared memory below `smem` + 2 tiles.
+template <int D>
+__device__ __forceinline__ void attn_part_to_smem(unsigned char* smem, float* ml, int x, int row_in_tile, bool have, uint32_t o_addr,
+                                                  float m_run, float l_run) {
+  float* row = reinterpret_cast<float*>(smem) + (x * 128 + row_in_tile) * kPartPitch;
+  if (have) {
+#pragma unroll 1
+    for (int c = 0; c < D / 32; ++c) {
+      uint32_t r[32];
+      tmem_ld32(o_addr + c * 32, r);
+      tmem_wait_ld();
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<uint4*>(row + c * 32 + 4 * i) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+    }
+  }
+  ml[x * 256 + row_in_tile] = have ? m_run : -INFINITY;
+  ml[x * 256 + 128 + row_in_tile] = have ? l_run : 0.f;
+}
+
+// One of 8 warps; the CTA of part p with this CTA's head has cluster rank p * stride + offset.  A warp takes kU rows at a
+// time, four elements of a row per lane.
+template <int D>
+__device__ __forceinline__ void attn_merge_cluster(const DevParams& P, unsigned char* smem, float* ml, int warp, int lane, int stride,
+                                                   int offset, int parts, int part, int r0, int s, int h,
+                                                   __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
+  constexpr int kU = 4, kMaxParts = 4;
+  const uint32_t o0 = smem_u32(smem), ml0 = smem_u32(ml);
+  const int rows = min(2 * kQTile, P.chunk - r0);
+  for (int j = warp * kU; part + parts * j < rows; j += 8 * kU) {
+    float m[kU], l[kU], wgt[kU], M[kU], L[kU];
+    float4 acc[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {                           // lane p holds part p's m and l
+      const int R = min(part + parts * (j + u), rows - 1), x = R >> 7, lr = R & 127;
+      const uint32_t at = map_to_cta(ml0 + (uint32_t)(x * 256 + lr) * 4u, (uint32_t)(min(lane, parts - 1) * stride + offset));
+      m[u] = ld_cluster_f(at);
+      l[u] = ld_cluster_f(at + 512u);
+      acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    // every part's elements before the first use of any (what a part without a result has there is not used)
+    float4 v[kMaxParts][kU];
+#pragma unroll
+    for (int p = 0; p < kMaxParts; ++p)
+      if (p < parts) {
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int R = min(part + parts * (j + u), rows - 1);
+          v[p][u] = ld_cluster_f4(map_to_cta(o0 + (uint32_t)(R * kPartPitch + 4 * (lane & (D / 4 - 1))) * 4u, (uint32_t)(p * stride + offset)));
+        }
+      }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      if (lane >= parts) { m[u] = -INFINITY; l[u] = 0.f; }
+      M[u] = m[u];
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) M[u] = fmaxf(M[u], __shfl_xor_sync(0xFFFFFFFFu, M[u], o));
+      M[u] = __shfl_sync(0xFFFFFFFFu, M[u], 0);
+      wgt[u] = m[u] == -INFINITY ? 0.f : ex2(m[u] - M[u]);
+      L[u] = 0.f;
+    }
+#pragma unroll
+    for (int p = 0; p < kMaxParts; ++p) {
+      if (p < parts) {
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const float w = __shfl_sync(0xFFFFFFFFu, wgt[u], p);
+          const float4 o = w != 0.f ? v[p][u] : make_float4(0.f, 0.f, 0.f, 0.f);
+          L[u] = fmaf(w, __shfl_sync(0xFFFFFFFFu, l[u], p), L[u]);
+          acc[u].x = fmaf(w, o.x, acc[u].x); acc[u].y = fmaf(w, o.y, acc[u].y);
+          acc[u].z = fmaf(w, o.z, acc[u].z); acc[u].w = fmaf(w, o.w, acc[u].w);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int R = part + parts * (j + u);
+      if (R >= rows) break;
+      const float inv = 1.f / L[u];
+      const __nv_bfloat162 a = __floats2bfloat162_rn(acc[u].x * inv, acc[u].y * inv), b = __floats2bfloat162_rn(acc[u].z * inv, acc[u].w * inv);
+      if (lane < D / 4)
+        *reinterpret_cast<uint2*>(out + (long long)s * P.o_sb + (long long)h * P.o_sh + (long long)(r0 + R) * P.o_st + 4 * lane) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      if (lse && lane == 0) lse[((long long)s * P.n_q + h) * P.chunk + r0 + R] = (M[u] + log2f(L[u])) * 0.6931471805599453f;
+    }
   }
 }
 

@@ -12,7 +12,8 @@ quoka_status launch_score_keys_tc(const quoka_params* p, const DevParams& P, con
 
 // Grids that leave SMs idle, all the time or in their last wave: the key tiles of the lightest `split_rb` row blocks of
 // every head are cut into `parts` parts, one CTA each (split_rb = 0: none).
-struct AttnPlan { int split_rb = 0, parts = 1; };
+// in_cluster: the parts of a row block are one cluster (and need no scratch)
+struct AttnPlan { int split_rb = 0, parts = 1; bool in_cluster = false; };
 AttnPlan attn_plan_sparse(const quoka_params* p, int budget_cap);
 AttnPlan attn_plan_dense(const quoka_params* p);
 // Scratch for the partial results

@@ -518,6 +518,34 @@ def test_attention_with_its_lightest_row_blocks_in_parts(n_q, n_kv, d, C, T, B):
         check_attention(f64(gp.out[0])[heads, rows], want, "bf16")
 
 
+@pytest.mark.parametrize("n_q,n_kv,C,T,B", [
+    (8, 2, 256, [4096], 2048),          # 4 clusters of eight CTAs
+    (8, 4, 257, [2500, 40], 2000),      # a row block of one row; a list shorter than a tile: parts without a tile
+    (32, 8, 130, [3000], 1500),         # 16 clusters of six
+    (32, 8, 2, [1030], 1024),           # two query rows
+    (32, 8, 400, [3000], 3000),         # 32 clusters of four, the list is the identity
+    (2, 1, 64, [1100], 1025),           # one cluster
+])
+def test_attention_parts_in_a_cluster(n_q, n_kv, C, T, B):
+    """Short grids of the pair kernel, whose parts merge through distributed shared memory: sparse (staged and fused, the
+    same bits) and dense, every row and its log-sum-exp against the oracle."""
+    gp = problem(1100 + C, batch=len(T), n_q=n_q, n_kv=n_kv, T=T, C=C, n_retain=16, kv_budget=B)
+    gp.run_staged()
+    check_chain(gp, attn_rows=400)
+    staged = gp.out.clone()
+    gp.out.zero_()
+    api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+    torch.cuda.synchronize()
+    assert torch.equal(gp.out, staged)
+    api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, gp.lse, gp.ws)
+    torch.cuda.synchronize()
+    for s in range(gp.b):
+        q, k, v, t = gp.oracle_inputs(s)
+        dense, lse = O.dense_chunk_attention(q, k, v, t)
+        check_attention(f64(gp.out[s]), dense, "bf16")
+        assert np.abs(f64(gp.lse[s]) - lse).max() <= 2e-3
+
+
 @pytest.mark.parametrize("paged", [False, True])
 @pytest.mark.parametrize("T,C,B,n_q,n_kv,d,n_retain", [
     (63, 2, 40, 4, 2, 128, 1),          # fewer keys than a tile, two query rows
