@@ -3,20 +3,26 @@
 // rank_queries : a thread-block cluster of 2 / 4 / 8 CTAs (by chunk length, about 256 rows per CTA) per
 //                (sequence, query head); each CTA owns a contiguous slice of the head's C query rows.
 //                Pass 1 brings the slice into shared memory with 16-byte cp.async in eight groups and sums
-//                the columns group by group as they land (a slice beyond the staging limit is re-read
-//                from L2 instead); the CTAs' shares of the mean query are added across the cluster
+//                the columns group by group as they land (of a longer slice the first rows; the rest is summed
+//                from registers); the CTAs' shares of the mean query are added across the cluster
 //                through distributed shared memory in a fixed order.  Pass 2 computes CosSim(q_r, M) for
-//                every row of the slice (two lanes per row), packs (order code of the cosine, position)
-//                into one 64-bit key, sorts 32-key runs in registers (bitonic network over shuffles) and
-//                merges the runs by counting (branch-free binary searches, keys are unique).  Each CTA
+//                every row of the slice (two lanes per two rows; the rows that were not kept come again from L2,
+//                a block of rows at a time) as an order code, and puts the slice in order: up to 256 rows by
+//                counting, for every row, the rows before it; more by 32-key runs sorted in registers
+//                (bitonic network over shuffles) and merged by branch-free binary searches.  Each CTA
 //                then copies the first codes of its peers' sorted slices into local shared memory and
 //                places each of its N smallest by global rank: own rank + number of smaller codes in
 //                every peer.  The N lowest cosines come out in ascending order, equal cosines by position.
+//                Bound by latency (a CTA's slice takes 2 us to arrive, four cluster barriers and the steps between
+//                them another 4) and, with two CTAs per SM, by shared memory and instruction issue.  Against every
+//                slice sorted in runs, M read once per row and long slices read again a row per lane pair, ranking and
+//                aggregation took before / now: 8 heads x 256 rows 12.4 / 10.3 us (f32 13.1 / 10.8), 32 x 512
+//                14.4 / 12.7, 32 x 2048 20.5 / 19.1, 256 x 1024 54.2 / 49.4, 32 x 4096 34.9 / 28.9.
 // aggregate    : one warp per (sequence, KV head, rank j): mean over the G heads of the group of
 //                their j-th retained query, each divided by its own norm; one rounding to dtype.
 #include <cooperative_groups.h>
 
-#include <type_traits>
+#include <algorithm>
 
 #include "common.cuh"
 #include "qbar.cuh"
@@ -27,9 +33,13 @@ namespace quoka {
 
 constexpr int kRankThreads = 512;
 constexpr int kRankCluster = 8;
-// A slice larger than this is not kept in shared memory but re-read from L2 in pass 2: two CTAs must still fit an
-// SM (with 128 KB slices, chunk 4096, one CTA per SM meant two waves of the grid and a fifth more time).
-constexpr size_t kRankStageLimit = 84 * 1024;
+// Shared memory of a CTA, where its sort leaves room for any rows at all: two CTAs must fit an SM (with 128 KB slices,
+// chunk 4096, one CTA per SM meant two waves of the grid and a fifth more time).
+constexpr size_t kRankSmem = 112 * 1024;
+// Slices up to this many rows are ordered by counting: quadratic, but with a handful of dependent steps (runs and
+// merge / counting, cycles of a CTA with two on the SM: 256 rows 5300 / 4000; alone on it, 128 rows 2700 / 1300).  512 rows
+// would count four times as long, the runs and their merge take 8500.
+constexpr int kRankCount = 256;
 
 template <typename T> struct Raw8;                // 8 consecutive elements as 16-byte words
 template <> struct Raw8<__nv_bfloat16> { uint4 w[1]; };
@@ -55,7 +65,7 @@ __device__ __forceinline__ void raw_to_f32(const Raw8<T>& r, float (&x)[8]) {
 template <typename T, int D, int CL>
 __global__ void __launch_bounds__(kRankThreads, 2) rank_queries_kernel(DevParams P, const T* __restrict__ q,
                                                                      int32_t* __restrict__ q_idx, int rpc, int n_sort,
-                                                                     int staged, int m_peer) {
+                                                                     int n_stage, int m_peer) {
   // The first kernel of a fused call is launched early as well (its launch runs under the tail of whatever is before it on
   // the stream); nothing is read or written, and no later kernel of the call starts, before that has completed.
   grid_dependency_wait();
@@ -69,10 +79,9 @@ __global__ void __launch_bounds__(kRankThreads, 2) rank_queries_kernel(DevParams
   unsigned long long* sorted = keys + n_sort;                                               // [n_sort] the sorted slice
   float* red = reinterpret_cast<float*>(smem_raw + (size_t)n_sort * 16);                    // [RPI][D]
   unsigned long long* peer_keys = reinterpret_cast<unsigned long long*>(red + RPI * D);     // [CL - 1][m_peer]
-  uint4* rows = reinterpret_cast<uint4*>(peer_keys + (((size_t)(CL - 1) * m_peer + 1) & ~(size_t)1));   // [rpc][LG][NW]
+  uint4* rows = reinterpret_cast<uint4*>(peer_keys + (((size_t)(CL - 1) * m_peer + 1) & ~(size_t)1));   // [n_stage][LG][NW]
   __shared__ float part[D];                 // this CTA's share of the column sums
-  __shared__ __align__(16) float M[D];
-  __shared__ float Mnorm;
+  __shared__ __align__(16) float M[D + 4];  // the second half 16 bytes on: the halves of a row read different banks
 
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
@@ -89,64 +98,71 @@ __global__ void __launch_bounds__(kRankThreads, 2) rank_queries_kernel(DevParams
   const int lo = min(C, rank * rpc), hi = min(C, lo + rpc);
   const int n_loc = hi - lo;
 
-  // ---- pass 1: the slice goes to shared memory with every 16-byte copy in flight at once, committed in 8
-  // groups of rows; the column sums are taken group by group as the copies land, so the arithmetic runs under
-  // the HBM transfer
-  const int n_iter = (n_loc + RPI - 1) / RPI;                // 32/64-row trips over the slice
-  const int grp_rows = ((n_iter + 7) / 8) * RPI;             // rows per copy group
-  if (staged) {
-    constexpr int WPR = LG * NW;                             // 16-byte words per row
-    constexpr int EPW = 16 / (int)sizeof(T);                 // elements per word
-    const uint32_t rows_s = (uint32_t)__cvta_generic_to_shared(rows);
-#pragma unroll 1
-    for (int gi = 0; gi < 8; ++gi) {
-      const int w_lo = min(n_loc, gi * grp_rows) * WPR, w_hi = min(n_loc, (gi + 1) * grp_rows) * WPR;
-      for (int w = w_lo + tid; w < w_hi; w += kRankThreads) {
-        const int r = w / WPR, c = w % WPR;
-        const T* src = qh + (long long)(lo + r) * P.q_st + c * EPW;
-        // word c of row r lives in slot c ^ (r & 7): both passes then read shared memory without bank conflicts
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(rows_s + (uint32_t)(r * WPR + (c ^ (r & 7))) * 16u), "l"(src) : "memory");
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
+  constexpr int WPR = LG * NW;                               // 16-byte words per row
+  constexpr int EPW = 16 / (int)sizeof(T);                   // elements per word
+  constexpr int HW = WPR / 2;                                // words per half row
+  // word c of row r lives in slot c ^ (r & 7): both passes then read shared memory without bank conflicts
+  const auto slot = [](int r, int c) { return r * WPR + (c ^ (r & 7)); };
+  const uint32_t rows_s = (uint32_t)__cvta_generic_to_shared(rows);
+  const auto copy_rows = [&](int first, int r_lo, int r_hi) {     // rows [r_lo, r_hi) of the buffer, which starts at row `first`
+    for (int w = r_lo * WPR + tid; w < r_hi * WPR; w += kRankThreads) {
+      const int r = w / WPR, c = w % WPR;
+      const T* src = qh + (long long)(lo + first + r) * P.q_st + c * EPW;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(rows_s + (uint32_t)slot(r, c) * 16u), "l"(src) : "memory");
     }
-  }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  // ---- pass 1: the slice's first n_stage rows go to shared memory with every 16-byte copy in flight at once, committed
+  // in 8 groups of rows; the column sums are taken group by group as the copies land, so the arithmetic runs under
+  // the HBM transfer
+  const int n_kept = min(n_loc, n_stage);
+  const int n_iter = (n_kept + RPI - 1) / RPI;               // 32/64-row trips over the kept rows
+  const int grp_rows = ((n_iter + 7) / 8) * RPI;             // rows per copy group
+#pragma unroll 1
+  for (int gi = 0; gi < 8; ++gi) copy_rows(0, min(n_kept, gi * grp_rows), min(n_kept, (gi + 1) * grp_rows));
   float acc[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+  const auto add_row = [&](const Raw8<T>& raw, bool live) {
+    float x[8];
+    raw_to_f32<T>(raw, x);
+    const float f = live ? 1.f : 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = fmaf(x[i], f, acc[i]);
+  };
 #pragma unroll
   for (int gi = 0; gi < 8; ++gi) {
-    if (staged) {
-      switch (gi) {                                          // all but the 7 - gi newest groups have landed
-        case 0: asm volatile("cp.async.wait_group 7;" ::: "memory"); break;
-        case 1: asm volatile("cp.async.wait_group 6;" ::: "memory"); break;
-        case 2: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
-        case 3: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
-        case 4: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
-        case 5: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
-        case 6: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
-        default: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
-      }
-      __syncthreads();
+    const int g_lo = gi * grp_rows, g_hi = min(n_kept, (gi + 1) * grp_rows);
+    if (g_lo >= n_kept) break;
+    switch (gi) {                                            // all but the 7 - gi newest groups have landed
+      case 0: asm volatile("cp.async.wait_group 7;" ::: "memory"); break;
+      case 1: asm volatile("cp.async.wait_group 6;" ::: "memory"); break;
+      case 2: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
+      case 3: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+      case 4: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+      case 5: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
+      case 6: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
+      default: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
     }
-    const int g_lo = min(n_loc, gi * grp_rows), g_hi = min(n_loc, (gi + 1) * grp_rows);
+    __syncthreads();
     for (int r0 = g_lo; r0 < g_hi; r0 += RPI) {
-      const int r = r0 + row_slot;
+      const int r = r0 + row_slot, rc = min(r, n_kept - 1);  // clamped: no branch around the loads
       Raw8<T> raw;
-      const int rc = min(r, n_loc - 1);                      // clamped: no branch around the loads
-      if (staged) {
 #pragma unroll
-        for (int w = 0; w < NW; ++w) raw.w[w] = rows[(size_t)rc * (LG * NW) + ((lane_in_row * NW + w) ^ (rc & 7))];
-      } else {
-        const uint4* src = reinterpret_cast<const uint4*>(qh + (long long)(lo + rc) * P.q_st + lane_in_row * 8);
-#pragma unroll
-        for (int w = 0; w < NW; ++w) raw.w[w] = __ldg(src + w);
-      }
-      float x[8];
-      raw_to_f32<T>(raw, x);
-      const float live = r < n_loc ? 1.f : 0.f;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) acc[i] = fmaf(x[i], live, acc[i]);
+      for (int w = 0; w < NW; ++w) raw.w[w] = rows[slot(rc, lane_in_row * NW + w)];
+      add_row(raw, r < n_kept);
     }
+  }
+  // (n_stage is a multiple of RPI where it is less than the slice: the sums are in row order either way)
+#pragma unroll 4
+  for (int r0 = n_stage; r0 < n_loc; r0 += RPI) {
+    const int r = r0 + row_slot, rc = min(r, n_loc - 1);
+    const uint4* src = reinterpret_cast<const uint4*>(qh + (long long)(lo + rc) * P.q_st + lane_in_row * 8);
+    Raw8<T> raw;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) raw.w[w] = __ldg(src + w);
+    add_row(raw, r < n_loc);
   }
 #pragma unroll
   for (int i = 0; i < 8; ++i) red[row_slot * D + lane_in_row * 8 + i] = acc[i];
@@ -161,117 +177,166 @@ __global__ void __launch_bounds__(kRankThreads, 2) rank_queries_kernel(DevParams
     float sum = 0.f;
 #pragma unroll
     for (int r = 0; r < CL; ++r) sum += cluster.map_shared_rank(part, r)[tid];   // fixed order
-    M[tid] = sum / (float)C;
+    M[tid + (tid >= D / 2 ? 4 : 0)] = sum / (float)C;
   }
   __syncthreads();
-  if (tid < 32) {
-    float p = 0.f;
-    for (int x = tid; x < D; x += 32) p += M[x] * M[x];
-    p = warp_sum(p);
-    if (tid == 0) Mnorm = fmaxf(sqrtf(p), kNormEps);
-  }
-  __syncthreads();
+  const int lane = tid & 31, wid = tid >> 5;
+  float mn = 0.f;                                            // |M|, in every warp
+  for (int x = lane; x < D; x += 32) { const float m = M[x + (x >= D / 2 ? 4 : 0)]; mn += m * m; }
+  mn = fmaxf(sqrtf(warp_sum(mn)), kNormEps);
 
-  // ---- pass 2: cosine of every row of the slice to M, packed as (order code << 32 | position).  Two adjacent
-  // lanes take one row (half of its 16-byte words each, the row's norm and its dot product with M in the same
-  // sweep, M read from shared memory as a broadcast); one shuffle joins the halves.
-  {
-    constexpr int WPR = LG * NW;                             // 16-byte words per row
-    constexpr int EPW = 16 / (int)sizeof(T);                 // elements per word
-    constexpr int HW = WPR / 2;                              // words per half row
-    const int half = tid & 1;
-    const float mn = Mnorm;
-    auto sweep = [&](auto from_smem) {                       // the staged / re-read choice is made once, not per word
-    for (int r0 = 0; r0 < n_sort; r0 += kRankThreads / 2) {
-      const int r = r0 + (tid >> 1);
-      const int rc = max(min(r, n_loc - 1), 0);              // clamped (an empty slice reads row 0 / the last row)
-      const uint4* grow = reinterpret_cast<const uint4*>(qh + (long long)min(lo + rc, C - 1) * P.q_st);
-      float dot = 0.f, nn = 0.f;
-#pragma unroll 4      // all eight words at once made the compiler spill
+  // ---- pass 2: cosine of every row of the slice to M as an order code.  A warp takes 32 rows, lanes l and l + 16 the
+  // halves of rows l and l + 16 (the rows' norms and dot products with M in the same sweep, M read from shared memory as a
+  // broadcast, which is two thirds of the words read with one row at a time); one shuffle joins the halves.
+  const bool count = n_sort <= kRankCount;
+  uint32_t* codes = reinterpret_cast<uint32_t*>(keys);       // [n_sort], with the counts [n_sort] behind them
+  uint32_t* counts = codes + n_sort;
+  const int half = lane >> 4;
+  for (int first = 0; first == 0 || first < n_loc; first += n_stage) {
+    if (first > 0) {                                         // the next rows, from L2
+      __syncthreads();
+      copy_rows(first, 0, min(n_loc - first, n_stage));
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+    }
+    // (the last block also writes the padding up to n_sort)
+    const int end = first + n_stage < n_loc ? first + n_stage : n_sort;
+    for (int r0 = first + wid * 32; r0 < end; r0 += kRankThreads) {
+      const uint4* row[2];
+      int x7[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {                          // clamped (an empty slice reads what is there)
+        const int rc = max(min(r0 + 16 * u + (lane & 15) - first, min(n_loc - first, n_stage) - 1), 0);
+        row[u] = rows + rc * WPR;
+        x7[u] = rc & 7;
+      }
+      float dot[2] = {0.f, 0.f}, nn[2] = {0.f, 0.f};
+#pragma unroll 2
       for (int i = 0; i < HW; ++i) {
         const int c = half * HW + i;
-        uint4 wv;
-        if constexpr (decltype(from_smem)::value) wv = rows[(size_t)rc * WPR + (c ^ (rc & 7))];
-        else wv = __ldg(grow + c);
-        float x[EPW];
-        if constexpr (sizeof(T) == 2) {
-          const uint32_t ww[4] = {wv.x, wv.y, wv.z, wv.w};
+        uint4 wv[2];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) { x[2 * j] = __uint_as_float(ww[j] << 16); x[2 * j + 1] = __uint_as_float(ww[j] & 0xFFFF0000u); }
-        } else {
-          x[0] = __uint_as_float(wv.x); x[1] = __uint_as_float(wv.y); x[2] = __uint_as_float(wv.z); x[3] = __uint_as_float(wv.w);
-        }
+        for (int u = 0; u < 2; ++u) wv[u] = row[u][c ^ x7[u]];
 #pragma unroll
         for (int j = 0; j < EPW; j += 4) {
-          const float4 mv = *reinterpret_cast<const float4*>(&M[c * EPW + j]);
-          dot = fmaf(x[j], mv.x, dot); dot = fmaf(x[j + 1], mv.y, dot);
-          dot = fmaf(x[j + 2], mv.z, dot); dot = fmaf(x[j + 3], mv.w, dot);
-          nn = fmaf(x[j], x[j], nn); nn = fmaf(x[j + 1], x[j + 1], nn);
-          nn = fmaf(x[j + 2], x[j + 2], nn); nn = fmaf(x[j + 3], x[j + 3], nn);
+          const float4 mv = *reinterpret_cast<const float4*>(&M[half * (D / 2 + 4) + i * EPW + j]);
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            float x[4];
+            if constexpr (sizeof(T) == 2) {
+              const uint32_t w0 = j ? wv[u].z : wv[u].x, w1 = j ? wv[u].w : wv[u].y;
+              x[0] = __uint_as_float(w0 << 16); x[1] = __uint_as_float(w0 & 0xFFFF0000u);
+              x[2] = __uint_as_float(w1 << 16); x[3] = __uint_as_float(w1 & 0xFFFF0000u);
+            } else {
+              x[0] = __uint_as_float(wv[u].x); x[1] = __uint_as_float(wv[u].y); x[2] = __uint_as_float(wv[u].z); x[3] = __uint_as_float(wv[u].w);
+            }
+            dot[u] = fmaf(x[0], mv.x, dot[u]); dot[u] = fmaf(x[1], mv.y, dot[u]);
+            dot[u] = fmaf(x[2], mv.z, dot[u]); dot[u] = fmaf(x[3], mv.w, dot[u]);
+            nn[u] = fmaf(x[0], x[0], nn[u]); nn[u] = fmaf(x[1], x[1], nn[u]);
+            nn[u] = fmaf(x[2], x[2], nn[u]); nn[u] = fmaf(x[3], x[3], nn[u]);
+          }
         }
       }
-      dot += __shfl_xor_sync(0xFFFFFFFFu, dot, 1);
-      nn += __shfl_xor_sync(0xFFFFFFFFu, nn, 1);
-      if (half == 0 && r < n_sort) {
-        unsigned long long code = ~0ull;                    // padding sorts last
-        if (r < n_loc) {
-          const float c = dot / (fmaxf(sqrtf(nn), kNormEps) * mn);
-          code = ((unsigned long long)float_order_key(c) << 32) | (unsigned)(lo + r);
-        }
-        keys[r] = code;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        dot[u] += __shfl_xor_sync(0xFFFFFFFFu, dot[u], 16);
+        nn[u] += __shfl_xor_sync(0xFFFFFFFFu, nn[u], 16);
+      }
+      // the first half's lanes write the first 16 rows, the second half's the others
+      const int r = r0 + lane;
+      const float d = half ? dot[1] : dot[0], n = half ? nn[1] : nn[0];
+      if (r < end) {
+        const uint32_t code = r < n_loc ? float_order_key(d / (fmaxf(sqrtf(n), kNormEps) * mn)) : 0xFFFFFFFFu;
+        if (count) { codes[r] = code; counts[r] = 0; }
+        else keys[r] = r < n_loc ? ((unsigned long long)code << 32) | (unsigned)(lo + r) : ~0ull;    // padding sorts last
       }
     }
-    };
-    if (staged) sweep(std::true_type{}); else sweep(std::false_type{});
   }
   __syncthreads();
 
-  // ---- sort of the slice, ascending.  Each warp sorts 32-key runs in registers (bitonic network over
-  // shuffles, no block barriers); then every key finds its place by counting the smaller keys of the other
-  // runs with branch-free binary searches (keys are unique) and is scattered to `sorted`.
-  const int lane = tid & 31, wid = tid >> 5;
-  const int n_runs = n_sort >> 5;
-  for (int run = wid; run < n_runs; run += kRankThreads / 32) {
-    unsigned long long v = keys[run * 32 + lane];
+  // ---- sort of the slice, ascending, equal codes by position.
+  if (count) {
+    // A warp holds 32 rows, one per lane, and counts those of 32 other rows (read as a broadcast) that come before each:
+    // two instructions a pair, the borrow of (other - mine) taken off the count.
+    const int log_blk = __popc(n_sort - 1) - 5, n_blk = (n_loc + 31) >> 5;
+    for (int e = wid; e < 1 << (2 * log_blk); e += kRankThreads / 32) {
+      const int mine = e & ((1 << log_blk) - 1), other = e >> log_blk;
+      if (max(mine, other) >= n_blk) continue;
+      const uint32_t code = codes[mine * 32 + lane];
+      const uint4* oc = reinterpret_cast<const uint4*>(codes + other * 32);
+      uint32_t n0 = 0, n1 = 0;                               // minus the number of smaller codes
+      const auto below = [](uint32_t& n, uint32_t a, uint32_t b) {   // n -= a < b
+        uint32_t t;
+        asm("sub.cc.u32 %0, %2, %3;\n\tsubc.u32 %1, %1, 0;" : "=r"(t), "+r"(n) : "r"(a), "r"(b));
+      };
+      if (other < mine) {                                    // rows before mine: n = 32 - those with a larger code
 #pragma unroll
-    for (int k = 2; k <= 32; k <<= 1) {
+        for (int j = 0; j < 8; ++j) {
+          const uint4 o = oc[j];
+          below(n0, code, o.x); below(n1, code, o.y); below(n0, code, o.z); below(n1, code, o.w);
+        }
+        n0 = 32u + (n0 + n1);
+      } else {
 #pragma unroll
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, v, j);
-        const bool up = (lane & k) == 0, lower = (lane & j) == 0;
-        const bool take_min = up == lower;
-        v = take_min ? (v < o ? v : o) : (v < o ? o : v);
+        for (int j = 0; j < 8; ++j) {
+          const uint4 o = oc[j];
+          below(n0, o.x, code); below(n1, o.y, code); below(n0, o.z, code); below(n1, o.w, code);
+        }
+        n0 = 0u - (n0 + n1);
+        if (other == mine && __reduce_add_sync(0xFFFFFFFFu, n0) != 32 * 31 / 2)      // not all different
+          n0 += __popc(__match_any_sync(0xFFFFFFFFu, code) & ((1u << lane) - 1));    // the equal ones before
       }
+      atomicAdd(&counts[mine * 32 + lane], n0);
     }
-    keys[run * 32 + lane] = v;
-  }
-  for (int i = tid; i < n_sort; i += kRankThreads) sorted[i] = ~0ull;   // slots the padding keys do not reach
-  __syncthreads();
-  for (int i = tid; i < n_sort; i += kRankThreads) {
-    const unsigned long long key = keys[i];
-    const int my_run = i >> 5;
-    int rk = i & 31;
+    __syncthreads();
+    for (int i = tid; i < n_sort; i += kRankThreads)
+      sorted[i < n_loc ? counts[i] : i] = i < n_loc ? ((unsigned long long)codes[i] << 32) | (unsigned)(lo + i) : ~0ull;
+  } else {
+    // Each warp sorts 32-key runs in registers (no block barriers); then every key finds its place by counting the smaller
+    // keys of the other runs with branch-free binary searches (keys are unique) and is scattered to `sorted`.
+    const int n_runs = n_sort >> 5;
+    for (int run = wid; run < n_runs; run += kRankThreads / 32) {
+      unsigned long long v = keys[run * 32 + lane];
+#pragma unroll
+      for (int k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+          const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, v, j);
+          const bool up = (lane & k) == 0, lower = (lane & j) == 0;
+          const bool take_min = up == lower;
+          v = take_min ? (v < o ? v : o) : (v < o ? o : v);
+        }
+      }
+      keys[run * 32 + lane] = v;
+    }
+    for (int i = tid; i < n_sort; i += kRankThreads) sorted[i] = ~0ull;   // slots the padding keys do not reach
+    __syncthreads();
+    for (int i = tid; i < n_sort; i += kRankThreads) {
+      const unsigned long long key = keys[i];
+      const int my_run = i >> 5;
+      int rk = i & 31;
 #pragma unroll 1
-    for (int run0 = 0; run0 < n_runs; run0 += 8) {        // eight searches side by side: their loads overlap
-      int pos[8];
+      for (int run0 = 0; run0 < n_runs; run0 += 8) {        // eight searches side by side: their loads overlap
+        int pos[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) pos[u] = 0;
+        for (int u = 0; u < 8; ++u) pos[u] = 0;
 #pragma unroll
-      for (int step = 16; step > 0; step >>= 1) {
+        for (int step = 16; step > 0; step >>= 1) {
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int run = min(run0 + u, n_runs - 1);
+            pos[u] += keys[run * 32 + pos[u] + step - 1] < key ? step : 0;
+          }
+        }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const int run = min(run0 + u, n_runs - 1);
-          pos[u] += keys[run * 32 + pos[u] + step - 1] < key ? step : 0;
+          pos[u] += keys[run * 32 + pos[u]] < key ? 1 : 0;
+          rk += (run0 + u < n_runs && run != my_run) ? pos[u] : 0;
         }
       }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int run = min(run0 + u, n_runs - 1);
-        pos[u] += keys[run * 32 + pos[u]] < key ? 1 : 0;
-        rk += (run0 + u < n_runs && run != my_run) ? pos[u] : 0;
-      }
+      sorted[rk] = key;                                     // padding keys are equal: they may collide, all ~0
     }
-    sorted[rk] = key;                                     // padding keys are equal: they may collide, all ~0
   }
   cluster.sync();                                         // every slice is sorted
 
@@ -284,6 +349,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) rank_queries_kernel(DevParams
     const int r = pr + (pr >= rank ? 1 : 0);
     peer_keys[e] = cluster.map_shared_rank(sorted, r)[j];
   }
+  cluster.barrier_arrive();                               // done with the peers' shared memory
   __syncthreads();
   const int n_cand = min(N, n_loc);
   for (int li = tid; li < n_cand; li += kRankThreads) {
@@ -304,7 +370,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) rank_queries_kernel(DevParams
     }
     if (rk < N) out[rk] = (int32_t)(key & 0xFFFFFFFFull);
   }
-  cluster.sync();                                         // my keys stay mapped until every peer is done
+  cluster.barrier_wait();                                 // my keys stay mapped until every peer is done
 }
 
 template <typename T, int D>
@@ -346,16 +412,20 @@ static cudaError_t launch_rank_t(const DevParams& P, const void* q, int32_t* q_i
   int rpc = (P.chunk + CL - 1) / CL;
   int n_sort = 32;
   while (n_sort < rpc) n_sort <<= 1;
-  const size_t row_bytes = (size_t)rpc * D * sizeof(T);
   int m_peer = 1;
   while (m_peer < P.n_sel && m_peer < n_sort) m_peer <<= 1;
+  const size_t row_bytes = (size_t)D * sizeof(T);
   const size_t fixed = (size_t)n_sort * 16 + (size_t)RPI * D * 4 + (((size_t)(CL - 1) * m_peer + 1) & ~(size_t)1) * 8;
-  const int staged = fixed + row_bytes <= kRankStageLimit + 48 * 1024 && row_bytes <= kRankStageLimit ? 1 : 0;
-  const size_t smem = fixed + (staged ? row_bytes : 0);
+  // the rows that stay in shared memory: all, or as many whole sweeps of pass 2 (of pass 1) as there is room for
+  int n_stage = fixed < kRankSmem ? (int)((kRankSmem - fixed) / row_bytes) : 0;
+  if (n_stage >= rpc) n_stage = rpc;
+  else if (n_stage >= kRankThreads / 2) n_stage -= n_stage % (kRankThreads / 2);
+  else n_stage = std::max(n_stage - n_stage % RPI, RPI);
+  const size_t smem = fixed + (size_t)n_stage * row_bytes;
   cudaError_t e = cudaFuncSetAttribute(rank_queries_kernel<T, D, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return launch_kernel("rank_queries", rank_queries_kernel<T, D, CL>, dim3(P.batch * P.n_q * CL), dim3(kRankThreads), smem, st, CL, chained, P,
-                       (const T*)q, q_idx, rpc, n_sort, staged, m_peer);
+                       (const T*)q, q_idx, rpc, n_sort, n_stage, m_peer);
 }
 
 // A cluster per (sequence, head), sized so that a CTA's slice is about 256 rows: shorter slices only multiply the

@@ -5,7 +5,7 @@ import torch
 
 from oracle import quoka_oracle as O
 from paper_2602_08722_b200 import api, synth
-from tests.parity import GpuProblem, attention_bound, check_attention, check_chain, f64, stratified_rows
+from tests.parity import GpuProblem, attention_bound, check_attention, check_chain, check_query_ranks, f64, stratified_rows
 
 pytestmark = pytest.mark.gpu
 
@@ -544,6 +544,36 @@ def test_attention_parts_in_a_cluster(n_q, n_kv, C, T, B):
         dense, lse = O.dense_chunk_attention(q, k, v, t)
         check_attention(f64(gp.out[s]), dense, "bf16")
         assert np.abs(f64(gp.lse[s]) - lse).max() <= 2e-3
+
+
+@pytest.mark.parametrize("C,n_retain,d,dtype", [
+    (2, 1, 128, "bf16"),                # one row per CTA
+    (65, 64, 64, "f32"),                # counted: a block of one row
+    (500, 200, 128, "bf16"),            # 250 rows per CTA, the last block not full
+    (1025, 130, 64, "bf16"),            # clusters of eight with a short last slice
+    (2047, 300, 128, "f32"),            # 256 rows, more than shared memory keeps; still counted
+    (2049, 40, 128, "bf16"),            # 257 rows: sorted in runs
+    (4099, 513, 128, "bf16"),           # 513 rows, kept in part
+])
+def test_query_ranks_at_the_edges_of_a_slice(C, n_retain, d, dtype):
+    """Slices that are counted, sorted, kept in part: the ranks of random rows against the oracle, and of rows that have one
+    of two values (equal cosines go by position) exactly."""
+    gp = problem(1200 + C, n_q=4, n_kv=2, d=d, T=40, C=C, dtype=dtype, n_retain=n_retain, kv_budget=8)
+    api.quoka_select_queries(gp.p, gp.q, gp.q_idx, gp.qbar, gp.ws)
+    torch.cuda.synchronize()
+    _, cos = O.select_queries(f64(gp.q[0]), n_retain)
+    check_query_ranks(gp.q_idx[0].cpu().numpy(), cos, n_retain)
+    pick = np.random.default_rng(C).random(C) < 0.3
+    q2 = gp.q[:, :, :1].expand_as(gp.q).clone()
+    q2[:, :, torch.from_numpy(np.nonzero(pick)[0]).cuda()] = -gp.q[:, :, 1:2]
+    api.quoka_select_queries(gp.p, q2, gp.q_idx, gp.qbar, gp.ws)
+    torch.cuda.synchronize()
+    mean = f64(q2[0]).mean(axis=1)
+    for h in range(4):
+        c = f64(q2[0, h]) @ mean[h] / np.linalg.norm(f64(q2[0, h]), axis=1)
+        low = c < 0.5 * (c.min() + c.max())
+        want = np.concatenate([np.nonzero(low)[0], np.nonzero(~low)[0]])[:n_retain] if pick.any() and not pick.all() else np.arange(n_retain)
+        assert np.array_equal(gp.q_idx[0, h].cpu().numpy(), want)
 
 
 @pytest.mark.parametrize("paged", [False, True])
