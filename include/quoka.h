@@ -228,8 +228,9 @@ quoka_status quoka_append_kv(const quoka_params* p, const void* k_new, const voi
  *   - Problems whose intermediates exceed QUOKA_STATIC_SCRATCH_BYTES are refused with
  *     QUOKA_ERR_STATIC_LIMIT before anything is launched (for scale: 32 q / 8 kv heads, d 128,
  *     131072 cached rows, N_Q 256 needs about 5.1 MiB; a batch of 8 at 65536 rows does not fit).
- *     The array has no room for the split attention kernel's partial results: small grids run
- *     unsplit here, so on those the output may differ from quoka_prefill_chunk's in the last bits.
+ *     The array has no room for the split attention kernel's partial results: grids whose parts
+ *     would pass them through memory run unsplit here, so on those the output may differ from
+ *     quoka_prefill_chunk's in the last bits.
  *   - The first call on each device looks up the array's device address (that device must be
  *     current); make that first call before any stream capture begins.
  *   - All calls in the process share the one array per device, and it keeps the previous call's

@@ -40,6 +40,7 @@ struct DevParams {
   int n_attn_counters;
   // plan of the attention call at hand (set by the launcher): the row blocks [0, attn_split_rb) of every head are cut
   // into attn_parts parts each, in a launch of their own after the one of the heavier row blocks above them, if any
+  int rank_heads;      // (sequence, query head) pairs of the whole problem: the ranking kernel's slices go by them
   int attn_one_part;   // f32 attention: keep row blocks whole (a slice of a problem that has waves enough)
   int attn_row_blocks, attn_split_rb, attn_parts, attn_after_whole;
 };

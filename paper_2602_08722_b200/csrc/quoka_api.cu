@@ -147,6 +147,7 @@ static DevParams make_dev(const quoka_params* p, void* ws, const Workspace& w) {
   P.k_inv_norm = p->k_inv_norm;
   P.kv_rows = p->kv_rows;
   P.attn_partials = w.attn_partials; P.attn_counters = w.attn_counters; P.n_attn_counters = w.n_attn_counters;
+  P.rank_heads = p->batch * p->n_q_heads;
   P.attn_one_part = 0; P.attn_row_blocks = 0; P.attn_split_rb = 0; P.attn_parts = 1; P.attn_after_whole = 0;
   return P;
 }
@@ -468,6 +469,7 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
     const Workspace w = carve(&sub, ws, /*with_split=*/false);
     DevParams P = make_dev(&sub, ws, w);
     P.attn_partials = whole.attn_partials; P.attn_counters = whole.attn_counters; P.n_attn_counters = whole.n_attn_counters;
+    P.rank_heads = p->batch * p->n_q_heads;
     P.attn_one_part = 1;
     st = run_prefill(&sub, P, w, plan, static_cast<char*>(q_dev) + (size_t)kv0 * G * head_bytes,
                      static_cast<char*>(k_cache) + (size_t)kv0 * p->kv_stride_h * es,

@@ -1,6 +1,6 @@
 // Query sub-selection, normalisation and GQA pre-aggregation (Algorithm 1, first two blocks).
 //
-// rank_queries : a thread-block cluster of 2 / 4 / 8 CTAs (by chunk length, about 256 rows per CTA) per
+// rank_queries : a thread-block cluster of 2 / 4 / 8 CTAs (slices of 64 to 512 rows, `launch_rank_d`) per
 //                (sequence, query head); each CTA owns a contiguous slice of the head's C query rows.
 //                Pass 1 brings the slice into shared memory with 16-byte cp.async in eight groups and sums
 //                the columns group by group as they land (of a longer slice the first rows; the rest is summed
@@ -17,7 +17,8 @@
 //                them another 4) and, with two CTAs per SM, by shared memory and instruction issue.  Against every
 //                slice sorted in runs, M read once per row and long slices read again a row per lane pair, ranking and
 //                aggregation took before / now: 8 heads x 256 rows 12.4 / 10.3 us (f32 13.1 / 10.8), 32 x 512
-//                14.4 / 12.7, 32 x 2048 20.5 / 19.1, 256 x 1024 54.2 / 49.4, 32 x 4096 34.9 / 28.9.
+//                14.4 / 12.7, 32 x 2048 20.5 / 19.1, 256 x 1024 54.2 / 49.4, 32 x 4096 34.9 / 28.9, all with the
+//                same slices; `launch_rank_d` has what their length is worth.
 // aggregate    : one warp per (sequence, KV head, rank j): mean over the G heads of the group of
 //                their j-th retained query, each divided by its own norm; one rounding to dtype.
 #include <cooperative_groups.h>
@@ -428,12 +429,23 @@ static cudaError_t launch_rank_t(const DevParams& P, const void* q, int32_t* q_i
                        (const T*)q, q_idx, rpc, n_sort, n_stage, m_peer);
 }
 
-// A cluster per (sequence, head), sized so that a CTA's slice is about 256 rows: shorter slices only multiply the
-// per-CTA costs (four cluster barriers, the sort, the merge).
+// A cluster per (sequence, head).  While every CTA has an SM of its own, shorter slices end sooner, down to 64 rows (8 heads x
+// 256 rows, f32, 2 / 4 CTAs per head: 10.8 / 9.6 us with the aggregation; 32 x 512 12.8 / 11.6); with two CTAs per SM slices
+// of 256 rows (32 x 777, 4 / 8 CTAs: 12.4 / 14.3; 32 x 2048 the same 19); and in grids of several waves the costs of a CTA
+// (barriers, order, merge) weigh more than the second read of what a slice of 512 rows cannot keep (256 x 1024, 4 / 2 CTAs:
+// 48.7 / 43.0).
 template <typename T, int D>
 static cudaError_t launch_rank_d(const DevParams& P, const void* q, int32_t* q_idx, cudaStream_t st, bool chained) {
-  if (P.chunk <= 512) return launch_rank_t<T, D, 2>(P, q, q_idx, st, chained);
-  if (P.chunk <= 1024) return launch_rank_t<T, D, 4>(P, q, q_idx, st, chained);
+  const long long heads = P.rank_heads, sms = device_sm_count();
+  int cl = 2;
+  while (cl < kRankCluster) {
+    const int rows = (P.chunk + cl - 1) / cl;
+    const long long ctas = 2 * heads * cl;                  // after doubling
+    if (!(rows > 512 || (rows > 256 && ctas <= 2 * sms) || (rows > 64 && ctas <= sms))) break;
+    cl *= 2;
+  }
+  if (cl == 2) return launch_rank_t<T, D, 2>(P, q, q_idx, st, chained);
+  if (cl == 4) return launch_rank_t<T, D, 4>(P, q, q_idx, st, chained);
   return launch_rank_t<T, D, kRankCluster>(P, q, q_idx, st, chained);
 }
 

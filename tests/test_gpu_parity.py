@@ -546,19 +546,21 @@ def test_attention_parts_in_a_cluster(n_q, n_kv, C, T, B):
         assert np.abs(f64(gp.lse[s]) - lse).max() <= 2e-3
 
 
-@pytest.mark.parametrize("C,n_retain,d,dtype", [
-    (2, 1, 128, "bf16"),                # one row per CTA
-    (65, 64, 64, "f32"),                # counted: a block of one row
-    (500, 200, 128, "bf16"),            # 250 rows per CTA, the last block not full
-    (1025, 130, 64, "bf16"),            # clusters of eight with a short last slice
-    (2047, 300, 128, "f32"),            # 256 rows, more than shared memory keeps; still counted
-    (2049, 40, 128, "bf16"),            # 257 rows: sorted in runs
-    (4099, 513, 128, "bf16"),           # 513 rows, kept in part
+@pytest.mark.parametrize("n_q,C,n_retain,d,dtype", [
+    (4, 2, 1, 128, "bf16"),             # one row per CTA
+    (4, 65, 64, 64, "f32"),             # 33 rows: a block of one row
+    (4, 500, 200, 128, "bf16"),         # clusters of eight, 63 rows
+    (4, 1025, 130, 64, "bf16"),         # clusters of eight with a short last slice
+    (4, 2047, 300, 128, "f32"),         # 256 rows, more than shared memory keeps; still counted
+    (4, 2049, 40, 128, "bf16"),         # 257 rows: sorted in runs
+    (4, 4099, 513, 128, "bf16"),        # 513 rows, kept in part
+    (80, 510, 200, 128, "bf16"),        # several waves: two CTAs of 255 rows, the last block not full
+    (80, 1023, 64, 128, "f32"),         # and of 512, kept in part
 ])
-def test_query_ranks_at_the_edges_of_a_slice(C, n_retain, d, dtype):
+def test_query_ranks_at_the_edges_of_a_slice(n_q, C, n_retain, d, dtype):
     """Slices that are counted, sorted, kept in part: the ranks of random rows against the oracle, and of rows that have one
     of two values (equal cosines go by position) exactly."""
-    gp = problem(1200 + C, n_q=4, n_kv=2, d=d, T=40, C=C, dtype=dtype, n_retain=n_retain, kv_budget=8)
+    gp = problem(1200 + C, n_q=n_q, n_kv=2, d=d, T=40, C=C, dtype=dtype, n_retain=n_retain, kv_budget=8)
     api.quoka_select_queries(gp.p, gp.q, gp.q_idx, gp.qbar, gp.ws)
     torch.cuda.synchronize()
     _, cos = O.select_queries(f64(gp.q[0]), n_retain)
@@ -569,7 +571,7 @@ def test_query_ranks_at_the_edges_of_a_slice(C, n_retain, d, dtype):
     api.quoka_select_queries(gp.p, q2, gp.q_idx, gp.qbar, gp.ws)
     torch.cuda.synchronize()
     mean = f64(q2[0]).mean(axis=1)
-    for h in range(4):
+    for h in range(n_q):
         c = f64(q2[0, h]) @ mean[h] / np.linalg.norm(f64(q2[0, h]), axis=1)
         low = c < 0.5 * (c.min() + c.max())
         want = np.concatenate([np.nonzero(low)[0], np.nonzero(~low)[0]])[:n_retain] if pick.any() and not pick.all() else np.arange(n_retain)
