@@ -101,8 +101,9 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
         tma_load_4d(q_smem + x * kPairQTileBytes + hh * 16384, &tm_q, q_full, hh * 64, r0 + x * kQTile, h, s);
   };
   // SPLIT: this CTA walks the tiles [t_lo, t_hi) of the row block's sequence only and leaves, per row, a partial
-  // result (reference point, sum, un-normalised output); the part that finishes last adds the parts up.  The list
-  // length has to be known before the range is, so nothing of the walk starts before the selection has ended.
+  // result (reference point, sum, un-normalised output); the part that finishes last, or the cluster, adds the
+  // parts up.  The list length has to be known before the range is, so nothing of the walk starts before the selection has
+  // ended.
   if (SPLIT) {
     if (warp == kMmaWarp && lane == 0) load_q();
     if (SPARSE) { if (P.attn_after_whole) learn_count(g, k_cnt, s); else resolve(g, k_cnt, s); }

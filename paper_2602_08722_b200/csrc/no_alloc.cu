@@ -44,7 +44,7 @@ extern "C" quoka_status quoka_prefill_chunk_static(const quoka_params* p, const 
   // every host-side refusal comes before the first thing put on the stream (the memset below)
   quoka_status st = quoka::check_prefill_args(p, q, k_cache, v_cache, out);
   if (st != QUOKA_OK) return st;
-  // the array has no room for the scratch of the split attention kernel: small grids run unsplit here
+  // the array has no room for the scratch of the split attention kernel: parts merge in clusters or not at all here
   if (quoka::workspace_bytes(p, /*with_split=*/false) > (size_t)QUOKA_STATIC_SCRATCH_BYTES) return QUOKA_ERR_STATIC_LIMIT;
   void* scratch = nullptr;
   if ((st = quoka::static_scratch_for_current_device(&scratch)) != QUOKA_OK) return st;

@@ -49,7 +49,7 @@ static AttnScratch attn_scratch(const quoka_params* p) {
   return a;
 }
 
-// with_split = false: the layout without the split-attention scratch (every call still works, small grids unsplit)
+// with_split = false: the layout without the split-attention scratch (every call still works, without parts that merge through memory)
 static Workspace carve(const quoka_params* p, void* ws, bool with_split = true) {
   Workspace w{};
   const size_t es = p->dtype == QUOKA_BF16 ? 2 : 4;
