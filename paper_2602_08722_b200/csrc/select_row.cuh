@@ -143,17 +143,20 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
   if (CL > 1) cluster_wait();
   if (P.score_dot) {
     row_range();
-    const float fmin = order_key_to_float(cmin), fmax = order_key_to_float(cmax);
-    mul_neg = mul_pos = fmax > fmin ? (float)kLinBins / (fmax - fmin) : 0.f;
-    add = -fmin * mul_pos;
+    const float fmin = order_key_to_float(cmin), range = order_key_to_float(cmax) - fmin;
+    const bool spread = range > 0.f && range < INFINITY;      // else (one value; infinities or NaN) all rows share a bin
+    mul_neg = mul_pos = spread ? (float)kLinBins / range : 0.f;
+    add = spread ? -fmin * mul_pos : nanf("");
   }
   int bin[ITEMS];                               // bin + 1, or 0 past the end of the row
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     if (i % GRAN == 0 && i >= n_it) break;
-    // Monotone in x.  Adding 2^23 + 1 rounds to an integer in the low mantissa bits (the conversion instruction runs at
-    // a quarter of the rate).
-    const float y = fminf(fmaxf(fmaf(x[i], x[i] < 0.f ? mul_neg : mul_pos, add), 0.f), (float)(kLinBins - 1));
+    // Monotone in the order code: a NaN, whose code is above every number's, falls into the last bin (one with the sign
+    // bit, below every number's, is read as -infinity).  Adding 2^23 + 1 rounds to an integer in the low mantissa bits (the
+    // conversion instruction runs at a quarter of the rate).
+    const float v = __uint_as_float(min(__float_as_uint(x[i]), 0xFF800000u));
+    const float y = fmaxf(fminf(fmaf(v, v < 0.f ? mul_neg : mul_pos, add), (float)(kLinBins - 1)), 0.f);
     bin[i] = base + 32 * i < T ? (int)(__float_as_uint(y + 8388609.f) & 0x7FFFFFu) : 0;
     if (bin[i] != 0) atomicAdd(&hist_all[bin[i] - 1], 1u);
   }
@@ -298,8 +301,8 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
     for (int r = 0; r < CL; ++r) before_cta += r < rank ? cnt_in[r][0] : 0u;
     mine_sel = cnt_in[rank][0];
   }
-  float thr = 0.f;                              // digit passes: the B-th largest score, and the last position that may
-  int cut = -1;                                 // still be taken among the rows with exactly that score
+  uint32_t thr = 0;                             // digit passes: the code of the B-th largest score, and the last position
+  int cut = -1;                                 // that may still be taken among the rows with exactly that code
   if (!found) {
     // ---- Many equal scores (or a range that these bins resolve badly): digit passes of 12 + 12 + 8 bits, most
     // significant first.  The codes of one row of scores share their leading bits: the digits are taken from
@@ -364,13 +367,14 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
       need = s_need;
       mask |= (uint32_t)(nb - 1) << shift;
     }
-    thr = order_key_to_float((prefix >> up) + cmin);
-    // rows above the threshold and equal to it, per warp, per CTA, and before this CTA
+    // Rows above the threshold and equal to it, per warp, per CTA, and before this CTA: by their codes, as the digits were
+    // (NaN scores among them are counted once and only once, so that B rows are listed whatever the scores are).
+    thr = (prefix >> up) + cmin;
     uint32_t w_gt = 0, w_eq = 0;
 #pragma unroll 4
     for (int i = 0; i < n_it; ++i) {
       const int pos = base + 32 * i;
-      const float v = __ldcg(row + min(pos, T - 1));
+      const uint32_t v = float_order_key(__ldcg(row + min(pos, T - 1)));
       w_gt += pos < T && v > thr ? 1u : 0u;
       w_eq += pos < T && v == thr ? 1u : 0u;
     }
@@ -404,7 +408,7 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
 #pragma unroll 1
         for (int i = 0; i < n_it; ++i) {
           const int pos = base + 32 * i;
-          const bool eq = pos < T && __ldcg(row + min(pos, T - 1)) == thr;
+          const bool eq = pos < T && float_order_key(__ldcg(row + min(pos, T - 1))) == thr;
           const uint32_t bal = __ballot_sync(0xFFFFFFFFu, eq);
           if (eq && seen + (uint32_t)__popc(bal & ((2u << lane) - 1u)) == need) s_cut = pos;
           seen += (uint32_t)__popc(bal);
@@ -451,7 +455,7 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
 #pragma unroll 4
     for (int i = 0; i < n_it; ++i) {
       const int pos = base + 32 * i;
-      const float v = __ldcg(row + min(pos, T - 1));
+      const uint32_t v = float_order_key(__ldcg(row + min(pos, T - 1)));
       put(i, __ballot_sync(0xFFFFFFFFu, pos < T && (v > thr || (v == thr && pos <= cut))));
     }
   }

@@ -413,6 +413,53 @@ def test_select_keys_constant_and_narrow_rows(T, B):
     np.testing.assert_array_equal(gp.k_idx[0, :, :B].cpu().numpy(), want)
 
 
+def largest_by_order_code(s, B):
+    """The B largest scores of each row by the kernels' order of floats: NaN above +inf (below -inf with the sign bit set),
+    -0 equal to +0, equal codes by position; ascending positions."""
+    u = s.view(np.uint32)
+    u = np.where((u << 1) == 0, 0, u).astype(np.uint32)
+    code = np.where(u >> 31, ~u, u | np.uint32(0x80000000)).astype(np.int64)
+    return np.sort(np.argsort(-code, axis=1, kind="stable")[:, :B], axis=1)
+
+
+@pytest.mark.parametrize("mode", ["cosine", "dot"])
+@pytest.mark.parametrize("T,B,n_kv", [(700, 100, 6), (5000, 600, 6), (20011, 3000, 6), (20011, 3000, 33), (40000, 39000, 14)])
+def test_select_keys_lists_b_rows_whatever_the_scores_are(T, B, n_kv, mode):
+    """NaN and infinite scores, alone and beside ties at the threshold: still exactly B rows, in the kernels' order."""
+    r = np.random.default_rng(T + B)
+    s = (0.2 * r.normal(size=(n_kv, T))).astype(np.float32)
+    s[0, :] = np.nan
+    s[1, :] = np.where(r.random(T) < 0.7, np.float32(0.25), s[1])           # ties at the threshold, with some NaN above it
+    s[1, r.permutation(T)[: B // 3]] = np.nan
+    s[2, r.permutation(T)[: B + 7]] = np.nan                                # the threshold lies among the NaN
+    s[3, r.permutation(T)[: T - B // 2]] = np.uint32(0xFFC00000).view(np.float32)     # among the NaN with the sign bit
+    s[4, r.permutation(T)[: B // 2]] = np.inf
+    s[4, r.permutation(T)[: T // 2]] = -np.inf
+    s[5, 11] = np.nan
+    gp = scores_only_problem(T, B, n_kv)
+    gp.p.score_mode = {"cosine": api.SCORE_COSINE, "dot": api.SCORE_DOT}[mode]
+    gp.scores[0] = torch.from_numpy(s).cuda()
+    api.quoka_select_keys(gp.p, gp.scores, gp.k_idx, gp.k_cnt, gp.ws)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(gp.k_idx[0, :, :B].cpu().numpy(), largest_by_order_code(s, B))
+
+
+@pytest.mark.parametrize("C,dtype", [(1, "bf16"), (1, "f32"), (40, "f32")])
+def test_queries_that_are_nan_leave_the_other_sequence_alone(C, dtype):
+    """One sequence's queries are NaN (all its scores too): its list is still one of valid rows, and the other sequence's
+    results are what they are without it."""
+    gp = problem(77, batch=2, n_q=8, n_kv=2, T=[5000, 4100], C=C, dtype=dtype, n_retain=64, kv_budget=300)
+    api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, gp.k_idx, gp.k_cnt, gp.ws)
+    torch.cuda.synchronize()
+    want = gp.out.clone()
+    gp.q[0] = float("nan")
+    api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, gp.k_idx, gp.k_cnt, gp.ws)
+    torch.cuda.synchronize()
+    assert api.quoka_last_device_status(gp.ws) == 0
+    assert (gp.k_idx[0].diff(dim=1) > 0).all() and gp.k_idx[0].min() >= 0 and gp.k_idx[0].max() < 5000
+    assert torch.equal(gp.out[1], want[1]) and torch.isnan(gp.out[0].float()).all()
+
+
 @pytest.mark.parametrize("d,dtype", [(128, "bf16"), (64, "bf16"), (128, "f32"), (64, "f32")])
 @pytest.mark.parametrize("n_q,n_kv,T,B", [
     (4, 4, 1, 5),              # one cached row, a head per KV group
