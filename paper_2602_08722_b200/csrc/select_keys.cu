@@ -1,16 +1,14 @@
-// Top-B key selection (Algorithm 1: I = topk(S^, B_SA)) as a radix select.
+// Top-B key selection (Algorithm 1: I = topk(S^, B_SA)).
 //
-// The fp32 scores are mapped to order-preserving uint32 codes; digit passes, most significant first,
-// narrow a (prefix, need) pair until `prefix` is the code of the B-th largest score and `need` is how
-// many rows with exactly that code are still to be taken.  The output pass walks the rows in position
-// order and computes each selected row's slot with warp ballots and prefix sums, so the list comes out
+// Scores are compared by order-preserving uint32 codes where it matters (the threshold and its ties).  The output pass walks
+// the rows in position order and computes each selected row's slot with warp ballots and prefix sums, so the list comes out
 // ascending and rows that tie at the threshold are taken lowest position first.
 //
 // select_keys_reg_kernel (the default): one CTA of 512 threads per (sequence, KV head), or a cluster
 // of 2/4/8 CTAs, holds the whole row of scores IN REGISTERS (as bins, up to 64 per thread: the scores are
 // read from memory once, coalesced); see select_row.cuh.
-// select_keys_kernel (one CTA per head, scores re-read from L2 every pass, 8-bit digits) serves rows
-// too long for that.
+// select_keys_kernel (one CTA per head, a radix select: scores re-read from L2 every pass, 8-bit digits of the codes, most
+// significant first) serves rows too long for that.
 #include "select_row.cuh"
 
 namespace quoka {

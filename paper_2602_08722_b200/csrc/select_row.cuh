@@ -1,9 +1,9 @@
 // Selection of the B largest of a row of scores by a CTA or a cluster of CTAs (Algorithm 1: I = topk(S^, B_SA)), for the
 // selection kernel and the fused selection + attention kernel of a generation step.
 //
-// First try: one histogram over bins linear in the score, the bin of the B-th largest, and that bin's few rows ranked
-// against each other.  Many equal scores: three digit passes of 12 + 12 + 8 bits over (code - smallest code of the row)
-// shifted up to the top bit.
+// One histogram over bins linear in the score, the bin of the B-th largest, and that bin's few rows ranked against each other.
+// Where that bin is crowded (equal scores, or scores in a narrow band): histograms over the row's order codes, each over the
+// bin of the one before, until a bin is a single code.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -20,9 +20,8 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
 constexpr int kRegThreads = 512, kRegWarps = kRegThreads / 32;
-constexpr int kDigitBins = 4096;          // 12-bit digits
-constexpr int kHistWords = 2 * kDigitBins + 256;
-constexpr int kLinBins = 8192;            // first try: bins linear in the score
+constexpr int kLinBits = 13, kLinBins = 1 << kLinBits;
+constexpr int kHistWords = kLinBins + 256;
 constexpr int kCoarse = 256;              // sums of 32 consecutive bins
 constexpr int kCandMax = 512;             // rows of the threshold's bin that are ranked against each other, all CTAs
 
@@ -30,7 +29,7 @@ template <int ITEMS, int CL>
 struct SelectSmem {
   static constexpr int kSeg = kCandMax / CL;    // listed rows per CTA
   static_assert(kRegThreads * ITEMS < 65536, "a CTA's sums are kept in 16 bits");
-  __align__(16) uint32_t hist_all[kHistWords];  // histograms, then the list
+  __align__(16) uint32_t hist_all[kHistWords];  // the histogram, then the list
   __align__(16) uint16_t coarse[kCoarse];       // this CTA's sums, and every CTA's (pushed by the peers)
   __align__(16) uint16_t coarse_in[CL][kCoarse];
   __align__(16) uint32_t sel_bits[kRegWarps * ITEMS];   // of the listed rows, the ones that are taken: bit = lane, word = item
@@ -107,14 +106,24 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
     }
     return v;
   };
+  // f(position, order code, is it a row) for this thread's rows, read again a few at a time: the loads of a batch overlap.
+  // (Kept small: unrolled further, this code costs the fused kernel 6 us that never runs it.)
+  const auto each_code = [&](auto&& f) {
+    constexpr int kBatch = ITEMS == 64 ? 8 : 4;
+#pragma unroll 1
+    for (int i = 0; i < n_it; i += kBatch) {
+      float v[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) v[u] = __ldcg(row + min(base + 32 * (i + u), T - 1));
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u)
+        f(base + 32 * (i + u), float_order_key(v[u]), base + 32 * (i + u) < T && (GRAN % kBatch == 0 || i + u < n_it));
+    }
+  };
   uint32_t cmin = 0u, cmax = 0xFFFFFFFFu;       // smallest and largest code of the row, where they are needed
   const auto row_range = [&]() {
     cmin = 0xFFFFFFFFu; cmax = 0u;
-#pragma unroll 4
-    for (int i = 0; i < n_it; ++i) {
-      const uint32_t c = float_order_key(__ldcg(row + min(base + 32 * i, T - 1)));     // (a row past the end repeats the last)
-      cmin = min(cmin, c); cmax = max(cmax, c);
-    }
+    each_code([&](int, uint32_t c, bool) { cmin = min(cmin, c); cmax = max(cmax, c); });       // (rows read past the end repeat the last)
     cmin = __reduce_min_sync(0xFFFFFFFFu, cmin);
     cmax = __reduce_max_sync(0xFFFFFFFFu, cmax);
     if (lane == 0) { warp_val[wid] = cmin; warp_off[wid] = cmax; }
@@ -127,6 +136,67 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
 #pragma unroll
       for (int r = 0; r < CL; ++r) { cmin = min(cmin, mm_in[r][0]); cmax = max(cmax, mm_in[r][1]); }
     }
+  };
+
+  // The bin of the histogram, over all CTAs, in which the running count from the top reaches `count`, + 1 (s_bin); what is
+  // still needed inside it (s_need); its size (s_cand).
+  const auto find_bin = [&](uint32_t count) {
+    {
+      // sums of 32 bins (two threads each), then to every CTA of the cluster, warp r to CTA r
+      static_assert(kRegThreads == 2 * kCoarse && kLinBins == 32 * kCoarse, "16 bins per thread");
+      uint32_t c = 0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {                       // (rotated: the two threads of a sum stay off each other's banks)
+        const uint4 h = reinterpret_cast<const uint4*>(hist_all)[4 * tid + ((j + (tid >> 1)) & 3)];
+        c += (h.x + h.y) + (h.z + h.w);
+      }
+      c += __shfl_xor_sync(0xFFFFFFFFu, c, 1);
+      const int cb = kCoarse - 1 - (tid >> 1);            // counted from the top
+      if ((tid & 1) == 0) (CL > 1 ? coarse : coarse_in[0])[cb] = (uint16_t)c;
+      if (CL > 1) {
+        __syncthreads();
+        if (wid < CL)
+          reinterpret_cast<uint4*>(peer(coarse_in[rank], wid))[lane] = reinterpret_cast<const uint4*>(coarse)[lane];
+      }
+    }
+    sync_all();
+    if (wid == 0) {
+      // the sum, then the bin, in which the running count from the top reaches `count`; lane l owns sums 8l .. 8l + 7
+      uint32_t c[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) c[j] = 0;
+#pragma unroll
+      for (int r = 0; r < CL; ++r) {
+        const uint4 a = *reinterpret_cast<const uint4*>(&coarse_in[r][8 * lane]);
+        c[0] += a.x & 0xFFFFu; c[1] += a.x >> 16; c[2] += a.y & 0xFFFFu; c[3] += a.y >> 16;
+        c[4] += a.z & 0xFFFFu; c[5] += a.z >> 16; c[6] += a.w & 0xFFFFu; c[7] += a.w >> 16;
+      }
+      uint32_t sum = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) sum += c[j];
+      const uint32_t incl = warp_scan(sum);
+      const int src = __ffs(__ballot_sync(0xFFFFFFFFu, incl >= count)) - 1;
+      uint32_t cum = incl - sum, at = 0;
+      bool hit = false;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (!hit && cum + c[j] >= count) { hit = true; at = j; }
+        if (!hit) cum += c[j];
+      }
+      const int cb = (int)__shfl_sync(0xFFFFFFFFu, 8 * lane + at, src);
+      const uint32_t want = count - __shfl_sync(0xFFFFFFFFu, cum, src);
+      const int bin0 = kLinBins - 1 - 32 * cb - lane;                    // lane's bin, from the top
+      uint32_t f = 0;
+#pragma unroll
+      for (int r = 0; r < CL; ++r) f += *peer(&hist_all[bin0], r);       // independent remote loads, all in flight together
+      const uint32_t fi = warp_scan(f);
+      if (lane == __ffs(__ballot_sync(0xFFFFFFFFu, fi >= want)) - 1) {
+        s_bin = (uint32_t)bin0 + 1;
+        s_need = want - (fi - f);
+        s_cand = f;
+      }
+    }
+    __syncthreads();
   };
 
   // ---- First try: one histogram over bins linear in the score.
@@ -161,62 +231,7 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
     if (bin[i] != 0) atomicAdd(&hist_all[bin[i] - 1], 1u);
   }
   __syncthreads();
-  {
-    // sums of 32 bins (two threads each), then to every CTA of the cluster, warp r to CTA r
-    static_assert(kRegThreads == 2 * kCoarse && kLinBins == 32 * kCoarse, "16 bins per thread");
-    uint32_t c = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {                       // (rotated: the two threads of a sum stay off each other's banks)
-      const uint4 h = reinterpret_cast<const uint4*>(hist_all)[4 * tid + ((j + (tid >> 1)) & 3)];
-      c += (h.x + h.y) + (h.z + h.w);
-    }
-    c += __shfl_xor_sync(0xFFFFFFFFu, c, 1);
-    const int cb = kCoarse - 1 - (tid >> 1);            // counted from the top
-    if ((tid & 1) == 0) (CL > 1 ? coarse : coarse_in[0])[cb] = (uint16_t)c;
-    if (CL > 1) {
-      __syncthreads();
-      if (wid < CL)
-        reinterpret_cast<uint4*>(peer(coarse_in[rank], wid))[lane] = reinterpret_cast<const uint4*>(coarse)[lane];
-    }
-  }
-  sync_all();
-  if (wid == 0) {
-    // the sum, then the bin, in which the running count from the top reaches B; lane l owns sums 8l .. 8l + 7
-    uint32_t c[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) c[j] = 0;
-#pragma unroll
-    for (int r = 0; r < CL; ++r) {
-      const uint4 a = *reinterpret_cast<const uint4*>(&coarse_in[r][8 * lane]);
-      c[0] += a.x & 0xFFFFu; c[1] += a.x >> 16; c[2] += a.y & 0xFFFFu; c[3] += a.y >> 16;
-      c[4] += a.z & 0xFFFFu; c[5] += a.z >> 16; c[6] += a.w & 0xFFFFu; c[7] += a.w >> 16;
-    }
-    uint32_t sum = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) sum += c[j];
-    const uint32_t incl = warp_scan(sum);
-    const int src = __ffs(__ballot_sync(0xFFFFFFFFu, incl >= (uint32_t)B)) - 1;
-    uint32_t cum = incl - sum, at = 0;
-    bool hit = false;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (!hit && cum + c[j] >= (uint32_t)B) { hit = true; at = j; }
-      if (!hit) cum += c[j];
-    }
-    const int cb = (int)__shfl_sync(0xFFFFFFFFu, 8 * lane + at, src);
-    const uint32_t want = (uint32_t)B - __shfl_sync(0xFFFFFFFFu, cum, src);
-    const int bin0 = kLinBins - 1 - 32 * cb - lane;                    // lane's bin, from the top
-    uint32_t f = 0;
-#pragma unroll
-    for (int r = 0; r < CL; ++r) f += *peer(&hist_all[bin0], r);       // independent remote loads, all in flight together
-    const uint32_t fi = warp_scan(f);
-    if (lane == __ffs(__ballot_sync(0xFFFFFFFFu, fi >= want)) - 1) {
-      s_bin = (uint32_t)bin0 + 1;
-      s_need = want - (fi - f);
-      s_cand = f;
-    }
-  }
-  __syncthreads();
+  find_bin((uint32_t)B);
   uint32_t before_cta = 0, mine_sel = 0;        // selected rows of the CTAs before this one, and of this one
   const int tb = (int)s_bin;
   uint32_t need = s_need;
@@ -260,7 +275,7 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
     for (int r = 0; r < CL; ++r) found = found && cnt_in[r][1] <= (uint32_t)kSeg;     // (uniform over the cluster)
   }
   if (found) {
-    // ---- the listed rows side by side (over the histograms, which are done with), each ranked by a thread
+    // ---- the listed rows side by side (over the histogram, which is done with), each ranked by a thread
     key64* all = reinterpret_cast<key64*>(hist_all);
     int n = 0;
     {
@@ -301,83 +316,40 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
     for (int r = 0; r < CL; ++r) before_cta += r < rank ? cnt_in[r][0] : 0u;
     mine_sel = cnt_in[rank][0];
   }
-  uint32_t thr = 0;                             // digit passes: the code of the B-th largest score, and the last position
+  uint32_t thr = 0;                             // a crowded bin: the code of the B-th largest score, and the last position
   int cut = -1;                                 // that may still be taken among the rows with exactly that code
   if (!found) {
-    // ---- Many equal scores (or a range that these bins resolve badly): digit passes of 12 + 12 + 8 bits, most
-    // significant first.  The codes of one row of scores share their leading bits: the digits are taken from
-    // (code - smallest code) shifted up to the top bit, a map that keeps the order and loses no bit.  The scores are
-    // read again for every pass.
-    row_range();
-    const int up = min(__clz((int)(cmax - cmin)), 31);
-    for (int i = tid; i < kHistWords; i += kRegThreads) hist_all[i] = 0;
-    __syncthreads();
-    uint32_t prefix = 0, mask = 0;
+    // ---- A crowded bin: more than 512 rows in 1/7680 (1/4096) of the cosine's range, or more than a CTA's share of those.
+    // The scores are read again for every pass: their range, a histogram per 13 bits of it, the counts, the list.  8 rows of
+    // 32768 scores, spread / within 1e-3 of each other / all equal: 6.7 / 14 / 10 us, 128 such rows 15 / 42 / 32 (digits of 12
+    // bits, every CTA reading all of every CTA's bins: 6.7 / 146 / 148 and 15 / 73 / 82).
+    row_range();                                              // (its barrier is behind every peer's look at the histogram)
+    uint32_t lo = cmin, hi = cmax;                            // the threshold's code lies in between
     need = (uint32_t)B;
 #pragma unroll 1
-    for (int pass = 0; pass < 3; ++pass) {
-      const int shift = pass == 0 ? 20 : (pass == 1 ? 8 : 0);
-      const int nb = pass == 2 ? 256 : kDigitBins;
-      uint32_t* hist = hist_all + pass * kDigitBins;
-#pragma unroll 4
-      for (int i = 0; i < n_it; ++i) {
-        const int pos = base + 32 * i;
-        const uint32_t c = (float_order_key(__ldcg(row + min(pos, T - 1))) - cmin) << up;
-        if (pos < T && (c & mask) == prefix) atomicAdd(&hist[(c >> shift) & (uint32_t)(nb - 1)], 1u);
-      }
-      sync_all();
-      // thread t owns the kPer bins nb-1-kPer*t and on downwards (counted from the top)
-      constexpr int kPer = kDigitBins / kRegThreads;
-      uint32_t c[kPer], sum = 0;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) c[k] = 0;
-      if (kPer * tid < nb) {
-#pragma unroll
-        for (int r = 0; r < CL; ++r) {
-          const uint32_t* ph = peer(hist, r);
-#pragma unroll
-          for (int k = 0; k < kPer; ++k) c[k] += ph[nb - 1 - (kPer * tid + k)];
-        }
-#pragma unroll
-        for (int k = 0; k < kPer; ++k) sum += c[k];
-      }
-      const uint32_t incl = warp_scan(sum);
-      if (lane == 31) warp_val[wid] = incl;
+    while (lo != hi) {
+      for (int i = tid; i < kLinBins / 4; i += kRegThreads) reinterpret_cast<uint4*>(hist_all)[i] = make_uint4(0, 0, 0, 0);
       __syncthreads();
-      if (wid == 0) {
-        const uint32_t v = lane < kRegWarps ? warp_val[lane] : 0u;
-        warp_off[lane] = warp_scan(v) - v;
-      }
+      const int shift = max(32 - kLinBits - __clz((int)(hi - lo)), 0);
+      each_code([&](int, uint32_t c, bool in) {
+        if (in && lo <= c && c <= hi) atomicAdd(&hist_all[(c - lo) >> shift], 1u);
+      });
       __syncthreads();
-      const uint32_t excl = warp_off[wid] + incl - sum;
-      if (excl < need && need <= excl + sum) {          // exactly one thread
-        uint32_t cum = excl;
-#pragma unroll
-        for (int k = 0; k < kPer; ++k) {
-          if (cum + c[k] >= need) {
-            s_bin = (uint32_t)(nb - 1 - (kPer * tid + k));
-            s_need = need - cum;
-            break;
-          }
-          cum += c[k];
-        }
-      }
-      __syncthreads();
-      prefix |= s_bin << shift;
+      find_bin(need);
       need = s_need;
-      mask |= (uint32_t)(nb - 1) << shift;
+      const uint32_t at = (s_bin - 1) << shift;
+      hi = lo + min(at + ((1u << shift) - 1), hi - lo);
+      lo += at;
+      sync_all();                                             // every peer has looked at this histogram
     }
-    // Rows above the threshold and equal to it, per warp, per CTA, and before this CTA: by their codes, as the digits were
+    // Rows above the threshold and equal to it, per warp, per CTA, and before this CTA: by their codes, as the bins were
     // (NaN scores among them are counted once and only once, so that B rows are listed whatever the scores are).
-    thr = (prefix >> up) + cmin;
+    thr = lo;
     uint32_t w_gt = 0, w_eq = 0;
-#pragma unroll 4
-    for (int i = 0; i < n_it; ++i) {
-      const int pos = base + 32 * i;
-      const uint32_t v = float_order_key(__ldcg(row + min(pos, T - 1)));
-      w_gt += pos < T && v > thr ? 1u : 0u;
-      w_eq += pos < T && v == thr ? 1u : 0u;
-    }
+    each_code([&](int, uint32_t c, bool in) {
+      w_gt += in && c > thr ? 1u : 0u;
+      w_eq += in && c == thr ? 1u : 0u;
+    });
     w_gt = __reduce_add_sync(0xFFFFFFFFu, w_gt);
     w_eq = __reduce_add_sync(0xFFFFFFFFu, w_eq);
     if (lane == 0) warp_val[wid] = w_gt | (w_eq << 16);      // at most 32 * n_it each
@@ -405,14 +377,12 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
     } else if (eq_cta < need) {
       if (eq_before < need && need <= eq_before + w_eq) {
         uint32_t seen = eq_before;
-#pragma unroll 1
-        for (int i = 0; i < n_it; ++i) {
-          const int pos = base + 32 * i;
-          const bool eq = pos < T && float_order_key(__ldcg(row + min(pos, T - 1))) == thr;
+        each_code([&](int pos, uint32_t c, bool in) {
+          const bool eq = in && c == thr;
           const uint32_t bal = __ballot_sync(0xFFFFFFFFu, eq);
           if (eq && seen + (uint32_t)__popc(bal & ((2u << lane) - 1u)) == need) s_cut = pos;
           seen += (uint32_t)__popc(bal);
-        }
+        });
       }
       __syncthreads();
       cut = s_cut;
@@ -423,18 +393,19 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
     if (lane == 0) warp_val[wid] = sel;
     __syncthreads();
   }
-  // ---- The list, in position order.  One ballot per item; it is collected in shared memory (over the histograms)
+  // ---- The list, in position order.  One ballot per item; it is collected in shared memory (over the histogram)
   // and copied out with full-width stores.
   const uint32_t lt = (1u << lane) - 1u;
   uint32_t run = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? warp_val[lane] : 0u);
   const bool staged = mine_sel <= (uint32_t)kHistWords;
   const uint32_t room = staged ? (uint32_t)kHistWords : (uint32_t)B - min((uint32_t)B, before_cta);
   uint32_t* dst = staged ? hist_all : reinterpret_cast<uint32_t*>(out) + before_cta;
-  const auto put = [&](int i, uint32_t bal) {
+  const auto put_at = [&](int pos, uint32_t bal) {
     const uint32_t slot = run + (uint32_t)__popc(bal & lt);
-    if ((bal >> lane & 1u) && slot < room) dst[slot] = (uint32_t)(base + 32 * i);
+    if ((bal >> lane & 1u) && slot < room) dst[slot] = (uint32_t)pos;
     run += (uint32_t)__popc(bal);
   };
+  const auto put = [&](int i, uint32_t bal) { put_at(base + 32 * i, bal); };
   if (found) {
 #pragma unroll
     for (int i = 0; i < ITEMS; i += 4) {
@@ -452,12 +423,9 @@ __device__ __forceinline__ Selected select_row(const DevParams& P, const float* 
       }
     }
   } else {
-#pragma unroll 4
-    for (int i = 0; i < n_it; ++i) {
-      const int pos = base + 32 * i;
-      const uint32_t v = float_order_key(__ldcg(row + min(pos, T - 1)));
-      put(i, __ballot_sync(0xFFFFFFFFu, pos < T && (v > thr || (v == thr && pos <= cut))));
-    }
+    each_code([&](int pos, uint32_t c, bool in) {
+      put_at(pos, __ballot_sync(0xFFFFFFFFu, in && (c > thr || (c == thr && pos <= cut))));
+    });
   }
   return Selected{before_cta, mine_sel};
 }

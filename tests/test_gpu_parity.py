@@ -444,6 +444,46 @@ def test_select_keys_lists_b_rows_whatever_the_scores_are(T, B, n_kv, mode):
     np.testing.assert_array_equal(gp.k_idx[0, :, :B].cpu().numpy(), largest_by_order_code(s, B))
 
 
+@pytest.mark.parametrize("T,B,n_kv", [(600, 71, 33), (9001, 1080, 15), (33000, 3960, 8), (33000, 3960, 80), (140000, 16800, 5)])
+def test_select_keys_of_rows_in_a_narrow_band(T, B, n_kv):
+    """More rows in the threshold's bin than are ranked against each other: bands of a few codes and of many (one, two and
+    three histograms over the codes), with a far-off row that widens the range.  Integer parity with the oracle."""
+    r = np.random.default_rng(T)
+    s = (0.25 + 1e-3 * r.normal(size=(n_kv, T))).astype(np.float32)
+    s[1] = np.float32(0.25) + r.integers(0, 9000, T).astype(np.float32) * np.float32(2.0 ** -25)
+    s[2] = (0.25 + 1e-4 * r.normal(size=T)).astype(np.float32)
+    s[2, T // 3], s[2, T // 2] = -1.0, 1.0
+    s[3, ::2] = np.float32(0.2505)
+    gp = scores_only_problem(T, B, n_kv)
+    gp.scores[0] = torch.from_numpy(s).cuda()
+    api.quoka_select_keys(gp.p, gp.scores, gp.k_idx, gp.k_cnt, gp.ws)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(gp.k_idx[0, :, :B].cpu().numpy(), O.select_keys(s.astype(np.float64), B))
+
+
+def test_select_keys_crowded_rows_are_not_far_slower_than_spread_ones():
+    """8 rows of 32768 scores: equal ones, or ones in a narrow band, may cost a few more passes over the row (6.7 us spread,
+    10 and 14 us crowded, back to back), not the 130 us of reading every CTA's histogram from every CTA."""
+    gp = scores_only_problem(32768, 3932, 8)
+    z = torch.randn(8, 32768, device="cuda", generator=torch.Generator("cuda").manual_seed(0))
+
+    def best_us(scores):
+        gp.scores[0] = scores
+        times = []
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                api.quoka_select_keys(gp.p, gp.scores, gp.k_idx, gp.k_cnt, gp.ws)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 50)
+        return min(times)
+
+    spread = best_us(0.25 + 0.06 * z)
+    assert best_us(torch.full_like(z, 0.25)) < 5 * spread and best_us(0.25 + 1e-3 * z) < 5 * spread
+
+
 @pytest.mark.parametrize("C,dtype", [(1, "bf16"), (1, "f32"), (40, "f32")])
 def test_queries_that_are_nan_leave_the_other_sequence_alone(C, dtype):
     """One sequence's queries are NaN (all its scores too): its list is still one of valid rows, and the other sequence's
