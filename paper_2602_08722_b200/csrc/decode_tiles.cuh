@@ -128,9 +128,10 @@ __device__ __forceinline__ void decode_attend(const DevParams& P, const T* __res
       float mx = fmaxf(m[i], x);
 #pragma unroll
       for (int o = LPR / UNR; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));   // rows of the same head
-      alpha[i] = __expf(m[i] - mx);                  // (0 on the first trip: m is -inf, mx is not, every warp has a row)
+      const float ref = mx == -INFINITY ? 0.f : mx;  // (logits of -infinity alone: weights of 0)
+      alpha[i] = __expf(m[i] - ref);                 // (0 on the first trip: m is -inf, ref is not)
       m[i] = mx;
-      lg[i] = __expf(x - mx);
+      lg[i] = __expf(x - ref);
       l[i] = fmaf(l[i], alpha[i], lg[i]);
     }
     if (u0 >= u_lo + kWarps * kRows) {               // not the warp's first trip

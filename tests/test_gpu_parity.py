@@ -522,6 +522,29 @@ def test_decode_attention_parts_and_groups(n_q, n_kv, T, B, d, dtype):
         assert np.abs(f64(gp.lse[s]) - lse).max() <= 2e-3
 
 
+@pytest.mark.parametrize("d,dtype", [(128, "bf16"), (64, "bf16"), (128, "f32"), (64, "f32")])
+@pytest.mark.parametrize("n_q,n_kv", [(4, 4), (8, 2)])
+def test_decode_attention_over_rows_whose_logits_overflow_to_minus_infinity(n_q, n_kv, d, dtype):
+    """Whole trips of a warp, and every key of one part, may have logits of minus infinity: weights of zero, not NaN."""
+    gp = problem(990 + d, n_q=n_q, n_kv=n_kv, d=d, T=400, C=1, dtype=dtype, n_retain=4, kv_budget=40)
+    gp.q.abs_().add_(0.5)
+    far = torch.cat([torch.arange(0, 140), torch.arange(200, 210)]).cuda()
+    gp.k[:, :, far] = -3e38
+    gp.k_idx[0] = torch.cat([far[:39], torch.tensor([399], device="cuda")]).int()
+    gp.k_cnt.fill_(40)
+    api.quoka_sparse_attn(gp.p, gp.q, gp.k, gp.v, gp.k_idx, gp.k_cnt, gp.out, gp.lse, gp.ws)
+    listed, listed_lse = gp.out.clone(), gp.lse.clone()
+    api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, gp.lse, gp.ws)
+    torch.cuda.synchronize()
+    q, k, v = f64(gp.q[0]), f64(gp.k[0]), f64(gp.v[0])
+    want, lse = O.sparse_attention(q, k, v, 400, [gp.k_idx[0, h].cpu().numpy() for h in range(n_kv)])
+    check_attention(f64(listed[0]), want, dtype)
+    assert np.abs(f64(listed_lse[0]) - lse).max() <= 2e-3
+    want, lse = O.dense_chunk_attention(q, k, v, 400)
+    check_attention(f64(gp.out[0]), want, dtype)
+    assert np.abs(f64(gp.lse[0]) - lse).max() <= 2e-3
+
+
 @pytest.mark.parametrize("paged", [False, True])
 @pytest.mark.parametrize("T,max_ctx,B,n_q,n_kv,d,dtype", [
     ([2049], 2049, 64, 8, 2, 128, "bf16"),        # just beyond the two-launch form: 258 positions per CTA
