@@ -47,6 +47,20 @@ __device__ __forceinline__ void transposing_sum(float (&v)[NV], int c) {
 
 constexpr int kDecodeUnroll = 4;
 
+// f32: the library's exp and compensated sums, as in the f32 attention of longer chunks (attn_f32.cu): a lane adds up thousands
+// of weights, and those below half an ulp of its sum must not vanish one by one.  bf16: the outputs are rounded to 8 bits.
+template <typename T>
+__device__ __forceinline__ float decode_exp(float x) {
+  if constexpr (sizeof(T) == 4) return expf(x); else return __expf(x);
+}
+// s += x; c: what the sum has lost so far, added once at the end (and left out where the sum has become infinite)
+__device__ __forceinline__ void add_compensated(float& s, float& c, float x) {
+  const float z = s + x;
+  c += (s - z) + x;
+  s = z;
+}
+__device__ __forceinline__ float compensated(float s, float c) { return c == c ? s + c : s; }
+
 // What the warps of a CTA leave for its sum, and what a CTA leaves for its cluster's: per head the reference point, the
 // sum of the weights and the un-normalised output.
 template <int D, int GH, int WARPS>
@@ -88,13 +102,21 @@ __device__ __forceinline__ void decode_attend(const DevParams& P, const T* __res
   constexpr int kRep = NV < LPR ? LPR / NV : 1;      // lanes that hold the same one
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int c = lane % LPR, rsub = lane / LPR;
+  constexpr bool kComp = sizeof(T) == 4;
   float m[PER], l[PER], acc[GH][NE];                 // m, l: of the head this lane's logits belong to
+  float cl[kComp ? PER : 1], cacc[kComp ? GH : 1][NE];
 #pragma unroll
-  for (int i = 0; i < PER; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
+  for (int i = 0; i < PER; ++i) {
+    m[i] = -INFINITY; l[i] = 0.f;
+    if constexpr (kComp) cl[i] = 0.f;
+  }
 #pragma unroll
   for (int g = 0; g < GH; ++g)
 #pragma unroll
-    for (int i = 0; i < NE; ++i) acc[g][i] = 0.f;
+    for (int i = 0; i < NE; ++i) {
+      acc[g][i] = 0.f;
+      if constexpr (kComp) cacc[g][i] = 0.f;
+    }
   for (int u0 = u_lo + warp * kRows; u0 < u_hi; u0 += kWarps * kRows) {
     int t[UNR];
 #pragma unroll
@@ -129,31 +151,65 @@ __device__ __forceinline__ void decode_attend(const DevParams& P, const T* __res
 #pragma unroll
       for (int o = LPR / UNR; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));   // rows of the same head
       const float ref = mx == -INFINITY ? 0.f : mx;  // (logits of -infinity alone: weights of 0)
-      alpha[i] = __expf(m[i] - ref);                 // (0 on the first trip: m is -inf, ref is not)
+      alpha[i] = decode_exp<T>(m[i] - ref);          // (0 on the first trip: m is -inf, ref is not)
       m[i] = mx;
-      lg[i] = __expf(x - ref);
-      l[i] = fmaf(l[i], alpha[i], lg[i]);
+      lg[i] = decode_exp<T>(x - ref);
+      if constexpr (kComp) {
+        l[i] *= alpha[i]; cl[i] *= alpha[i];
+        add_compensated(l[i], cl[i], lg[i]);
+      } else {
+        l[i] = fmaf(l[i], alpha[i], lg[i]);
+      }
     }
     if (u0 >= u_lo + kWarps * kRows) {               // not the warp's first trip
 #pragma unroll
       for (int g = 0; g < GH; ++g) {
         const float a = __shfl_sync(0xFFFFFFFFu, alpha[g % PER], g / PER * kRep, LPR);
 #pragma unroll
-        for (int i = 0; i < NE; ++i) acc[g][i] *= a;
+        for (int i = 0; i < NE; ++i) {
+          acc[g][i] *= a;
+          if constexpr (kComp) cacc[g][i] *= a;
+        }
       }
     }
+    if constexpr (kComp) {
 #pragma unroll
-    for (int j = 0; j < UNR; ++j) {
-      float x[NE];
-      word_to_f32<T>(vw[j], x);
+      for (int g = 0; g < GH; ++g) {                 // the trip's rows first, then to the running sum
+        float pv[NE];
 #pragma unroll
-      for (int g = 0; g < GH; ++g) {
-        const int id = j * GH + g;
-        const float p = __shfl_sync(0xFFFFFFFFu, lg[id % PER], id / PER * kRep, LPR);
+        for (int j = 0; j < UNR; ++j) {
+          const int id = j * GH + g;
+          const float p = __shfl_sync(0xFFFFFFFFu, lg[id % PER], id / PER * kRep, LPR);
+          float x[NE];
+          word_to_f32<T>(vw[j], x);
 #pragma unroll
-        for (int i = 0; i < NE; ++i) acc[g][i] = fmaf(p, x[i], acc[g][i]);
+          for (int i = 0; i < NE; ++i) pv[i] = j == 0 ? p * x[i] : fmaf(p, x[i], pv[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < NE; ++i) add_compensated(acc[g][i], cacc[g][i], pv[i]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < UNR; ++j) {
+        float x[NE];
+        word_to_f32<T>(vw[j], x);
+#pragma unroll
+        for (int g = 0; g < GH; ++g) {
+          const int id = j * GH + g;
+          const float p = __shfl_sync(0xFFFFFFFFu, lg[id % PER], id / PER * kRep, LPR);
+#pragma unroll
+          for (int i = 0; i < NE; ++i) acc[g][i] = fmaf(p, x[i], acc[g][i]);
+        }
       }
     }
+  }
+  if constexpr (kComp) {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) l[i] = compensated(l[i], cl[i]);
+#pragma unroll
+    for (int g = 0; g < GH; ++g)
+#pragma unroll
+      for (int i = 0; i < NE; ++i) acc[g][i] = compensated(acc[g][i], cacc[g][i]);
   }
   __syncthreads();
   // ---- the warp's result: lanes that hold the same word of different rows, and the sums of the weights
@@ -186,7 +242,7 @@ __device__ __forceinline__ void decode_attend(const DevParams& P, const T* __res
     for (int i = 0; i < kWarps; ++i) M = fmaxf(M, w.m[i][g]);
 #pragma unroll
     for (int i = 0; i < kWarps; ++i) {
-      const float wgt = w.m[i][g] == -INFINITY ? 0.f : __expf(w.m[i][g] - M);
+      const float wgt = w.m[i][g] == -INFINITY ? 0.f : decode_exp<T>(w.m[i][g] - M);
       L = fmaf(wgt, w.l[i][g], L);
       o = fmaf(wgt, w.o[i][g][x], o);
     }
@@ -215,7 +271,7 @@ __device__ __forceinline__ void decode_merge(const DevParams& P, DecodePart<D, G
     for (int p = 0; p < 8; ++p) M = fmaxf(M, pm[p]);
 #pragma unroll
     for (int p = 0; p < 8; ++p) {
-      const float wgt = pm[p] == -INFINITY ? 0.f : __expf(pm[p] - M);
+      const float wgt = pm[p] == -INFINITY ? 0.f : decode_exp<T>(pm[p] - M);
       L = fmaf(wgt, pl[p], L);
       o = fmaf(wgt, po[p], o);
     }

@@ -545,6 +545,50 @@ def test_decode_attention_over_rows_whose_logits_overflow_to_minus_infinity(n_q,
     assert np.abs(f64(gp.lse[0]) - lse).max() <= 2e-3
 
 
+@pytest.mark.parametrize("listed", [False, True])
+@pytest.mark.parametrize("group,d", [(1, 64), (4, 128)])
+def test_f32_generation_step_keeps_the_thousands_of_small_weights(group, d, listed):
+    """f32, one query, 16000 keys in one part (more KV groups than the GPU has room to cut): the first key of every lane's
+    share has a weight e^17 times the others', of which a thousand and more follow, each below half an ulp of the lane's sum.
+    Added one by one they all vanished (7e-4 of 16, times values of 3)."""
+    b, n_kv, T = 19, 8, 16000
+    first = torch.arange(8)[:, None] * (512 // d) + torch.arange(128 // d)
+    g = torch.Generator("cuda").manual_seed(5)
+    q = torch.zeros(b, n_kv * group, 1, d, device="cuda")
+    q[..., 0] = d ** 0.5                                         # logits are the keys' first elements
+    k = 0.1 * torch.randn(b, n_kv, T + 1, d, device="cuda", generator=g)
+    k[:, :, first.flatten().cuda(), 0] = 17.0
+    v = 3.0 + torch.rand(b, n_kv, T + 1, d, device="cuda", generator=g)
+    v[:, :, first.flatten().cuda()] = -5.0
+    out, lse = torch.empty_like(q), torch.empty(b, n_kv * group, 1, device="cuda")
+    ctx = torch.full((b,), T, dtype=torch.int32, device="cuda")
+    p = api.make_params(q, k, out, ctx, n_retain=4, kv_budget=T - 3, max_ctx_len=T)
+    ws = api.alloc_workspace(p)
+    if listed:
+        idx = torch.arange(T - 3, dtype=torch.int32, device="cuda").expand(b, n_kv, T - 3).contiguous()
+        api.quoka_sparse_attn(p, q, k, v, idx, torch.full_like(ctx, T - 3), out, lse, ws)
+    else:
+        api.quoka_dense_chunk_attn(p, q, k, v, out, lse, ws)
+    torch.cuda.synchronize()
+    rows = torch.cat([torch.arange(T - 3 if listed else T), torch.tensor([T])]).cuda()
+    w = torch.exp(k[:, :, rows, 0].double())
+    want = (w[:, :, None] @ v[:, :, rows].double())[:, :, 0] / w.sum(-1, keepdim=True)
+    want = want.repeat_interleave(group, 1)
+    assert (out[:, :, 0].double() - want).abs().max() <= 2e-5
+    assert (lse[:, :, 0].double() - torch.log(w.sum(-1)).repeat_interleave(group, 1)).abs().max() <= 1e-5
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_generation_step_over_an_infinite_value(dtype):
+    """An infinite value among hundreds makes its output infinite, not NaN, and no other."""
+    gp = problem(79, n_q=4, n_kv=2, d=64, T=900, C=1, dtype=dtype, n_retain=4, kv_budget=900)
+    gp.v[:, 0, 5, 7], gp.v[:, 0, 600, 9] = float("inf"), float("-inf")
+    api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+    torch.cuda.synchronize()
+    assert (gp.out[0, :2, 0, 7] == float("inf")).all() and (gp.out[0, :2, 0, 9] == float("-inf")).all()
+    assert int(torch.isfinite(gp.out).sum()) == gp.out.numel() - 4
+
+
 @pytest.mark.parametrize("paged", [False, True])
 @pytest.mark.parametrize("T,max_ctx,B,n_q,n_kv,d,dtype", [
     ([2049], 2049, 64, 8, 2, 128, "bf16"),        # just beyond the two-launch form: 258 positions per CTA
