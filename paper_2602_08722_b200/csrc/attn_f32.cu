@@ -12,6 +12,8 @@
 // thousands of weights below half an ulp of a sum that one key dominates must not vanish one by one.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "f32_tiles.cuh"
 
 namespace cg = cooperative_groups;
@@ -126,34 +128,53 @@ attn_f32_kernel(DevParams P, const float* __restrict__ q, const float* __restric
     cp_async_wait<1>();                          // V has landed, the next K may still be in flight
     __syncthreads();                             // (and P is written: its rows are read by the same half warp only)
     // (in halves of 32 keys, each added to the running output with compensation)
+    const int seen = cnt + r0 + 1 - t * kF32Tile;               // columns that every row of the block sees
 #pragma unroll 1
     for (int u0 = 0; u0 < kF32Tile; u0 += kF32Tile / 2) {
       uint64_t pv[4][2 * NC];
+      const auto sum_half = [&](auto leave_out) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 2 * NC; ++j) pv[i][j] = 0ull;
+          for (int j = 0; j < 2 * NC; ++j) pv[i][j] = 0ull;
 #pragma unroll 2
-      for (int u = u0; u < u0 + kF32Tile / 2; u += 4) {
-        float4 p[4];
+        for (int u = u0; u < u0 + kF32Tile / 2; u += 4) {
+          float4 p[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) p[i] = *reinterpret_cast<const float4*>(ps + (4 * ty + i) * kPPitch + u);
+          for (int i = 0; i < 4; ++i) p[i] = *reinterpret_cast<const float4*>(ps + (4 * ty + i) * kPPitch + u);
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          ulonglong2 vv[NC];
+          for (int w = 0; w < 4; ++w) {
+            ulonglong2 vv[NC];
 #pragma unroll
-          for (int g = 0; g < NC; ++g) vv[g] = *reinterpret_cast<const ulonglong2*>(vs + (u + w) * D + 64 * g + 4 * tx);
+            for (int g = 0; g < NC; ++g) vv[g] = *reinterpret_cast<const ulonglong2*>(vs + (u + w) * D + 64 * g + 4 * tx);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float pw = w == 0 ? p[i].x : (w == 1 ? p[i].y : (w == 2 ? p[i].z : p[i].w));
-            const uint64_t p2 = pack2(pw, pw);
+            for (int i = 0; i < 4; ++i) {
+              if constexpr (decltype(leave_out)::value) {
+                if (u + w >= seen + 4 * ty + i) continue;       // row r0 + 4 ty + i does not see this key
+              }
+              const float pw = w == 0 ? p[i].x : (w == 1 ? p[i].y : (w == 2 ? p[i].z : p[i].w));
+              const uint64_t p2 = pack2(pw, pw);
 #pragma unroll
-            for (int g = 0; g < NC; ++g) {
-              pv[i][2 * g] = fma2(p2, vv[g].x, pv[i][2 * g]);
-              pv[i][2 * g + 1] = fma2(p2, vv[g].y, pv[i][2 * g + 1]);
+              for (int g = 0; g < NC; ++g) {
+                pv[i][2 * g] = fma2(p2, vv[g].x, pv[i][2 * g]);
+                pv[i][2 * g + 1] = fma2(p2, vv[g].y, pv[i][2 * g + 1]);
+              }
             }
           }
         }
+      };
+      sum_half(std::false_type{});
+      if (seen < kF32Tile) {
+        // Rows of the chunk that some of these query rows do not see.  Their weights are 0, and 0 times a value that is
+        // not finite is NaN: then once more without them.
+        uint64_t all = 0ull;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 2 * NC; ++j) all = fma2(pv[i][j], 0ull, all);
+        float x[2];
+        unpack2(all, x[0], x[1]);
+        if (!(x[0] + x[1] == 0.f)) sum_half(std::true_type{});
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i)

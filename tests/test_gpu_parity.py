@@ -752,6 +752,28 @@ def test_f32_tiles_at_their_edges(T, C, B, n_q, n_kv, d, n_retain, paged):
     assert np.abs(f64(gp.lse[0]) - lse).max() <= 2e-3
 
 
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+@pytest.mark.parametrize("T,C,B,n_q,n_kv,d", [(2000, 200, 300, 4, 2, 128), (100, 64, 30, 2, 1, 64), (700, 650, 100, 32, 8, 64)])
+def test_f32_values_of_later_rows_do_not_reach_earlier_ones(T, C, B, n_q, n_kv, d, bad):
+    """A value that is not finite reaches the rows that attend it and no others, although a tile holds both."""
+    gp = problem(960 + T, n_q=n_q, n_kv=n_kv, d=d, T=T, C=C, dtype="f32", n_retain=16, kv_budget=B)
+    for call in ("sparse", "dense"):
+        got = []
+        for row in (None, C // 2 + 3):
+            if row is not None:
+                gp.v[:, :, T + row, d // 3] = bad
+            if call == "sparse":
+                api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+            else:
+                api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, None, gp.ws)
+            torch.cuda.synchronize()
+            got.append(gp.out.clone())
+        gp.v[:, :, T + row, d // 3] = 0.5
+        assert torch.isfinite(got[0]).all()
+        assert torch.equal(got[1][:, :, :row], got[0][:, :, :row])
+        assert not torch.isfinite(got[1][:, :, row:, d // 3]).any()
+
+
 @pytest.mark.parametrize("mode", ["cosine", "dot"])
 @pytest.mark.parametrize("T,n_kv", [(513, 3), (8193, 8), (16385, 8), (16385, 33), (20011, 73), (32768, 14), (32769, 15)])
 def test_select_keys_every_cluster_width(T, n_kv, mode):
