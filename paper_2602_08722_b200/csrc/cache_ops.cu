@@ -10,14 +10,14 @@
 
 namespace quoka {
 
-template <typename E>
+template <typename E, int D>
 __global__ void __launch_bounds__(256) append_kv_kernel(DevParams P, const uint4* __restrict__ k_new,
                                                          const uint4* __restrict__ v_new, uint4* __restrict__ k_cache,
                                                          uint4* __restrict__ v_cache, float* __restrict__ k_inv_norm) {
   constexpr int ES = (int)sizeof(E);
   grid_dependency_wait();
   grid_launch_dependents();
-  const int wpr = P.d * ES / 16;                                     // 16-byte words per row: 8, 16 or 32
+  constexpr int wpr = D * ES / 16;                                   // 16-byte words per row: 8, 16 or 32
   const int64_t total = (int64_t)P.batch * P.n_kv * P.chunk * wpr;
   const int lane = threadIdx.x & 31;
   for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; e0 < total; e0 += (int64_t)gridDim.x * blockDim.x) {
@@ -39,20 +39,30 @@ __global__ void __launch_bounds__(256) append_kv_kernel(DevParams P, const uint4
       v_cache[dst] = vw;
     }
     if (k_inv_norm != nullptr) {
+      // The sum of squares in key_norms_kernel's order, for its bits: D / 32 elements in a row, then the 32 such pieces of the
+      // row by a butterfly from the far halves to the neighbours.  A word holds kPieces of them, next to each other.
+      constexpr int NE = D / 32, kPieces = 16 / ES / NE;
       const uint32_t v[4] = {kw.x, kw.y, kw.z, kw.w};
-      float nn = 0.f;
+      float nn[kPieces];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if constexpr (ES == 2) {
-          const float a = __uint_as_float(v[j] << 16), b = __uint_as_float(v[j] & 0xFFFF0000u);
-          nn = fmaf(a, a, fmaf(b, b, nn));
-        } else {
-          const float a = __uint_as_float(v[j]);
-          nn = fmaf(a, a, nn);
+      for (int i = 0; i < kPieces; ++i) {
+        nn[i] = 0.f;
+#pragma unroll
+        for (int j = i * NE; j < (i + 1) * NE; ++j) {
+          const uint32_t w32 = v[j * ES / 4];
+          const float x = ES == 4 ? __uint_as_float(w32) : __uint_as_float(j % 2 ? w32 & 0xFFFF0000u : w32 << 16);
+          nn[i] = fmaf(x, x, nn[i]);
         }
       }
-      for (int o = wpr / 2; o > 0; o >>= 1) nn += __shfl_xor_sync(0xFFFFFFFFu, nn, o);
-      if (live && w == 0) k_inv_norm[kv_norm_index(P, s, h, t)] = 1.f / fmaxf(sqrtf(nn), kNormEps);
+#pragma unroll
+      for (int o = wpr / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) nn[i] += __shfl_xor_sync(0xFFFFFFFFu, nn[i], o);
+#pragma unroll
+      for (int o = kPieces / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < o; ++i) nn[i] += nn[i + o];
+      if (live && w == 0) k_inv_norm[kv_norm_index(P, s, h, t)] = 1.f / fmaxf(sqrtf(nn[0]), kNormEps);
     }
   }
 }
@@ -66,10 +76,12 @@ cudaError_t launch_append_kv(const DevParams& P, int dtype, const void* k_new, c
   if (blocks > 148 * 16) blocks = 148 * 16;
   const dim3 grid((unsigned)blocks), block(256);
   cudaError_t e;
-  if (es == 2)
-    e = launch_kernel("append_kv", append_kv_kernel<__nv_bfloat16>, grid, block, 0, st, 1, true, P, (const uint4*)k_new, (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache, k_inv_norm);
-  else
-    e = launch_kernel("append_kv", append_kv_kernel<float>, grid, block, 0, st, 1, true, P, (const uint4*)k_new, (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache, k_inv_norm);
+#define QUOKA_APPEND(E_, D_)                                                                                        \
+  e = launch_kernel("append_kv", append_kv_kernel<E_, D_>, grid, block, 0, st, 1, true, P, (const uint4*)k_new,     \
+                    (const uint4*)v_new, (uint4*)k_cache, (uint4*)v_cache, k_inv_norm)
+  if (es == 2) { if (P.d == 128) QUOKA_APPEND(__nv_bfloat16, 128); else QUOKA_APPEND(__nv_bfloat16, 64); }
+  else { if (P.d == 128) QUOKA_APPEND(float, 128); else QUOKA_APPEND(float, 64); }
+#undef QUOKA_APPEND
   if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();

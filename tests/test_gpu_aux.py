@@ -81,6 +81,23 @@ def test_append_kv_f32_contiguous():
     assert torch.equal(gp.k, want_k) and torch.equal(gp.v, want_v)
 
 
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("d,dtype", [(128, "bf16"), (64, "bf16"), (128, "f32"), (64, "f32")])
+def test_append_kv_writes_the_inverse_norms_that_update_key_norms_writes(d, dtype, paged):
+    """The same bits: a cache of norms kept by the one and rebuilt by the other scores, and so selects, the same keys."""
+    inp = synth.make_chunk_inputs(61, 2, 4, 2, d, [300, 77], 65, dtype)
+    if paged:
+        inp = synth.to_paged(inp, 61)
+    gp = GpuProblem(inp, 8, kv_budget=16, paged=paged)
+    k_new = torch.randn(2, 2, 65, d, device="cuda").to(gp.k.dtype)
+    kept = torch.zeros(gp.k.shape[:3], device="cuda")
+    rebuilt = torch.zeros_like(kept)
+    api.quoka_append_kv(gp.p, k_new, k_new, gp.k, gp.v, kept, gp.ws)
+    api.quoka_update_key_norms(gp.p, gp.k, rebuilt, False, gp.ws)
+    torch.cuda.synchronize()
+    assert torch.equal(kept, rebuilt) and int((kept != 0).sum()) == 2 * 2 * 65
+
+
 # ---------------------------------------------------------------- the bounded device wait
 def test_a_wait_that_nobody_satisfies_gives_up_and_reports():
     inp = synth.make_chunk_inputs(33, 1, 4, 2, 128, 500, 130, "bf16")
