@@ -31,10 +31,10 @@ __global__ void __launch_bounds__(256) append_kv_kernel(DevParams P, const uint4
     uint4 kw = make_uint4(0, 0, 0, 0);
     int t = 0;
     if (live) {
-      kw = __ldg(k_new + e);
-      const uint4 vw = __ldg(v_new + e);
-      t = __ldg(P.ctx_len + s) + r;
-      const int64_t dst = kv_row_offset(P, s, h, t) * ES / 16 + w;   // strides are multiples of 8 elements
+      kw = load_input<true>(k_new + e);
+      const uint4 vw = load_input<true>(v_new + e);
+      t = load_input<true>(P.ctx_len + s) + r;
+      const int64_t dst = kv_row_offset<true>(P, s, h, t) * ES / 16 + w;   // strides are multiples of 8 elements
       k_cache[dst] = kw;
       v_cache[dst] = vw;
     }
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(256) append_kv_kernel(DevParams P, const uint4
       for (int o = kPieces / 2; o > 0; o >>= 1)
 #pragma unroll
         for (int i = 0; i < o; ++i) nn[i] += nn[i + o];
-      if (live && w == 0) k_inv_norm[kv_norm_index(P, s, h, t)] = 1.f / fmaxf(sqrtf(nn[0]), kNormEps);
+      if (live && w == 0) k_inv_norm[kv_norm_index<true>(P, s, h, t)] = 1.f / fmaxf(sqrtf(nn[0]), kNormEps);
     }
   }
 }

@@ -53,17 +53,26 @@ __host__ __device__ inline int key_budget(int T, int kv_budget, float frac) {
   return B < T ? B : T;
 }
 
+// Reads by a kernel that may be resident before the caller's data is complete (the first kernel of a call, see "programmatic
+// dependent launch" below) go to L2: the read-only path is for what nobody writes while the kernel lives.
+template <bool FIRST, typename T>
+__device__ __forceinline__ T load_input(const T* p) {
+  if constexpr (FIRST) return __ldcg(p); else return __ldg(p);
+}
+
 // Element offset of row t of (sequence s, KV head h) in a contiguous or paged cache.
+template <bool FIRST = false>
 __device__ __forceinline__ int64_t kv_row_offset(const DevParams& P, int s, int h, int t) {
   if (P.page_size == 0) return (int64_t)s * P.kv_sb + (int64_t)h * P.kv_sh + (int64_t)t * P.kv_st;
-  const int page = __ldg(P.block_table + (int64_t)s * P.max_pages + (t >> 6));
+  const int page = load_input<FIRST>(P.block_table + (int64_t)s * P.max_pages + (t >> 6));
   return (int64_t)page * P.kv_sb + (int64_t)h * P.kv_sh + (int64_t)(t & (kPage - 1)) * P.kv_st;
 }
 
 // Index of row t of (sequence s, KV head h) in the cached inverse-norm array (the cache's layout without head_dim).
+template <bool FIRST = false>
 __device__ __forceinline__ int64_t kv_norm_index(const DevParams& P, int s, int h, int t) {
   if (P.page_size == 0) return ((int64_t)s * P.n_kv + h) * P.kv_rows + t;
-  const int page = __ldg(P.block_table + (int64_t)s * P.max_pages + (t >> 6));
+  const int page = load_input<FIRST>(P.block_table + (int64_t)s * P.max_pages + (t >> 6));
   return ((int64_t)page * P.n_kv + h) * kPage + (t & (kPage - 1));
 }
 
@@ -75,20 +84,20 @@ template <> __device__ __forceinline__ float from_f32<float>(float x) { return x
 template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
 
 // Load NE consecutive elements (NE*sizeof(T) is 8, 16 or 32 bytes, pointer aligned to min(16, that)) as floats.
-template <typename T, int NE>
+template <typename T, int NE, bool FIRST = false>
 __device__ __forceinline__ void load_vec(const T* __restrict__ p, float (&out)[NE]) {
   if constexpr (sizeof(T) == 4) {
     if constexpr (NE % 4 == 0) {
 #pragma unroll
       for (int i = 0; i < NE / 4; ++i) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(p) + i);
+        const float4 v = load_input<FIRST>(reinterpret_cast<const float4*>(p) + i);
         out[4 * i + 0] = v.x; out[4 * i + 1] = v.y; out[4 * i + 2] = v.z; out[4 * i + 3] = v.w;
       }
     } else {
       static_assert(NE % 2 == 0, "NE");
 #pragma unroll
       for (int i = 0; i < NE / 2; ++i) {
-        const float2 v = __ldg(reinterpret_cast<const float2*>(p) + i);
+        const float2 v = load_input<FIRST>(reinterpret_cast<const float2*>(p) + i);
         out[2 * i] = v.x; out[2 * i + 1] = v.y;
       }
     }
@@ -96,7 +105,7 @@ __device__ __forceinline__ void load_vec(const T* __restrict__ p, float (&out)[N
     if constexpr (NE % 8 == 0) {
 #pragma unroll
       for (int i = 0; i < NE / 8; ++i) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(p) + i);
+        const uint4 v = load_input<FIRST>(reinterpret_cast<const uint4*>(p) + i);
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -107,7 +116,7 @@ __device__ __forceinline__ void load_vec(const T* __restrict__ p, float (&out)[N
     } else if constexpr (NE % 4 == 0) {
 #pragma unroll
       for (int i = 0; i < NE / 4; ++i) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2*>(p) + i);
+        const uint2 v = load_input<FIRST>(reinterpret_cast<const uint2*>(p) + i);
         out[4 * i + 0] = __uint_as_float(v.x << 16); out[4 * i + 1] = __uint_as_float(v.x & 0xFFFF0000u);
         out[4 * i + 2] = __uint_as_float(v.y << 16); out[4 * i + 3] = __uint_as_float(v.y & 0xFFFF0000u);
       }
@@ -115,7 +124,7 @@ __device__ __forceinline__ void load_vec(const T* __restrict__ p, float (&out)[N
       static_assert(NE % 2 == 0, "NE");
 #pragma unroll
       for (int i = 0; i < NE / 2; ++i) {
-        const uint32_t v = __ldg(reinterpret_cast<const uint32_t*>(p) + i);
+        const uint32_t v = load_input<FIRST>(reinterpret_cast<const uint32_t*>(p) + i);
         out[2 * i] = __uint_as_float(v << 16); out[2 * i + 1] = __uint_as_float(v & 0xFFFF0000u);
       }
     }
@@ -151,10 +160,17 @@ __device__ __forceinline__ float warp_sum(float x) {
 // launched with programmatic stream serialisation may become resident while the kernel before it still runs;
 // it must then execute grid_dependency_wait() before its first access to anything that kernel writes (the wait
 // returns once that grid has completed and its writes are visible; without the launch attribute it returns at
-// once).  A kernel lets the one after it start early with grid_launch_dependents(), which every CTA executes at
-// its start; the dependent grid is launched when all of them have, so it never holds resources that this
-// grid's own CTAs still need.  The first kernel of a call is launched this way too, whatever is before it on the stream;
-// it waits before anything else and lets the second one start only after that.
+// once), and read it through L2, not the read-only path.  A kernel lets the one after it start early with
+// grid_launch_dependents(); the dependent grid is launched when every CTA has executed it or ended, so it never holds
+// resources that this grid's own CTAs still need.  No CTA of a chained kernel ends without having waited, so that the
+// completion of the last link is the completion of all.  Where the signal stands:
+//  - In the first kernel of a call, after its wait: it may be launched early itself (generation steps, appended rows, and
+//    prefill whose attention grid is below a wave), behind whatever the caller has on the stream, and the second kernel reads
+//    the caller's inputs before it waits.
+//  - In the sparse attention of whole row blocks, after it has learnt the list length, that is after its wait: the parts
+//    launched behind it (learn_count) read the list without a wait of their own.  Do not move it to the start.
+//  - Parts do not signal; the last CTA of a launch of parts waits for the whole row blocks before it ends.
+//  - Everywhere else at the start.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -37,16 +37,17 @@ constexpr size_t kGemvSmem = (size_t)(kGemvThreads / 32) * kGemvStages * (kGemvU
 template <typename T, int D>
 constexpr int gemv_unit_rows() { return kGemvUnitBytes / (D * (int)sizeof(T)); }
 
-// Position in the list of units: the u-th unit of (sequence s, KV head kv), `left` units before the warp's share ends.
+// Position in the list of units: the u-th unit of (sequence s, KV head kv), `left` units before the warp's share ends; T rows
+// in the sequence.
 struct UnitWalk {
-  int s, kv, u, units_s, left;
+  int s, kv, u, units_s, left, T;
   __device__ __forceinline__ void next(const DevParams& P, int unit_rows) {
     --left;
     if (++u < units_s || left <= 0) return;
     u = 0;
     if (++kv < P.n_kv) return;
     kv = 0;
-    do { units_s = (__ldg(P.ctx_len + ++s) + unit_rows - 1) / unit_rows; } while (units_s == 0);
+    do { T = load_input<true>(P.ctx_len + ++s); units_s = (T + unit_rows - 1) / unit_rows; } while (units_s == 0);
   }
 };
 
@@ -74,7 +75,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) score_keys_gemv_kernel(DevPar
   {
     int total = 0;
     for (int s0 = 0; s0 < P.batch; s0 += 32) {
-      const int T_l = s0 + lane < P.batch ? __ldg(P.ctx_len + s0 + lane) : 0;
+      const int T_l = s0 + lane < P.batch ? load_input<true>(P.ctx_len + s0 + lane) : 0;
       total += __reduce_add_sync(0xFFFFFFFFu, (T_l + ROWS - 1) / ROWS * P.n_kv);
     }
     const int n_warps = gridDim.x * (kGemvThreads / 32), id = blockIdx.x + gridDim.x * warp;   // (a short list: all SMs)
@@ -82,7 +83,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) score_keys_gemv_kernel(DevPar
     w.left = (int)((long long)total * (id + 1) / n_warps) - lo;
     if (w.left == 0) return;
     for (int s0 = 0;; s0 += 32) {
-      const int T_l = s0 + lane < P.batch ? __ldg(P.ctx_len + s0 + lane) : 0;
+      const int T_l = s0 + lane < P.batch ? load_input<true>(P.ctx_len + s0 + lane) : 0;
       const int u_l = (T_l + ROWS - 1) / ROWS, n_l = u_l * P.n_kv;
       int incl = n_l;
 #pragma unroll
@@ -96,6 +97,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) score_keys_gemv_kernel(DevPar
         lo -= __shfl_sync(0xFFFFFFFFu, incl - n_l, src);
         w.s = s0 + src;
         w.units_s = __shfl_sync(0xFFFFFFFFu, u_l, src);
+        w.T = __shfl_sync(0xFFFFFFFFu, T_l, src);
         w.kv = lo / w.units_s;
         w.u = lo % w.units_s;
         break;
@@ -109,12 +111,12 @@ __global__ void __launch_bounds__(kGemvThreads, 1) score_keys_gemv_kernel(DevPar
   // ---- filling the ring: one group per unit, empty past the share
   UnitWalk in = w;
   const auto page_of = [&](const UnitWalk& at) {
-    return P.page_size != 0 && at.left > 0 ? __ldg(P.block_table + (long long)at.s * P.max_pages + at.u * ROWS / kPage) : 0;
+    return P.page_size != 0 && at.left > 0 ? load_input<true>(P.block_table + (long long)at.s * P.max_pages + at.u * ROWS / kPage) : 0;
   };
   int page = page_of(in);
   const auto fill = [&](int stage) {
     if (in.left > 0) {
-      const int t0 = in.u * ROWS, T_s = __ldg(P.ctx_len + in.s);
+      const int t0 = in.u * ROWS, T_s = in.T;
       const T* base = P.page_size == 0 ? k + (long long)in.s * P.kv_sb + (long long)in.kv * P.kv_sh + (long long)t0 * P.kv_st
                                        : k + (long long)page * P.kv_sb + (long long)in.kv * P.kv_sh + (long long)(t0 & (kPage - 1)) * P.kv_st;
 #pragma unroll
@@ -191,7 +193,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) score_keys_gemv_kernel(DevPar
       val /= fmaxf(sqrtf(nn[0]), kNormEps);
     }
     const int t = w.u * ROWS + my_row;
-    if (c % kRep == 0 && t < __ldg(P.ctx_len + s_cur)) scores[((long long)s_cur * P.n_kv + kv_cur) * P.max_ctx + t] = val;
+    if (c % kRep == 0 && t < w.T) scores[((long long)s_cur * P.n_kv + kv_cur) * P.max_ctx + t] = val;
     fill(stage);
     if (++stage == kGemvStages) stage = 0;
   }

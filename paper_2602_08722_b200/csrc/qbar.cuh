@@ -25,7 +25,7 @@ __device__ __forceinline__ void mean_normalised_query(const DevParams& P, const 
         const int r = __shfl_sync(0xFFFFFFFFu, r_lane, g & 31);
         if (g < g_end) {
           const int h = kv * P.group + g0 + g;
-          load_vec<T, NE>(q + (int64_t)s * P.q_sb + (int64_t)h * P.q_sh + (int64_t)r * P.q_st + lane * NE, x[u]);
+          load_vec<T, NE, /*FIRST=*/true>(q + (int64_t)s * P.q_sb + (int64_t)h * P.q_sh + (int64_t)r * P.q_st + lane * NE, x[u]);
         } else {
 #pragma unroll
           for (int i = 0; i < NE; ++i) x[u][i] = 0.f;

@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kSelThreads) select_keys_kernel(DevParams P, c
     for (int t0 = 0; t0 < T; t0 += kSelThreads) {
       const int t = t0 + tid;
       const bool in = t < T;
-      const uint32_t key = in ? float_order_key(__ldg(row + t)) : 0u;
+      const uint32_t key = in ? float_order_key(__ldcg(row + t)) : 0u;
       const bool live = in && ((key & mask) == prefix);
       const uint32_t digit = live ? ((key >> shift) & 255u) : 256u + (uint32_t)lane;   // dead lanes match nobody
       const uint32_t peers = __match_any_sync(0xFFFFFFFFu, digit);
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kSelThreads) select_keys_kernel(DevParams P, c
   uint32_t run_gt = 0, run_eq = 0;
   for (int t0 = 0; t0 < T; t0 += kSelThreads) {
     const int t = t0 + tid;
-    const uint32_t key = (t < T) ? float_order_key(__ldg(row + t)) : 0u;
+    const uint32_t key = (t < T) ? float_order_key(__ldcg(row + t)) : 0u;
     const bool gt = (t < T) && key > thr;
     const bool eq = (t < T) && key == thr;
     const uint32_t b_gt = __ballot_sync(0xFFFFFFFFu, gt);

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) rank_queries_kernel(DevParams
     const uint4* src = reinterpret_cast<const uint4*>(qh + (long long)(lo + rc) * P.q_st + lane_in_row * 8);
     Raw8<T> raw;
 #pragma unroll
-    for (int w = 0; w < NW; ++w) raw.w[w] = __ldg(src + w);
+    for (int w = 0; w < NW; ++w) raw.w[w] = load_input<true>(src + w);
     add_row(raw, r < n_loc);
   }
 #pragma unroll

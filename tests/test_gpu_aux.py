@@ -1,6 +1,8 @@
 """Algorithm 2 as a loop with a growing cache (append, select, attend, every chunk against the oracle), and the
 library's diagnostics: the bounded device wait, the debug build's index checks, the host-side block-table check."""
 import ctypes as C
+import shutil
+import subprocess
 
 import numpy as np
 import pytest
@@ -96,6 +98,103 @@ def test_append_kv_writes_the_inverse_norms_that_update_key_norms_writes(d, dtyp
     api.quoka_update_key_norms(gp.p, gp.k, rebuilt, False, gp.ws)
     torch.cuda.synchronize()
     assert torch.equal(kept, rebuilt) and int((kept != 0).sum()) == 2 * 2 * 65
+
+
+# ---------------------------------------------------------------- a caller's kernel that signals its dependents early
+EARLY_PRODUCER = """
+// Reads `data` (through L1, in every CTA), lets the next kernel of the stream start, and writes it 30 us later.
+__global__ void produce(const uint4* fresh, uint4* data, int words, uint4* sink) {
+  uint4 w = make_uint4(0, 0, 0, 0);
+  const auto look = [&]() {
+    for (int i = threadIdx.x; i < words; i += blockDim.x) {
+      uint4 v;
+      asm volatile("ld.global.ca.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(data + i));
+      w.x ^= v.x; w.y ^= v.y; w.z ^= v.z; w.w ^= v.w;
+    }
+  };
+  look();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const long long t0 = clock64();
+  while (clock64() - t0 < 60000) {}
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < words; i += blockDim.x) data[i] = fresh[i];
+  else
+    while (clock64() - t0 < 120000) look();
+  sink[blockIdx.x * blockDim.x + threadIdx.x] = w;
+}
+extern "C" int launch(const void* fresh, void* data, int words, void* sink, int ctas, void* stream) {
+  produce<<<ctas, 256, 0, (cudaStream_t)stream>>>((const uint4*)fresh, (uint4*)data, words, (uint4*)sink);
+  return (int)cudaGetLastError();
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def early_producer(tmp_path_factory):
+    d = tmp_path_factory.mktemp("early")
+    (d / "produce.cu").write_text(EARLY_PRODUCER)
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-shared", "-Xcompiler", "-fPIC",
+                    "-o", str(d / "produce.so"), str(d / "produce.cu")], check=True)
+    return C.CDLL(str(d / "produce.so"))
+
+
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("call,chunk,n_retain", [("append", 1, 8), ("prefill", 1, 8), ("prefill", 40, 64), ("prefill", 60, 16)],
+                         ids=["append", "generation", "every-query-kept", "ranked"])
+def test_first_kernel_of_a_call_behind_one_that_signals_early(early_producer, call, chunk, n_retain, paged):
+    """The first kernel of a call may be resident while the kernel before it still writes its inputs (queries, new rows,
+    cached lengths, block table): it sees what that kernel has written, not what was there when it started."""
+    n_q, n_kv, d, T = 4, 2, 64, 900
+    inp = synth.make_chunk_inputs(83, 2, n_q, n_kv, d, [T, T - 130], chunk, "bf16")
+    if paged:
+        inp = synth.to_paged(inp, 83)
+    gp = GpuProblem(inp, n_retain, kv_budget=100, paged=paged, max_ctx_len=T)
+    parts = {"q": gp.q, "k_new": torch.randn(2, n_kv, chunk, d, device="cuda").bfloat16(),
+             "v_new": torch.randn(2, n_kv, chunk, d, device="cuda").bfloat16(), "ctx": gp.ctx_len}
+    if paged:
+        parts["table"] = gp.block_table
+    size = {k: -(-v.numel() * v.element_size() // 256) * 256 for k, v in parts.items()}
+    fresh = torch.zeros(sum(size.values()), dtype=torch.uint8, device="cuda")
+    data = torch.zeros_like(fresh)
+    view, at = {}, 0
+    for k, v in parts.items():
+        n = v.numel() * v.element_size()
+        fresh[at:at + n] = v.contiguous().view(-1).view(torch.uint8)
+        view[k] = data[at:at + n].view(v.dtype).view(v.shape)
+        at += size[k]
+    stale = fresh.clone()
+    off = size["q"] + size["k_new"] + size["v_new"]
+    stale[:off] = 0
+    stale[off:off + 8].view(torch.int32).fill_(T // 2)                # valid as well, but not what is asked for
+    if paged:
+        stale[off + size["ctx"]:] = fresh[off + size["ctx"]:].view(2, -1).flip(0).reshape(-1)
+    gp.p.ctx_len = view["ctx"].data_ptr()
+    if paged:
+        gp.p.block_table = view["table"].data_ptr()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sink = torch.empty(sms * 256 * 16, dtype=torch.uint8, device="cuda")
+    k0, v0 = gp.k.clone(), gp.v.clone()
+
+    def run(early):
+        gp.k.copy_(k0); gp.v.copy_(v0); gp.out.zero_()
+        norms = torch.zeros(gp.k.shape[:3], device="cuda")
+        data.copy_(stale if early else fresh)
+        torch.cuda.synchronize()
+        if early:
+            assert early_producer.launch(C.c_void_p(fresh.data_ptr()), C.c_void_p(data.data_ptr()), fresh.numel() // 16,
+                                         C.c_void_p(sink.data_ptr()), sms, C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+        if call == "append":
+            api.quoka_append_kv(gp.p, view["k_new"], view["v_new"], gp.k, gp.v, norms, gp.ws)
+        else:
+            api.quoka_prefill_chunk(gp.p, view["q"], gp.k, gp.v, gp.out, None, None, gp.ws)
+        torch.cuda.synchronize()
+        return gp.k.clone(), gp.v.clone(), gp.out.clone(), norms
+
+    want = run(False)
+    for _ in range(3):
+        assert all(torch.equal(a, b) for a, b in zip(run(True), want))
+    assert api.quoka_last_device_status(gp.ws) == 0
 
 
 # ---------------------------------------------------------------- the bounded device wait
