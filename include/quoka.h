@@ -56,7 +56,7 @@ typedef enum {
   QUOKA_OK = 0,
   QUOKA_ERR_INVALID_ARG = 1,  /* null pointer, non-positive size, n_Q % n_KV != 0, misaligned stride */
   QUOKA_ERR_UNSUPPORTED = 2,  /* head_dim not in {64,128}, page_size not in {0,64}, chunk_len > 8192 with selection */
-  QUOKA_ERR_WORKSPACE = 3,    /* workspace pointer null / misaligned / smaller than quoka_workspace_size */
+  QUOKA_ERR_WORKSPACE = 3,    /* workspace pointer null / misaligned / too small (see quoka_workspace_size) */
   QUOKA_ERR_CUDA = 4,         /* a CUDA runtime or driver call failed (launch, tensor-map encode) */
   QUOKA_ERR_TIMEOUT = 5,      /* device status word: a bounded wait inside a kernel ran out */
   QUOKA_ERR_STATIC_LIMIT = 6, /* quoka_prefill_chunk_static: the problem needs more scratch than the built-in array */
@@ -115,17 +115,23 @@ typedef struct {
 /* Row pitch of k_idx: the largest B_s any sequence can have, from max_ctx_len. */
 quoka_status quoka_kv_budget_cap(const quoka_params* p, int32_t* cap);
 
-/* Bytes of workspace that every call below accepts (256-byte aligned pointer).
+/* Bytes of workspace with which every call below runs as fast as it can (256-byte aligned pointer).
  * The first 256 bytes hold the device status word, which the caller sets to zero
  * once after allocating; the rest is scratch whose contents mean nothing between
  * calls.  Two calls that share a workspace must not overlap on the GPU.
  * For problems whose attention grid is smaller than the GPU (few heads, a short
  * chunk) or leaves much of its last wave empty, the size includes room for the
- * partial results of the split attention kernel, at most 128 MiB of them on large
- * grids (the keys of the lightest row blocks, or of all, are cut into up to 8 parts,
- * one CTA each, and added up in part order: results are reproducible from run to
- * run, and differ from the unsplit kernel's in the last bits only).
- */
+ * partial results of the split attention kernel (the keys of the lightest row
+ * blocks, or of all, are cut into up to 8 parts, one CTA each, and added up in part
+ * order: results are reproducible from run to run, and differ from the unsplit
+ * kernel's in the last bits only).  It comes last and is sized for whichever of
+ * quoka_prefill_chunk / quoka_sparse_attn and quoka_dense_chunk_attn needs more.
+ * On grids of a wave or more (batch * n_Q * ceil(C / 256) no less than the number of
+ * SMs) it is at most 128 MiB, mostly the dense call's (32 heads, C 2048, 32768 cached
+ * rows: 65 MiB, nothing for the sparse call), and may be missing in part or
+ * altogether: a call that does not find room for its own parts leaves the row blocks
+ * whole.  So a workspace made for the longest chunk of a prompt serves the shorter
+ * ones, although their size by this function may be larger. */
 quoka_status quoka_workspace_size(const quoka_params* p, size_t* bytes);
 
 /* Alg. 1, "Query Sub-selection", then the normalisation and the mean over the G

@@ -247,11 +247,10 @@ cudaError_t launch_append_kv(const DevParams& P, int dtype, const void* k_new, c
 // Host checks shared by the fused entry points (everything but the workspace); nothing is enqueued before they pass.
 quoka_status check_prefill_args(const quoka_params* p, const void* q, const void* k_cache, const void* v_cache,
                                 const void* out);
-// the fused call behind quoka_prefill_chunk, and its workspace need, with or without the split-attention scratch
+// the fused call behind quoka_prefill_chunk, arguments checked; and what its buffers take without split-attention scratch
 quoka_status prefill_chunk_impl(const quoka_params* p, const void* q, const void* k_cache, const void* v_cache, void* out,
-                                int32_t* k_idx_out, int32_t* k_cnt_out, void* ws, size_t ws_bytes, void* stream,
-                                bool with_split);
-size_t workspace_bytes(const quoka_params* p, bool with_split);
+                                int32_t* k_idx_out, int32_t* k_cnt_out, void* ws, size_t ws_bytes, void* stream);
+size_t workspace_bytes_unsplit(const quoka_params* p);
 // Device address of the built-in scratch array on the current device (looked up once per device).
 quoka_status static_scratch_for_current_device(void** out);
 

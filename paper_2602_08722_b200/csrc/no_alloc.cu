@@ -45,12 +45,12 @@ extern "C" quoka_status quoka_prefill_chunk_static(const quoka_params* p, const 
   quoka_status st = quoka::check_prefill_args(p, q, k_cache, v_cache, out);
   if (st != QUOKA_OK) return st;
   // the array has no room for the scratch of the split attention kernel: parts merge in clusters or not at all here
-  if (quoka::workspace_bytes(p, /*with_split=*/false) > (size_t)QUOKA_STATIC_SCRATCH_BYTES) return QUOKA_ERR_STATIC_LIMIT;
+  const size_t bytes = quoka::workspace_bytes_unsplit(p);
+  if (bytes > (size_t)QUOKA_STATIC_SCRATCH_BYTES) return QUOKA_ERR_STATIC_LIMIT;
   void* scratch = nullptr;
   if ((st = quoka::static_scratch_for_current_device(&scratch)) != QUOKA_OK) return st;
   // The array keeps whatever the previous call left.  Only the status word has to start at zero;
   // everything else is written before it is read.
   if (cudaMemsetAsync(scratch, 0, 256, static_cast<cudaStream_t>(stream)) != cudaSuccess) return QUOKA_ERR_CUDA;
-  return quoka::prefill_chunk_impl(p, q, k_cache, v_cache, out, k_idx_out, k_cnt_out, scratch,
-                                   (size_t)QUOKA_STATIC_SCRATCH_BYTES, stream, /*with_split=*/false);
+  return quoka::prefill_chunk_impl(p, q, k_cache, v_cache, out, k_idx_out, k_cnt_out, scratch, bytes, stream);
 }

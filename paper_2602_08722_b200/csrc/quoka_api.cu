@@ -35,30 +35,18 @@ static int budget_cap_of(const quoka_params* p) {
   return cap < 1 ? 1 : cap;
 }
 
-// The two plans an attention call of this problem may follow, and the scratch that serves either.
-struct AttnScratch { AttnPlan sparse, dense; size_t counters = 0, partials = 0; };
-static AttnScratch attn_scratch(const quoka_params* p) {
-  AttnScratch a;
-  a.sparse = attn_plan_sparse(p, budget_cap_of(p));
-  a.dense = attn_plan_dense(p);
-  for (const AttnPlan& plan : {a.sparse, a.dense}) {
-    const size_t c = attn_split_counter_bytes(p, plan), b = attn_split_partial_bytes(p, plan);
-    a.counters = c > a.counters ? c : a.counters;
-    a.partials = b > a.partials ? b : a.partials;
-  }
-  return a;
-}
-
-// with_split = false: the layout without the split-attention scratch (every call still works, without parts that merge through memory)
-static Workspace carve(const quoka_params* p, void* ws, bool with_split = true) {
+// The buffers of a call in a workspace of ws_bytes.  The scratch of `plan` (partial results and arrival counters of row
+// blocks in parts that merge through memory), where the plan has any, comes last and only if there is room for it: the
+// attention leaves the row blocks whole without it.
+static Workspace carve(const quoka_params* p, void* ws, size_t ws_bytes = 0, const AttnPlan* plan = nullptr) {
   Workspace w{};
   const size_t es = p->dtype == QUOKA_BF16 ? 2 : 4;
   const int N = p->n_retain < p->chunk_len ? p->n_retain : p->chunk_len;
-  const int cap = budget_cap_of(p);
-  char* base = static_cast<char*>(ws);
+  const size_t cap = (size_t)budget_cap_of(p);
+  unsigned char* base = static_cast<unsigned char*>(ws);
   size_t off = 0;
   auto take = [&](size_t bytes) {
-    char* r = base ? base + off : nullptr;
+    unsigned char* r = base ? base + off : nullptr;
     off += align_up(bytes);
     return r;
   };
@@ -68,16 +56,30 @@ static Workspace carve(const quoka_params* p, void* ws, bool with_split = true) 
   w.scores = reinterpret_cast<float*>(take((size_t)p->batch * p->n_kv_heads * (size_t)(p->max_ctx_len > 0 ? p->max_ctx_len : 1) * 4));
   w.k_idx = reinterpret_cast<int32_t*>(take((size_t)p->batch * p->n_kv_heads * cap * 4));
   w.k_cnt = reinterpret_cast<int32_t*>(take((size_t)p->batch * 4));
-  if (with_split) {
-    const AttnScratch a = attn_scratch(p);
-    if (a.counters > 0) {
-      w.attn_counters = reinterpret_cast<int32_t*>(take(a.counters));
-      w.attn_partials = reinterpret_cast<float*>(take(a.partials));
-      w.n_attn_counters = (int)(a.counters / sizeof(int32_t));
-    }
+  const size_t counters = plan ? attn_split_counter_bytes(p, *plan) : 0;
+  if (counters > 0 && off + align_up(counters) + align_up(attn_split_partial_bytes(p, *plan)) <= ws_bytes) {
+    w.attn_counters = reinterpret_cast<int32_t*>(take(counters));
+    w.attn_partials = reinterpret_cast<float*>(take(attn_split_partial_bytes(p, *plan)));
+    w.n_attn_counters = (int)(counters / sizeof(int32_t));
   }
   w.total = off;
   return w;
+}
+
+// The scratch of the larger of the two plans an attention call of this problem may follow.
+static size_t attn_scratch_bytes(const quoka_params* p) {
+  size_t bytes = 0;
+  for (const AttnPlan& plan : {attn_plan_sparse(p, budget_cap_of(p)), attn_plan_dense(p)}) {
+    const size_t b = align_up(attn_split_counter_bytes(p, plan)) + align_up(attn_split_partial_bytes(p, plan));
+    bytes = b > bytes ? b : bytes;
+  }
+  return bytes;
+}
+// The least a call takes.  A grid below a wave needs its scratch (its parts are what fills the GPU); that of a larger grid
+// only levels the last wave and may be missing: it does not grow with the chunk or the context (2048 queries of 32 heads at
+// 4096 rows have none, 1500 have 12 MiB), and a workspace made for the longest chunk serves the shorter ones.
+static size_t workspace_least(const quoka_params* p) {
+  return carve(p, nullptr).total + (attn_below_a_wave(p) ? attn_scratch_bytes(p) : 0);
 }
 
 static quoka_status validate(const quoka_params* p) {
@@ -120,13 +122,13 @@ quoka_status check_prefill_args(const quoka_params* p, const void* q, const void
   return QUOKA_OK;
 }
 
-static quoka_status check_ws(const quoka_params* p, void* ws, size_t ws_bytes, bool with_split = true) {
+static quoka_status check_ws(const quoka_params* p, void* ws, size_t ws_bytes) {
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0) return QUOKA_ERR_WORKSPACE;
-  if (ws_bytes < carve(p, nullptr, with_split).total) return QUOKA_ERR_WORKSPACE;
+  if (ws_bytes < workspace_least(p)) return QUOKA_ERR_WORKSPACE;
   return QUOKA_OK;
 }
 
-size_t workspace_bytes(const quoka_params* p, bool with_split) { return carve(p, nullptr, with_split).total; }
+size_t workspace_bytes_unsplit(const quoka_params* p) { return carve(p, nullptr).total; }
 
 static DevParams make_dev(const quoka_params* p, void* ws, const Workspace& w) {
   DevParams P{};
@@ -193,7 +195,7 @@ static quoka_status run_score_keys(const quoka_params* p, const DevParams& P, co
 
 static quoka_status run_attn(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                              const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
-                             bool after_selection = false, const AttnPlan* plan = nullptr) {
+                             const AttnPlan& plan, bool after_selection = false) {
   if (p->impl == QUOKA_IMPL_AUTO && P.chunk == 1) {
     // (a fused call that gets here does not have the one-launch form: run_prefill would have taken it)
     if (k_idx && !after_selection && decode_path_applies(P) && decode_select_attn_applies(P))
@@ -203,8 +205,7 @@ static quoka_status run_attn(const quoka_params* p, const DevParams& P, const vo
     return QUOKA_OK;
   }
   if (use_tensor(p) && attn_tc_supported(p))
-    return launch_attn_tc(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection,
-                          plan ? *plan : (k_idx ? attn_plan_sparse(p, P.budget_cap) : attn_plan_dense(p)));
+    return launch_attn_tc(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection, plan);
   if (p->impl == QUOKA_IMPL_TENSOR) return QUOKA_ERR_UNSUPPORTED;
   if (p->impl == QUOKA_IMPL_AUTO && p->dtype == QUOKA_F32) {
     QUOKA_TRY_CUDA(launch_attn_f32(P, static_cast<const float*>(q), static_cast<const float*>(k), static_cast<const float*>(v),
@@ -272,19 +273,16 @@ static quoka_status run_prefill(const quoka_params* p, const DevParams& P, const
   }
   // with an empty cache the selection kernel only writes k_cnt = 0 and the -1 padding
   QUOKA_TRY_CUDA(launch_select_keys(P, w.scores, k_idx, k_cnt, cs, /*chained=*/p->max_ctx_len > 0));
-  return run_attn(p, P, q, k_cache, v_cache, k_idx, k_cnt, out, nullptr, cs, /*after_selection=*/true, &plan);
+  return run_attn(p, P, q, k_cache, v_cache, k_idx, k_cnt, out, nullptr, cs, plan, /*after_selection=*/true);
 }
 
-// with_split = false keeps to the workspace layout without the split-attention scratch (the built-in array of the
-// no-allocation entry point has no room for it).
+// The fused call on a workspace known to be large enough (the built-in array of the no-allocation entry point, which has no
+// room for the split attention's scratch, among them).
 quoka_status prefill_chunk_impl(const quoka_params* p, const void* q, const void* k_cache, const void* v_cache, void* out,
-                                int32_t* k_idx_out, int32_t* k_cnt_out, void* ws, size_t ws_bytes, void* stream,
-                                bool with_split) {
-  quoka_status st = check_prefill_args(p, q, k_cache, v_cache, out);
-  if (st != QUOKA_OK) return st;
-  if ((st = check_ws(p, ws, ws_bytes, with_split)) != QUOKA_OK) return st;
-  const Workspace w = carve(p, ws, with_split);
-  return run_prefill(p, make_dev(p, ws, w), w, attn_plan_sparse(p, budget_cap_of(p)), q, k_cache, v_cache, out,
+                                int32_t* k_idx_out, int32_t* k_cnt_out, void* ws, size_t ws_bytes, void* stream) {
+  const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p));
+  const Workspace w = carve(p, ws, ws_bytes, &plan);
+  return run_prefill(p, make_dev(p, ws, w), w, plan, q, k_cache, v_cache, out,
                      k_idx_out ? k_idx_out : w.k_idx, k_cnt_out ? k_cnt_out : w.k_cnt, static_cast<cudaStream_t>(stream));
 }
 
@@ -304,7 +302,7 @@ quoka_status quoka_workspace_size(const quoka_params* p, size_t* bytes) {
   if (!bytes) return QUOKA_ERR_INVALID_ARG;
   quoka_status st = validate(p);
   if (st != QUOKA_OK) return st;
-  *bytes = carve(p, nullptr).total;
+  *bytes = carve(p, nullptr).total + attn_scratch_bytes(p);
   return QUOKA_OK;
 }
 
@@ -356,8 +354,9 @@ quoka_status quoka_sparse_attn(const quoka_params* p, const void* q, const void*
   if (!q || !k_cache || !v_cache || !k_idx || !k_cnt || !out) return QUOKA_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k_cache) || !aligned16(v_cache) || !aligned16(out)) return QUOKA_ERR_INVALID_ARG;
   if ((st = check_ws(p, ws, ws_bytes)) != QUOKA_OK) return st;
-  return run_attn(p, make_dev(p, ws), q, k_cache, v_cache, k_idx, k_cnt, out, lse,
-                  static_cast<cudaStream_t>(stream));
+  const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p));
+  return run_attn(p, make_dev(p, ws, carve(p, ws, ws_bytes, &plan)), q, k_cache, v_cache, k_idx, k_cnt, out, lse,
+                  static_cast<cudaStream_t>(stream), plan);
 }
 
 quoka_status quoka_dense_chunk_attn(const quoka_params* p, const void* q, const void* k_cache, const void* v_cache,
@@ -367,14 +366,18 @@ quoka_status quoka_dense_chunk_attn(const quoka_params* p, const void* q, const 
   if (!q || !k_cache || !v_cache || !out) return QUOKA_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k_cache) || !aligned16(v_cache) || !aligned16(out)) return QUOKA_ERR_INVALID_ARG;
   if ((st = check_ws(p, ws, ws_bytes)) != QUOKA_OK) return st;
-  return run_attn(p, make_dev(p, ws), q, k_cache, v_cache, nullptr, nullptr, out, lse,
-                  static_cast<cudaStream_t>(stream));
+  const AttnPlan plan = attn_plan_dense(p);
+  return run_attn(p, make_dev(p, ws, carve(p, ws, ws_bytes, &plan)), q, k_cache, v_cache, nullptr, nullptr, out, lse,
+                  static_cast<cudaStream_t>(stream), plan);
 }
 
 quoka_status quoka_prefill_chunk(const quoka_params* p, const void* q, const void* k_cache, const void* v_cache,
                                  void* out, int32_t* k_idx_out, int32_t* k_cnt_out, void* ws, size_t ws_bytes,
                                  void* stream) {
-  return prefill_chunk_impl(p, q, k_cache, v_cache, out, k_idx_out, k_cnt_out, ws, ws_bytes, stream, /*with_split=*/true);
+  quoka_status st = check_prefill_args(p, q, k_cache, v_cache, out);
+  if (st != QUOKA_OK) return st;
+  if ((st = check_ws(p, ws, ws_bytes)) != QUOKA_OK) return st;
+  return prefill_chunk_impl(p, q, k_cache, v_cache, out, k_idx_out, k_cnt_out, ws, ws_bytes, stream);
 }
 
 quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_len_host, const void* q_host,
@@ -454,7 +457,7 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
     return QUOKA_OK;
   }
   if ((st = check_prefill_args(p, q_dev, k_cache, v_cache, out_dev)) != QUOKA_OK) return st;
-  const Workspace whole = carve(p, ws);
+  const Workspace whole = carve(p, ws, ws_bytes, &plan);
   QUOKA_TRY_CUDA(cudaEventRecord(hp->fork, cs));
   QUOKA_TRY_CUDA(cudaStreamWaitEvent(hp->h2d, hp->fork, 0));
   QUOKA_TRY_CUDA(copy_in_kv(hp->h2d));
@@ -466,7 +469,7 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
     sub.n_kv_heads = slice[i];
     sub.n_q_heads = slice[i] * G;
     // (a slice's intermediates end below the whole problem's split-attention scratch)
-    const Workspace w = carve(&sub, ws, /*with_split=*/false);
+    const Workspace w = carve(&sub, ws);
     DevParams P = make_dev(&sub, ws, w);
     P.attn_partials = whole.attn_partials; P.attn_counters = whole.attn_counters; P.n_attn_counters = whole.n_attn_counters;
     P.rank_heads = p->batch * p->n_q_heads;

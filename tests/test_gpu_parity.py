@@ -672,6 +672,35 @@ def test_attention_with_its_lightest_row_blocks_in_parts(n_q, n_kv, d, C, T, B):
         check_attention(f64(gp.out[0])[heads, rows], want, "bf16")
 
 
+@pytest.mark.parametrize("n_q,n_kv,d,C,tail,T", [
+    (32, 8, 128, 2048, 1500, 4096),       # no parts for the whole chunk, 12 MiB of them for the rest of the prompt
+    (40, 8, 64, 2048, 1270, 8192),        # parts in both, more of them for the shorter chunk
+])
+def test_a_workspace_made_for_the_longest_chunk_serves_the_shorter_ones(n_q, n_kv, d, C, tail, T):
+    """The scratch of grids of a wave or more may be missing: what was sized for another chunk of the same prompt is accepted,
+    the results are right, nothing behind the given bytes is touched; below the intermediates it is still refused."""
+    gp = problem(1300 + tail, n_q=n_q, n_kv=n_kv, d=d, T=T, C=tail, n_retain=64, kv_budget=T // 8)
+    full = GpuProblem(synth.make_chunk_inputs(0, 1, n_q, n_kv, d, 8, C, "bf16"), 64, kv_budget=T // 8)
+    full.p.max_ctx_len, full.p.kv_rows = T, T + C
+    n = api.quoka_workspace_size(full.p)
+    assert n < gp.ws.numel()
+    guarded = torch.full((n + (1 << 20),), 0x5A, dtype=torch.uint8, device="cuda")
+    guarded[:256] = 0
+    ws, q, k, v = guarded[:n], *gp.oracle_inputs(0)[:3]
+    heads, rows = stratified_rows(n_q, tail, 64, 5)
+    api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, gp.k_idx, gp.k_cnt, ws)
+    torch.cuda.synchronize()
+    idx = [gp.k_idx[0, h].cpu().numpy() for h in range(n_kv)]
+    check_attention(f64(gp.out[0])[heads, rows], O.sparse_attention_rows(q, k, v, T, idx, heads, rows), "bf16")
+    api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, None, ws)
+    torch.cuda.synchronize()
+    check_attention(f64(gp.out[0])[heads, rows], O.sparse_attention_rows(q, k, v, T, [np.arange(T)] * n_kv, heads, rows), "bf16")
+    assert (guarded[n:] == 0x5A).all() and api.quoka_last_device_status(ws) == 0
+    with pytest.raises(api.QuokaError) as e:
+        api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, ws[:n_kv * T * 4])
+    assert e.value.status == api.ERR_WORKSPACE
+
+
 @pytest.mark.parametrize("n_q,n_kv,C,T,B", [
     (8, 2, 256, [4096], 2048),          # 4 clusters of eight CTAs
     (8, 4, 257, [2500, 40], 2000),      # a row block of one row; a list shorter than a tile: parts without a tile
