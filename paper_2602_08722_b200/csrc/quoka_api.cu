@@ -119,6 +119,8 @@ quoka_status check_prefill_args(const quoka_params* p, const void* q, const void
   if (st != QUOKA_OK) return st;
   if (!q || !k_cache || !v_cache || !out) return QUOKA_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k_cache) || !aligned16(v_cache) || !aligned16(out)) return QUOKA_ERR_INVALID_ARG;
+  if (p->impl == QUOKA_IMPL_TENSOR && ((p->max_ctx_len > 0 && !score_keys_tc_supported(p)) || !attn_tc_supported(p)))
+    return QUOKA_ERR_UNSUPPORTED;
   return QUOKA_OK;
 }
 
@@ -398,6 +400,7 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
     return QUOKA_ERR_INVALID_ARG;
   for (int s = 0; s < p->batch; ++s)
     if (ctx_len_host[s] < 0 || ctx_len_host[s] > p->max_ctx_len) return QUOKA_ERR_INVALID_ARG;
+  if ((st = check_prefill_args(p, q_dev, k_cache, v_cache, out_dev)) != QUOKA_OK) return st;
   if ((st = check_ws(p, ws, ws_bytes)) != QUOKA_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   // Copies of the KV heads [kv0, kv0 + n_kv) and their query heads; every (sequence, head) block is contiguous on
@@ -451,41 +454,51 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
   if (!hp) {
     QUOKA_TRY_CUDA(copy_in_q(0, p->n_kv_heads, cs));
     QUOKA_TRY_CUDA(copy_in_kv(cs));
-    st = quoka_prefill_chunk(p, q_dev, k_cache, v_cache, out_dev, nullptr, nullptr, ws, ws_bytes, stream);
+    st = prefill_chunk_impl(p, q_dev, k_cache, v_cache, out_dev, nullptr, nullptr, ws, ws_bytes, stream);
     if (st != QUOKA_OK) return st;
     QUOKA_TRY_CUDA(copy_out(0, p->n_kv_heads, cs));
     return QUOKA_OK;
   }
-  if ((st = check_prefill_args(p, q_dev, k_cache, v_cache, out_dev)) != QUOKA_OK) return st;
   const Workspace whole = carve(p, ws, ws_bytes, &plan);
+  // Whatever happens between, the caller's stream ends up behind everything that was put on the side streams: the call must
+  // not leave copies in flight behind an error, nor forked streams in a capture.
+  bool out_forked = false;
+  const auto run_slices = [&]() -> quoka_status {
+    QUOKA_TRY_CUDA(copy_in_kv(hp->h2d));
+    for (int i = 0, kv0 = 0; i < n_slices; kv0 += slice[i++]) {
+      QUOKA_TRY_CUDA(copy_in_q(kv0, slice[i], hp->h2d));
+      QUOKA_TRY_CUDA(cudaEventRecord(hp->in[i], hp->h2d));
+      QUOKA_TRY_CUDA(cudaStreamWaitEvent(cs, hp->in[i], 0));
+      quoka_params sub = *p;
+      sub.n_kv_heads = slice[i];
+      sub.n_q_heads = slice[i] * G;
+      // (a slice's intermediates end below the whole problem's split-attention scratch)
+      const Workspace w = carve(&sub, ws);
+      DevParams P = make_dev(&sub, ws, w);
+      P.attn_partials = whole.attn_partials; P.attn_counters = whole.attn_counters; P.n_attn_counters = whole.n_attn_counters;
+      P.rank_heads = p->batch * p->n_q_heads;
+      P.attn_one_part = 1;
+      const quoka_status s = run_prefill(&sub, P, w, plan, static_cast<char*>(q_dev) + (size_t)kv0 * G * head_bytes,
+                                         static_cast<char*>(k_cache) + (size_t)kv0 * p->kv_stride_h * es,
+                                         static_cast<char*>(v_cache) + (size_t)kv0 * p->kv_stride_h * es,
+                                         static_cast<char*>(out_dev) + (size_t)kv0 * G * head_bytes, w.k_idx, w.k_cnt, cs);
+      if (s != QUOKA_OK) return s;
+      QUOKA_TRY_CUDA(cudaEventRecord(hp->done[i], cs));
+      QUOKA_TRY_CUDA(cudaStreamWaitEvent(hp->d2h, hp->done[i], 0));
+      out_forked = true;
+      QUOKA_TRY_CUDA(copy_out(kv0, slice[i], hp->d2h));
+    }
+    return QUOKA_OK;
+  };
   QUOKA_TRY_CUDA(cudaEventRecord(hp->fork, cs));
   QUOKA_TRY_CUDA(cudaStreamWaitEvent(hp->h2d, hp->fork, 0));
-  QUOKA_TRY_CUDA(copy_in_kv(hp->h2d));
-  for (int i = 0, kv0 = 0; i < n_slices; kv0 += slice[i++]) {
-    QUOKA_TRY_CUDA(copy_in_q(kv0, slice[i], hp->h2d));
-    QUOKA_TRY_CUDA(cudaEventRecord(hp->in[i], hp->h2d));
-    QUOKA_TRY_CUDA(cudaStreamWaitEvent(cs, hp->in[i], 0));
-    quoka_params sub = *p;
-    sub.n_kv_heads = slice[i];
-    sub.n_q_heads = slice[i] * G;
-    // (a slice's intermediates end below the whole problem's split-attention scratch)
-    const Workspace w = carve(&sub, ws);
-    DevParams P = make_dev(&sub, ws, w);
-    P.attn_partials = whole.attn_partials; P.attn_counters = whole.attn_counters; P.n_attn_counters = whole.n_attn_counters;
-    P.rank_heads = p->batch * p->n_q_heads;
-    P.attn_one_part = 1;
-    st = run_prefill(&sub, P, w, plan, static_cast<char*>(q_dev) + (size_t)kv0 * G * head_bytes,
-                     static_cast<char*>(k_cache) + (size_t)kv0 * p->kv_stride_h * es,
-                     static_cast<char*>(v_cache) + (size_t)kv0 * p->kv_stride_h * es,
-                     static_cast<char*>(out_dev) + (size_t)kv0 * G * head_bytes, w.k_idx, w.k_cnt, cs);
-    if (st != QUOKA_OK) return st;
-    QUOKA_TRY_CUDA(cudaEventRecord(hp->done[i], cs));
-    QUOKA_TRY_CUDA(cudaStreamWaitEvent(hp->d2h, hp->done[i], 0));
-    QUOKA_TRY_CUDA(copy_out(kv0, slice[i], hp->d2h));
-  }
-  QUOKA_TRY_CUDA(cudaEventRecord(hp->join, hp->d2h));
-  QUOKA_TRY_CUDA(cudaStreamWaitEvent(cs, hp->join, 0));
-  return QUOKA_OK;
+  st = run_slices();
+  bool joined = true;
+  if (st != QUOKA_OK)                          // (else the last slice's wait is behind all that came in)
+    joined = cudaEventRecord(hp->in[0], hp->h2d) == cudaSuccess && cudaStreamWaitEvent(cs, hp->in[0], 0) == cudaSuccess;
+  if (out_forked)
+    joined = cudaEventRecord(hp->join, hp->d2h) == cudaSuccess && cudaStreamWaitEvent(cs, hp->join, 0) == cudaSuccess && joined;
+  return st == QUOKA_OK && !joined ? QUOKA_ERR_CUDA : st;
 }
 
 quoka_status quoka_append_kv(const quoka_params* p, const void* k_new, const void* v_new, void* k_cache,

@@ -296,6 +296,34 @@ def test_host_buffer_slices_give_the_whole_calls_bits(dtype, n_q, n_kv, C):
     assert torch.equal(out_host, want) and torch.equal(gp.k, want_k)
 
 
+def test_a_host_buffer_call_that_is_refused_puts_nothing_on_any_stream():
+    """The tensor-core kernels asked for, and more retained queries than they take: refused before the first copy, so that
+    neither copies of it are in flight nor side streams forked in a capture."""
+    T, C = 2000, 2048
+    gp = problem(15, n_q=32, n_kv=8, T=T, C=C, n_retain=600, kv_budget=500, impl=api.IMPL_TENSOR)
+    host = [x.contiguous().pin_memory() for x in (gp.inp.q, gp.inp.k[:, :, T:T + C], gp.inp.v[:, :, T:T + C])]
+    out_host, q_dev, before = torch.zeros_like(host[0]).pin_memory(), torch.zeros_like(gp.q), api.quoka_launch_count()
+
+    def call():
+        with pytest.raises(api.QuokaError) as e:
+            api.quoka_prefill_chunk_host(gp.p, gp.inp.ctx_len.clone(), *host, out_host, q_dev, gp.k, gp.v, gp.out, gp.ws)
+        assert e.value.status == api.ERR_UNSUPPORTED
+
+    call()
+    torch.cuda.synchronize()
+    assert not q_dev.any() and api.quoka_launch_count() == before
+    with pytest.raises(api.QuokaError):
+        api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+    assert api.quoka_launch_count() == before
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        q_dev.add_(0)
+        call()
+    g.replay()
+    torch.cuda.synchronize()
+    assert not q_dev.any()
+
+
 def test_host_buffer_entry_point_replayed_from_a_cuda_graph():
     # the sliced call forks to the library's two copy streams and joins again: captured as one graph and replayed
     shape = dict(n_q=32, n_kv=8, T=3000, C=2048, n_retain=64, kv_budget=700)
