@@ -435,8 +435,11 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
   };
   // A large chunk is cut into slices of whole KV groups (the selection and the attention of a KV group need nothing
   // of another group): the next slice's queries come in and the last one's output goes out while a slice is computed.
-  // Every slice's attention follows the whole problem's plan, so that it gives the same bits as the whole.  Not for grids
-  // below a wave, without a cache of key norms (indexed by the whole problem's head count), and when the side streams exist.
+  // Every slice's attention follows the whole problem's plan, so that it gives the same bits as the whole.  Only without a
+  // cache of key norms (indexed by the whole problem's head count), and when the side streams exist.  A bf16 grid below a wave
+  // is cut into two halves, unless its row blocks are cut into parts (8 query heads, 4096 queries at 16K / 4K, 2 / 4 KV heads:
+  // 523 / 571 us whole, 481 / 484 in halves, 483 / 528 in slices as below; f32, whose kernels are the longer part, 954 whole, 1572
+  // in slices).
   // What bounds it: the host link, and on it the number of copies: one that starts while the other direction is busy costs
   // about 17 us.  So all keys and values first, then the queries in three pieces, the first the smallest.  32 query / 8 KV
   // heads, 2048 queries at 32K (25.2 MB in: 500 us alone, 16.8 MB out): slices of 2, 3 and 3 KV groups 745 us, of 2 / 2 / 2 / 2
@@ -444,10 +447,12 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
   int n_slices = 1, slice[kHostSlices] = {p->n_kv_heads, 0, 0};
   const size_t q_bytes = (size_t)p->batch * p->n_q_heads * head_bytes;
   const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p));
-  if (!p->k_inv_norm && !attn_below_a_wave(p) && q_bytes >= ((size_t)8 << 20) && p->n_kv_heads > 1) {
-    slice[0] = p->n_kv_heads / 4 > 0 ? p->n_kv_heads / 4 : 1;
-    slice[1] = p->n_kv_heads == 2 ? 1 : (p->n_kv_heads - slice[0]) / 2;
-    slice[2] = p->n_kv_heads - slice[0] - slice[1];
+  const bool below = attn_below_a_wave(p), whole_below = plan.split_rb > 0 || p->dtype != QUOKA_BF16;
+  const int n_kv = p->n_kv_heads;
+  if (!p->k_inv_norm && !(below && whole_below) && q_bytes >= ((size_t)8 << 20) && n_kv > 1) {
+    slice[0] = below ? n_kv / 2 : (n_kv / 4 > 0 ? n_kv / 4 : 1);
+    slice[1] = below || n_kv == 2 ? n_kv - slice[0] : (n_kv - slice[0]) / 2;
+    slice[2] = n_kv - slice[0] - slice[1];
     n_slices = slice[2] > 0 ? 3 : 2;
   }
   HostPipe* hp = n_slices > 1 ? host_pipe_for_current_device() : nullptr;

@@ -296,6 +296,25 @@ def test_host_buffer_slices_give_the_whole_calls_bits(dtype, n_q, n_kv, C):
     assert torch.equal(out_host, want) and torch.equal(gp.k, want_k)
 
 
+@pytest.mark.parametrize("n_q,n_kv,sliced", [(8, 2, True), (8, 4, True), (8, 8, True), (9, 3, True), (7, 1, False)])
+def test_host_buffer_slices_of_a_grid_just_below_a_wave(n_q, n_kv, sliced):
+    """128 to 144 row blocks that are not cut into parts: still copied in and out slice by slice (more launches than the
+    device call's), with its bits."""
+    C, T = 4096 if n_q < 9 else 4000, 3000
+    gp = problem(16, n_q=n_q, n_kv=n_kv, T=T, C=C if n_q > 7 else 4700, n_retain=32, kv_budget=700)
+    C = gp.C
+    n0 = api.quoka_launch_count()
+    api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+    torch.cuda.synchronize()
+    n1 = api.quoka_launch_count()
+    want = gp.out.cpu()
+    host = [x.contiguous().pin_memory() for x in (gp.inp.q, gp.inp.k[:, :, T:T + C], gp.inp.v[:, :, T:T + C])]
+    out_host = torch.zeros_like(host[0]).pin_memory()
+    api.quoka_prefill_chunk_host(gp.p, gp.inp.ctx_len.clone(), *host, out_host, torch.zeros_like(gp.q), gp.k, gp.v, gp.out, gp.ws)
+    torch.cuda.synchronize()
+    assert torch.equal(out_host, want) and (api.quoka_launch_count() - n1 >= 2 * (n1 - n0)) == sliced
+
+
 def test_a_host_buffer_call_that_is_refused_puts_nothing_on_any_stream():
     """The tensor-core kernels asked for, and more retained queries than they take: refused before the first copy, so that
     neither copies of it are in flight nor side streams forked in a capture."""
