@@ -14,6 +14,9 @@ import torch
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libquoka.so")
 _lib = None
+# torch's own names for these may go away
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_STATIC_LIMIT, ERR_BAD_INDEX = range(8)
 STATIC_SCRATCH_BYTES = 8 << 20
@@ -116,7 +119,9 @@ def _stream(stream):
     if stream is None:
         # torch.cuda.current_stream() builds a Stream object: 3.2 us per call, a third of the host time of a generation
         # step; the raw handle takes 0.1 us
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        if _raw_stream is None or _current_device is None:
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(_current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -3,8 +3,10 @@ arguments on the host before anything is launched.  No GPU needed (no compute ca
 import ctypes as C
 import os
 import re
+import types
 
 import pytest
+import torch
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -110,6 +112,18 @@ def test_missing_library_is_an_error(monkeypatch, tmp_path):
     monkeypatch.setattr(api, "_LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="no fallback"):
         api.load()
+
+
+def test_current_stream_with_and_without_torchs_private_names(monkeypatch):
+    from paper_2602_08722_b200 import api
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    monkeypatch.setattr(api, "_current_device", lambda: 3)
+    monkeypatch.setattr(api, "_raw_stream", {3: 55}.__getitem__)
+    assert api._stream(None) == 55 and api._stream(9) == 9
+    for name in ("_raw_stream", "_current_device"):
+        with monkeypatch.context() as m:
+            m.setattr(api, name, None)
+            assert api._stream(None) == 77
 
 
 def test_block_table_check_on_the_host(lib):
