@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kRegThreads, 1) decode_listed_attn_kernel(DevP
   decode_load_q<T, D, GH>(P, q, s, h0, n_heads, (tid & 31) % (D / VecOf<T>::N), qv);
   if (tid == 0) { s_lo = 0; s_hi = 0; }
   __syncthreads();
-  int lo = (int)((long long)rank * T_s / kFuseCl), hi = (int)((long long)(rank + 1) * T_s / kFuseCl);
+  int lo = (int)((long long)rank * cnt / kFuseCl), hi = (int)((long long)(rank + 1) * cnt / kFuseCl);    // (cnt >= T_s: all)
   if (cnt < T_s) {                                   // entries below the first position of this CTA, and of the next
     const int piece = P.max_ctx <= kFuseShort ? select_piece<kFuseCl, 1>(T_s) : select_piece<kFuseCl, 8>(T_s);
     int a = 0, b = 0;

@@ -625,6 +625,21 @@ def test_f32_generation_step_keeps_the_thousands_of_small_weights(group, d, list
     assert (lse[:, :, 0].double() - torch.log(w.sum(-1)).repeat_interleave(group, 1)).abs().max() <= 1e-5
 
 
+@pytest.mark.parametrize("T,max_ctx", [(100, 4096), (100, 1000), (4000, 4096)])
+def test_generation_step_over_a_callers_own_list(T, max_ctx):
+    """A list in any order, with repeated rows, longer than the cache even: every entry counts."""
+    inp = synth.make_chunk_inputs(78, 1, 8, 2, 128, T, 1, "bf16", capacity=max_ctx + 1)
+    gp = GpuProblem(inp, 4, kv_budget=300, max_ctx_len=max_ctx)
+    gp.k_idx.copy_(torch.randint(0, T, gp.k_idx.shape, generator=torch.Generator().manual_seed(T)))
+    gp.k_cnt.fill_(300)
+    api.quoka_sparse_attn(gp.p, gp.q, gp.k, gp.v, gp.k_idx, gp.k_cnt, gp.out, gp.lse, gp.ws)
+    torch.cuda.synchronize()
+    q, k, v, _ = gp.oracle_inputs(0)
+    want, lse = O.sparse_attention(q, k, v, T, [gp.k_idx[0, h].cpu().numpy() for h in range(2)])
+    check_attention(f64(gp.out[0]), want, "bf16")
+    assert np.abs(f64(gp.lse[0]) - lse).max() <= 2e-3
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_generation_step_over_an_infinite_value(dtype):
     """An infinite value among hundreds makes its output infinite, not NaN, and no other."""
