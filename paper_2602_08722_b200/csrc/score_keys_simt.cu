@@ -103,9 +103,11 @@ __global__ void __launch_bounds__(kF32Threads) score_keys_f32_kernel(DevParams P
 #pragma unroll
   for (int i = 0; i < 4; ++i) { best[i] = -INFINITY; total[i] = 0.f; nn[i] = 0.f; }
   for (int j0 = 0; j0 < N; j0 += kQ) {
-    for (int e = tid; e < kQ * W; e += kF32Threads) {
+    // (only the rows there are: a last one repeated in their place had every CTA of the grid at the same lines of L2; the
+    // products with what lies in the other rows are not used)
+    for (int e = tid; e < min(kQ, N - j0) * W; e += kF32Threads) {
       const int r = e / W, c = e % W;
-      ptx::cp_async_16(ptx::smem_u32(qs + r * LD + 4 * c), qb + (long long)min(j0 + r, N - 1) * D + 4 * c, true);
+      ptx::cp_async_16(ptx::smem_u32(qs + r * LD + 4 * c), qb + (long long)(j0 + r) * D + 4 * c, true);
     }
     ptx::cp_async_wait_all();
     __syncthreads();

@@ -843,6 +843,22 @@ def test_f32_tiles_at_their_edges(T, C, B, n_q, n_kv, d, n_retain, paged):
     assert np.abs(f64(gp.lse[0]) - lse).max() <= 2e-3
 
 
+def test_f32_scoring_of_few_queries_is_not_slower_than_of_a_full_block():
+    """2 retained queries against 32 (20 us each at this size; 58 us for 2 while a block repeated its last row)."""
+    best = {}
+    for n in (2, 32):
+        gp = problem(31, n_q=2, n_kv=2, d=64, T=32768, C=n, dtype="f32", n_retain=64, kv_budget=64)
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                api.quoka_score_keys(gp.p, gp.qbar, gp.k, gp.scores, gp.ws)
+            b.record()
+            torch.cuda.synchronize()
+            best[n] = min(best.get(n, 1e9), a.elapsed_time(b))
+    assert best[2] < 1.5 * best[32]
+
+
 @pytest.mark.parametrize("bad", [float("inf"), float("nan")])
 @pytest.mark.parametrize("T,C,B,n_q,n_kv,d", [(2000, 200, 300, 4, 2, 128), (100, 64, 30, 2, 1, 64), (700, 650, 100, 32, 8, 64)])
 def test_f32_values_of_later_rows_do_not_reach_earlier_ones(T, C, B, n_q, n_kv, d, bad):
