@@ -94,6 +94,13 @@ attn_f32_kernel(DevParams P, const float* __restrict__ q, const float* __restric
   for (int t = t_lo; t < t_hi; ++t) {
     const int next = rows_of(t + 1);
     cp_async_wait<1>();                          // Q and K have landed, V may still be in flight
+    if (t == t_lo) {                             // the softmax scale goes into the queries (every thread its own words): a
+#pragma unroll                                   // product may overflow where the logit would not
+      for (int i = 0; i < RPW / RPI; ++i) {
+        float4* w = reinterpret_cast<float4*>(qs + (warp * RPW + i * RPI + rsub) * LD + 4 * c);
+        *w = make_float4(w->x * P.scale, w->y * P.scale, w->z * P.scale, w->w * P.scale);
+      }
+    }
     __syncthreads();
     float sc[4][4];
     f32_dot_tile<D, 4>(qs, ks, ty, tx, sc);
@@ -107,7 +114,7 @@ attn_f32_kernel(DevParams P, const float* __restrict__ q, const float* __restric
       float mx = -INFINITY;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        sc[i][j] = tx + 16 * j < lim && r < C ? sc[i][j] * P.scale : -INFINITY;
+        sc[i][j] = tx + 16 * j < lim && r < C ? sc[i][j] : -INFINITY;
         mx = fmaxf(mx, sc[i][j]);
       }
       const float m_new = fmaxf(m[i], half_warp_max(mx));

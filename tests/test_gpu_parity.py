@@ -859,6 +859,20 @@ def test_f32_scoring_of_few_queries_is_not_slower_than_of_a_full_block():
     assert best[2] < 1.5 * best[32]
 
 
+@pytest.mark.parametrize("d,C", [(128, 70), (64, 70), (128, 1)])
+def test_f32_products_beyond_the_range_of_logits_within_it(d, C):
+    """q . k overflows, q . k / sqrt(d) does not: the row is one-hot, not NaN."""
+    gp = problem(83, n_q=4, n_kv=2, d=d, T=300, C=C, dtype="f32", n_retain=8, kv_budget=60)
+    gp.q[0, 1, C // 2] = 0
+    gp.q[0, 1, C // 2, 5] = 2e38
+    gp.inp.q = gp.q.cpu()
+    api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, gp.lse, gp.ws)
+    torch.cuda.synchronize()
+    q, k, v, T = gp.oracle_inputs(0)
+    check_attention(f64(gp.out[0]), O.dense_chunk_attention(q, k, v, T)[0], "f32")
+    assert torch.isfinite(gp.lse).all()
+
+
 @pytest.mark.parametrize("bad", [float("inf"), float("nan")])
 @pytest.mark.parametrize("T,C,B,n_q,n_kv,d", [(2000, 200, 300, 4, 2, 128), (100, 64, 30, 2, 1, 64), (700, 650, 100, 32, 8, 64)])
 def test_f32_values_of_later_rows_do_not_reach_earlier_ones(T, C, B, n_q, n_kv, d, bad):
