@@ -73,7 +73,8 @@ cudaError_t launch_append_kv(const DevParams& P, int dtype, const void* k_new, c
   const int64_t total = (int64_t)P.batch * P.n_kv * P.chunk * (P.d * es / 16);
   if (total <= 0) return cudaSuccess;
   int64_t blocks = (total + 255) / 256;
-  if (blocks > 148 * 16) blocks = 148 * 16;
+  const int64_t most = 16ll * device_sm_count();                     // two waves of eight CTAs per SM; longer appends loop
+  if (blocks > most && most > 0) blocks = most;
   const dim3 grid((unsigned)blocks), block(256);
   cudaError_t e;
 #define QUOKA_APPEND(E_, D_)                                                                                        \

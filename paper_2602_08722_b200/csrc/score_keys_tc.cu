@@ -10,8 +10,8 @@
 // which a sum of squares does not care about) and applied in fp32: score = max_j(Qbar_j . k)/|k|.
 //
 // Persistent CTAs (one per SM), each taking a contiguous, equal share of the valid (sequence, KV
-// head, key tile) list.  Warp 0 = TMA producer, warp 1 = MMA issuer, warps 2..5 = epilogue.  K tiles
-// stream through a multi-stage ring (32 KiB per stage at d = 128); accumulators are double-buffered
+// head, key tile) list.  Warp 0 = TMA producer, warp 1 = MMA issuer, warps 2..9 = two epilogue groups of four on
+// alternate tiles.  K tiles stream through a multi-stage ring (32 KiB per stage at d = 128); accumulators are double-buffered
 // in TMEM when N <= 256 so the epilogue of tile i overlaps the MMAs of tile i+1.
 // Arithmetic intensity is N flop per byte of K: HBM-bound below N ~ 200, tensor-bound above.
 #include <cstdio>
