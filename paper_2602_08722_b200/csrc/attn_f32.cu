@@ -6,10 +6,13 @@
 // 4 x 4 per thread, the output 4 x D/16 per thread, so that a 16-byte shared-memory read feeds 8 to 11 FMAs.  A problem
 // with fewer row blocks than SMs has every row block's keys cut into up to 8 parts, one CTA of a cluster each; the parts
 // are added up through distributed shared memory, in part order.
-//   8 heads x 256 queries over 512 listed rows + the chunk: 353 -> 36 us (one warp per query row, key by key, before).
+//   8 heads x 256 queries over 512 listed rows + the chunk: 353 -> 37 us (one warp per query row, key by key, before).
 // K of the next tile is in flight under this tile's softmax and PV, V of the next one under the next scores: one buffer
 // of each.  Half a tile's PV sum is formed in fresh accumulators and added to the running output with compensation:
 // thousands of weights below half an ulp of a sum that one key dominates must not vanish one by one.
+// Error against 64 bits (relative, 2-norm, 60 problems of 300 to 16000 keys): 2.9e-7; 3.4e-7 with dot products in chains over 32
+// elements and the last sums in 32 bits (for 3 % less time), 2.6e-7 in the scalar kernel, whose every sum is compensated.
+// Quarters of a tile instead of halves 2.8e-7 and 8 % more time.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -23,6 +26,13 @@ namespace quoka {
 using namespace ptx;
 
 constexpr int kPPitch = kF32Tile + 4;
+
+__device__ __forceinline__ uint64_t neg2(uint64_t a) { return a ^ 0x8000000080000000ull; }      // of a pair of floats
+// 1 / x beyond fp32: what all elements of a row are multiplied with should not round them all alike.
+__device__ __forceinline__ double inverse(double x) {
+  const double r = (double)(1.f / (float)x);
+  return isfinite(r) ? r * (2. - x * r) : r;
+}
 
 template <int D>
 constexpr size_t attn_f32_smem() {
@@ -81,12 +91,13 @@ attn_f32_kernel(DevParams P, const float* __restrict__ q, const float* __restric
     }
     cp_async_commit();
   };
-  float m[4], l[4], cl[4], o[4][4 * NC], co[4][4 * NC];             // co, cl: what the sums have lost so far
+  float m[4], l[4], cl[4];                       // cl, co: what the sums have gained too much so far
+  uint64_t o[4][2 * NC], co[4][2 * NC];          // in pairs
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     m[i] = -INFINITY; l[i] = 0.f; cl[i] = 0.f;
 #pragma unroll
-    for (int j = 0; j < 4 * NC; ++j) { o[i][j] = 0.f; co[i][j] = 0.f; }
+    for (int j = 0; j < 2 * NC; ++j) { o[i][j] = 0ull; co[i][j] = 0ull; }
   }
   int rows = rows_of(t_lo);
   fetch(k, ks, LD, rows);
@@ -103,7 +114,7 @@ attn_f32_kernel(DevParams P, const float* __restrict__ q, const float* __restric
     }
     __syncthreads();
     float sc[4][4];
-    f32_dot_tile<D, 4>(qs, ks, ty, tx, sc);
+    f32_dot_tile<D, 4, 8>(qs, ks, ty, tx, sc);
     __syncthreads();                             // K may be overwritten
     fetch(k, ks, LD, next);
     // ---- softmax of the tile; row 4 ty + i is shared by the 16 lanes of a half warp
@@ -184,40 +195,46 @@ attn_f32_kernel(DevParams P, const float* __restrict__ q, const float* __restric
         if (!(x[0] + x[1] == 0.f)) sum_half(std::true_type{});
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 4; ++i) {
+        const float f = u0 == 0 ? alpha[i] : 1.f;
+        const uint64_t f2 = pack2(f, f);
 #pragma unroll
         for (int j = 0; j < 2 * NC; ++j) {
-          float x[2];
-          unpack2(pv[i][j], x[0], x[1]);
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            float& oo = o[i][2 * j + e];
-            float& cc = co[i][2 * j + e];
-            if (u0 == 0) { oo *= alpha[i]; cc *= alpha[i]; }
-            const float y = x[e] - cc, z = oo + y;
-            cc = (z - oo) - y;
-            oo = z;
-          }
+          const uint64_t oo = fma2(o[i][j], f2, 0ull), y = fma2(neg2(co[i][j]), f2, pv[i][j]), z = add2(oo, y);
+          co[i][j] = add2(add2(z, neg2(oo)), neg2(y));
+          o[i][j] = z;
         }
+      }
     }
     __syncthreads();                             // V may be overwritten
     fetch(v, vs, D, next);
   }
   cp_async_wait_all();
+  // What is left is in 64 bits: a handful of sums and one product per element, whose roundings would add up to those above.
+  double ld[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) l[i] = half_warp_sum(l[i]);
+  for (int i = 0; i < 4; ++i) {
+    ld[i] = (double)l[i] - (double)cl[i];
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) ld[i] += __shfl_xor_sync(0xFFFFFFFFu, ld[i], off);
+  }
   float* oh = out + (long long)s * P.o_sb + (long long)h * P.o_sh;
   if (parts == 1) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int r = r0 + 4 * ty + i;
       if (r >= C) continue;
-      const float inv = 1.f / l[i];
+      const double inv = inverse(ld[i]);
 #pragma unroll
-      for (int g = 0; g < NC; ++g)
-        *reinterpret_cast<float4*>(oh + (long long)r * P.o_st + 64 * g + 4 * tx) =
-            make_float4(o[i][4 * g] * inv, o[i][4 * g + 1] * inv, o[i][4 * g + 2] * inv, o[i][4 * g + 3] * inv);
-      if (lse && tx == 0) lse[((long long)s * P.n_q + h) * C + r] = m[i] + logf(l[i]);
+      for (int g = 0; g < NC; ++g) {
+        float x[4], c4[4];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) { unpack2(o[i][2 * g + j], x[2 * j], x[2 * j + 1]); unpack2(co[i][2 * g + j], c4[2 * j], c4[2 * j + 1]); }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j] = (float)(((double)x[j] - (double)c4[j]) * inv);
+        *reinterpret_cast<float4*>(oh + (long long)r * P.o_st + 64 * g + 4 * tx) = make_float4(x[0], x[1], x[2], x[3]);
+      }
+      if (lse && tx == 0) lse[((long long)s * P.n_q + h) * C + r] = m[i] + logf((float)ld[i]);
     }
     return;
   }
@@ -228,15 +245,15 @@ attn_f32_kernel(DevParams P, const float* __restrict__ q, const float* __restric
   for (int i = 0; i < 4; ++i) {
 #pragma unroll
     for (int g = 0; g < NC; ++g)
-      *reinterpret_cast<float4*>(vs + (4 * ty + i) * D + 64 * g + 4 * tx) = make_float4(o[i][4 * g], o[i][4 * g + 1], o[i][4 * g + 2], o[i][4 * g + 3]);
-    if (tx == 0) { part_m[4 * ty + i] = m[i]; part_l[4 * ty + i] = l[i]; }
+      *reinterpret_cast<ulonglong2*>(vs + (4 * ty + i) * D + 64 * g + 4 * tx) = make_ulonglong2(o[i][2 * g], o[i][2 * g + 1]);
+    if (tx == 0) { part_m[4 * ty + i] = m[i]; part_l[4 * ty + i] = (float)ld[i]; }
   }
   cluster.sync();
   for (int e = tid; e < (kF32Tile / parts + 1) * W; e += kF32Threads) {
     const int lr = (e / W) * parts + part, w = e % W;
     if (lr >= kF32Tile || r0 + lr >= C) continue;
-    float pm[8], M = -INFINITY, L = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float pm[8], M = -INFINITY;
+    double L = 0., acc[4] = {0., 0., 0., 0.};
 #pragma unroll
     for (int p = 0; p < 8; ++p) {
       pm[p] = p < parts ? *cluster.map_shared_rank(part_m + lr, p) : -INFINITY;
@@ -245,14 +262,15 @@ attn_f32_kernel(DevParams P, const float* __restrict__ q, const float* __restric
 #pragma unroll
     for (int p = 0; p < 8; ++p)
       if (p < parts && pm[p] != -INFINITY) {
-        const float wgt = expf(pm[p] - M);
-        L += wgt * *cluster.map_shared_rank(part_l + lr, p);
+        const double wgt = (double)expf(pm[p] - M);
+        L += wgt * (double)*cluster.map_shared_rank(part_l + lr, p);
         const float4 x = *cluster.map_shared_rank(reinterpret_cast<const float4*>(vs + lr * D + 4 * w), p);
-        acc.x = fmaf(wgt, x.x, acc.x); acc.y = fmaf(wgt, x.y, acc.y); acc.z = fmaf(wgt, x.z, acc.z); acc.w = fmaf(wgt, x.w, acc.w);
+        acc[0] += wgt * (double)x.x; acc[1] += wgt * (double)x.y; acc[2] += wgt * (double)x.z; acc[3] += wgt * (double)x.w;
       }
-    const float inv = 1.f / L;
-    *reinterpret_cast<float4*>(oh + (long long)(r0 + lr) * P.o_st + 4 * w) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
-    if (lse && w == 0) lse[((long long)s * P.n_q + h) * C + r0 + lr] = M + logf(L);
+    const double inv = inverse(L);
+    *reinterpret_cast<float4*>(oh + (long long)(r0 + lr) * P.o_st + 4 * w) =
+        make_float4((float)(acc[0] * inv), (float)(acc[1] * inv), (float)(acc[2] * inv), (float)(acc[3] * inv));
+    if (lse && w == 0) lse[((long long)s * P.n_q + h) * C + r0 + lr] = M + logf((float)L);
   }
   cluster.sync();                                // my part stays mapped until every peer has read it
 }

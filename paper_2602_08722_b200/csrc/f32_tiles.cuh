@@ -14,9 +14,9 @@ constexpr int kF32Tile = 64;
 template <int D> __host__ __device__ constexpr int f32_pitch() { return D + 4; }      // floats
 
 // acc[i][j] = A[4 ty + i] . B[tx + 16 j] over D elements; fp32 FMAs, even and odd elements in the halves of a pair
-// (16 J FMAs for 4 + J shared-memory reads of 16 bytes).  Summed in blocks of 32 elements: chains of 64 FMAs doubled the
-// rounding error of the attention output.
-template <int D, int J>
+// (16 J FMAs for 4 + J shared-memory reads of 16 bytes).  Summed in chains over BLOCK elements, those in blocks of 32: chains
+// of 64 FMAs doubled the rounding error of the attention output, chains over 32 elements leave a tenth more than over 8.
+template <int D, int J, int BLOCK>
 __device__ __forceinline__ void f32_dot_tile(const float* __restrict__ A, const float* __restrict__ B, int ty, int tx,
                                              float (&acc)[4][J]) {
   constexpr int LD = f32_pitch<D>();
@@ -29,27 +29,32 @@ __device__ __forceinline__ void f32_dot_tile(const float* __restrict__ A, const 
   const float* bp = B + tx * LD;
 #pragma unroll 1
   for (int c0 = 0; c0 < D; c0 += 32) {
-    uint64_t t2[4][J];
+    uint64_t u2[4][J];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int c1 = 0; c1 < 32; c1 += BLOCK) {
+      uint64_t t2[4][J];
 #pragma unroll
-      for (int j = 0; j < J; ++j) t2[i][j] = 0ull;
+      for (int c = c0 + c1; c < c0 + c1 + BLOCK; c += 4) {
+        ulonglong2 a[4], b[J];
 #pragma unroll
-    for (int c = c0; c < c0 + 32; c += 4) {
-      ulonglong2 a[4], b[J];
+        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(ap + i * LD + c);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(ap + i * LD + c);
+        for (int j = 0; j < J; ++j) b[j] = *reinterpret_cast<const ulonglong2*>(bp + 16 * j * LD + c);
 #pragma unroll
-      for (int j = 0; j < J; ++j) b[j] = *reinterpret_cast<const ulonglong2*>(bp + 16 * j * LD + c);
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < J; ++j)
+            t2[i][j] = ptx::fma2(a[i].y, b[j].y, ptx::fma2(a[i].x, b[j].x, c == c0 + c1 ? 0ull : t2[i][j]));
+      }
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < J; ++j) t2[i][j] = ptx::fma2(a[i].y, b[j].y, ptx::fma2(a[i].x, b[j].x, t2[i][j]));
+        for (int j = 0; j < J; ++j) u2[i][j] = c1 == 0 ? t2[i][j] : ptx::add2(u2[i][j], t2[i][j]);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < J; ++j) a2[i][j] = ptx::add2(a2[i][j], t2[i][j]);
+      for (int j = 0; j < J; ++j) a2[i][j] = ptx::add2(a2[i][j], u2[i][j]);
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i)

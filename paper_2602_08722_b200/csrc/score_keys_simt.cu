@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kF32Threads) score_keys_f32_kernel(DevParams P
     ptx::cp_async_wait_all();
     __syncthreads();
     float acc[4][J];
-    f32_dot_tile<D, J>(ks, qs, ty, tx, acc);
+    f32_dot_tile<D, J, 32>(ks, qs, ty, tx, acc);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
