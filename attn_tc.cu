@@ -1,0 +1,519 @@
+// Flash-style attention on the 5th-generation tensor cores over
+//   [selected cached rows | the chunk's own causal rows]      (Algorithm 2's attention line, Eq. 2)
+// or, without an index list, over every cached row (Eq. 2, dense chunk attention).  bf16 in, fp32
+// softmax and accumulation, P rounded to bf16 for the PV product.
+//
+// One CTA owns 256 consecutive chunk rows of one query head as two 128-row Q tiles (A, B) and walks
+// the key tiles (128 keys) once for both.  Roles:
+//   warps 0-3 / 4-7  softmax of Q tile A / B: one thread per query row, S read from tensor memory,
+//                    running max / sum in registers, P written back to tensor memory over S,
+//                    lazy rescale of the O accumulator (only when the max grew by more than 2^32),
+//                    final normalisation and the global store.
+//   warps 8-10       loaders: every K / V row of a tile is fetched with 16-byte cp.async straight
+//                    into the 128-byte-swizzled layout the MMA descriptors expect.  The row address
+//                    comes from the selected-index list (the gather), the chunk offset, or the page
+//                    table, so no compacted copy of K or V is ever made; rows past the end are
+//                    zero-filled.  A slot's "full" barrier is armed by the copies themselves.
+//   warp 11          MMA issuer (one thread): S = Q K^T (both operands in shared memory) and
+//                    O += P V (P from tensor memory, V in shared memory, MN-major).
+// Tensor memory (512 columns): S_A | S_B | O_A | O_B, P aliasing the first 64 columns of its S.
+// K and V tiles share one ring of shared-memory slots in the order K0 V0 K1 V1 ...
+// 384 threads and no register re-balancing between roles: every thread may use 168 registers
+// (with 512 threads and setmaxnreg the compiler still scheduled the softmax for 128 registers,
+// which halved its speed).
+#include <algorithm>
+#include "attn_tiles.cuh"
+
+namespace quoka {
+
+template <int HALVES, bool SPARSE, bool SPLIT>
+__global__ void __launch_bounds__(kAttnThreads, 1)
+attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+               const __grid_constant__ CUtensorMap tm_v, const __nv_bfloat16* __restrict__ kc,
+               const __nv_bfloat16* __restrict__ vc, const int32_t* __restrict__ k_idx,
+               const int32_t* __restrict__ k_cnt, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
+  constexpr int D = HALVES * 64;
+  constexpr uint32_t kHalfBytes = 128 * 128;                 // 128 rows x 128 B
+  constexpr uint32_t kTileBytes = HALVES * kHalfBytes;       // one Q / K / V tile
+  constexpr int kSlots = HALVES == 2 ? 5 : 8;
+  // tensor memory: S buffers | P_A | P_B | O_A | O_B
+  constexpr int NBUF = HALVES == 2 ? 1 : 2;
+  constexpr uint32_t P_COL = NBUF * 128, O_COL = P_COL + 128;   // Q tile B's are 64 and D columns on
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  unsigned char* q_smem = smem;                               // [2][HALVES][128][128 B]
+  unsigned char* kv_smem = smem + 2 * kTileBytes;             // [kSlots][HALVES][128][128 B]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(kv_smem + (size_t)kSlots * kTileBytes);
+  uint64_t* kv_full = bars;                 // [kSlots]  the loader threads' cp.async arrivals
+  uint64_t* kv_empty = bars + kSlots;       // [kSlots]  MMA commit
+  uint64_t* s_full = bars + 2 * kSlots;     // [2][2]    MMA commit, per Q tile and S buffer
+  uint64_t* s_free = s_full + 4;            // [2]       S has been read: 4 softmax warps arrive, per S buffer
+  uint64_t* p_full = s_free + 2;            // [2][2]    4 softmax warps arrive, per Q tile and half of the key tile
+  uint64_t* p_done = p_full + 4;            // [2]       MMA commit: P has been multiplied
+  uint64_t* o_full = p_done + 2;            // [2]       MMA commit after the last PV
+  uint64_t* q_full = o_full + 2;            // TMA
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q_full + 1);
+  __shared__ int abort_flag;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const WaitCtx wc{&abort_flag, P.status};
+  // grid = (heads, row blocks, batch): heads vary fastest so the CTAs resident together share a KV head's
+  // rows in L2, and the row blocks run heaviest (most causal tiles) first, lightest last, the sequences longest first
+  const int s = longest_first(P, blockIdx.z), h = blockIdx.x, kv = h / P.group;
+  // (SPLIT: grid.y = row blocks times the parts a row block's key tiles are cut into)
+  const int n_parts = SPLIT ? P.attn_parts : 1;
+  const int rb = (SPLIT ? P.attn_split_rb : P.attn_row_blocks) - 1 - blockIdx.y / n_parts;
+  const int r0 = rb * 2 * kQTile;
+  AttnGeom g = make_geom<SPARSE>(P, s, r0);
+  // SPLIT: this CTA walks the tiles [t_lo, t_hi) of the row block's sequence only and leaves, per row, a partial
+  // result; the part that finishes last adds the parts up.  The list length has to be known before the range is, so
+  // nothing of the walk starts before the selection has ended.
+  int t_lo = 0;
+  if (SPLIT) {
+    if (SPARSE) { if (P.attn_after_whole) learn_count(g, k_cnt, s); else resolve(g, k_cnt, s); }
+    const int part = blockIdx.y % n_parts;
+    t_lo = (int)(((long long)part * g.n_known) / n_parts);
+    g.n_known = (int)(((long long)(part + 1) * g.n_known) / n_parts);
+  }
+
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int i = 0; i < kSlots; ++i) { mbar_init(&kv_full[i], kLoaderWarps * 32); mbar_init(&kv_empty[i], 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&s_free[i], 4); mbar_init(&p_done[i], 1); mbar_init(&o_full[i], 1); }
+    for (int i = 0; i < 4; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 4); }
+    mbar_init(q_full, 1);
+    fence_mbar_init();
+    tma_prefetch_desc(&tm_q);
+    tma_prefetch_desc(&tm_k);
+    tma_prefetch_desc(&tm_v);
+  }
+  if (warp == kQkWarp) tmem_alloc(tmem_slot, 512);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  if (!SPARSE && !SPLIT) grid_launch_dependents();
+
+  if (warp < 8) {
+    // ================================================================== softmax + epilogue
+    const int x = warp >> 2;                                  // Q tile A (0) or B (1)
+    const int quarter = warp & 3;
+    const int row_in_tile = quarter * 32 + lane;
+    const int row = r0 + x * kQTile + row_in_tile;            // chunk row
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+    const uint32_t p_addr = lane_addr + P_COL + x * 64, o_addr = lane_addr + O_COL + x * D;
+    const float scale_log2 = P.scale * 1.4426950408889634f;
+    float m_run = -INFINITY, l_run = 0.f;
+    uint32_t phase = 0, s_phase = 0;
+    // S buffers go by items (see attn_issue_qk): with both Q tiles at work each keeps one, a single one alternates
+    int buf = NBUF == 2 && (x ? t_lo >= g.skip_a : g.skip_a > t_lo) ? 1 : 0;
+    bool ok = true;
+    const int skip_x = max(x ? 0 : g.skip_a, t_lo);         // first tile this Q tile takes part in
+    const bool active_x = (x ? g.active_b : true) && (!SPLIT || skip_x < g.n_known);
+    VisibleCols<SPARSE> vis(g, skip_x, row);
+    for (int t = skip_x; active_x; ++t, vis.advance()) {
+      if (t == g.n_known) {                                   // end of what is known: the list length, or the end
+        if (g.resolved) break;
+        resolve(g, k_cnt, s);
+        if (t == g.n_known) break;
+      }
+      vis.at(g, t, row);
+      const bool masked = !__all_sync(0xFFFFFFFFu, vis.lim >= kKeyTile);
+      if (!mbar_wait(&s_full[2 * x + buf], (s_phase >> buf) & 1u, wc)) { ok = false; break; }
+      s_phase ^= 1u << buf;
+      tc_fence_after();
+      ok = attn_softmax_tile<D>(
+          lane_addr + buf * 128, p_addr, o_addr, vis.lim, masked, scale_log2, t == skip_x, lane, m_run, l_run, [&]() { mbar_arrive(&s_free[buf]); },
+          [&]() {
+            if (!mbar_wait_done(&p_done[x], phase ^ 1, wc)) return false;
+            tc_fence_after();
+            return true;
+          },
+          [&](int half) { mbar_arrive(&p_full[2 * x + half]); });
+      if (!ok) break;
+      phase ^= 1;
+      if (NBUF == 2 && !g.active_b) buf ^= 1;
+    }
+    // ---- epilogue: O / l -> bf16 -> global
+    if constexpr (!SPLIT) {
+      if (ok && active_x && mbar_wait(&o_full[x], 0, wc)) {
+        tc_fence_after();
+        attn_store_row<D>(P, o_addr, m_run, l_run, s, h, row, out, lse);
+      }
+    } else {
+      const bool have = ok && active_x && mbar_wait(&o_full[x], 0, wc);
+      if (have) tc_fence_after();
+      attn_split_epilogue<D>(P, (s * P.n_q + h) * P.attn_split_rb + rb, blockIdx.y % n_parts, n_parts, x, quarter, lane, row_in_tile, row, have,
+                             o_addr, m_run, l_run, s, h, out, lse);
+    }
+  } else if (warp < 8 + kLoaderWarps) {
+    // ================================================================== K / V row loaders (gather)
+    // One warp instruction copies 32 / PIECES whole rows (16 lanes x 16 bytes cover a 256-byte row); the
+    // row groups of a tile are dealt round-robin to the loader warps.
+    const int lw = warp - 8;
+    constexpr int PIECES = D / 8;                             // 16-byte pieces per row (16 or 8)
+    constexpr int ROWS_PER_INSTR = 32 / PIECES;               // 2 or 4
+    constexpr int GROUPS = kKeyTile / ROWS_PER_INSTR;         // 64 or 32 row groups per tile
+    constexpr int RPT = (GROUPS + kLoaderWarps - 1) / kLoaderWarps;   // row groups per warp (last one may be idle)
+    const int c16 = lane % PIECES;                            // this thread's piece of the row
+    const int rsub = lane / PIECES;
+    const int32_t* idx = SPARSE ? k_idx + ((long long)s * P.n_kv + kv) * P.budget_cap : nullptr;
+    uint32_t phase = 0;
+    int slot = 0;
+    const uint32_t kv_base = smem_u32(kv_smem);
+    // Row addressing in 16-byte units, 32 bits wide (the host refuses caches beyond 2^32 units; strides are
+    // multiples of 8 elements): sequence/head base plus this thread's piece, row stride, page stride.
+    const uint32_t st16 = (uint32_t)(P.kv_st >> 3), sb16 = (uint32_t)(P.kv_sb >> 3);
+    const uint32_t base16 = (uint32_t)(((P.page_size == 0 ? (long long)s * P.kv_sb : 0ll) + (long long)kv * P.kv_sh) >> 3) +
+                            (uint32_t)c16;
+    const int32_t* table = P.block_table + (long long)s * P.max_pages;
+    // Row numbers of this warp's rows of a tile of the selected list (-1 past the end), `base` = the tile's first
+    // list entry, `count` = entries left from there.  The warp's RPT * ROWS_PER_INSTR rows are numbered
+    // p = i * ROWS_PER_INSTR + rsub; lane l keeps rows p = l and p = 32 + l (two registers instead of one per row
+    // group), and the thread that copies row p fetches its number with a shuffle.  Except for the first list tile
+    // they are fetched when the previous tile's copies have been issued and only looked at when this tile's copies
+    // are issued (the loader normally waits for a free slot in between), so the loader does not wait on them.
+    // The per-row code below is kept free of branches (clamped loads, selects): a branch per row costs a single
+    // warp far more than the arithmetic it skips.
+    constexpr int LIST_REGS = (RPT * ROWS_PER_INSTR + 31) / 32;
+    static_assert(32 % ROWS_PER_INSTR == 0, "a row group's entries must sit in one register");
+    int t_list[LIST_REGS];
+    auto list_rows = [&](int base, int count) {
+      const int last = min(count, kKeyTile) - 1;                   // last valid row of the tile
+      if (last >= 0) {
+#pragma unroll
+        for (int k = 0; k < LIST_REGS; ++k) {
+          const int pp = 32 * k + lane;
+          const int rr = (lw + (pp / ROWS_PER_INSTR) * kLoaderWarps) * ROWS_PER_INSTR + pp % ROWS_PER_INSTR;
+          const int v = __ldcg(idx + base + min(rr, last));        // written by the kernel before: L2, not the read-only path
+          t_list[k] = rr <= last ? v : -1;
+        }
+      }
+    };
+#pragma unroll
+    for (int k = 0; k < LIST_REGS; ++k) t_list[k] = -1;
+    for (int tile = t_lo;; ++tile) {
+      if (tile == g.n_known) {                                // end of what is known: the list length, or the end
+        if (g.resolved) break;
+        resolve(g, k_cnt, s);
+        if (tile == g.n_known) break;
+      }
+      const TileRows tr = tile_rows<SPARSE>(g, tile);
+      bool stop = false;
+#pragma unroll 1
+      for (int kvi = 0; kvi < 2; ++kvi) {                     // the tile's K rows, then its V rows
+        if (!mbar_wait(&kv_empty[slot], phase ^ 1, wc)) { stop = true; break; }
+        // A whole tile of consecutive rows (page-aligned in a paged cache) is fetched by the copy engine as 64-row
+        // boxes: one thread issues them, the others only keep the barrier's arrival count.  Ragged tiles (rows past
+        // the end must read as zeros, not as whatever the cache holds there) and listed rows take the copies below.
+        if (!tr.from_list && tr.count >= kKeyTile && (P.page_size == 0 || (tr.first & (kPage - 1)) == 0)) {
+          if (lw == 0 && lane == 0) {
+            fence_proxy_async_smem();             // earlier contents of the slot were written through the generic proxy
+            mbar_arrive_expect_tx(&kv_full[slot], kTileBytes);
+            unsigned char* dst = kv_smem + (size_t)slot * kTileBytes;
+            const CUtensorMap* tm = kvi ? &tm_v : &tm_k;
+#pragma unroll
+            for (int sub = 0; sub < 2; ++sub) {
+              int c1 = tr.first + sub * 64, c3 = s;
+              if (P.page_size != 0) { c1 = 0; c3 = __ldg(table + (tr.first >> 6) + sub); }
+#pragma unroll
+              for (int hh = 0; hh < HALVES; ++hh)
+                tma_load_4d(dst + hh * kHalfBytes + sub * 64 * 128, tm, &kv_full[slot], hh * 64, c1, kv, c3);
+            }
+          } else {
+            mbar_arrive(&kv_full[slot]);
+          }
+          if (++slot == kSlots) { slot = 0; phase ^= 1; }
+          continue;
+        }
+        if (kvi == 0 && tr.from_list && tile == max(g.n_chunk, t_lo)) list_rows(tr.first, tr.count);   // first list tile
+        const uint4* src_base = reinterpret_cast<const uint4*>(kvi ? vc : kc);
+        const uint32_t dst_tile = kv_base + slot * kTileBytes + (c16 >> 3) * kHalfBytes;
+        int t[RPT];                                               // row number, or -1
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+          const int rr = (lw + i * kLoaderWarps) * ROWS_PER_INSTR + rsub;
+          const int listed = __shfl_sync(0xFFFFFFFFu, t_list[(i * ROWS_PER_INSTR) / 32], (i * ROWS_PER_INSTR + rsub) & 31);
+          t[i] = tr.from_list ? listed : (rr < tr.count ? tr.first + rr : -1);
+        }
+#ifdef QUOKA_DEBUG
+        // debug build: a listed row outside [0, T) is recorded and treated as absent (zero-filled) instead of read
+#pragma unroll
+        for (int i = 0; i < RPT; ++i)
+          if (tr.from_list && (t[i] < -1 || t[i] >= g.T)) { atomicExch(P.status, (int32_t)QUOKA_ERR_BAD_INDEX); t[i] = -1; }
+#endif
+        uint32_t off[RPT];
+        if (P.page_size == 0) {
+#pragma unroll
+          for (int i = 0; i < RPT; ++i) off[i] = base16 + (uint32_t)max(t[i], 0) * st16;
+        } else {
+#pragma unroll
+          for (int i = 0; i < RPT; ++i) {
+            const int tc = max(t[i], 0);
+            int page = __ldg(table + (tc >> 6));
+#ifdef QUOKA_DEBUG
+            // debug build: a page id outside the pool is recorded and the row treated as absent
+            if (t[i] >= 0 && (page < 0 || (long long)page >= P.kv_rows)) {
+              atomicExch(P.status, (int32_t)QUOKA_ERR_BAD_INDEX);
+              t[i] = -1;
+            }
+            if (page < 0 || (long long)page >= P.kv_rows) page = 0;
+#endif
+            off[i] = (uint32_t)page * sb16 + base16 + (uint32_t)(tc & (kPage - 1)) * st16;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+          const int rr = (lw + i * kLoaderWarps) * ROWS_PER_INSTR + rsub;
+          if (rr < kKeyTile)                                      // false only for the last group of some warps
+            cp_async_16(dst_tile + rr * 128 + (((c16 & 7) ^ (rr & 7)) << 4), src_base + off[i], t[i] >= 0);
+        }
+        // this thread's share of the slot is signalled by the copy engine itself when the bytes have landed:
+        // no wait in the loader, every slot of the ring can be in flight
+        cp_async_mbar_arrive_noinc(&kv_full[slot]);
+        if (kvi == 1 && tr.from_list) list_rows(tr.first + kKeyTile, tr.count - kKeyTile);   // next list tile
+        if (++slot == kSlots) { slot = 0; phase ^= 1; }
+      }
+      if (stop) break;
+    }
+    cp_async_wait_all();                                      // nothing of this thread is in flight at exit
+  } else {
+    // ================================================================== MMA issuers: warp 11 QK^T, warp 10 PV
+    if (warp == kQkWarp && lane == 0) {
+      mbar_arrive_expect_tx(q_full, 2 * kTileBytes);
+      for (int x = 0; x < 2; ++x)
+        for (int hh = 0; hh < HALVES; ++hh)
+          tma_load_4d(q_smem + x * kTileBytes + hh * kHalfBytes, &tm_q, q_full, hh * 64, r0 + x * kQTile, h, s);
+    }
+    __syncwarp();
+    const bool leader = elect_one();
+    const uint32_t tmem = (uint32_t)warp_uniform((int)tmem_base);
+    t_lo = warp_uniform(t_lo);
+    uniform_geom(g);
+    const uint32_t kv_base = smem_u32(kv_smem);
+    const auto acquire = [&](int sl, uint32_t phase) {
+      if (!warp_all(mbar_wait(&kv_full[sl], phase, wc))) return false;
+      fence_proxy_async_smem();               // cp.async wrote through the generic proxy, the MMA reads through the async one
+      tc_fence_after();
+      return true;
+    };
+    const auto release = [&](int sl) { if (leader) mma_commit(&kv_empty[sl]); };
+    // Operand descriptors are built once; a tile, slot or k-step offset is an addition to the 16-byte-unit
+    // address field (shared memory addresses stay far below the field's 14 bits).
+    // The sparse sequence's length is learnt (resolve) just before the walk past the chunk's own tiles.
+    if (warp == kQkWarp) {
+      const uint32_t idesc_qk = idesc_bf16_f32(128, kKeyTile, false, false);
+      const uint64_t desc_q = smem_desc_sw128(smem_u32(q_smem), 16, 1024);
+      const uint64_t desc_k = smem_desc_sw128(kv_base, 16, 1024);            // K-major rows (K tiles)
+      if (warp_all(mbar_wait(q_full, 0, wc)))
+        attn_issue_qk<NBUF, kSlots>(
+            g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); grid_launch_dependents(); }, acquire,
+            [&](unsigned buf, uint32_t parity) {
+              if (!warp_all(mbar_wait(&s_free[buf], parity, wc))) return false;
+              tc_fence_after();
+              return true;
+            },
+            [&](int x, unsigned buf, int ks) {
+              const uint64_t da = desc_q + (uint64_t)(x * (kTileBytes >> 4));
+              const uint64_t db = desc_k + (uint64_t)((uint32_t)ks * (kTileBytes >> 4));
+#pragma unroll
+              for (int hh = 0; hh < HALVES; ++hh)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                  const uint64_t off = (uint64_t)((hh * kHalfBytes + kk * 32) >> 4);
+                  if (leader) mma_ss(tmem + buf * 128, da + off, db + off, idesc_qk, (hh | kk) ? 1u : 0u);
+                }
+              if (leader) mma_commit(&s_full[2 * x + buf]);
+            },
+            release);
+    } else {
+      const uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true);
+      const uint64_t desc_v = smem_desc_sw128(kv_base, kHalfBytes, 1024);    // MN-major rows (V tiles)
+      uint32_t p_phase = 0;
+      attn_issue_pv<kSlots>(
+          g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); }, acquire,
+          [&](int x, int half, int vs, bool add) {
+            if (!warp_all(mbar_wait(&p_full[2 * x + half], (p_phase >> x) & 1u, wc))) return false;
+            tc_fence_after();
+            const uint64_t dv = desc_v + (uint64_t)((uint32_t)vs * (kTileBytes >> 4) + half * 4 * (2048 >> 4));
+            const uint32_t pa = tmem + P_COL + x * 64 + half * 32, oa = tmem + O_COL + x * D;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)             // 16 keys per MMA: 8 packed columns of P, 16 rows of V
+              if (leader) mma_ts(oa, pa + kk * 8, dv + (uint64_t)(kk * (2048 >> 4)), idesc_pv, add || kk ? 1u : 0u);
+            if (half) {
+              if (leader) mma_commit(&p_done[x]);
+              p_phase ^= 1u << x;
+            }
+            return true;
+          },
+          release, [&](int x) { if (leader) mma_commit(&o_full[x]); });
+    }
+  }
+  if (SPLIT && attn_last_cta()) grid_dependency_wait();       // this grid's end is the whole row blocks' end too
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kQkWarp) tmem_dealloc(tmem_base, 512);
+}
+
+// ---------------------------------------------------------------------------------------------- host
+// Split attention.  A grid of fewer CTAs than SMs (short chunks, few heads) leaves part of the GPU idle while
+// every CTA walks its whole key sequence; cutting each row block's tiles into parts, one CTA each, fills it.
+// The number of parts minimises  waves(parts) * (tiles / parts + 6):  a part costs about six tiles' time of
+// start-up, partial results and merge (the model fits the measured times of 1 to 5 parts on grids of 32 to 288 CTAs
+// within 3 %), parts keep at least six tiles, and a split has to promise 3 % to be taken.
+// The pair kernel's parts merge in a cluster of 2 * parts CTAs where all of a grid's clusters are resident at once: the
+// device holds 33, 22 or 15 of 4, 6 or 8 CTAs of this shared memory, the limits leave one or two free (a second wave costs
+// more than any split gives: 16 clusters of eight took 38 us where the 14 that fit take 30).  A part then costs about one
+// tile on top of the walk against parts through memory, and four and a half against a whole row block (a sparse part's step
+// is slower than a whole row block's).  Sparse attention, whole or parts through memory / clusters: 32 heads, 128 queries
+// over 2396 listed rows 32.8 / 24.5 us, over 1024 22.0 / 17.2; 256 over 3600 42.9 / 38.0; 512 over 1966 41.6 / 36.4; 8 heads,
+// 256 queries over 1024 25.3 / 19.6, over 2048 35.7 / 23.9.  Below the line: 8 heads, 256 over 512 18.5 / 19.4; 32 heads,
+// 512 queries over 1024 in a whole prefill call 58.0 / 59.2.  Dense, 8 heads, 256 over 4096 37.0 / 30.4.
+// A grid of q full waves and a rest has its lightest row blocks, as many as the rest, cut instead: the whole ones then
+// end after about q waves and the parts level the end.  The model is the total work over the SMs plus a third of a part
+// for the uneven end, against q + 1 waves of average jobs; list-scheduling simulations agree with it within 4 %.  Dense
+// calls take 3 % promised, sparse ones 7 % and equal lengths (their parts run a quarter slower per tile than whole row
+// blocks, and a batch's budgets differ): 32 heads, without / with parts: 1536 queries at 64K, a quarter listed 508 / 420 us,
+// 4096 at 128K 1039 / 990, 3072 at 32K, half listed 789 / 746; 40 heads, 1536 at 32K, promised 4 %: 290 / 309; dense 1536 at
+// 32K 920 / 692, 2048 at 32K 942 / 908, 4096 at 128K 7412 / 6689.
+// Partial results above 128 MB are not written: such jobs have waves enough.
+static long long attn_row_blocks(const quoka_params* p) { return (p->chunk_len + 2 * kQTile - 1) / (2 * kQTile); }
+static long long attn_jobs(const quoka_params* p) { return p->n_q_heads * attn_row_blocks(p) * p->batch; }
+static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
+  constexpr double kPartCost = 6.0;
+  AttnPlan plan;
+  if (p->dtype != QUOKA_BF16 || p->impl == QUOKA_IMPL_SIMT || p->chunk_len <= 1) return plan;
+  const long long n_rb = attn_row_blocks(p), per_rb = (long long)p->n_q_heads * p->batch, jobs = per_rb * n_rb;
+  const long long sms = device_sm_count();
+  if (sms <= 0) return plan;
+  if (jobs < sms) {
+    const double t = tiles + n_rb;                                          // plus the chunk's own tiles, on average
+    double best = t;
+    for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
+      const long long waves = (jobs * parts + sms - 1) / sms;
+      const double cost = (double)waves * (t / parts + kPartCost);
+      if (cost < 0.97 * best) { plan.split_rb = (int)n_rb; plan.parts = parts; plan.in_cluster = false; best = cost; }
+    }
+    // the pair kernel's, in clusters
+    const int group = p->n_q_heads / p->n_kv_heads;
+    if (p->head_dim == 128 && group % 2 == 0) {
+      for (int parts = 2; parts <= 4 && parts <= tiles / 2; ++parts) {
+        const double cost = t / parts + 1.0, limit = std::min(0.95 * best, 0.97 * t - 4.5);
+        if (jobs / 2 <= (parts == 2 ? 32 : parts == 3 ? 20 : 14) && cost < limit) {
+          plan.split_rb = (int)n_rb; plan.parts = parts; plan.in_cluster = true; best = cost / 0.95;
+        }
+      }
+    }
+    return plan;
+  }
+  const long long q = jobs / sms, rest = jobs % sms;
+  if (rest == 0 || (sparse && p->batch > 1)) return plan;
+  const long long split = (rest + per_rb - 1) / per_rb;                      // row blocks to cut; block r has 2 r + 2 own tiles
+  const double t_all = tiles + 2 + n_rb, t_whole = tiles + 2 + split + n_rb, t_split = tiles + 2 + split;
+  double best = (sparse ? 0.93 : 0.97) * (double)(q + 1) * t_all;
+  for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
+    const double t_part = t_split / parts + kPartCost;
+    const double cost = ((double)(jobs - split * per_rb) * t_whole + (double)(split * per_rb * parts) * t_part) / (double)sms + 0.3 * t_part;
+    AttnPlan cand;
+    cand.split_rb = (int)split; cand.parts = parts;
+    if (cost < best && attn_split_partial_bytes(p, cand) <= ((size_t)128 << 20)) { best = cost; plan = cand; }
+  }
+  return plan;
+}
+AttnPlan attn_plan_sparse(const quoka_params* p, int budget_cap) { return attn_plan(p, (budget_cap + kKeyTile - 1) / kKeyTile + 1, true); }
+AttnPlan attn_plan_dense(const quoka_params* p) { return attn_plan(p, (p->max_ctx_len + kKeyTile - 1) / kKeyTile + 1, false); }
+static size_t attn_split_jobs(const quoka_params* p, const AttnPlan& plan) { return (size_t)p->n_q_heads * p->batch * plan.split_rb; }
+size_t attn_split_partial_bytes(const quoka_params* p, const AttnPlan& plan) {
+  return plan.in_cluster ? 0 : attn_split_jobs(p, plan) * plan.parts * 2 * kSplitTileFloats * sizeof(float);
+}
+size_t attn_split_counter_bytes(const quoka_params* p, const AttnPlan& plan) { return plan.in_cluster ? 0 : attn_split_jobs(p, plan) * 8 * sizeof(int32_t); }
+
+// The launches of an attention call: the whole row blocks, then the ones in parts.
+//
+// Programmatic stream serialisation, (1) inside the fused call: the first launch may start while the kernel before it on
+// the stream (the key selection, which signals early and writes none of this kernel's other inputs) still runs; it touches
+// the selection's outputs only after its own griddepcontrol.wait.  A stand-alone call keeps the ordinary stream order:
+// whatever ran before it may have written q, k or v.  (2) The parts always: their CTAs take the SMs that the whole row
+// blocks' last wave leaves idle.  The whole row blocks let them start once every CTA has begun (dense) or has learnt the
+// list length (sparse: the selection is complete by then, so the parts need not wait for it), and the parts' last CTA
+// waits for the whole row blocks before it ends.
+quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const AttnPlan& plan, AttnKernel (*pick)(bool, bool, bool),
+                              const char* name, int cluster, size_t smem, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
+                              const CUtensorMap& tm_v, const void* k, const void* v, const int32_t* k_idx, const int32_t* k_cnt,
+                              void* out, float* lse, cudaStream_t st, bool after_selection) {
+  const bool sparse = k_idx != nullptr, split = plan.split_rb > 0 && (P.attn_partials || plan.in_cluster);
+  DevParams PP = P;
+  PP.attn_row_blocks = (int)attn_row_blocks(p);
+  PP.attn_split_rb = split ? plan.split_rb : 0;
+  PP.attn_parts = split ? plan.parts : 1;
+  const int whole = PP.attn_row_blocks - PP.attn_split_rb;
+  PP.attn_after_whole = whole > 0 ? 1 : 0;
+  if (split && !plan.in_cluster && !after_selection &&          // (the fused call clears the counters in an earlier kernel)
+      cudaMemsetAsync(P.attn_counters, 0, attn_split_counter_bytes(p, plan), st) != cudaSuccess)
+    return QUOKA_ERR_CUDA;
+  for (int parts = whole > 0 ? 0 : 1; parts <= (split ? 1 : 0); ++parts) {
+    AttnKernel kernel = pick(sparse, parts != 0, plan.in_cluster);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return QUOKA_ERR_CUDA;
+    const bool early = parts && whole > 0 ? true : sparse && after_selection;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(P.n_q, parts ? PP.attn_split_rb * PP.attn_parts : whole, P.batch);   // (pairs: n_q is even)
+    cfg.blockDim = dim3(kAttnThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    if (early) {
+      attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (parts && plan.in_cluster) {           // (the other kernels' clusters are part of the kernel)
+      attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+      attr[cfg.numAttrs].val.clusterDim.x = (unsigned)cluster;
+      attr[cfg.numAttrs].val.clusterDim.y = (unsigned)PP.attn_parts;
+      attr[cfg.numAttrs++].val.clusterDim.z = 1;
+    }
+    log_launch(name, cfg.gridDim, cfg.blockDim, smem, cluster, early);
+    if (cudaLaunchKernelEx(&cfg, kernel, PP, tm_q, tm_k, tm_v, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, k_idx, k_cnt,
+                           (__nv_bfloat16*)out, lse) != cudaSuccess)
+      return QUOKA_ERR_CUDA;
+    count_launch();
+  }
+  return cudaGetLastError() == cudaSuccess ? QUOKA_OK : QUOKA_ERR_CUDA;
+}
+
+bool attn_below_a_wave(const quoka_params* p) { return attn_jobs(p) < device_sm_count(); }
+
+bool attn_tc_supported(const quoka_params* p) {
+  if (p->dtype != QUOKA_BF16) return false;
+  // the loaders address cache rows in 32-bit units of 16 bytes
+  const int64_t extent = (p->page_size ? p->kv_rows : (int64_t)p->batch) * p->kv_stride_b;
+  if (extent / 8 >= (int64_t)0xFFFFFFFFll) return false;
+  return true;
+}
+
+template <int HALVES>
+static AttnKernel pick_attn_tc(bool sparse, bool parts, bool) {
+  if (parts) return sparse ? attn_tc_kernel<HALVES, true, true> : attn_tc_kernel<HALVES, false, true>;
+  return sparse ? attn_tc_kernel<HALVES, true, false> : attn_tc_kernel<HALVES, false, false>;
+}
+
+quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
+                            const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
+                            bool after_selection, const AttnPlan& plan) {
+  if (attn_tc_pair_applies(P)) return launch_attn_tc_pair(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection, plan);
+  CUtensorMap tm_q;
+  {
+    const uint64_t dims[4] = {(uint64_t)P.d, (uint64_t)P.chunk, (uint64_t)P.n_q, (uint64_t)P.batch};
+    const uint64_t strides[3] = {(uint64_t)P.q_st * 2, (uint64_t)P.q_sh * 2, (uint64_t)P.q_sb * 2};
+    const uint32_t box[4] = {64, 128, 1, 1};
+    if (!encode_tensor_map_bf16(&tm_q, q, 4, dims, strides, box)) return QUOKA_ERR_CUDA;
+  }
+  CUtensorMap tm_k, tm_v;
+  if (!encode_kv_tensor_map(&tm_k, p, k, 64) || !encode_kv_tensor_map(&tm_v, p, v, 64)) return QUOKA_ERR_CUDA;
+  const int halves = P.d / 64;
+  const size_t tile = (size_t)halves * 128 * 128;
+  const size_t smem = 1024 + (2 + (halves == 2 ? 5 : 8)) * tile + 512;
+  return launch_attn_plan(p, P, plan, halves == 2 ? pick_attn_tc<2> : pick_attn_tc<1>, "attn_tc", /*cluster=*/1, smem, tm_q, tm_k, tm_v, k, v, k_idx, k_cnt, out, lse, st, after_selection);
+}
+
+}  // namespace quoka

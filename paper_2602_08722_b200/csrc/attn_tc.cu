@@ -6,21 +6,21 @@
 // One CTA owns 256 consecutive chunk rows of one query head as two 128-row Q tiles (A, B) and walks
 // the key tiles (128 keys) once for both.  Roles:
 //   warps 0-3 / 4-7  softmax of Q tile A / B: one thread per query row, S read from tensor memory,
-//                    running max / sum in registers, P written back to tensor memory over S,
-//                    lazy rescale of the O accumulator (only when the max grew by more than 2^32),
-//                    final normalisation and the global store.
-//   warps 8-10       loaders: every K / V row of a tile is fetched with 16-byte cp.async straight
+//                    running max / sum in registers, P written back to tensor memory, lazy rescale of
+//                    the O accumulator (only when the max grew by more than 2^32), final
+//                    normalisation and the global store.
+//   warps 8-9        loaders: every K / V row of a tile is fetched with 16-byte cp.async straight
 //                    into the 128-byte-swizzled layout the MMA descriptors expect.  The row address
 //                    comes from the selected-index list (the gather), the chunk offset, or the page
 //                    table, so no compacted copy of K or V is ever made; rows past the end are
 //                    zero-filled.  A slot's "full" barrier is armed by the copies themselves.
-//   warp 11          MMA issuer (one thread): S = Q K^T (both operands in shared memory) and
-//                    O += P V (P from tensor memory, V in shared memory, MN-major).
-// Tensor memory (512 columns): S_A | S_B | O_A | O_B, P aliasing the first 64 columns of its S.
+//   warp 10          issues O += P V (P from tensor memory, V in shared memory, MN-major)
+//   warp 11          issues S = Q K^T (both operands in shared memory)
+// Where S and P live and what the products wait for: "order of the products" in attn_tiles.cuh.
 // K and V tiles share one ring of shared-memory slots in the order K0 V0 K1 V1 ...
-// 384 threads and no register re-balancing between roles: every thread may use 168 registers
-// (with 512 threads and setmaxnreg the compiler still scheduled the softmax for 128 registers,
-// which halved its speed).
+// 384 threads and no register re-balancing between roles: every thread may use 168 registers, a thirteenth warp would
+// leave it 128.  Sixteen softmax warps with half a row each (96 registers) were slower: 121 us where these take 100
+// (777 queries of 32 heads over 5000 listed rows, head_dim 64, the whole call).
 #include <algorithm>
 #include "attn_tiles.cuh"
 
@@ -35,7 +35,11 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
   constexpr int D = HALVES * 64;
   constexpr uint32_t kHalfBytes = 128 * 128;                 // 128 rows x 128 B
   constexpr uint32_t kTileBytes = HALVES * kHalfBytes;       // one Q / K / V tile
-  constexpr uint32_t S_COL[2] = {0, 128}, O_COL[2] = {256, 384};
+  constexpr int kSlots = HALVES == 2 ? 5 : 8;
+  // tensor memory (see "order of the products"): S | P_A | P_B | O_A | O_B, or S | S | S | O_A | O_B with P in place
+  constexpr bool APART = HALVES == 2;
+  constexpr int NBUF = APART ? 1 : 3;
+  constexpr uint32_t P_COL = 128, O_COL = APART ? 256 : 384;    // (Q tile B's P is 64, its O D columns on)
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char* q_smem = smem;                               // [2][HALVES][128][128 B]
@@ -43,9 +47,13 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
   uint64_t* bars = reinterpret_cast<uint64_t*>(kv_smem + (size_t)kSlots * kTileBytes);
   uint64_t* kv_full = bars;                 // [kSlots]  the loader threads' cp.async arrivals
   uint64_t* kv_empty = bars + kSlots;       // [kSlots]  MMA commit
-  uint64_t* s_full = bars + 2 * kSlots;     // [2]       MMA commit
-  uint64_t* p_full = s_full + 2;            // [2][2]    4 softmax warps arrive, per Q tile and half of the key tile
-  uint64_t* o_full = p_full + 4;            // [2]       MMA commit after the last PV
+  // (N = per Q tile if APART, per S buffer otherwise)
+  constexpr int N = APART ? 2 : NBUF;
+  uint64_t* s_full = bars + 2 * kSlots;     // [N]       MMA commit
+  uint64_t* p_full = s_full + N;            // [N][2]    4 softmax warps arrive, per half of the key tile
+  uint64_t* p_done = p_full + 2 * N;        // [N]       MMA commit: P has been multiplied
+  uint64_t* s_free = p_done + N;            // APART only: 4 softmax warps have read S
+  uint64_t* o_full = s_free + 1;            // [2]       MMA commit after the last PV
   uint64_t* q_full = o_full + 2;            // TMA
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q_full + 1);
   __shared__ int abort_flag;
@@ -74,15 +82,17 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int i = 0; i < kSlots; ++i) { mbar_init(&kv_full[i], kLoaderWarps * 32); mbar_init(&kv_empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&s_full[i], 1); mbar_init(&o_full[i], 1); }
-    for (int i = 0; i < 4; ++i) mbar_init(&p_full[i], 4);
+    for (int i = 0; i < N; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_done[i], 1); }
+    for (int i = 0; i < 2 * N; ++i) mbar_init(&p_full[i], 4);
+    for (int i = 0; i < 2; ++i) mbar_init(&o_full[i], 1);
+    mbar_init(s_free, 4);
     mbar_init(q_full, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tm_q);
     tma_prefetch_desc(&tm_k);
     tma_prefetch_desc(&tm_v);
   }
-  if (warp == kMmaWarp) tmem_alloc(tmem_slot, 512);
+  if (warp == kQkWarp) tmem_alloc(tmem_slot, 512);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -96,26 +106,42 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     const int row_in_tile = quarter * 32 + lane;
     const int row = r0 + x * kQTile + row_in_tile;            // chunk row
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t s_addr = lane_addr + S_COL[x], o_addr = lane_addr + O_COL[x];
+    const uint32_t o_addr = lane_addr + O_COL + x * D;
     const float scale_log2 = P.scale * 1.4426950408889634f;
     float m_run = -INFINITY, l_run = 0.f;
+    // APART: this Q tile's barriers.  Otherwise those of the S buffers, which go by items: the first of this Q tile's is item 0,
+    // or 1 where the other comes first, the next one is `step` items on.
     uint32_t phase = 0;
+    int buf = APART ? x : (x ? t_lo >= g.skip_a : g.skip_a > t_lo) ? 1 : 0;
+    const int step = APART ? 0 : g.active_b ? 2 : 1;
     bool ok = true;
     const int skip_x = max(x ? 0 : g.skip_a, t_lo);         // first tile this Q tile takes part in
     const bool active_x = (x ? g.active_b : true) && (!SPLIT || skip_x < g.n_known);
-    for (int t = skip_x; active_x; ++t) {
+    VisibleCols<SPARSE> vis(g, skip_x, row);
+    for (int t = skip_x; active_x; ++t, vis.advance()) {
       if (t == g.n_known) {                                   // end of what is known: the list length, or the end
         if (g.resolved) break;
         resolve(g, k_cnt, s);
         if (t == g.n_known) break;
       }
-      if (!mbar_wait(&s_full[x], phase, wc)) { ok = false; break; }
-      phase ^= 1;
+      vis.at(g, t, row);
+      const bool masked = !__all_sync(0xFFFFFFFFu, vis.lim >= kKeyTile);
+      if (!mbar_wait(&s_full[buf], phase, wc)) { ok = false; break; }
       tc_fence_after();
-      const int lim = visible_cols(tile_rows<SPARSE>(g, t), row);
-      const bool masked = !__all_sync(0xFFFFFFFFu, lim >= kKeyTile);
-      attn_softmax_tile<D>(s_addr, o_addr, lim, masked, scale_log2, t == skip_x, lane, m_run, l_run,
-                           [&](int half) { mbar_arrive(&p_full[2 * x + half]); });
+      const uint32_t s_addr = lane_addr + (APART ? 0 : buf * 128);
+      const auto products_done = [&]() {                      // of this Q tile's item before
+        const int before = buf - step;
+        if (!mbar_wait_done(&p_done[before < 0 ? before + N : before], APART || before < 0 ? phase ^ 1 : phase, wc)) return false;
+        tc_fence_after();
+        return true;
+      };
+      ok = attn_softmax_tile<D, APART>(
+          s_addr, APART ? lane_addr + P_COL + x * 64 : s_addr, o_addr, vis.lim, masked, scale_log2, t == skip_x, lane, m_run, l_run,
+          [&]() { mbar_arrive(s_free); }, [&]() { return APART ? products_done() : true; },
+          [&]() { return APART ? true : products_done(); }, [&](int half) { mbar_arrive(&p_full[2 * buf + half]); });
+      if (!ok) break;
+      buf += step;
+      if (APART || buf >= N) { phase ^= 1; buf -= APART ? 0 : N; }
     }
     // ---- epilogue: O / l -> bf16 -> global
     if constexpr (!SPLIT) {
@@ -137,44 +163,45 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     constexpr int PIECES = D / 8;                             // 16-byte pieces per row (16 or 8)
     constexpr int ROWS_PER_INSTR = 32 / PIECES;               // 2 or 4
     constexpr int GROUPS = kKeyTile / ROWS_PER_INSTR;         // 64 or 32 row groups per tile
-    constexpr int RPT = (GROUPS + kLoaderWarps - 1) / kLoaderWarps;   // row groups per warp (last one may be idle)
+    constexpr int RPT = GROUPS / kLoaderWarps;                // row groups per warp
     const int c16 = lane % PIECES;                            // this thread's piece of the row
     const int rsub = lane / PIECES;
     const int32_t* idx = SPARSE ? k_idx + ((long long)s * P.n_kv + kv) * P.budget_cap : nullptr;
     uint32_t phase = 0;
     int slot = 0;
     const uint32_t kv_base = smem_u32(kv_smem);
-    // Row addressing in 16-byte units, 32 bits wide (the host refuses caches beyond 2^32 units; strides are
+    // Row addressing in 16-byte units, 32 bits wide (the host refuses caches of 2^32 - 1 units and more; strides are
     // multiples of 8 elements): sequence/head base plus this thread's piece, row stride, page stride.
     const uint32_t st16 = (uint32_t)(P.kv_st >> 3), sb16 = (uint32_t)(P.kv_sb >> 3);
     const uint32_t base16 = (uint32_t)(((P.page_size == 0 ? (long long)s * P.kv_sb : 0ll) + (long long)kv * P.kv_sh) >> 3) +
                             (uint32_t)c16;
     const int32_t* table = P.block_table + (long long)s * P.max_pages;
-    // Row numbers of this warp's rows of a tile of the selected list (-1 past the end), `base` = the tile's first
-    // list entry, `count` = entries left from there.  The warp's RPT * ROWS_PER_INSTR rows are numbered
-    // p = i * ROWS_PER_INSTR + rsub; lane l keeps rows p = l and p = 32 + l (two registers instead of one per row
-    // group), and the thread that copies row p fetches its number with a shuffle.  Except for the first list tile
-    // they are fetched when the previous tile's copies have been issued and only looked at when this tile's copies
-    // are issued (the loader normally waits for a free slot in between), so the loader does not wait on them.
-    // The per-row code below is kept free of branches (clamped loads, selects): a branch per row costs a single
-    // warp far more than the arithmetic it skips.
-    constexpr int LIST_REGS = (RPT * ROWS_PER_INSTR + 31) / 32;
-    static_assert(32 % ROWS_PER_INSTR == 0, "a row group's entries must sit in one register");
-    int t_list[LIST_REGS];
+    // The warp's RPT * ROWS_PER_INSTR rows of a tile are numbered p = i * ROWS_PER_INSTR + rsub (i = its i-th row group); lane
+    // l looks after rows p = l and p = 32 + l: their row numbers (-1 past the end), for listed rows fetched when the
+    // previous tile's copies have been issued and looked at when this tile's are, and their offsets, worked out once per
+    // tile.  The thread that copies a row fetches its offset by shuffle.  The per-row code is kept free of branches: a branch
+    // per row costs a single warp far more than the arithmetic it skips.
+    constexpr int LIST_REGS = RPT * ROWS_PER_INSTR / 32;
+    static_assert(GROUPS % kLoaderWarps == 0 && RPT * ROWS_PER_INSTR % 32 == 0, "whole registers of rows");
+    int rows[LIST_REGS], rr_of[LIST_REGS];
+    uint32_t offs[LIST_REGS];
+#pragma unroll
+    for (int k = 0; k < LIST_REGS; ++k) {
+      const int pp = 32 * k + lane;
+      rr_of[k] = (lw + (pp / ROWS_PER_INSTR) * kLoaderWarps) * ROWS_PER_INSTR + pp % ROWS_PER_INSTR;
+      rows[k] = -1;
+      offs[k] = kNoRow;
+    }
     auto list_rows = [&](int base, int count) {
       const int last = min(count, kKeyTile) - 1;                   // last valid row of the tile
       if (last >= 0) {
 #pragma unroll
         for (int k = 0; k < LIST_REGS; ++k) {
-          const int pp = 32 * k + lane;
-          const int rr = (lw + (pp / ROWS_PER_INSTR) * kLoaderWarps) * ROWS_PER_INSTR + pp % ROWS_PER_INSTR;
-          const int v = __ldcg(idx + base + min(rr, last));        // written by the kernel before: L2, not the read-only path
-          t_list[k] = rr <= last ? v : -1;
+          const int v = __ldcg(idx + base + min(rr_of[k], last));  // written by the kernel before: L2, not the read-only path
+          rows[k] = rr_of[k] <= last ? v : -1;
         }
       }
     };
-#pragma unroll
-    for (int k = 0; k < LIST_REGS; ++k) t_list[k] = -1;
     for (int tile = t_lo;; ++tile) {
       if (tile == g.n_known) {                                // end of what is known: the list length, or the end
         if (g.resolved) break;
@@ -209,47 +236,21 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
           if (++slot == kSlots) { slot = 0; phase ^= 1; }
           continue;
         }
-        if (kvi == 0 && tr.from_list && tile == max(g.n_chunk, t_lo)) list_rows(tr.first, tr.count);   // first list tile
-        const uint4* src_base = reinterpret_cast<const uint4*>(kvi ? vc : kc);
-        const uint32_t dst_tile = kv_base + slot * kTileBytes + (c16 >> 3) * kHalfBytes;
-        int t[RPT];                                               // row number, or -1
+        if (kvi == 0) {
+          if (tr.from_list && tile == max(g.n_chunk, t_lo)) list_rows(tr.first, tr.count);   // first list tile
 #pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-          const int rr = (lw + i * kLoaderWarps) * ROWS_PER_INSTR + rsub;
-          const int listed = __shfl_sync(0xFFFFFFFFu, t_list[(i * ROWS_PER_INSTR) / 32], (i * ROWS_PER_INSTR + rsub) & 31);
-          t[i] = tr.from_list ? listed : (rr < tr.count ? tr.first + rr : -1);
-        }
-#ifdef QUOKA_DEBUG
-        // debug build: a listed row outside [0, T) is recorded and treated as absent (zero-filled) instead of read
-#pragma unroll
-        for (int i = 0; i < RPT; ++i)
-          if (tr.from_list && (t[i] < -1 || t[i] >= g.T)) { atomicExch(P.status, (int32_t)QUOKA_ERR_BAD_INDEX); t[i] = -1; }
-#endif
-        uint32_t off[RPT];
-        if (P.page_size == 0) {
-#pragma unroll
-          for (int i = 0; i < RPT; ++i) off[i] = base16 + (uint32_t)max(t[i], 0) * st16;
-        } else {
-#pragma unroll
-          for (int i = 0; i < RPT; ++i) {
-            const int tc = max(t[i], 0);
-            int page = __ldg(table + (tc >> 6));
-#ifdef QUOKA_DEBUG
-            // debug build: a page id outside the pool is recorded and the row treated as absent
-            if (t[i] >= 0 && (page < 0 || (long long)page >= P.kv_rows)) {
-              atomicExch(P.status, (int32_t)QUOKA_ERR_BAD_INDEX);
-              t[i] = -1;
-            }
-            if (page < 0 || (long long)page >= P.kv_rows) page = 0;
-#endif
-            off[i] = (uint32_t)page * sb16 + base16 + (uint32_t)(tc & (kPage - 1)) * st16;
+          for (int k = 0; k < LIST_REGS; ++k) {
+            if (!tr.from_list) rows[k] = rr_of[k] < tr.count ? tr.first + rr_of[k] : -1;
+            offs[k] = kv_row_off16(P, table, st16, sb16, rows[k], tr.from_list, g.T);
           }
         }
+        const uint4* src_base = reinterpret_cast<const uint4*>(kvi ? vc : kc) + base16;
+        const uint32_t dst_tile = kv_base + slot * kTileBytes + (c16 >> 3) * kHalfBytes;
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
+          const uint32_t off = __shfl_sync(0xFFFFFFFFu, offs[(i * ROWS_PER_INSTR) / 32], (i * ROWS_PER_INSTR + rsub) & 31);
           const int rr = (lw + i * kLoaderWarps) * ROWS_PER_INSTR + rsub;
-          if (rr < kKeyTile)                                      // false only for the last group of some warps
-            cp_async_16(dst_tile + rr * 128 + (((c16 & 7) ^ (rr & 7)) << 4), src_base + off[i], t[i] >= 0);
+          cp_async_16(dst_tile + rr * 128 + (((c16 & 7) ^ (rr & 7)) << 4), src_base + (off == kNoRow ? 0u : off), off != kNoRow);
         }
         // this thread's share of the slot is signalled by the copy engine itself when the bytes have landed:
         // no wait in the loader, every slot of the ring can be in flight
@@ -260,99 +261,83 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
       if (stop) break;
     }
     cp_async_wait_all();                                      // nothing of this thread is in flight at exit
-  } else if (lane == 0) {
-    // ================================================================== MMA issuer (one thread)
-    mbar_arrive_expect_tx(q_full, 2 * kTileBytes);
-    for (int x = 0; x < 2; ++x)
-      for (int hh = 0; hh < HALVES; ++hh)
-        tma_load_4d(q_smem + x * kTileBytes + hh * kHalfBytes, &tm_q, q_full, hh * 64, r0 + x * kQTile, h, s);
-    const uint32_t idesc_qk = idesc_bf16_f32(128, kKeyTile, false, false);
-    const uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true);
-    const uint32_t q_base = smem_u32(q_smem), kv_base = smem_u32(kv_smem);
-    int slot = 0;
-    uint32_t kv_phase = 0;
-    uint32_t p_phase[2] = {0, 0};
-    int k_slot = -1, v_slot = -1;
-    bool ok = mbar_wait(q_full, 0, wc);
-    auto acquire = [&]() -> int {           // next ring item (K or V) becomes readable
-      if (!mbar_wait(&kv_full[slot], kv_phase, wc)) { ok = false; return 0; }
-      fence_proxy_async_smem();             // cp.async wrote through the generic proxy, the MMA reads through the async one
+  } else {
+    // ================================================================== warp 11: QK^T, warp 10: PV
+    if (warp == kQkWarp && lane == 0) {
+      mbar_arrive_expect_tx(q_full, 2 * kTileBytes);
+      for (int x = 0; x < 2; ++x)
+        for (int hh = 0; hh < HALVES; ++hh)
+          tma_load_4d(q_smem + x * kTileBytes + hh * kHalfBytes, &tm_q, q_full, hh * 64, r0 + x * kQTile, h, s);
+    }
+    __syncwarp();
+    const bool leader = elect_one();
+    const uint32_t tmem = (uint32_t)warp_uniform((int)tmem_base);
+    t_lo = warp_uniform(t_lo);
+    uniform_geom(g);
+    const uint32_t kv_base = smem_u32(kv_smem);
+    const auto acquire = [&](int sl, uint32_t phase) {
+      if (!warp_all(mbar_wait(&kv_full[sl], phase, wc))) return false;
+      fence_proxy_async_smem();               // cp.async wrote through the generic proxy, the MMA reads through the async one
       tc_fence_after();
-      const int got = slot;
-      if (++slot == kSlots) { slot = 0; kv_phase ^= 1; }
-      return got;
+      return true;
     };
+    const auto release = [&](int sl) { if (leader) mma_commit(&kv_empty[sl]); };
     // Operand descriptors are built once; a tile, slot or k-step offset is an addition to the 16-byte-unit
-    // address field (shared memory addresses stay far below the field's 14 bits), which keeps the issuing
-    // thread's instruction count per MMA small.
-    const uint64_t desc_q = smem_desc_sw128(q_base, 16, 1024);
-    const uint64_t desc_k = smem_desc_sw128(kv_base, 16, 1024);            // K-major rows (K tiles)
-    const uint64_t desc_v = smem_desc_sw128(kv_base, kHalfBytes, 1024);    // MN-major rows (V tiles)
-    auto issue_qk = [&](int x, int ks) {
-      const uint64_t da = desc_q + (uint64_t)(x * (kTileBytes >> 4));
-      const uint64_t db = desc_k + (uint64_t)((uint32_t)ks * (kTileBytes >> 4));
+    // address field (shared memory addresses stay far below the field's 14 bits).
+    // The sparse sequence's length is learnt (resolve) just before the walk past the chunk's own tiles.
+    if (warp == kQkWarp) {
+      const uint32_t idesc_qk = idesc_bf16_f32(128, kKeyTile, false, false);
+      const uint64_t desc_q = smem_desc_sw128(smem_u32(q_smem), 16, 1024);
+      const uint64_t desc_k = smem_desc_sw128(kv_base, 16, 1024);            // K-major rows (K tiles)
+      if (warp_all(mbar_wait(q_full, 0, wc)))
+        attn_issue_qk<NBUF, kSlots>(
+            g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); grid_launch_dependents(); }, acquire,
+            [&](unsigned buf, uint32_t parity) {
+              if (!warp_all(mbar_wait(APART ? s_free : &p_done[buf], parity, wc))) return false;
+              tc_fence_after();
+              return true;
+            },
+            [&](int x, unsigned buf, int ks) {
+              const uint64_t da = desc_q + (uint64_t)(x * (kTileBytes >> 4));
+              const uint64_t db = desc_k + (uint64_t)((uint32_t)ks * (kTileBytes >> 4));
 #pragma unroll
-      for (int hh = 0; hh < HALVES; ++hh)
+              for (int hh = 0; hh < HALVES; ++hh)
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint64_t off = (uint64_t)((hh * kHalfBytes + kk * 32) >> 4);
-          mma_ss(tmem_base + S_COL[x], da + off, db + off, idesc_qk, (hh | kk) ? 1u : 0u);
-        }
-      mma_commit(&s_full[x]);
-    };
-    auto issue_pv = [&](int x, int vs, bool first) {
-      const uint64_t dv = desc_v + (uint64_t)((uint32_t)vs * (kTileBytes >> 4));
+                for (int kk = 0; kk < 4; ++kk) {
+                  const uint64_t off = (uint64_t)((hh * kHalfBytes + kk * 32) >> 4);
+                  if (leader) mma_ss(tmem + buf * 128, da + off, db + off, idesc_qk, (hh | kk) ? 1u : 0u);
+                }
+              if (leader) mma_commit(&s_full[APART ? x : buf]);
+            },
+            release);
+    } else {
+      const uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true);
+      const uint64_t desc_v = smem_desc_sw128(kv_base, kHalfBytes, 1024);    // MN-major rows (V tiles)
+      uint32_t p_phase = 0;
+      attn_issue_pv<NBUF, kSlots>(
+          g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); }, acquire,
+          [&](int x, int half, unsigned buf, int vs, bool add) {
+            const unsigned n = APART ? x : buf;
+            if (!warp_all(mbar_wait(&p_full[2 * n + half], (p_phase >> n) & 1u, wc))) return false;
+            tc_fence_after();
+            const uint64_t dv = desc_v + (uint64_t)((uint32_t)vs * (kTileBytes >> 4) + half * 4 * (2048 >> 4));
+            const uint32_t pa = tmem + (APART ? P_COL + x * 64 : buf * 128) + half * 32, oa = tmem + O_COL + x * D;
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        if (!mbar_wait(&p_full[2 * x + half], p_phase[x], wc)) { ok = false; return; }
-        tc_fence_after();
-#pragma unroll
-        for (int kk = half * 4; kk < half * 4 + 4; ++kk) {   // 16 keys per MMA: 8 packed columns of P, 16 rows of V
-          mma_ts(tmem_base + O_COL[x], tmem_base + S_COL[x] + kk * 8, dv + (uint64_t)(kk * (2048 >> 4)), idesc_pv,
-                 (!first || kk) ? 1u : 0u);
-        }
-      }
-      p_phase[x] ^= 1;
-    };
-    // Tile t: O += P_t V_t for each Q tile taking part (as the two halves of P arrive), then S = Q K_{t+1}^T.
-    // K_{t+1} and V_t are both acquired before the P waits, so those never sit on the P -> PV -> QK chain.
-    // The sparse sequence's length is learnt (resolve) just before the look-ahead past the chunk's own tiles.
-    const auto part = [&](int x, int t) { return x ? g.active_b : t >= g.skip_a; };
-    if (ok && t_lo < g.n_known) {
-      k_slot = acquire();
-      if (ok) {
-        if (part(0, t_lo)) issue_qk(0, k_slot);
-        if (part(1, t_lo)) issue_qk(1, k_slot);
-        mma_commit(&kv_empty[k_slot]);
-      }
-      for (int t = t_lo; ok; ++t) {
-        if (t + 1 == g.n_known && !g.resolved) { resolve(g, k_cnt, s); grid_launch_dependents(); }
-        const bool more = t + 1 < g.n_known;
-        v_slot = acquire();
-        if (ok && more) k_slot = acquire();
-        if (!ok) break;
-        if (part(0, t)) {
-          issue_pv(0, v_slot, t == max(g.skip_a, t_lo));
-          if (!ok) break;
-          if (!more) mma_commit(&o_full[0]);
-        }
-        if (more && part(0, t + 1)) issue_qk(0, k_slot);
-        if (part(1, t)) {
-          issue_pv(1, v_slot, t == t_lo);
-          if (!ok) break;
-          if (!more) mma_commit(&o_full[1]);
-        }
-        mma_commit(&kv_empty[v_slot]);
-        if (!more) break;
-        if (part(1, t + 1)) issue_qk(1, k_slot);
-        mma_commit(&kv_empty[k_slot]);
-      }
+            for (int kk = 0; kk < 4; ++kk)             // 16 keys per MMA: 8 packed columns of P, 16 rows of V
+              if (leader) mma_ts(oa, pa + kk * 8, dv + (uint64_t)(kk * (2048 >> 4)), idesc_pv, add || kk ? 1u : 0u);
+            if (half) {
+              if (leader) mma_commit(&p_done[n]);
+              p_phase ^= 1u << n;
+            }
+            return true;
+          },
+          release, [&](int x) { if (leader) mma_commit(&o_full[x]); });
     }
   }
   if (SPLIT && attn_last_cta()) grid_dependency_wait();       // this grid's end is the whole row blocks' end too
   tc_fence_before();
   __syncthreads();
-  if (warp == kMmaWarp) tmem_dealloc(tmem_base, 512);
+  if (warp == kQkWarp) tmem_dealloc(tmem_base, 512);
 }
 
 // ---------------------------------------------------------------------------------------------- host
@@ -512,7 +497,7 @@ quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P, const voi
   if (!encode_kv_tensor_map(&tm_k, p, k, 64) || !encode_kv_tensor_map(&tm_v, p, v, 64)) return QUOKA_ERR_CUDA;
   const int halves = P.d / 64;
   const size_t tile = (size_t)halves * 128 * 128;
-  const size_t smem = 1024 + (2 + kSlots) * tile + 512;
+  const size_t smem = 1024 + (2 + (halves == 2 ? 5 : 8)) * tile + 512;
   return launch_attn_plan(p, P, plan, halves == 2 ? pick_attn_tc<2> : pick_attn_tc<1>, "attn_tc", /*cluster=*/1, smem, tm_q, tm_k, tm_v, k, v, k_idx, k_cnt, out, lse, st, after_selection);
 }
 

@@ -8,18 +8,20 @@
 //   O += P V  : each CTA supplies its own P (tensor memory) and 64 of V's 128 columns (all 128 keys).
 // So a CTA fetches HALF of every K and V tile (the 16-byte cp.async gather of listed rows tops out near 20 bytes per
 // clock and SM, which a one-CTA step of 64 KB all but needs), its loaders execute half the instructions, and per
-// key tile and Q tile the tensor core reads 48 KB + 16 KB of a CTA's shared memory instead of 64 KB + 32 KB.  A
-// step's time itself is set by one Q tile's chain S ready -> softmax -> P ready -> PV -> next QK^T and changes little:
-// measured against the one-CTA kernel, 1 % (listed rows) to 4 % (whole tiles, paged serving mix) faster.
+// key tile and Q tile the tensor core reads 48 KB + 16 KB of a CTA's shared memory instead of 64 KB + 32 KB.
+// What bounds a step (one key tile for both Q tiles; the products alone take 2050 cycles, the exponentials 2100): the chain
+// S ready -> read by the softmax warps of both CTAs -> next QK^T, twice, which meets the second half of the PV products of
+// the other Q tile; about 2750 cycles where P over S and one issuing thread took 3550.  2048 queries at 32K: sparse call 211
+// -> 196 us, dense 1052 -> 952; 4096 at 128K 1245 -> 1140; paged mix of 8 sequences 950 -> 875.
 //
-// Roles per CTA as in the one-CTA kernel (8 softmax warps, 3 loader warps, warp 11), except:
-//   * only the first CTA's warp 11 issues MMAs.  A slot of its ring is ready when its own loaders AND the second
-//     CTA's have filled it: warp 11 of the second CTA forwards its slots' "full" barriers, in ring order, to a
-//     barrier of the first CTA;
-//   * completions (S ready, slot free, O final) are delivered to both CTAs' barriers by one multicast commit;
-//   * the softmax warps of both CTAs announce P on the first CTA's barriers;
+// Roles per CTA as in the one-CTA kernel, except:
+//   * only the first CTA's warps 10 and 11 issue MMAs.  A slot of its ring is ready when its own loaders AND the second
+//     CTA's have filled it: the second CTA's warps 10 and 11 forward the "full" barriers of its V and K slots to a barrier
+//     of the first CTA;
+//   * completions (S ready, P multiplied, slot free, O final) are delivered to both CTAs' barriers by one multicast commit;
+//   * the softmax warps of both CTAs announce "S read" and "P ready" on the first CTA's barriers;
 //   * nobody leaves before a cluster barrier: the other CTA's MMAs read this one's shared and tensor memory.
-// Tensor memory (512 columns per CTA): S_A | S_B | O_A | O_B, P aliasing the first 64 columns of its S.
+// Tensor memory (512 columns per CTA): S | P_A | P_B | O_A | O_B.
 // Ring slots are 16 KB: a K item holds [2 halves of d][64 keys][128 B], a V item [128 keys][128 B], both in the
 // 128-byte-swizzled layout of the operand descriptors.
 #include "attn_tiles.cuh"
@@ -27,7 +29,7 @@
 namespace quoka {
 
 constexpr int kPairSlots = 8;
-constexpr int kPairLoaderWarps = 3;
+constexpr int kPairLoaderWarps = kLoaderWarps;
 constexpr uint32_t kPairSlotBytes = 16384;
 constexpr uint32_t kPairQTileBytes = 32768;
 
@@ -41,7 +43,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
                   float* __restrict__ lse) {
   constexpr bool SPLIT = MODE != kWhole;
   constexpr int D = 128;
-  constexpr uint32_t S_COL[2] = {0, 128}, O_COL[2] = {256, 384};
+  constexpr uint32_t S_COL = 0, P_COL = 128, O_COL = 256;     // Q tile B's P and O are 64 and 128 columns on
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char* q_smem = smem;                               // [2][2 halves][128][128 B]
@@ -51,8 +53,10 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
   uint64_t* kv_empty = kv_full + kPairSlots;      // [kPairSlots]  MMA commit (both CTAs)
   uint64_t* peer_full = kv_empty + kPairSlots;    // [kPairSlots]  first CTA only: the second CTA's slot is full
   uint64_t* s_full = peer_full + kPairSlots;      // [2]           MMA commit (both CTAs)
-  uint64_t* p_full = s_full + 2;                  // [2][2]        first CTA only: 4 softmax warps of each CTA
-  uint64_t* o_full = p_full + 4;                  // [2]           MMA commit (both CTAs)
+  uint64_t* s_free = s_full + 2;                  //               first CTA only: S has been read, 4 softmax warps of each CTA
+  uint64_t* p_full = s_free + 1;                  // [2][2]        first CTA only: 4 softmax warps of each CTA
+  uint64_t* p_done = p_full + 4;                  // [2]           MMA commit (both CTAs): P has been multiplied
+  uint64_t* o_full = p_done + 2;                  // [2]           MMA commit (both CTAs)
   uint64_t* q_full = o_full + 2;                  // this CTA's Q tiles (TMA)
   uint64_t* peer_q = q_full + 1;                  // first CTA only: the second CTA's Q tiles have landed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(peer_q + 1);
@@ -79,8 +83,9 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
       mbar_init(&kv_empty[i], 1);
       mbar_init(&peer_full[i], 1);
     }
-    for (int i = 0; i < 2; ++i) { mbar_init(&s_full[i], 1); mbar_init(&o_full[i], 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_done[i], 1); mbar_init(&o_full[i], 1); }
     for (int i = 0; i < 4; ++i) mbar_init(&p_full[i], 8);
+    mbar_init(s_free, 8);
     mbar_init(q_full, 1);
     mbar_init(peer_q, 1);
     fence_mbar_init();
@@ -88,7 +93,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     tma_prefetch_desc(&tm_k);
     tma_prefetch_desc(&tm_v);
   }
-  if (warp == kMmaWarp) tmem_alloc_pair(tmem_slot, 512);
+  if (warp == kQkWarp) tmem_alloc_pair(tmem_slot, 512);
   tc_fence_before();
   cluster_sync_all();                                         // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
@@ -105,7 +110,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
   // parts up.  The list length has to be known before the range is, so nothing of the walk starts before the selection has
   // ended.
   if (SPLIT) {
-    if (warp == kMmaWarp && lane == 0) load_q();
+    if (warp == kQkWarp && lane == 0) load_q();
     if (SPARSE) { if (P.attn_after_whole) learn_count(g, k_cnt, s); else resolve(g, k_cnt, s); }
     const int part = blockIdx.y % n_parts;
     t_lo = (int)(((long long)part * g.n_known) / n_parts);
@@ -121,28 +126,36 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     const int row_in_tile = quarter * 32 + lane;
     const int row = r0 + x * kQTile + row_in_tile;            // chunk row
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    const uint32_t s_addr = lane_addr + S_COL[x], o_addr = lane_addr + O_COL[x];
+    const uint32_t p_addr = lane_addr + P_COL + x * 64, o_addr = lane_addr + O_COL + x * D;
     const float scale_log2 = P.scale * 1.4426950408889634f;
-    const uint32_t p_bar0 = map_to_cta(smem_u32(&p_full[2 * x]), first);   // the first CTA's barriers
-    const uint32_t p_bar1 = map_to_cta(smem_u32(&p_full[2 * x + 1]), first);
+    const uint32_t s_bar = map_to_cta(smem_u32(s_free), first);            // the first CTA's barriers
+    const uint32_t p_bar = map_to_cta(smem_u32(&p_full[2 * x]), first);
     float m_run = -INFINITY, l_run = 0.f;
     uint32_t phase = 0;
     bool ok = true;
     const int skip_x = max(x ? 0 : g.skip_a, t_lo);         // first tile this Q tile takes part in
     const bool active_x = (x ? g.active_b : true) && (!SPLIT || skip_x < g.n_known);
-    for (int t = skip_x; active_x; ++t) {
+    VisibleCols<SPARSE> vis(g, skip_x, row);
+    for (int t = skip_x; active_x; ++t, vis.advance()) {
       if (t == g.n_known) {                                   // end of what is known: the list length, or the end
         if (g.resolved) break;
         resolve(g, k_cnt, s);
         if (t == g.n_known) break;
       }
+      vis.at(g, t, row);
+      const bool masked = !__all_sync(0xFFFFFFFFu, vis.lim >= kKeyTile);
       if (!mbar_wait(&s_full[x], phase, wc)) { ok = false; break; }
-      phase ^= 1;
       tc_fence_after();
-      const int lim = visible_cols(tile_rows<SPARSE>(g, t), row);
-      const bool masked = !__all_sync(0xFFFFFFFFu, lim >= kKeyTile);
-      attn_softmax_tile<D>(s_addr, o_addr, lim, masked, scale_log2, t == skip_x, lane, m_run, l_run,
-                           [&](int half) { mbar_arrive_cluster(half ? p_bar1 : p_bar0); });
+      ok = attn_softmax_tile<D, true>(
+          lane_addr + S_COL, p_addr, o_addr, vis.lim, masked, scale_log2, t == skip_x, lane, m_run, l_run, [&]() { mbar_arrive_cluster(s_bar); },
+          [&]() {
+            if (!mbar_wait_done(&p_done[x], phase ^ 1, wc)) return false;
+            tc_fence_after();
+            return true;
+          },
+          []() { return true; }, [&](int half) { mbar_arrive_cluster(p_bar + 8u * half); });
+      if (!ok) break;
+      phase ^= 1;
     }
     // ---- epilogue: O / l -> bf16 -> global
     if constexpr (!SPLIT) {
@@ -170,7 +183,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     // Either way an item is 32 row groups, dealt round-robin to the loader warps.
     const int lw = warp - 8;
     constexpr int GROUPS = 32;
-    constexpr int RPT = (GROUPS + kPairLoaderWarps - 1) / kPairLoaderWarps;   // row groups per warp (the last may be idle)
+    constexpr int RPT = GROUPS / kPairLoaderWarps;             // row groups per warp
     const int kc16 = lane & 15, krsub = lane >> 4;
     const int vc16 = lane & 7, vrsub = lane >> 3;
     const int krow0 = (int)rank * 64;
@@ -178,35 +191,32 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     uint32_t phase = 0;
     int slot = 0;
     const uint32_t kv_base = smem_u32(kv_smem);
-    // Row addressing in 16-byte units, 32 bits wide (the host refuses caches beyond 2^32 units; strides are
+    // Row addressing in 16-byte units, 32 bits wide (the host refuses caches of 2^32 - 1 units and more; strides are
     // multiples of 8 elements): sequence/head base plus this thread's piece, row stride, page stride.
     const uint32_t st16 = (uint32_t)(P.kv_st >> 3), sb16 = (uint32_t)(P.kv_sb >> 3);
     const uint32_t head16 = (uint32_t)(((P.page_size == 0 ? (long long)s * P.kv_sb : 0ll) + (long long)kv * P.kv_sh) >> 3);
     const uint32_t kbase16 = head16 + (uint32_t)kc16, vbase16 = head16 + rank * 8u + (uint32_t)vc16;
     const int32_t* table = P.block_table + (long long)s * P.max_pages;
-    // Row numbers of this warp's rows of a tile of the selected list (-1 past the end), fetched one tile ahead.
-    // The warp's K rows are numbered p = 2 i + rsub (i = its i-th row group), its V rows p = 4 i + rsub; lane l
-    // keeps K row p = l and V rows p = l, 32 + l, and the thread that copies a row fetches its number by shuffle.
-    int tk_list = -1, tv_list[2] = {-1, -1};
+    // The warp's K rows of a tile are numbered p = 2 i + rsub (i = its i-th row group), its V rows p = 4 i + rsub; lane l
+    // looks after K row p = l and V rows p = l, 32 + l: their row numbers (-1 past the end), for listed rows fetched one
+    // tile ahead, and their offsets, worked out once per tile.  The thread that copies a row fetches its offset by shuffle.
+    int k_row = -1, v_row[2] = {-1, -1};
+    uint32_t k_off = kNoRow, v_off[2] = {kNoRow, kNoRow};
+    const int krr = krow0 + (lw + (lane >> 1) * kPairLoaderWarps) * 2 + (lane & 1);
+    const int vrr = (lw + (lane >> 2) * kPairLoaderWarps) * 4 + (lane & 3);       // the second one is kVStep rows on
+    constexpr int kVStep = 8 * kPairLoaderWarps * 4;
+    static_assert(GROUPS % kPairLoaderWarps == 0 && RPT == 16, "a lane per K row, two V rows per lane");
     auto list_rows = [&](int base, int count) {
       const int last = min(count, kKeyTile) - 1;                   // last valid row of the tile
-      if (last >= 0) {
-        {
-          const int gi = lw + (lane >> 1) * kPairLoaderWarps;
-          const int rr = krow0 + gi * 2 + (lane & 1);
-          const int v = __ldcg(idx + base + min(rr, last));        // written by the kernel before: L2, not the read-only path
-          tk_list = (lane < 2 * RPT && gi < GROUPS && rr <= last) ? v : -1;
-        }
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const int pp = 32 * k + lane;
-          const int gi = lw + (pp >> 2) * kPairLoaderWarps;
-          const int rr = gi * 4 + (pp & 3);
-          const int v = __ldcg(idx + base + min(rr, last));
-          tv_list[k] = (pp < 4 * RPT && gi < GROUPS && rr <= last) ? v : -1;
-        }
+      if (last >= 0) {                                             // written by the kernel before: L2, not the read-only path
+        const int vk = __ldcg(idx + base + min(krr, last));
+        const int v0 = __ldcg(idx + base + min(vrr, last)), v1 = __ldcg(idx + base + min(vrr + kVStep, last));
+        k_row = krr <= last ? vk : -1;
+        v_row[0] = vrr <= last ? v0 : -1;
+        v_row[1] = vrr + kVStep <= last ? v1 : -1;
       }
     };
+    auto row_off = [&](int t, bool listed) -> uint32_t { return kv_row_off16(P, table, st16, sb16, t, listed, g.T); };
     // One ring item of tile `tr`: K (is_v = false) or V.  Returns false when a wait gave up.
     auto item = [&](auto is_v_c, const TileRows& tr, bool first_list_tile) -> bool {
       constexpr bool V = decltype(is_v_c)::value;
@@ -234,51 +244,26 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
           mbar_arrive(&kv_full[slot]);
         }
       } else {
-        if (!V && first_list_tile) list_rows(tr.first, tr.count);
-        const int c16 = V ? vc16 : kc16, rsub = V ? vrsub : krsub;
-        const uint32_t base16 = V ? vbase16 : kbase16;
-        const uint4* src_base = reinterpret_cast<const uint4*>(V ? vc : kc);
-        const uint32_t dst_item = kv_base + (uint32_t)slot * kPairSlotBytes + (V ? 0u : (uint32_t)(c16 >> 3) * 8192u);
-        int t[RPT];                                               // row number, or -1
-#pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-          const int rr = (V ? 0 : krow0) + (lw + i * kPairLoaderWarps) * RPI + rsub;   // row of the tile
-          const int listed = V ? __shfl_sync(0xFFFFFFFFu, tv_list[(i * 4) / 32], (i * 4 + rsub) & 31)
-                               : __shfl_sync(0xFFFFFFFFu, tk_list, i * 2 + rsub);
-          t[i] = tr.from_list ? listed : (rr < tr.count ? tr.first + rr : -1);
-        }
-#ifdef QUOKA_DEBUG
-        // debug build: a listed row outside [0, T) is recorded and treated as absent (zero-filled) instead of read
-#pragma unroll
-        for (int i = 0; i < RPT; ++i)
-          if (tr.from_list && (t[i] < -1 || t[i] >= g.T)) { atomicExch(P.status, (int32_t)QUOKA_ERR_BAD_INDEX); t[i] = -1; }
-#endif
-        uint32_t off[RPT];
-        if (P.page_size == 0) {
-#pragma unroll
-          for (int i = 0; i < RPT; ++i) off[i] = base16 + (uint32_t)max(t[i], 0) * st16;
-        } else {
-#pragma unroll
-          for (int i = 0; i < RPT; ++i) {
-            const int tc = max(t[i], 0);
-            int page = __ldg(table + (tc >> 6));
-#ifdef QUOKA_DEBUG
-            // debug build: a page id outside the pool is recorded and the row treated as absent
-            if (t[i] >= 0 && (page < 0 || (long long)page >= P.kv_rows)) {
-              atomicExch(P.status, (int32_t)QUOKA_ERR_BAD_INDEX);
-              t[i] = -1;
-            }
-            if (page < 0 || (long long)page >= P.kv_rows) page = 0;
-#endif
-            off[i] = (uint32_t)page * sb16 + base16 + (uint32_t)(tc & (kPage - 1)) * st16;
+        if (!V) {
+          if (tr.from_list) {
+            if (first_list_tile) list_rows(tr.first, tr.count);
+          } else {
+            k_row = krr < tr.count ? tr.first + krr : -1;
+            v_row[0] = vrr < tr.count ? tr.first + vrr : -1;
+            v_row[1] = vrr + kVStep < tr.count ? tr.first + vrr + kVStep : -1;
           }
+          k_off = row_off(k_row, tr.from_list);
+          v_off[0] = row_off(v_row[0], tr.from_list);
+          v_off[1] = row_off(v_row[1], tr.from_list);
         }
+        const int c16 = V ? vc16 : kc16, rsub = V ? vrsub : krsub;
+        const uint4* src_base = reinterpret_cast<const uint4*>(V ? vc : kc) + (V ? vbase16 : kbase16);
+        const uint32_t dst_item = kv_base + (uint32_t)slot * kPairSlotBytes + (V ? 0u : (uint32_t)(c16 >> 3) * 8192u);
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
-          const int gi = lw + i * kPairLoaderWarps;
-          const int lr = gi * RPI + rsub;                         // row of the item in shared memory
-          if (gi < GROUPS)                                        // false only for the last group of some warps
-            cp_async_16(dst_item + lr * 128 + (((c16 & 7) ^ (lr & 7)) << 4), src_base + off[i], t[i] >= 0);
+          const uint32_t off = V ? __shfl_sync(0xFFFFFFFFu, v_off[i / 8], (i * 4 + rsub) & 31) : __shfl_sync(0xFFFFFFFFu, k_off, i * 2 + rsub);
+          const int lr = (lw + i * kPairLoaderWarps) * RPI + rsub;   // row of the item in shared memory
+          cp_async_16(dst_item + lr * 128 + (((c16 & 7) ^ (lr & 7)) << 4), src_base + (off == kNoRow ? 0u : off), off != kNoRow);
         }
         // this thread's share of the slot is signalled by the copy engine itself when the bytes have landed
         cp_async_mbar_arrive_noinc(&kv_full[slot]);
@@ -299,115 +284,93 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
       if (!item(std::true_type{}, tr, first_list_tile)) break;
     }
     cp_async_wait_all();                                      // nothing of this thread is in flight at exit
-  } else if (lane == 0) {
-    // ================================================================== warp 11, one thread
-    if (!SPLIT) load_q();
-    bool ok = mbar_wait(q_full, 0, wc);
-    if (rank != 0) {
-      // ---------------------------------------------------------------- second CTA: forward "full" to the first
-      if (ok) mbar_arrive_cluster(map_to_cta(smem_u32(peer_q), first));
+  } else if (rank != 0) {
+    // ================================================================== second CTA, one thread of warps 10 and 11: forward
+    // the "full" of the V (10) and K (11) slots to the first CTA
+    if (lane == 0) {
+      bool ok = true;
+      if (warp == kQkWarp) {
+        if (!SPLIT) load_q();
+        ok = mbar_wait(q_full, 0, wc);
+        if (ok) mbar_arrive_cluster(map_to_cta(smem_u32(peer_q), first));
+      }
       const uint32_t peer_full0 = map_to_cta(smem_u32(peer_full), first);
-      int slot = 0;
-      uint32_t phase = 0;
-      for (int tile = t_lo; ok; ++tile) {
+      RingCursor<kPairSlots> r(warp == kQkWarp ? 0 : 1);
+      for (int tile = t_lo; ok; ++tile, r.advance()) {
         if (tile == g.n_known) {
           if (g.resolved) break;
           resolve(g, k_cnt, s);
-          grid_launch_dependents();
+          if (warp == kQkWarp) grid_launch_dependents();
           if (tile == g.n_known) break;
         }
-#pragma unroll 1
-        for (int kvi = 0; kvi < 2; ++kvi) {
-          if (!mbar_wait(&kv_full[slot], phase, wc)) { ok = false; break; }
-          fence_proxy_async_all();            // the loaders' cp.async wrote through the generic proxy
-          mbar_arrive_cluster(peer_full0 + (uint32_t)slot * 8u);
-          if (++slot == kPairSlots) { slot = 0; phase ^= 1; }
-        }
+        ok = mbar_wait(&kv_full[r.slot], r.phase, wc);
+        if (!ok) break;
+        fence_proxy_async_smem();             // the loaders' cp.async wrote through the generic proxy
+        mbar_arrive_cluster(peer_full0 + (uint32_t)r.slot * 8u);
       }
-    } else {
-      // ---------------------------------------------------------------- first CTA: MMA issuer for the pair
+    }
+  } else {
+    // ================================================================== first CTA, warps 10 and 11: issue the pair's products
+    if (!SPLIT && warp == kQkWarp && lane == 0) load_q();
+    __syncwarp();
+    const bool leader = elect_one();
+    const uint32_t tmem = (uint32_t)warp_uniform((int)tmem_base);
+    t_lo = warp_uniform(t_lo);
+    uniform_geom(g);
+    // Descriptors are built once; a tile, slot or k-step offset is an addition to the 16-byte-unit address field.
+    const uint64_t desc_kv = smem_desc_sw128(smem_u32(kv_smem), 16, 1024);
+    const auto acquire = [&](int sl, uint32_t phase) {
+      if (!warp_all(mbar_wait(&kv_full[sl], phase, wc) && mbar_wait(&peer_full[sl], phase, wc))) return false;
+      fence_proxy_async_smem();               // cp.async wrote through the generic proxy, the MMA reads through the async one
+      tc_fence_after();
+      return true;
+    };
+    const auto release = [&](int sl) { if (leader) mma_pair_commit(both, &kv_empty[sl]); };
+    if (warp == kQkWarp) {
       const uint32_t idesc_qk = idesc_bf16_f32(256, kKeyTile, false, false);
+      const uint64_t desc_q = smem_desc_sw128(smem_u32(q_smem), 16, 1024);
+      if (warp_all(mbar_wait(q_full, 0, wc) && mbar_wait(peer_q, 0, wc)))
+        attn_issue_qk<1, kPairSlots>(
+            g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); grid_launch_dependents(); }, acquire,
+            [&](unsigned, uint32_t parity) {
+              if (!warp_all(mbar_wait(s_free, parity, wc))) return false;
+              tc_fence_after();
+              return true;
+            },
+            [&](int x, unsigned, int ks) {
+              const uint64_t da = desc_q + (uint64_t)(x * (kPairQTileBytes >> 4));
+              const uint64_t db = desc_kv + (uint64_t)((uint32_t)ks * (kPairSlotBytes >> 4));
+#pragma unroll
+              for (int hh = 0; hh < 2; ++hh)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                  const uint64_t offa = (uint64_t)((hh * 16384 + kk * 32) >> 4);   // Q: halves of 128 rows
+                  const uint64_t offb = (uint64_t)((hh * 8192 + kk * 32) >> 4);    // K: halves of 64 rows
+                  if (leader) mma_pair_ss(tmem + S_COL, da + offa, db + offb, idesc_qk, (hh | kk) ? 1u : 0u);
+                }
+              if (leader) mma_pair_commit(both, &s_full[x]);
+            },
+            release);
+    } else {
       const uint32_t idesc_pv = idesc_bf16_f32(256, D, false, true);
-      const uint32_t q_base = smem_u32(q_smem), kv_base = smem_u32(kv_smem);
-      int slot = 0;
-      uint32_t kv_phase = 0;
-      uint32_t p_phase[2] = {0, 0};
-      int k_slot = -1, v_slot = -1;
-      if (ok) ok = mbar_wait(peer_q, 0, wc);
-      auto acquire = [&]() -> int {           // next ring item (K or V) is readable in both CTAs
-        if (!mbar_wait(&kv_full[slot], kv_phase, wc) || !mbar_wait(&peer_full[slot], kv_phase, wc)) {
-          ok = false;
-          return 0;
-        }
-        fence_proxy_async_smem();             // cp.async wrote through the generic proxy, the MMA reads through the async one
-        tc_fence_after();
-        const int got = slot;
-        if (++slot == kPairSlots) { slot = 0; kv_phase ^= 1; }
-        return got;
-      };
-      // Descriptors are built once; a tile, slot or k-step offset is an addition to the 16-byte-unit address field.
-      const uint64_t desc_q = smem_desc_sw128(q_base, 16, 1024);
-      const uint64_t desc_kv = smem_desc_sw128(kv_base, 16, 1024);
-      auto issue_qk = [&](int x, int ks) {
-        const uint64_t da = desc_q + (uint64_t)(x * (kPairQTileBytes >> 4));
-        const uint64_t db = desc_kv + (uint64_t)((uint32_t)ks * (kPairSlotBytes >> 4));
+      uint32_t p_phase = 0;
+      attn_issue_pv<1, kPairSlots>(
+          g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); }, acquire,
+          [&](int x, int half, unsigned, int vs, bool add) {
+            if (!warp_all(mbar_wait(&p_full[2 * x + half], (p_phase >> x) & 1u, wc))) return false;
+            tc_fence_after();
+            const uint64_t dv = desc_kv + (uint64_t)((uint32_t)vs * (kPairSlotBytes >> 4) + half * 4 * (2048 >> 4));
+            const uint32_t pa = tmem + P_COL + x * 64 + half * 32, oa = tmem + O_COL + x * D;
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh)
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t offa = (uint64_t)((hh * 16384 + kk * 32) >> 4);   // Q: halves of 128 rows
-            const uint64_t offb = (uint64_t)((hh * 8192 + kk * 32) >> 4);    // K: halves of 64 rows
-            mma_pair_ss(tmem_base + S_COL[x], da + offa, db + offb, idesc_qk, (hh | kk) ? 1u : 0u);
-          }
-        mma_pair_commit(both, &s_full[x]);
-      };
-      auto issue_pv = [&](int x, int vs, bool first) {
-        const uint64_t dv = desc_kv + (uint64_t)((uint32_t)vs * (kPairSlotBytes >> 4));
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          if (!mbar_wait(&p_full[2 * x + half], p_phase[x], wc)) { ok = false; return; }
-          tc_fence_after();
-#pragma unroll
-          for (int kk = half * 4; kk < half * 4 + 4; ++kk) {   // 16 keys per MMA: 8 packed columns of P, 16 rows of V
-            mma_pair_ts(tmem_base + O_COL[x], tmem_base + S_COL[x] + kk * 8, dv + (uint64_t)(kk * (2048 >> 4)), idesc_pv,
-                        (!first || kk) ? 1u : 0u);
-          }
-        }
-        p_phase[x] ^= 1;
-      };
-      // Tile t: O += P_t V_t for each Q tile taking part (as the two halves of P arrive), then S = Q K_{t+1}^T.
-      // K_{t+1} and V_t are both acquired before the P waits, so those never sit on the P -> PV -> QK chain.
-      const auto part = [&](int x, int t) { return x ? g.active_b : t >= g.skip_a; };
-      if (ok && t_lo < g.n_known) {
-        k_slot = acquire();
-        if (ok) {
-          if (part(0, t_lo)) issue_qk(0, k_slot);
-          if (part(1, t_lo)) issue_qk(1, k_slot);
-          mma_pair_commit(both, &kv_empty[k_slot]);
-        }
-        for (int t = t_lo; ok; ++t) {
-          if (t + 1 == g.n_known && !g.resolved) { resolve(g, k_cnt, s); grid_launch_dependents(); }
-          const bool more = t + 1 < g.n_known;
-          v_slot = acquire();
-          if (ok && more) k_slot = acquire();
-          if (!ok) break;
-          if (part(0, t)) {
-            issue_pv(0, v_slot, t == max(g.skip_a, t_lo));
-            if (!ok) break;
-            if (!more) mma_pair_commit(both, &o_full[0]);
-          }
-          if (more && part(0, t + 1)) issue_qk(0, k_slot);
-          if (part(1, t)) {
-            issue_pv(1, v_slot, t == t_lo);
-            if (!ok) break;
-            if (!more) mma_pair_commit(both, &o_full[1]);
-          }
-          mma_pair_commit(both, &kv_empty[v_slot]);
-          if (!more) break;
-          if (part(1, t + 1)) issue_qk(1, k_slot);
-          mma_pair_commit(both, &kv_empty[k_slot]);
-        }
-      }
+            for (int kk = 0; kk < 4; ++kk)             // 16 keys per MMA: 8 packed columns of P, 16 rows of V
+              if (leader) mma_pair_ts(oa, pa + kk * 8, dv + (uint64_t)(kk * (2048 >> 4)), idesc_pv, add || kk ? 1u : 0u);
+            if (half) {
+              if (leader) mma_pair_commit(both, &p_done[x]);
+              p_phase ^= 1u << x;
+            }
+            return true;
+          },
+          release, [&](int x) { if (leader) mma_pair_commit(both, &o_full[x]); });
     }
   }
   if (SPLIT && attn_last_cta()) grid_dependency_wait();       // this grid's end is the whole row blocks' end too
@@ -417,7 +380,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     if (warp < 8) attn_merge_cluster<D>(P, smem, part_ml, warp, lane, 2, (int)rank, n_parts, blockIdx.y % n_parts, r0, s, h, out, lse);
   }
   cluster_sync_all();                                         // the other CTA's MMAs no longer read this CTA
-  if (warp == kMmaWarp) tmem_dealloc_pair(tmem_base, 512);
+  if (warp == kQkWarp) tmem_dealloc_pair(tmem_base, 512);
 }
 
 #define QUOKA_PAIR_PARAMS                                                                                               \

@@ -10,11 +10,10 @@ namespace quoka {
 using namespace ptx;
 
 constexpr int kAttnThreads = 12 * 32;
-constexpr int kLoaderWarps = 3;
-constexpr int kMmaWarp = 11;
+constexpr int kLoaderWarps = 2;
+constexpr int kPvWarp = 10, kQkWarp = 11;
 constexpr int kQTile = 128;
 constexpr int kKeyTile = 128;
-constexpr int kSlots = 5;
 // The reference point m of the exponentials 2^(s - m) is raised, and O and l rescaled, only when a row's maximum
 // exceeds it by more than this many powers of two.  Until then P, l and O are simply larger by a common factor of at
 // most 2^32, which floating point carries without loss (bf16 and fp32 both reach 2^127; l <= 2^32 * keys and
@@ -110,6 +109,14 @@ __device__ __forceinline__ void resolve(AttnGeom& g, const int32_t* k_cnt, int s
   g.resolved = true;
 }
 
+// For the warps that issue the products: their loops' bounds in a form the compiler knows to be the same in every lane.
+__device__ __forceinline__ void uniform_geom(AttnGeom& g) {
+  g.skip_a = warp_uniform(g.skip_a);
+  g.active_b = warp_all(g.active_b);
+  g.n_known = warp_uniform(g.n_known);
+  g.resolved = warp_all(g.resolved);
+}
+
 // The same where the selection is known to be complete.
 __device__ __forceinline__ void learn_count(AttnGeom& g, const int32_t* k_cnt, int s) {
   g.cnt = __ldcg(k_cnt + s);
@@ -161,17 +168,53 @@ __device__ __forceinline__ TileRows tile_rows(const AttnGeom& g, int t) {
   return r;
 }
 
-// Number of visible columns of tile t for chunk row `row` (columns [0, lim) are visible).
-__device__ __forceinline__ int visible_cols(const TileRows& tr, int row) {
-  const int lim = tr.causal ? row - tr.col0 + 1 : tr.count;
-  return max(0, min(kKeyTile, lim));
+// Offset of cache row t of a (sequence, head) in 16-byte units, kNoRow for t < 0 (`listed`: an entry of the selected list).
+constexpr uint32_t kNoRow = 0xFFFFFFFFu;
+__device__ __forceinline__ uint32_t kv_row_off16(const DevParams& P, const int32_t* table, uint32_t st16, uint32_t sb16, int t,
+                                                 bool listed, int T) {
+#ifdef QUOKA_DEBUG
+  // debug build: a listed row outside [0, T) is recorded and treated as absent (zero-filled) instead of read
+  if (listed && (t < -1 || t >= T)) { atomicExch(P.status, (int32_t)QUOKA_ERR_BAD_INDEX); t = -1; }
+#endif
+  const int tc = max(t, 0);
+  uint32_t off = (uint32_t)tc * st16;
+  if (P.page_size != 0) {
+    int page = __ldg(table + (tc >> 6));
+#ifdef QUOKA_DEBUG
+    // debug build: a page id outside the pool is recorded and the row treated as absent
+    if (page < 0 || (long long)page >= P.kv_rows) {
+      if (t >= 0) atomicExch(P.status, (int32_t)QUOKA_ERR_BAD_INDEX);
+      t = -1;
+      page = 0;
+    }
+#endif
+    off = (uint32_t)page * sb16 + (uint32_t)(tc & (kPage - 1)) * st16;
+  }
+  return t < 0 ? kNoRow : off;
 }
 
-// Maximum of 32 score columns starting at col0; columns at and beyond `lim` are masked out.
-__device__ __forceinline__ float max32(uint32_t (&v)[32], bool masked, int col0, int lim) {
+// Number of visible columns of tile t for chunk row `row` (columns [0, lim) are visible; may lie outside [0, 128]).
+// A softmax thread keeps it up from tile to tile: it changes by one tile's columns except where the chunk's own rows or
+// the selected list begin.
+template <bool SPARSE>
+struct VisibleCols {
+  int lim;
+  __device__ __forceinline__ VisibleCols(const AttnGeom& g, int t, int row) {
+    const TileRows tr = tile_rows<SPARSE>(g, t);
+    lim = tr.causal ? row - tr.col0 + 1 : tr.count;
+  }
+  __device__ __forceinline__ void at(const AttnGeom& g, int t, int row) {
+    if (SPARSE && t == g.b_first) lim = row + 1;
+    if (SPARSE && t == g.n_chunk) lim = g.cnt;
+  }
+  __device__ __forceinline__ void advance() { lim += SPARSE ? -kKeyTile : kKeyTile; }
+};
+
+// Maximum of 32 score columns starting at col0; columns at and beyond `lim` are masked out (-inf: exp2 gives exactly 0).
+__device__ __forceinline__ float max32(uint32_t* v, bool masked, int col0, int lim) {
   if (masked) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) if (col0 + i >= lim) v[i] = 0xFF800000u;    // -inf
+    for (int i = 0; i < 32; ++i) if (col0 + i >= lim) v[i] = 0xFF800000u;
   }
   float m0 = __uint_as_float(v[0]), m1 = __uint_as_float(v[1]);
 #pragma unroll
@@ -183,41 +226,48 @@ __device__ __forceinline__ float max32(uint32_t (&v)[32], bool masked, int col0,
 }
 
 // ---------------------------------------------------------------------------------------------- softmax of one tile
-// One thread = one query row of a 128-row Q tile against one 128-key tile: S is read from tensor memory at s_addr,
-// bf16 P written back over its first 64 columns, the running reference point m_run (log2 units) and sum l_run kept
-// up, the accumulator at o_addr rescaled when the reference point moves.  `lim` = visible columns of this row,
-// `masked` = some row of the warp sees fewer than all; `announce(half)` (lane 0) tells the MMA issuer that a half of
-// P is in place.  first_tile: nothing has been accumulated yet.
-template <int D, typename Announce>
-__device__ __forceinline__ void attn_softmax_tile(uint32_t s_addr, uint32_t o_addr, int lim, bool masked, float scale_log2,
-                                                  bool first_tile, int lane, float& m_run, float& l_run,
-                                                  Announce&& announce) {
-  // ---- pass 1: the row maximum.  All four 32-column loads are issued together (one tensor-memory round
-  // trip).  The first 96 scores stay in registers for pass 2, the last 32 are read once more there (under the
-  // third block's exponentials): all 128 alive next to a block of exponentials in flight do not fit the 168
-  // registers, and 96 fit only because P is stored 16 columns at a time and the rare rescale below works in
-  // 8-column pieces.
+// One thread = one query row of a 128-row Q tile against one 128-key tile: S is read from tensor memory at s_addr, bf16 P
+// written at p_addr, 16 columns at a time, the running reference point m_run (log2 units) and sum l_run kept up, the
+// accumulator at o_addr rescaled when the reference point moves.  `lim` = visible columns of this row, `masked` = some row
+// of the warp sees fewer than all; first_tile: nothing has been accumulated yet; announce(half) (lane 0): a half of P is in
+// place; o_idle: no product into O is on its way.  False when a wait gave up.
+// APART: P has columns of its own.  All of S is read at once and `s_read` (lane 0) tells so, for the next tile's QK^T to go
+// into its columns while the exponentials run; `p_free` waits for the products of the tile before, which read P (as a rule
+// they are done; one wait, ahead of the exponentials, which the compiler would not interleave across it).
+// Otherwise P goes over the first 64 columns of S and the last 32 scores are read once more, under the third block's
+// exponentials: 128 scores and a block of exponentials in flight are a few registers more than the 168.
+template <int D, bool APART, typename SRead, typename PFree, typename OIdle, typename Announce>
+__device__ __forceinline__ bool attn_softmax_tile(uint32_t s_addr, uint32_t p_addr, uint32_t o_addr, int lim, bool masked,
+                                                  float scale_log2, bool first_tile, int lane, float& m_run, float& l_run,
+                                                  SRead&& s_read, PFree&& p_free, OIdle&& o_idle, Announce&& announce) {
+  // ---- pass 1: the row maximum; all four 32-column loads are issued together (one tensor-memory round trip)
+  constexpr int kHeld = APART ? 128 : 96;
+  uint32_t v0[kHeld];
   float mx;
-  uint32_t v0[96];                                         // the first 96 scores stay in registers for pass 2
   {
-    uint32_t c3[32];
+    uint32_t c3[APART ? 1 : 32];
+    uint32_t* last = APART ? v0 + (kHeld - 32) : c3;
     tmem_ld32(s_addr, v0);
     tmem_ld32(s_addr + 32, v0 + 32);
     tmem_ld32(s_addr + 64, v0 + 64);
-    tmem_ld32(s_addr + 96, c3);
+    tmem_ld32(s_addr + 96, last);
     tmem_wait_ld();
-    uint32_t (&a0)[32] = *reinterpret_cast<uint32_t (*)[32]>(v0);
-    uint32_t (&a1)[32] = *reinterpret_cast<uint32_t (*)[32]>(v0 + 32);
-    uint32_t (&a2)[32] = *reinterpret_cast<uint32_t (*)[32]>(v0 + 64);
-    mx = fmaxf(fmaxf(max32(a0, masked, 0, lim), max32(a1, masked, 32, lim)),
-               fmaxf(max32(a2, masked, 64, lim), max32(c3, masked, 96, lim)));
+    if (APART) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) s_read();
+    }
+    mx = fmaxf(fmaxf(max32(v0, masked, 0, lim), max32(v0 + 32, masked, 32, lim)),
+               fmaxf(max32(v0 + 64, masked, 64, lim), max32(last, masked, 96, lim)));
   }
   const float m_tile = mx * scale_log2;
   // ---- lazy rescale of the accumulator: only when some row's maximum grew by more than the threshold
   const bool grow = m_tile > m_run + kRescaleThreshold;
+  if (!p_free()) return false;
   if (__any_sync(0xFFFFFFFFu, grow)) {
     const float m_new = fmaxf(m_run, m_tile);
     if (!first_tile) {
+      if (!o_idle()) return false;
       const float alpha = (m_run == -INFINITY) ? 0.f : ex2(m_run - m_new);
       l_run *= alpha;
 #pragma unroll 1
@@ -234,34 +284,33 @@ __device__ __forceinline__ void attn_softmax_tile(uint32_t s_addr, uint32_t o_ad
     m_run = m_new;
   }
   const float m_use = (m_run == -INFINITY) ? 0.f : m_run;
-  // ---- pass 2: p = 2^(s*scale - m) in four blocks of 32 keys.  bf16 P goes over the first 64 columns of S
-  // (block b of P lands on columns 16b..16b+15, all of them read already) and each half of the tile is handed to
-  // the MMA issuer as soon as it is stored, so the first PV products run under the second half's arithmetic.
+  // ---- pass 2: p = 2^(s*scale - m) in four blocks of 32 keys, each half of the tile handed to the issuing warp as soon as
+  // it is stored, so the first PV products run under the second half's arithmetic.
   const uint64_t sc2 = pack2(scale_log2, scale_log2), nm2 = pack2(-m_use, -m_use);
   uint64_t psa[2] = {0ull, 0ull};                           // four running sums as two packed pairs
-  uint32_t vb[32];
+  uint32_t vb[APART ? 1 : 32];
 #pragma unroll
   for (int blk = 0; blk < 4; ++blk) {
-    if (blk == 2) tmem_ld32(s_addr + 96, vb);              // under the third block's exponentials
-    if (blk == 3) {
+    if (!APART && blk == 2) tmem_ld32(s_addr + 96, vb);
+    if (!APART && blk == 3) {
       tmem_wait_ld();
       if (masked) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) if (96 + i >= lim) vb[i] = 0xFF800000u;   // -inf: exp2 gives exactly 0
+        for (int i = 0; i < 32; ++i) if (96 + i >= lim) vb[i] = 0xFF800000u;
       }
     }
     uint32_t pk[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      const uint32_t e0 = blk < 3 ? v0[blk * 32 + 2 * i] : vb[2 * i], e1 = blk < 3 ? v0[blk * 32 + 2 * i + 1] : vb[2 * i + 1];
+      const uint32_t* v = APART || blk < 3 ? v0 + blk * 32 : vb;
       float x0, x1;
-      unpack2(fma2(pack2u(e0, e1), sc2, nm2), x0, x1);
+      unpack2(fma2(pack2u(v[2 * i], v[2 * i + 1]), sc2, nm2), x0, x1);
       const float p0 = ex2(x0), p1 = ex2(x1);
       psa[i & 1] = add2(psa[i & 1], pack2(p0, p1));
       const __nv_bfloat162 b2 = __floats2bfloat162_rn(p0, p1);
       pk[i] = *reinterpret_cast<const uint32_t*>(&b2);
     }
-    tmem_st16(s_addr + blk * 16, pk);
+    tmem_st16(p_addr + blk * 16, pk);
     if (blk & 1) {
       tmem_wait_st();
       tc_fence_before();
@@ -273,6 +322,82 @@ __device__ __forceinline__ void attn_softmax_tile(uint32_t s_addr, uint32_t o_ad
   unpack2(psa[0], ps0, ps1);
   unpack2(psa[1], ps2, ps3);
   l_run += (ps0 + ps1) + (ps2 + ps3);
+  return true;
+}
+
+// ---------------------------------------------------------------------------------------------- order of the products
+// Two warps issue the products, each in order: one every S = Q K^T, one every O += P V.  An item is one Q tile against one
+// key tile; items run A0 B0 A1 B1 ... (a Q tile that does not take part in a key tile has no item there).  S has NBUF
+// tensor-memory buffers, used in turn; the QK^T of item i + NBUF waits until item i's is free, and nothing else orders it
+// against PV.
+//   head_dim 128: O takes 256 of the 512 columns, one S and two P (one per Q tile) the rest: S is free when item i's scores
+//     have been READ, the next QK^T then runs under item i's exponentials.
+//   head_dim 64: O takes 128 columns, three S the rest, P in place: free when item i's weights have been multiplied, which
+//     is an item and a half before its next scores are wanted.
+// So a softmax warp finds its next scores ready, or nearly, when it is done with a tile.  Two warps because a wait on a
+// barrier that is complete already costs 75 to 100 cycles and there are five to a pair of products, which take 1024: one
+// warp for both left the tensor core idle for 45 % of a step (3650 cycles at head_dim 128).  Products of two warps
+// interleave without loss (2050 cycles for 32, alone).
+// The ring holds K0 V0 K1 V1 ...; a slot is released as its last product is issued.
+template <int SLOTS>
+struct RingCursor {                                         // every second item of the ring
+  int slot;
+  uint32_t phase = 0;
+  __device__ __forceinline__ explicit RingCursor(int first) : slot(first) {}
+  __device__ __forceinline__ void advance() {
+    slot += 2;
+    if (slot >= SLOTS) { slot -= SLOTS; phase ^= 1; }
+  }
+};
+
+// acquire(slot, phase): the slot's K rows are readable; s_free(buf, parity): S buffer `buf` is free again (both false
+// when a wait gave up); qk(x, buf, slot): the products and their commit; release(slot): commit of the slot.
+template <int NBUF, int SLOTS, typename Resolve, typename Acquire, typename SFree, typename Qk, typename Release>
+__device__ __forceinline__ void attn_issue_qk(AttnGeom& g, int t_lo, Resolve&& resolve_list, Acquire&& acquire, SFree&& s_free,
+                                              Qk&& qk, Release&& release) {
+  RingCursor<SLOTS> k(0);
+  unsigned item = 0;
+#pragma unroll 1
+  for (int t = t_lo;; ++t, k.advance()) {
+    if (t == g.n_known && !g.resolved) resolve_list();
+    if (t >= g.n_known) return;
+    if (!acquire(k.slot, k.phase)) return;
+#pragma unroll 1
+    for (int x = t >= g.skip_a ? 0 : 1; x < (g.active_b ? 2 : 1); ++x, ++item) {
+      const unsigned buf = item % NBUF;
+      if (item >= NBUF && !s_free(buf, (item / NBUF + 1) & 1)) return;
+      qk(x, buf, k.slot);
+    }
+    release(k.slot);
+  }
+}
+
+// acquire(slot, phase): the slot's V rows are readable; pv(x, half, buf, slot, add): waits for that half of P, products, commit;
+// final(x): commit of the finished O.
+template <int NBUF, int SLOTS, typename Resolve, typename Acquire, typename Pv, typename Release, typename Final>
+__device__ __forceinline__ void attn_issue_pv(AttnGeom& g, int t_lo, Resolve&& resolve_list, Acquire&& acquire, Pv&& pv,
+                                              Release&& release, Final&& final) {
+  RingCursor<SLOTS> v(1);
+  const int first_a = max(g.skip_a, t_lo);
+  unsigned item = 0;
+#pragma unroll 1
+  for (int t = t_lo;; ++t, v.advance()) {
+    if (t == g.n_known && !g.resolved) resolve_list();
+    if (t >= g.n_known) break;
+    if (!acquire(v.slot, v.phase)) return;
+#pragma unroll 1
+    for (int x = t >= g.skip_a ? 0 : 1; x < (g.active_b ? 2 : 1); ++x, ++item) {
+      const unsigned buf = item % NBUF;
+      if (!pv(x, 0, buf, v.slot, t != (x ? t_lo : first_a)) || !pv(x, 1, buf, v.slot, true)) return;
+      if (g.resolved && t == g.n_known - 1) final(x);
+    }
+    release(v.slot);
+    if (!g.resolved && t == g.n_known - 1) {                // (an empty list: the chunk's last tile was the last)
+      resolve_list();
+      if (t == g.n_known - 1)
+        for (int x = t >= g.skip_a ? 0 : 1; x < (g.active_b ? 2 : 1); ++x) final(x);
+    }
+  }
 }
 
 // Epilogue of a softmax thread: its row of O from tensor memory, divided by l, to global memory as bf16 (and the

@@ -37,6 +37,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Every wait in the kernels goes through here.  It gives up after about a second (or as soon as
 // another thread of the CTA has given up), records QUOKA_ERR_TIMEOUT in the device status word and
 // returns false; the caller then leaves its loop and runs the normal teardown.
@@ -61,6 +73,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
     }
   }
   return true;
+}
+
+// The same where the barrier is expected to be complete: a plain test first (about 30 cycles where try_wait takes 75).
+__device__ __forceinline__ bool mbar_wait_done(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
+  return mbar_test_wait(bar, parity) || mbar_wait(bar, parity, w);
 }
 
 // ---------------------------------------------------------------------------------- CTA pairs (clusters of two)
@@ -299,6 +316,20 @@ template <int N> __device__ __forceinline__ void setmaxnreg_dec() { asm volatile
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// ---------------------------------------------------------------------------------- warp-uniform control
+// One lane of the (converged) warp.  MMAs are issued under this predicate by a warp that runs its whole loop converged, not by
+// a lane in a branch of its own: only then does the compiler keep descriptors and addresses in uniform registers, which is
+// where the instruction wants them.  In a divergent branch an MMA takes 51 to 57 cycles to issue (products alone, head_dim
+// 64: 1368 cycles per step of 24 MMAs, 1049 by a converged warp, which is the tensor core's time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e != 0;
+}
+// The same value in every lane, in a form the compiler knows to be so.
+__device__ __forceinline__ int warp_uniform(int v) { return (int)__reduce_or_sync(0xFFFFFFFFu, (unsigned)v); }
+__device__ __forceinline__ bool warp_all(bool v) { return __all_sync(0xFFFFFFFFu, v) != 0; }
 
 // ---------------------------------------------------------------------------------- packed fp32, max3
 // Packed pairs of fp32 (one instruction for two lanes of arithmetic) and the three-input maximum: the

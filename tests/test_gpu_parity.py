@@ -706,6 +706,36 @@ def test_decode_scoring_units(T, d, dtype, group, cached_norms, paged):
     assert torch.equal(gp.out, want_out) and torch.equal(gp.k_idx, want_idx)
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_q,n_kv,d,C,T,B,paged", [
+    (32, 4, 64, 777, 6000, 1500, False),    # P in place, three S buffers; the last row block has one Q tile, of nine rows
+    (32, 4, 64, 384, 3000, 2999, True),     # and of 128
+    (32, 8, 128, 633, 6000, 1500, True),    # pairs: one S buffer, P apart
+    (32, 32, 128, 640, 2500, 700, False),   # the same in the one-CTA kernel
+])
+def test_q_tiles_that_walk_many_key_tiles(n_q, n_kv, d, C, T, B, paged):
+    """Row blocks of two Q tiles and of one over dozens of key tiles: the buffers of scores and weights go round many times.
+    Sparse (staged, and the fused call five times with the same bits) and dense, against the oracle."""
+    gp = problem(2000 + C, n_q=n_q, n_kv=n_kv, d=d, T=T, C=C, n_retain=32, kv_budget=B, paged=paged)
+    gp.run_staged()
+    check_chain(gp, attn_rows=200)
+    staged = gp.out.clone()
+    for _ in range(5):
+        gp.out.zero_()
+        api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+        torch.cuda.synchronize()
+        assert torch.equal(gp.out, staged)
+    q, k, v, _ = gp.oracle_inputs(0)
+    heads, rows = stratified_rows(n_q, C, 200, 5)
+    want = O.sparse_attention_rows(q, k, v, T, [np.arange(T)] * n_kv, heads, rows)
+    for _ in range(2):
+        gp.out.zero_()
+        api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, gp.lse, gp.ws)
+        torch.cuda.synchronize()
+        check_attention(f64(gp.out[0])[heads, rows], want, "bf16")
+    assert api.quoka_last_device_status(gp.ws) == 0
+
+
 @pytest.mark.parametrize("n_q,n_kv,d,C,T,B", [
     (32, 8, 128, 1300, 9000, 5000),     # pairs, 6 row blocks: the lightest in parts after the whole ones, ragged last block
     (24, 8, 64, 1800, 7000, 6000),      # one-CTA kernel, 8 row blocks
