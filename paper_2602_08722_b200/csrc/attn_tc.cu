@@ -276,7 +276,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     uniform_geom(g);
     const uint32_t kv_base = smem_u32(kv_smem);
     const auto acquire = [&](int sl, uint32_t phase) {
-      if (!warp_all(mbar_wait(&kv_full[sl], phase, wc))) return false;
+      if (!warp_all(mbar_poll(&kv_full[sl], phase, wc))) return false;
       fence_proxy_async_smem();               // cp.async wrote through the generic proxy, the MMA reads through the async one
       tc_fence_after();
       return true;
@@ -289,11 +289,11 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
       const uint32_t idesc_qk = idesc_bf16_f32(128, kKeyTile, false, false);
       const uint64_t desc_q = smem_desc_sw128(smem_u32(q_smem), 16, 1024);
       const uint64_t desc_k = smem_desc_sw128(kv_base, 16, 1024);            // K-major rows (K tiles)
-      if (warp_all(mbar_wait(q_full, 0, wc)))
+      if (warp_all(mbar_poll(q_full, 0, wc)))
         attn_issue_qk<NBUF, kSlots>(
             g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); grid_launch_dependents(); }, acquire,
             [&](unsigned buf, uint32_t parity) {
-              if (!warp_all(mbar_wait(APART ? s_free : &p_done[buf], parity, wc))) return false;
+              if (!warp_all(mbar_poll(APART ? s_free : &p_done[buf], parity, wc))) return false;
               tc_fence_after();
               return true;
             },
@@ -318,7 +318,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
           g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); }, acquire,
           [&](int x, int half, unsigned buf, int vs, bool add) {
             const unsigned n = APART ? x : buf;
-            if (!warp_all(mbar_wait(&p_full[2 * n + half], (p_phase >> n) & 1u, wc))) return false;
+            if (!warp_all(mbar_poll(&p_full[2 * n + half], (p_phase >> n) & 1u, wc))) return false;
             tc_fence_after();
             const uint64_t dv = desc_v + (uint64_t)((uint32_t)vs * (kTileBytes >> 4) + half * 4 * (2048 >> 4));
             const uint32_t pa = tmem + (APART ? P_COL + x * 64 : buf * 128) + half * 32, oa = tmem + O_COL + x * D;

@@ -320,7 +320,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     // Descriptors are built once; a tile, slot or k-step offset is an addition to the 16-byte-unit address field.
     const uint64_t desc_kv = smem_desc_sw128(smem_u32(kv_smem), 16, 1024);
     const auto acquire = [&](int sl, uint32_t phase) {
-      if (!warp_all(mbar_wait(&kv_full[sl], phase, wc) && mbar_wait(&peer_full[sl], phase, wc))) return false;
+      if (!warp_all(mbar_poll(&kv_full[sl], phase, wc) && mbar_poll(&peer_full[sl], phase, wc))) return false;
       fence_proxy_async_smem();               // cp.async wrote through the generic proxy, the MMA reads through the async one
       tc_fence_after();
       return true;
@@ -329,11 +329,11 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     if (warp == kQkWarp) {
       const uint32_t idesc_qk = idesc_bf16_f32(256, kKeyTile, false, false);
       const uint64_t desc_q = smem_desc_sw128(smem_u32(q_smem), 16, 1024);
-      if (warp_all(mbar_wait(q_full, 0, wc) && mbar_wait(peer_q, 0, wc)))
+      if (warp_all(mbar_poll(q_full, 0, wc) && mbar_poll(peer_q, 0, wc)))
         attn_issue_qk<1, kPairSlots>(
             g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); grid_launch_dependents(); }, acquire,
             [&](unsigned, uint32_t parity) {
-              if (!warp_all(mbar_wait(s_free, parity, wc))) return false;
+              if (!warp_all(mbar_poll(s_free, parity, wc))) return false;
               tc_fence_after();
               return true;
             },
@@ -357,7 +357,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
       attn_issue_pv<1, kPairSlots>(
           g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); }, acquire,
           [&](int x, int half, unsigned, int vs, bool add) {
-            if (!warp_all(mbar_wait(&p_full[2 * x + half], (p_phase >> x) & 1u, wc))) return false;
+            if (!warp_all(mbar_poll(&p_full[2 * x + half], (p_phase >> x) & 1u, wc))) return false;
             tc_fence_after();
             const uint64_t dv = desc_kv + (uint64_t)((uint32_t)vs * (kPairSlotBytes >> 4) + half * 4 * (2048 >> 4));
             const uint32_t pa = tmem + P_COL + x * 64 + half * 32, oa = tmem + O_COL + x * D;

@@ -80,6 +80,24 @@ __device__ __forceinline__ bool mbar_wait_done(uint64_t* bar, uint32_t parity, c
   return mbar_test_wait(bar, parity) || mbar_wait(bar, parity, w);
 }
 
+// The same by polling, for the two warps that issue products: try_wait suspends the thread, and waking up takes a few hundred
+// cycles of the time between a barrier's completion and the products that it lets go.
+__device__ __forceinline__ bool mbar_poll(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
+  if (mbar_test_wait(bar, parity)) return true;
+  const long long t0 = clock64();
+  uint32_t it = 0;
+  while (!mbar_test_wait(bar, parity)) {
+    if ((++it & 255u) == 0) {
+      if (*w.abort_flag || clock64() - t0 > w.limit) {
+        *w.abort_flag = 1;
+        atomicExch(w.status, (int32_t)QUOKA_ERR_TIMEOUT);
+        return false;
+      }
+    }
+  }
+  return true;
+}
+
 // ---------------------------------------------------------------------------------- CTA pairs (clusters of two)
 __device__ __forceinline__ uint32_t cluster_cta_rank() {
   uint32_t r;
