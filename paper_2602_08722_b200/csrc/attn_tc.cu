@@ -3,8 +3,9 @@
 // or, without an index list, over every cached row (Eq. 2, dense chunk attention).  bf16 in, fp32
 // softmax and accumulation, P rounded to bf16 for the PV product.
 //
-// One CTA owns 256 consecutive chunk rows of one query head as two 128-row Q tiles (A, B) and walks
-// the key tiles (128 keys) once for both.  Roles:
+// This file: the kernel for head_dim 64, and the plan and the launches of both (attn_tc_pair.cu has the one for head_dim
+// 128).  A CTA owns two Q tiles (A, B) of 128 rows, or one, chunk positions of all heads of a KV group, and walks the key
+// tiles (128 keys) once for both.  Roles:
 //   warps 0-3 / 4-7  softmax of Q tile A / B: one thread per query row, S read from tensor memory,
 //                    running max / sum in registers, P written back to tensor memory, lazy rescale of
 //                    the O accumulator (only when the max grew by more than 2^32), final
@@ -26,48 +27,45 @@
 
 namespace quoka {
 
-template <int HALVES, bool SPARSE, bool SPLIT>
+constexpr int kSlots = 8;
+
+template <bool SPARSE, bool SPLIT>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __nv_bfloat16* __restrict__ kc,
                const __nv_bfloat16* __restrict__ vc, const int32_t* __restrict__ k_idx,
                const int32_t* __restrict__ k_cnt, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
-  constexpr int D = HALVES * 64;
-  constexpr uint32_t kHalfBytes = 128 * 128;                 // 128 rows x 128 B
-  constexpr uint32_t kTileBytes = HALVES * kHalfBytes;       // one Q / K / V tile
-  constexpr int kSlots = HALVES == 2 ? 5 : 8;
-  // tensor memory (see "order of the products"): S | P_A | P_B | O_A | O_B, or S | S | S | O_A | O_B with P in place
-  constexpr bool APART = HALVES == 2;
-  constexpr int NBUF = APART ? 1 : 3;
-  constexpr uint32_t P_COL = 128, O_COL = APART ? 256 : 384;    // (Q tile B's P is 64, its O D columns on)
+  constexpr int D = 64;
+  constexpr uint32_t kTileBytes = 128 * 128;                 // one Q / K / V tile: 128 rows x 128 B
+  // tensor memory (see "order of the products"): S | S | S | O_A | O_B, P in place
+  constexpr int NBUF = 3;
+  constexpr uint32_t O_COL = NBUF * 128;                     // (Q tile B's O is 64 columns on)
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  unsigned char* q_smem = smem;                               // [2][HALVES][128][128 B]
-  unsigned char* kv_smem = smem + 2 * kTileBytes;             // [kSlots][HALVES][128][128 B]
+  unsigned char* q_smem = smem;                               // [2][128][128 B]
+  unsigned char* kv_smem = smem + 2 * kTileBytes;             // [kSlots][128][128 B]
   uint64_t* bars = reinterpret_cast<uint64_t*>(kv_smem + (size_t)kSlots * kTileBytes);
   uint64_t* kv_full = bars;                 // [kSlots]  the loader threads' cp.async arrivals
   uint64_t* kv_empty = bars + kSlots;       // [kSlots]  MMA commit
-  // (N = per Q tile if APART, per S buffer otherwise)
-  constexpr int N = APART ? 2 : NBUF;
-  uint64_t* s_full = bars + 2 * kSlots;     // [N]       MMA commit
-  uint64_t* p_full = s_full + N;            // [N][2]    4 softmax warps arrive, per half of the key tile
-  uint64_t* p_done = p_full + 2 * N;        // [N]       MMA commit: P has been multiplied
-  uint64_t* s_free = p_done + N;            // APART only: 4 softmax warps have read S
-  uint64_t* o_full = s_free + 1;            // [2]       MMA commit after the last PV
+  uint64_t* s_full = bars + 2 * kSlots;     // [NBUF]    MMA commit
+  uint64_t* p_full = s_full + NBUF;         // [NBUF][2] 4 softmax warps arrive, per half of the key tile
+  uint64_t* p_done = p_full + 2 * NBUF;     // [NBUF]    MMA commit: P has been multiplied, the buffer is free
+  uint64_t* o_full = p_done + NBUF;         // [2]       MMA commit after the last PV
   uint64_t* q_full = o_full + 2;            // TMA
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q_full + 1);
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WaitCtx wc{&abort_flag, P.status};
-  // grid = (heads, row blocks, batch): heads vary fastest so the CTAs resident together share a KV head's
-  // rows in L2, and the row blocks run heaviest (most causal tiles) first, lightest last, the sequences longest first
-  const int s = longest_first(P, blockIdx.z), h = blockIdx.x, kv = h / P.group;
+  // grid = (head groups, row blocks, batch): head groups vary fastest, the row blocks run heaviest (most causal tiles)
+  // first, lightest last, the sequences longest first
+  const int s = longest_first(P, blockIdx.z), hg = blockIdx.x;
   // (SPLIT: grid.y = row blocks times the parts a row block's key tiles are cut into)
   const int n_parts = SPLIT ? P.attn_parts : 1;
   const int rb = (SPLIT ? P.attn_split_rb : P.attn_row_blocks) - 1 - blockIdx.y / n_parts;
-  const int r0 = rb * 2 * kQTile;
-  AttnGeom g = make_geom<SPARSE>(P, s, r0);
+  const QRows qr{hg * P.attn_pack, rb * P.attn_qtiles * P.attn_span};
+  const int kv = qr.head0 / P.group;
+  AttnGeom g = make_geom<SPARSE>(P, s, qr.p0, 1);
   // SPLIT: this CTA walks the tiles [t_lo, t_hi) of the row block's sequence only and leaves, per row, a partial
   // result; the part that finishes last adds the parts up.  The list length has to be known before the range is, so
   // nothing of the walk starts before the selection has ended.
@@ -82,10 +80,9 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int i = 0; i < kSlots; ++i) { mbar_init(&kv_full[i], kLoaderWarps * 32); mbar_init(&kv_empty[i], 1); }
-    for (int i = 0; i < N; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_done[i], 1); }
-    for (int i = 0; i < 2 * N; ++i) mbar_init(&p_full[i], 4);
+    for (int i = 0; i < NBUF; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_done[i], 1); }
+    for (int i = 0; i < 2 * NBUF; ++i) mbar_init(&p_full[i], 4);
     for (int i = 0; i < 2; ++i) mbar_init(&o_full[i], 1);
-    mbar_init(s_free, 4);
     mbar_init(q_full, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tm_q);
@@ -93,6 +90,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     tma_prefetch_desc(&tm_v);
   }
   if (warp == kQkWarp) tmem_alloc(tmem_slot, 512);
+  zero_spare_q_rows<D>(P, q_smem, threadIdx.x, kAttnThreads);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -104,16 +102,15 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     const int x = warp >> 2;                                  // Q tile A (0) or B (1)
     const int quarter = warp & 3;
     const int row_in_tile = quarter * 32 + lane;
-    const int row = r0 + x * kQTile + row_in_tile;            // chunk row
+    const int row = qr.position(P, x, row_in_tile);           // chunk position
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
     const uint32_t o_addr = lane_addr + O_COL + x * D;
     const float scale_log2 = P.scale * 1.4426950408889634f;
     float m_run = -INFINITY, l_run = 0.f;
-    // APART: this Q tile's barriers.  Otherwise those of the S buffers, which go by items: the first of this Q tile's is item 0,
-    // or 1 where the other comes first, the next one is `step` items on.
+    // S buffers go by items: the first of this Q tile's is item 0, or 1 where the other comes first, the next one `step` on
     uint32_t phase = 0;
-    int buf = APART ? x : (x ? t_lo >= g.skip_a : g.skip_a > t_lo) ? 1 : 0;
-    const int step = APART ? 0 : g.active_b ? 2 : 1;
+    int buf = (x ? t_lo >= g.skip_a : g.skip_a > t_lo) ? 1 : 0;
+    const int step = g.active_b ? 2 : 1;
     bool ok = true;
     const int skip_x = max(x ? 0 : g.skip_a, t_lo);         // first tile this Q tile takes part in
     const bool active_x = (x ? g.active_b : true) && (!SPLIT || skip_x < g.n_known);
@@ -128,37 +125,36 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
       const bool masked = !__all_sync(0xFFFFFFFFu, vis.lim >= kKeyTile);
       if (!mbar_wait(&s_full[buf], phase, wc)) { ok = false; break; }
       tc_fence_after();
-      const uint32_t s_addr = lane_addr + (APART ? 0 : buf * 128);
-      const auto products_done = [&]() {                      // of this Q tile's item before
-        const int before = buf - step;
-        if (!mbar_wait_done(&p_done[before < 0 ? before + N : before], APART || before < 0 ? phase ^ 1 : phase, wc)) return false;
-        tc_fence_after();
-        return true;
-      };
-      ok = attn_softmax_tile<D, APART>(
-          s_addr, APART ? lane_addr + P_COL + x * 64 : s_addr, o_addr, vis.lim, masked, scale_log2, t == skip_x, lane, m_run, l_run,
-          [&]() { mbar_arrive(s_free); }, [&]() { return APART ? products_done() : true; },
-          [&]() { return APART ? true : products_done(); }, [&](int half) { mbar_arrive(&p_full[2 * buf + half]); });
+      const uint32_t s_addr = lane_addr + buf * 128;
+      ok = attn_softmax_tile<D, false>(
+          s_addr, s_addr, o_addr, vis.lim, masked, scale_log2, t == skip_x, lane, m_run, l_run, []() {}, []() { return true; },
+          [&]() {                                             // products of this Q tile's item before
+            const int before = buf - step;
+            if (!mbar_wait_done(&p_done[before < 0 ? before + NBUF : before], before < 0 ? phase ^ 1 : phase, wc)) return false;
+            tc_fence_after();
+            return true;
+          },
+          [&](int half) { mbar_arrive(&p_full[2 * buf + half]); });
       if (!ok) break;
       buf += step;
-      if (APART || buf >= N) { phase ^= 1; buf -= APART ? 0 : N; }
+      if (buf >= NBUF) { phase ^= 1; buf -= NBUF; }
     }
     // ---- epilogue: O / l -> bf16 -> global
     if constexpr (!SPLIT) {
       if (ok && active_x && mbar_wait(&o_full[x], 0, wc)) {
         tc_fence_after();
-        attn_store_row<D>(P, o_addr, m_run, l_run, s, h, row, out, lse);
+        attn_store_row<D>(P, o_addr, m_run, l_run, s, qr.head(P, row_in_tile), row, row_in_tile < qr.count(P, x), out, lse);
       }
     } else {
       const bool have = ok && active_x && mbar_wait(&o_full[x], 0, wc);
       if (have) tc_fence_after();
-      attn_split_epilogue<D>(P, (s * P.n_q + h) * P.attn_split_rb + rb, blockIdx.y % n_parts, n_parts, x, quarter, lane, row_in_tile, row, have,
-                             o_addr, m_run, l_run, s, h, out, lse);
+      attn_split_epilogue<D>(P, (s * QRows::groups(P) + hg) * P.attn_split_rb + rb, blockIdx.y % n_parts, n_parts, x, quarter, lane,
+                             row_in_tile, row, row_in_tile < qr.count(P, x), have, o_addr, m_run, l_run, s, qr.head(P, row_in_tile),
+                             out, lse);
     }
   } else if (warp < 8 + kLoaderWarps) {
     // ================================================================== K / V row loaders (gather)
-    // One warp instruction copies 32 / PIECES whole rows (16 lanes x 16 bytes cover a 256-byte row); the
-    // row groups of a tile are dealt round-robin to the loader warps.
+    // One warp instruction copies four whole rows (eight lanes x 16 bytes cover a 128-byte row); the row groups of a tile are dealt round-robin to the loader warps.
     const int lw = warp - 8;
     constexpr int PIECES = D / 8;                             // 16-byte pieces per row (16 or 8)
     constexpr int ROWS_PER_INSTR = 32 / PIECES;               // 2 or 4
@@ -226,9 +222,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
             for (int sub = 0; sub < 2; ++sub) {
               int c1 = tr.first + sub * 64, c3 = s;
               if (P.page_size != 0) { c1 = 0; c3 = __ldg(table + (tr.first >> 6) + sub); }
-#pragma unroll
-              for (int hh = 0; hh < HALVES; ++hh)
-                tma_load_4d(dst + hh * kHalfBytes + sub * 64 * 128, tm, &kv_full[slot], hh * 64, c1, kv, c3);
+              tma_load_4d(dst + sub * 64 * 128, tm, &kv_full[slot], 0, c1, kv, c3);
             }
           } else {
             mbar_arrive(&kv_full[slot]);
@@ -245,12 +239,12 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
           }
         }
         const uint4* src_base = reinterpret_cast<const uint4*>(kvi ? vc : kc) + base16;
-        const uint32_t dst_tile = kv_base + slot * kTileBytes + (c16 >> 3) * kHalfBytes;
+        const uint32_t dst_tile = kv_base + slot * kTileBytes;
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
           const uint32_t off = __shfl_sync(0xFFFFFFFFu, offs[(i * ROWS_PER_INSTR) / 32], (i * ROWS_PER_INSTR + rsub) & 31);
           const int rr = (lw + i * kLoaderWarps) * ROWS_PER_INSTR + rsub;
-          cp_async_16(dst_tile + rr * 128 + (((c16 & 7) ^ (rr & 7)) << 4), src_base + (off == kNoRow ? 0u : off), off != kNoRow);
+          cp_async_16(dst_tile + rr * 128 + ((c16 ^ (rr & 7)) << 4), src_base + (off == kNoRow ? 0u : off), off != kNoRow);
         }
         // this thread's share of the slot is signalled by the copy engine itself when the bytes have landed:
         // no wait in the loader, every slot of the ring can be in flight
@@ -263,12 +257,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     cp_async_wait_all();                                      // nothing of this thread is in flight at exit
   } else {
     // ================================================================== warp 11: QK^T, warp 10: PV
-    if (warp == kQkWarp && lane == 0) {
-      mbar_arrive_expect_tx(q_full, 2 * kTileBytes);
-      for (int x = 0; x < 2; ++x)
-        for (int hh = 0; hh < HALVES; ++hh)
-          tma_load_4d(q_smem + x * kTileBytes + hh * kHalfBytes, &tm_q, q_full, hh * 64, r0 + x * kQTile, h, s);
-    }
+    if (warp == kQkWarp && lane == 0) load_q_tiles<D>(P, qr, q_smem, &tm_q, q_full, s);
     __syncwarp();
     const bool leader = elect_one();
     const uint32_t tmem = (uint32_t)warp_uniform((int)tmem_base);
@@ -293,7 +282,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
         attn_issue_qk<NBUF, kSlots>(
             g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); grid_launch_dependents(); }, acquire,
             [&](unsigned buf, uint32_t parity) {
-              if (!warp_all(mbar_poll(APART ? s_free : &p_done[buf], parity, wc))) return false;
+              if (!warp_all(mbar_poll(&p_done[buf], parity, wc))) return false;
               tc_fence_after();
               return true;
             },
@@ -301,33 +290,28 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
               const uint64_t da = desc_q + (uint64_t)(x * (kTileBytes >> 4));
               const uint64_t db = desc_k + (uint64_t)((uint32_t)ks * (kTileBytes >> 4));
 #pragma unroll
-              for (int hh = 0; hh < HALVES; ++hh)
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                  const uint64_t off = (uint64_t)((hh * kHalfBytes + kk * 32) >> 4);
-                  if (leader) mma_ss(tmem + buf * 128, da + off, db + off, idesc_qk, (hh | kk) ? 1u : 0u);
-                }
-              if (leader) mma_commit(&s_full[APART ? x : buf]);
+              for (int kk = 0; kk < 4; ++kk)
+                if (leader) mma_ss(tmem + buf * 128, da + (uint64_t)(kk * 32 >> 4), db + (uint64_t)(kk * 32 >> 4), idesc_qk, kk ? 1u : 0u);
+              if (leader) mma_commit(&s_full[buf]);
             },
             release);
     } else {
       const uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true);
-      const uint64_t desc_v = smem_desc_sw128(kv_base, kHalfBytes, 1024);    // MN-major rows (V tiles)
+      const uint64_t desc_v = smem_desc_sw128(kv_base, 16, 1024);            // MN-major rows (V tiles)
       uint32_t p_phase = 0;
       attn_issue_pv<NBUF, kSlots>(
           g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); }, acquire,
           [&](int x, int half, unsigned buf, int vs, bool add) {
-            const unsigned n = APART ? x : buf;
-            if (!warp_all(mbar_poll(&p_full[2 * n + half], (p_phase >> n) & 1u, wc))) return false;
+            if (!warp_all(mbar_poll(&p_full[2 * buf + half], (p_phase >> buf) & 1u, wc))) return false;
             tc_fence_after();
             const uint64_t dv = desc_v + (uint64_t)((uint32_t)vs * (kTileBytes >> 4) + half * 4 * (2048 >> 4));
-            const uint32_t pa = tmem + (APART ? P_COL + x * 64 : buf * 128) + half * 32, oa = tmem + O_COL + x * D;
+            const uint32_t pa = tmem + buf * 128 + half * 32, oa = tmem + O_COL + x * D;
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)             // 16 keys per MMA: 8 packed columns of P, 16 rows of V
               if (leader) mma_ts(oa, pa + kk * 8, dv + (uint64_t)(kk * (2048 >> 4)), idesc_pv, add || kk ? 1u : 0u);
             if (half) {
-              if (leader) mma_commit(&p_done[n]);
-              p_phase ^= 1u << n;
+              if (leader) mma_commit(&p_done[buf]);
+              p_phase ^= 1u << buf;
             }
             return true;
           },
@@ -362,39 +346,69 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
 // 4096 at 128K 1039 / 990, 3072 at 32K, half listed 789 / 746; 40 heads, 1536 at 32K, promised 4 %: 290 / 309; dense 1536 at
 // 32K 920 / 692, 2048 at 32K 942 / 908, 4096 at 128K 7412 / 6689.
 // Partial results above 128 MB are not written: such jobs have waves enough.
-static long long attn_row_blocks(const quoka_params* p) { return (p->chunk_len + 2 * kQTile - 1) / (2 * kQTile); }
-static long long attn_jobs(const quoka_params* p) { return p->n_q_heads * attn_row_blocks(p) * p->batch; }
+// How the query rows of a call are laid out: see QRows.
+struct AttnShape {
+  int pack, span;                  // heads and chunk positions of a Q tile
+  int ctas, block;                 // CTAs and positions of a row block
+  long long blocks, per_rb, jobs;  // row blocks of a head group; CTAs of one row block of every head; CTAs
+};
+static AttnShape attn_shape(const quoka_params* p, int q_tiles) {
+  AttnShape a;
+  const int group = p->n_q_heads / p->n_kv_heads;
+  a.pack = 1;
+  for (int d = 2; d <= 32 && d <= group; ++d)
+    if (group % d == 0) a.pack = d;
+  a.span = kQTile / a.pack;
+  a.ctas = p->head_dim == 128 ? 2 : 1;
+  a.block = q_tiles * a.ctas * a.span;
+  a.blocks = (p->chunk_len + a.block - 1) / a.block;
+  a.per_rb = (long long)(p->n_q_heads / a.pack) * a.ctas * p->batch;
+  a.jobs = a.per_rb * a.blocks;
+  return a;
+}
 static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
-  constexpr double kPartCost = 6.0;
+  constexpr double kPartCost = 6.0, kOneTile = 0.75;
   AttnPlan plan;
   if (p->dtype != QUOKA_BF16 || p->impl == QUOKA_IMPL_SIMT || p->chunk_len <= 1) return plan;
-  const long long n_rb = attn_row_blocks(p), per_rb = (long long)p->n_q_heads * p->batch, jobs = per_rb * n_rb;
   const long long sms = device_sm_count();
   if (sms <= 0) return plan;
-  if (jobs < sms) {
-    const double t = tiles + n_rb;                                          // plus the chunk's own tiles, on average
-    double best = t;
-    for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
-      const long long waves = (jobs * parts + sms - 1) / sms;
-      const double cost = (double)waves * (t / parts + kPartCost);
-      if (cost < 0.97 * best) { plan.split_rb = (int)n_rb; plan.parts = parts; plan.in_cluster = false; best = cost; }
-    }
-    // the pair kernel's, in clusters
-    const int group = p->n_q_heads / p->n_kv_heads;
-    if (p->head_dim == 128 && group % 2 == 0) {
-      for (int parts = 2; parts <= 4 && parts <= tiles / 2; ++parts) {
-        const double cost = t / parts + 1.0, limit = std::min(0.95 * best, 0.97 * t - 4.5);
-        if (jobs / 2 <= (parts == 2 ? 32 : parts == 3 ? 20 : 14) && cost < limit) {
-          plan.split_rb = (int)n_rb; plan.parts = parts; plan.in_cluster = true; best = cost / 0.95;
+  const AttnShape two = attn_shape(p, 2);
+  if (two.jobs < sms) {
+    double best_of_all = 0;
+    for (int q_tiles = 2; q_tiles >= 1; --q_tiles) {
+      const AttnShape a = attn_shape(p, q_tiles);
+      if (a.jobs > sms) break;
+      AttnPlan cand;
+      cand.q_tiles = q_tiles;
+      // plus the chunk's own tiles, on average; in steps of two Q tiles
+      const double step = q_tiles == 1 ? kOneTile : 1.0;
+      const double t = tiles + 0.5 * (double)a.block / kKeyTile * (double)a.blocks;
+      double best = step * t, cost = best;
+      for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
+        const long long waves = (a.jobs * parts + sms - 1) / sms;
+        cost = (double)waves * (step * t / parts + kPartCost);
+        if (cost < 0.97 * best) { cand.split_rb = (int)a.blocks; cand.parts = parts; cand.in_cluster = false; best = cost; }
+      }
+      // the pair kernel's, in clusters
+      if (a.ctas == 2) {
+        for (int parts = 2; parts <= 4 && parts <= tiles / 2; ++parts) {
+          cost = step * t / parts + 1.0;
+          const double limit = std::min(0.95 * best, 0.97 * step * t - 4.5);
+          if (a.jobs / 2 <= (parts == 2 ? 32 : parts == 3 ? 20 : 14) && cost < limit) {
+            cand.split_rb = (int)a.blocks; cand.parts = parts; cand.in_cluster = true; best = cost / 0.95;
+          }
         }
       }
+      if (q_tiles == 2 || best < best_of_all) { plan = cand; best_of_all = best; }
     }
     return plan;
   }
+  const long long n_rb = two.blocks, per_rb = two.per_rb, jobs = two.jobs;
+  const double own = (double)two.block / kKeyTile;                           // the chunk's own tiles grow by this per row block
   const long long q = jobs / sms, rest = jobs % sms;
   if (rest == 0 || (sparse && p->batch > 1)) return plan;
-  const long long split = (rest + per_rb - 1) / per_rb;                      // row blocks to cut; block r has 2 r + 2 own tiles
-  const double t_all = tiles + 2 + n_rb, t_whole = tiles + 2 + split + n_rb, t_split = tiles + 2 + split;
+  const long long split = (rest + per_rb - 1) / per_rb;                      // row blocks to cut; block r has about (r + 1) * own of its own tiles
+  const double t_all = tiles + 2 + 0.5 * own * n_rb, t_whole = tiles + 2 + 0.5 * own * (split + n_rb), t_split = tiles + 2 + 0.5 * own * split;
   double best = (sparse ? 0.93 : 0.97) * (double)(q + 1) * t_all;
   for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
     const double t_part = t_split / parts + kPartCost;
@@ -407,7 +421,7 @@ static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
 }
 AttnPlan attn_plan_sparse(const quoka_params* p, int budget_cap) { return attn_plan(p, (budget_cap + kKeyTile - 1) / kKeyTile + 1, true); }
 AttnPlan attn_plan_dense(const quoka_params* p) { return attn_plan(p, (p->max_ctx_len + kKeyTile - 1) / kKeyTile + 1, false); }
-static size_t attn_split_jobs(const quoka_params* p, const AttnPlan& plan) { return (size_t)p->n_q_heads * p->batch * plan.split_rb; }
+static size_t attn_split_jobs(const quoka_params* p, const AttnPlan& plan) { return (size_t)attn_shape(p, plan.q_tiles).per_rb * plan.split_rb; }
 size_t attn_split_partial_bytes(const quoka_params* p, const AttnPlan& plan) {
   return plan.in_cluster ? 0 : attn_split_jobs(p, plan) * plan.parts * 2 * kSplitTileFloats * sizeof(float);
 }
@@ -428,7 +442,8 @@ quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const A
                               void* out, float* lse, cudaStream_t st, bool after_selection) {
   const bool sparse = k_idx != nullptr, split = plan.split_rb > 0 && (P.attn_partials || plan.in_cluster);
   DevParams PP = P;
-  PP.attn_row_blocks = (int)attn_row_blocks(p);
+  const AttnShape shape = attn_shape(p, plan.q_tiles);
+  PP.attn_row_blocks = (int)shape.blocks;
   PP.attn_split_rb = split ? plan.split_rb : 0;
   PP.attn_parts = split ? plan.parts : 1;
   const int whole = PP.attn_row_blocks - PP.attn_split_rb;
@@ -441,7 +456,7 @@ quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const A
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return QUOKA_ERR_CUDA;
     const bool early = parts && whole > 0 ? true : sparse && after_selection;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(P.n_q, parts ? PP.attn_split_rb * PP.attn_parts : whole, P.batch);   // (pairs: n_q is even)
+    cfg.gridDim = dim3((unsigned)(shape.per_rb / P.batch), parts ? PP.attn_split_rb * PP.attn_parts : whole, P.batch);
     cfg.blockDim = dim3(kAttnThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -466,7 +481,7 @@ quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const A
   return cudaGetLastError() == cudaSuccess ? QUOKA_OK : QUOKA_ERR_CUDA;
 }
 
-bool attn_below_a_wave(const quoka_params* p) { return attn_jobs(p) < device_sm_count(); }
+bool attn_below_a_wave(const quoka_params* p) { return attn_shape(p, 2).jobs < device_sm_count(); }
 
 bool attn_tc_supported(const quoka_params* p) {
   if (p->dtype != QUOKA_BF16) return false;
@@ -476,29 +491,32 @@ bool attn_tc_supported(const quoka_params* p) {
   return true;
 }
 
-template <int HALVES>
-static AttnKernel pick_attn_tc(bool sparse, bool parts, bool) {
-  if (parts) return sparse ? attn_tc_kernel<HALVES, true, true> : attn_tc_kernel<HALVES, false, true>;
-  return sparse ? attn_tc_kernel<HALVES, true, false> : attn_tc_kernel<HALVES, false, false>;
+bool encode_q_tensor_map(CUtensorMap* out, const DevParams& P, const void* q) {
+  const uint64_t dims[5] = {(uint64_t)P.d, (uint64_t)P.attn_pack, (uint64_t)P.chunk, (uint64_t)(P.n_q / P.attn_pack), (uint64_t)P.batch};
+  const uint64_t strides[4] = {(uint64_t)P.q_sh * 2, (uint64_t)P.q_st * 2, (uint64_t)P.q_sh * 2 * P.attn_pack, (uint64_t)P.q_sb * 2};
+  const uint32_t box[5] = {64, (uint32_t)P.attn_pack, (uint32_t)P.attn_span, 1, 1};
+  return encode_tensor_map_bf16(out, q, 5, dims, strides, box);
 }
 
-quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
+static AttnKernel pick_attn_tc(bool sparse, bool parts, bool) {
+  if (parts) return sparse ? attn_tc_kernel<true, true> : attn_tc_kernel<false, true>;
+  return sparse ? attn_tc_kernel<true, false> : attn_tc_kernel<false, false>;
+}
+
+quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P0, const void* q, const void* k, const void* v,
                             const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                             bool after_selection, const AttnPlan& plan) {
-  if (attn_tc_pair_applies(P)) return launch_attn_tc_pair(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection, plan);
-  CUtensorMap tm_q;
-  {
-    const uint64_t dims[4] = {(uint64_t)P.d, (uint64_t)P.chunk, (uint64_t)P.n_q, (uint64_t)P.batch};
-    const uint64_t strides[3] = {(uint64_t)P.q_st * 2, (uint64_t)P.q_sh * 2, (uint64_t)P.q_sb * 2};
-    const uint32_t box[4] = {64, 128, 1, 1};
-    if (!encode_tensor_map_bf16(&tm_q, q, 4, dims, strides, box)) return QUOKA_ERR_CUDA;
-  }
-  CUtensorMap tm_k, tm_v;
+  DevParams P = P0;
+  const AttnShape shape = attn_shape(p, plan.q_tiles);
+  P.attn_pack = shape.pack;
+  P.attn_span = shape.span;
+  P.attn_qtiles = plan.q_tiles;
+  if (shape.ctas == 2) return launch_attn_tc_pair(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection, plan);
+  CUtensorMap tm_q, tm_k, tm_v;
+  if (!encode_q_tensor_map(&tm_q, P, q)) return QUOKA_ERR_CUDA;
   if (!encode_kv_tensor_map(&tm_k, p, k, 64) || !encode_kv_tensor_map(&tm_v, p, v, 64)) return QUOKA_ERR_CUDA;
-  const int halves = P.d / 64;
-  const size_t tile = (size_t)halves * 128 * 128;
-  const size_t smem = 1024 + (2 + (halves == 2 ? 5 : 8)) * tile + 512;
-  return launch_attn_plan(p, P, plan, halves == 2 ? pick_attn_tc<2> : pick_attn_tc<1>, "attn_tc", /*cluster=*/1, smem, tm_q, tm_k, tm_v, k, v, k_idx, k_cnt, out, lse, st, after_selection);
+  const size_t smem = 1024 + (2 + kSlots) * 16384 + 512;
+  return launch_attn_plan(p, P, plan, pick_attn_tc, "attn_tc", /*cluster=*/1, smem, tm_q, tm_k, tm_v, k, v, k_idx, k_cnt, out, lse, st, after_selection);
 }
 
 }  // namespace quoka

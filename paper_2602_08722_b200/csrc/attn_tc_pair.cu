@@ -1,9 +1,9 @@
-// The tensor-core attention kernel for head_dim 128 with an even number of query heads per KV head: the CTAs of
-// two query heads of one KV group run as a PAIR (a cluster of two on neighbouring SMs) and share every K / V tile.
+// The tensor-core attention kernel for head_dim 128: two CTAs with neighbouring chunk positions of one KV group run as a
+// PAIR (a cluster of two on neighbouring SMs) and share every K / V tile.
 //
-// Both heads of a pair walk the same key tiles in the same order (the selected list, the chunk's own rows and the
-// causal limits depend on the KV head and the chunk row only), so one `tcgen05.mma.cta_group::2` covers both:
-// 256 rows of S (or O), 128 per CTA, with the K (or V) operand split between the two CTAs' shared memories.
+// Both walk the same key tiles in the same order (the selected list depends on the KV head only; the causal limits end
+// within a few tiles of each other), so one `tcgen05.mma.cta_group::2` covers both: 256 rows of S (or O), 128 per CTA, with
+// the K (or V) operand split between the two CTAs' shared memories.
 //   S = Q K^T : each CTA supplies its own Q tile and 64 of the tile's 128 keys (all 128 elements of each).
 //   O += P V  : each CTA supplies its own P (tensor memory) and 64 of V's 128 columns (all 128 keys).
 // So a CTA fetches HALF of every K and V tile (the 16-byte cp.async gather of listed rows tops out near 20 bytes per
@@ -66,14 +66,15 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WaitCtx wc{&abort_flag, P.status};
   const uint32_t cta = cluster_cta_rank();
-  const uint32_t rank = MODE == kPartsCluster ? cta & 1u : cta;   // 0: issues the MMAs; the pair is heads (2j, 2j + 1)
+  const uint32_t rank = MODE == kPartsCluster ? cta & 1u : cta;   // 0: issues the MMAs, has the first positions
   const uint32_t first = MODE == kPartsCluster ? cta & ~1u : 0u;  // the pair's first CTA
-  const int s = longest_first(P, blockIdx.z), h = blockIdx.x, kv = h / P.group;
+  const int s = longest_first(P, blockIdx.z), hg = blockIdx.x >> 1;
   // grid.y = row blocks (heaviest first), times the parts a row block's key tiles are cut into (SPLIT)
   const int n_parts = SPLIT ? P.attn_parts : 1;
   const int rb = (SPLIT ? P.attn_split_rb : P.attn_row_blocks) - 1 - blockIdx.y / n_parts;
-  const int r0 = rb * 2 * kQTile;
-  AttnGeom g = make_geom<SPARSE>(P, s, r0);
+  const QRows qr{hg * P.attn_pack, (rb * 2 + (int)rank) * P.attn_qtiles * P.attn_span};
+  const int kv = qr.head0 / P.group;
+  AttnGeom g = make_geom<SPARSE>(P, s, rb * 2 * P.attn_qtiles * P.attn_span, 2);
   int t_lo = 0;
 
   if (threadIdx.x == 0) {
@@ -94,17 +95,13 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     tma_prefetch_desc(&tm_v);
   }
   if (warp == kQkWarp) tmem_alloc_pair(tmem_slot, 512);
+  zero_spare_q_rows<D>(P, q_smem, threadIdx.x, kAttnThreads);
   tc_fence_before();
   cluster_sync_all();                                         // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const uint16_t both = MODE == kPartsCluster ? (uint16_t)(3u << first) : (uint16_t)3;   // this pair in the cluster
-  const auto load_q = [&]() {
-    mbar_arrive_expect_tx(q_full, 2 * kPairQTileBytes);
-    for (int x = 0; x < 2; ++x)
-      for (int hh = 0; hh < 2; ++hh)
-        tma_load_4d(q_smem + x * kPairQTileBytes + hh * 16384, &tm_q, q_full, hh * 64, r0 + x * kQTile, h, s);
-  };
+  const auto load_q = [&]() { load_q_tiles<D>(P, qr, q_smem, &tm_q, q_full, s); };
   // SPLIT: this CTA walks the tiles [t_lo, t_hi) of the row block's sequence only and leaves, per row, a partial
   // result (reference point, sum, un-normalised output); the part that finishes last, or the cluster, adds the
   // parts up.  The list length has to be known before the range is, so nothing of the walk starts before the selection has
@@ -124,7 +121,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     const int x = warp >> 2;                                  // Q tile A (0) or B (1)
     const int quarter = warp & 3;
     const int row_in_tile = quarter * 32 + lane;
-    const int row = r0 + x * kQTile + row_in_tile;            // chunk row
+    const int row = qr.position(P, x, row_in_tile);           // chunk position
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
     const uint32_t p_addr = lane_addr + P_COL + x * 64, o_addr = lane_addr + O_COL + x * D;
     const float scale_log2 = P.scale * 1.4426950408889634f;
@@ -161,7 +158,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     if constexpr (!SPLIT) {
       if (ok && active_x && mbar_wait(&o_full[x], 0, wc)) {
         tc_fence_after();
-        attn_store_row<D>(P, o_addr, m_run, l_run, s, h, row, out, lse);
+        attn_store_row<D>(P, o_addr, m_run, l_run, s, qr.head(P, row_in_tile), row, row_in_tile < qr.count(P, x), out, lse);
       }
     } else if constexpr (MODE == kPartsCluster) {
       // every product of the CTA has been formed when both are final: the ring and the Q tiles are free
@@ -173,8 +170,9 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     } else {
       const bool have = ok && active_x && mbar_wait(&o_full[x], 0, wc);
       if (have) tc_fence_after();
-      attn_split_epilogue<D>(P, (s * P.n_q + h) * P.attn_split_rb + rb, blockIdx.y % n_parts, n_parts, x, quarter, lane, row_in_tile, row, have,
-                             o_addr, m_run, l_run, s, h, out, lse);
+      attn_split_epilogue<D>(P, ((s * QRows::groups(P) + hg) * P.attn_split_rb + rb) * 2 + (int)rank, blockIdx.y % n_parts, n_parts, x,
+                             quarter, lane, row_in_tile, row, row_in_tile < qr.count(P, x), have, o_addr, m_run, l_run, s,
+                             qr.head(P, row_in_tile), out, lse);
     }
   } else if (warp < 8 + kPairLoaderWarps) {
     // ================================================================== K / V loaders: this CTA's half of every tile
@@ -377,7 +375,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
   tc_fence_before();
   if constexpr (MODE == kPartsCluster) {
     cluster_sync_all();                                       // every part's result is in its shared memory
-    if (warp < 8) attn_merge_cluster<D>(P, smem, part_ml, warp, lane, 2, (int)rank, n_parts, blockIdx.y % n_parts, r0, s, h, out, lse);
+    if (warp < 8) attn_merge_cluster<D>(P, smem, part_ml, warp, lane, 2, (int)rank, n_parts, blockIdx.y % n_parts, qr, s, out, lse);
   }
   cluster_sync_all();                                         // the other CTA's MMAs no longer read this CTA
   if (warp == kQkWarp) tmem_dealloc_pair(tmem_base, 512);
@@ -398,18 +396,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_pair_cluster_kernel(Q
 }
 
 // ---------------------------------------------------------------------------------------------- host
-bool attn_tc_pair_applies(const DevParams& P) { return P.d == 128 && P.group % 2 == 0; }
-
 quoka_status launch_attn_tc_pair(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                                  const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                                  bool after_selection, const AttnPlan& plan) {
   CUtensorMap tm_q;
-  {
-    const uint64_t dims[4] = {(uint64_t)P.d, (uint64_t)P.chunk, (uint64_t)P.n_q, (uint64_t)P.batch};
-    const uint64_t strides[3] = {(uint64_t)P.q_st * 2, (uint64_t)P.q_sh * 2, (uint64_t)P.q_sb * 2};
-    const uint32_t box[4] = {64, 128, 1, 1};
-    if (!encode_tensor_map_bf16(&tm_q, q, 4, dims, strides, box)) return QUOKA_ERR_CUDA;
-  }
+  if (!encode_q_tensor_map(&tm_q, P, q)) return QUOKA_ERR_CUDA;
   CUtensorMap tm_k, tm_v;
   if (!encode_kv_tensor_map(&tm_k, p, k, 64) || !encode_kv_tensor_map(&tm_v, p, v, 64)) return QUOKA_ERR_CUDA;
   const size_t smem = 1024 + 2 * kPairQTileBytes + (size_t)kPairSlots * kPairSlotBytes + 512 + (plan.in_cluster ? 2048 : 0);

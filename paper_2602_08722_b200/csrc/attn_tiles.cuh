@@ -52,18 +52,60 @@ __device__ __forceinline__ int longest_first(const DevParams& P, int z) {
   return __ffs(__ballot_sync(0xFFFFFFFFu, lane < P.batch && before == z)) - 1;
 }
 
-// Every CTA walks ONE sequence of key tiles t = 0 .. n_total-1 for both of its Q tiles; Q tile x takes part in
-// the tiles t >= skip[x] (a suffix, so both finish on the same tile).
-//   dense : the tiles of rows [0, T + C) in DESCENDING order (the tiles only Q tile B sees come first).
-//   sparse: first the chunk's own tiles (the one only B sees, then tiles 0 .. c_a-1), THEN the tiles of the
-//           selected list.  The chunk's tiles do not depend on the key selection, so this kernel is launched
-//           with programmatic stream serialisation: it starts while the selection kernel still runs, works
-//           through the chunk tiles, and only then waits for the selection (`resolve`) to learn the list length.
+// The query rows of a Q tile: `pack` heads of one KV group at `span` consecutive chunk positions, position by position, so
+// that the heads of a group share every key tile and a tile's rows end at nearly the same causal limit.  A KV group's heads
+// all go into one tile where they are up to 32 (else its largest divisor does): 128 / pack positions each, the rows that are
+// left over, seven at most, are zero.  Against 128 positions of one head each: a chunk of 777 with eight heads per KV head
+// takes 49 tiles instead of 56, one of 68 with three heads 2 instead of 3, the chunk's own tiles that a row block walks end
+// 32 positions after its first row and not 256 (four heads), and any number of heads per KV head makes pairs.
+// A row block is the Q tiles of one CTA (A, or A and B), or of both CTAs of a pair (A, B of the first, A, B of the second).
+struct QRows {
+  int head0;            // first head
+  int p0;               // first chunk position of this CTA
+  __device__ __forceinline__ static int groups(const DevParams& P) { return P.n_q / P.attn_pack; }
+  __device__ __forceinline__ int position(const DevParams& P, int x, int row_in_tile) const {
+    return p0 + x * P.attn_span + row_in_tile / P.attn_pack;
+  }
+  __device__ __forceinline__ int head(const DevParams& P, int row_in_tile) const { return head0 + row_in_tile % P.attn_pack; }
+  // rows of tile x that exist: the first ones
+  __device__ __forceinline__ int count(const DevParams& P, int x) const {
+    return x < P.attn_qtiles ? P.attn_pack * max(0, min(P.attn_span, P.chunk - p0 - x * P.attn_span)) : 0;
+  }
+};
+
+// This CTA's Q tiles by the copy engine: boxes of [span][pack][64 elements].
+template <int D>
+__device__ __forceinline__ void load_q_tiles(const DevParams& P, const QRows& qr, unsigned char* q_smem, const CUtensorMap* tm_q,
+                                             uint64_t* q_full, int s) {
+  mbar_arrive_expect_tx(q_full, P.attn_qtiles * (D / 64) * 128 * P.attn_pack * P.attn_span);
+  for (int x = 0; x < P.attn_qtiles; ++x)
+    for (int hh = 0; hh < D / 64; ++hh)
+      tma_load_5d(q_smem + (x * (D / 64) + hh) * 16384, tm_q, q_full, hh * 64, 0, qr.p0 + x * P.attn_span, qr.head0 / P.attn_pack, s);
+}
+// The rows left over: by the calling threads, before the barrier that the issuing warps pass.
+template <int D>
+__device__ __forceinline__ void zero_spare_q_rows(const DevParams& P, unsigned char* q_smem, int thread, int threads) {
+  const int used = P.attn_pack * P.attn_span, spare = (128 - used) * 8;      // 16-byte pieces of a half tile
+  if (spare == 0) return;
+  for (int i = thread; i < 2 * (D / 64) * spare; i += threads)
+    reinterpret_cast<uint4*>(q_smem + (i / spare) * 16384 + used * 128)[i % spare] = make_uint4(0, 0, 0, 0);
+  fence_proxy_async_smem();
+}
+bool encode_q_tensor_map(CUtensorMap* out, const DevParams& P, const void* q);
+
+// Every CTA walks ONE sequence of key tiles t = 0 .. n_total-1 for both of its Q tiles (a pair, for all four); Q tile B takes
+// part in all of them, A in the tiles t >= skip_a (a suffix, so both finish on the same tile).
+//   dense : the tiles of rows [0, T + C) in DESCENDING order.
+//   sparse: first the chunk's own tiles, those that not all rows of the block see descending and then the others ascending,
+//           THEN the tiles of the selected list.  The chunk's tiles do not depend on the key selection, so this kernel is
+//           launched with programmatic stream serialisation: it starts while the selection kernel still runs, works through
+//           the chunk tiles, and only then waits for the selection (`resolve`) to learn the list length.
+// So the tiles that a row does not see come before the first one that it does: whatever they add to O (their weights are
+// zero, but a value may be infinite) is wiped when the row's reference point is first set.
 struct AttnGeom {
   int T, C;
   int n_chunk;        // sparse: tiles of the chunk's own rows in the sequence; dense: 0
-  int c_a;            // sparse: chunk tiles Q tile A sees
-  int b_first;        // sparse: 1 when the sequence starts with the tile only B sees
+  int lead;           // sparse: as many of them are not seen by all rows
   int skip_a;         // first tile Q tile A takes part in (B takes part in all); scalars, not arrays: the struct
   bool active_b;      // must live in registers (an indexed member would put it in local memory)
   int n_known;        // tiles known so far (sparse: n_chunk until resolved, then n_chunk + n_sel)
@@ -72,29 +114,29 @@ struct AttnGeom {
   bool resolved;
 };
 
+// The row block of `ctas` CTAs that begins at chunk position p.
 template <bool SPARSE>
-__device__ __forceinline__ AttnGeom make_geom(const DevParams& P, int s, int r0) {
+__device__ __forceinline__ AttnGeom make_geom(const DevParams& P, int s, int p, int ctas) {
   AttnGeom g;
   g.T = __ldg(P.ctx_len + s);
   g.C = P.chunk;
-  const bool b_active = r0 + kQTile < g.C;
-  g.active_b = b_active;
+  const int span = P.attn_span, per_cta = P.attn_qtiles * span;
+  g.active_b = P.attn_qtiles == 2 && p + span < g.C;
+  // last positions of any A tile and of any tile
+  const int last = min(p + ctas * per_cta, g.C) - 1;
+  const int last_a = min(p + span + (ctas == 2 && p + per_cta < g.C ? per_cta : 0), g.C) - 1;
   g.cnt = 0;
   if (SPARSE) {
-    g.c_a = r0 / kQTile + 1;
-    g.b_first = b_active ? 1 : 0;
-    g.n_chunk = g.c_a + g.b_first;
-    g.skip_a = g.b_first;
+    g.n_chunk = last / kKeyTile + 1;
+    g.lead = g.n_chunk - (p / kKeyTile + 1);
+    g.skip_a = g.active_b ? g.n_chunk - (last_a / kKeyTile + 1) : 0;       // 0 or 1: a Q tile spans at most 128 positions
     g.n_known = g.n_chunk;
     g.n_dense = 0;
     g.resolved = false;
   } else {
-    const int last_a = min(r0 + kQTile - 1, g.C - 1), last_b = min(r0 + 2 * kQTile - 1, g.C - 1);
-    const int n_a = (g.T + last_a) / kKeyTile + 1;
-    const int n_b = b_active ? (g.T + last_b) / kKeyTile + 1 : 0;
-    g.n_dense = max(n_a, n_b);
-    g.skip_a = g.n_dense - n_a;
-    g.n_chunk = 0; g.c_a = 0; g.b_first = 0;
+    g.n_dense = (g.T + last) / kKeyTile + 1;
+    g.skip_a = g.active_b ? g.n_dense - ((g.T + last_a) / kKeyTile + 1) : 0;
+    g.n_chunk = 0; g.lead = 0;
     g.n_known = g.n_dense;
     g.resolved = true;
   }
@@ -142,7 +184,7 @@ __device__ __forceinline__ TileRows tile_rows(const AttnGeom& g, int t) {
   TileRows r;
   if (SPARSE) {
     if (t < g.n_chunk) {
-      const int ct = g.b_first ? (t == 0 ? g.c_a : t - 1) : t;
+      const int ct = t < g.lead ? g.n_chunk - 1 - t : t - g.lead;
       r.from_list = false;
       r.causal = true;
       r.first = g.T + ct * kKeyTile;
@@ -194,20 +236,20 @@ __device__ __forceinline__ uint32_t kv_row_off16(const DevParams& P, const int32
 }
 
 // Number of visible columns of tile t for chunk row `row` (columns [0, lim) are visible; may lie outside [0, 128]).
-// A softmax thread keeps it up from tile to tile: it changes by one tile's columns except where the chunk's own rows or
-// the selected list begin.
+// A softmax thread keeps it up from tile to tile.
 template <bool SPARSE>
 struct VisibleCols {
-  int lim;
+  int lim, step;
   __device__ __forceinline__ VisibleCols(const AttnGeom& g, int t, int row) {
     const TileRows tr = tile_rows<SPARSE>(g, t);
     lim = tr.causal ? row - tr.col0 + 1 : tr.count;
+    step = !SPARSE || t < g.lead ? kKeyTile : -kKeyTile;
   }
   __device__ __forceinline__ void at(const AttnGeom& g, int t, int row) {
-    if (SPARSE && t == g.b_first) lim = row + 1;
+    if (SPARSE && t == g.lead) { lim = row + 1; step = -kKeyTile; }
     if (SPARSE && t == g.n_chunk) lim = g.cnt;
   }
-  __device__ __forceinline__ void advance() { lim += SPARSE ? -kKeyTile : kKeyTile; }
+  __device__ __forceinline__ void advance() { lim += step; }
 };
 
 // Maximum of 32 score columns starting at col0; columns at and beyond `lim` are masked out (-inf: exp2 gives exactly 0).
@@ -268,7 +310,7 @@ __device__ __forceinline__ bool attn_softmax_tile(uint32_t s_addr, uint32_t p_ad
     const float m_new = fmaxf(m_run, m_tile);
     if (!first_tile) {
       if (!o_idle()) return false;
-      const float alpha = (m_run == -INFINITY) ? 0.f : ex2(m_run - m_new);
+      const float alpha = (m_run == -INFINITY) ? 0.f : ex2(m_run - m_new);      // (nothing seen yet: O is wiped)
       l_run *= alpha;
 #pragma unroll 1
       for (int c = 0; c < D / 8; ++c) {                       // rare: small pieces, few registers
@@ -276,7 +318,7 @@ __device__ __forceinline__ bool attn_softmax_tile(uint32_t s_addr, uint32_t p_ad
         tmem_ld8(o_addr + c * 8, r);
         tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 8; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
+        for (int i = 0; i < 8; ++i) r[i] = m_run == -INFINITY ? 0u : __float_as_uint(__uint_as_float(r[i]) * alpha);
         tmem_st8(o_addr + c * 8, r);
       }
       tmem_wait_st();
@@ -404,9 +446,8 @@ __device__ __forceinline__ void attn_issue_pv(AttnGeom& g, int t_lo, Resolve&& r
 // row's log-sum-exp when asked for).
 template <int D>
 __device__ __forceinline__ void attn_store_row(const DevParams& P, uint32_t o_addr, float m_run, float l_run, int s, int h,
-                                               int row, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
+                                               int row, bool store, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
   const float inv = 1.f / l_run;
-  const bool store = row < P.chunk;
   __nv_bfloat16* orow = out + (long long)s * P.o_sb + (long long)h * P.o_sh + (long long)row * P.o_st;
 #pragma unroll
   for (int c = 0; c < D / 32; ++c) {
@@ -438,7 +479,7 @@ constexpr int kSplitTileFloats = 130 * 128;     // one part's partial result of 
 // Epilogue of a softmax warp of a split launch.
 template <int D>
 __device__ __forceinline__ void attn_split_epilogue(const DevParams& P, int job, int part, int n_parts, int x, int quarter,
-                                                    int lane, int row_in_tile, int row, bool have, uint32_t o_addr,
+                                                    int lane, int row_in_tile, int row, bool store, bool have, uint32_t o_addr,
                                                     float m_run, float l_run, int s, int h, __nv_bfloat16* out,
                                                     float* lse) {
   // ---- this part's partial result (reference point m, sum l, un-normalised O; a part without tiles for this
@@ -484,7 +525,6 @@ __device__ __forceinline__ void attn_split_epilogue(const DevParams& P, int job,
       wgt[q] = w;
     }
     const float inv = 1.f / l;
-    const bool store = row < P.chunk;
     __nv_bfloat16* orow = out + (long long)s * P.o_sb + (long long)h * P.o_sh + (long long)row * P.o_st;
 #pragma unroll 1
     for (int c = 0; c < D / 32; ++c) {
@@ -547,17 +587,18 @@ __device__ __forceinline__ void attn_part_to_smem(unsigned char* smem, float* ml
 // time, four elements of a row per lane.
 template <int D>
 __device__ __forceinline__ void attn_merge_cluster(const DevParams& P, unsigned char* smem, float* ml, int warp, int lane, int stride,
-                                                   int offset, int parts, int part, int r0, int s, int h,
+                                                   int offset, int parts, int part, const QRows& qr, int s,
                                                    __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
   constexpr int kU = 4, kMaxParts = 4;
   const uint32_t o0 = smem_u32(smem), ml0 = smem_u32(ml);
-  const int rows = min(2 * kQTile, P.chunk - r0);
+  const int rows_a = qr.count(P, 0), rows = rows_a + qr.count(P, 1);
+  const auto row_of = [&](int i) { return i < rows_a ? i : 128 + i - rows_a; };       // i-th row that exists -> tile * 128 + row
   for (int j = warp * kU; part + parts * j < rows; j += 8 * kU) {
     float m[kU], l[kU], wgt[kU], M[kU], L[kU];
     float4 acc[kU];
 #pragma unroll
     for (int u = 0; u < kU; ++u) {                           // lane p holds part p's m and l
-      const int R = min(part + parts * (j + u), rows - 1), x = R >> 7, lr = R & 127;
+      const int R = row_of(min(part + parts * (j + u), rows - 1)), x = R >> 7, lr = R & 127;
       const uint32_t at = map_to_cta(ml0 + (uint32_t)(x * 256 + lr) * 4u, (uint32_t)(min(lane, parts - 1) * stride + offset));
       m[u] = ld_cluster_f(at);
       l[u] = ld_cluster_f(at + 512u);
@@ -570,7 +611,7 @@ __device__ __forceinline__ void attn_merge_cluster(const DevParams& P, unsigned 
       if (p < parts) {
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
-          const int R = min(part + parts * (j + u), rows - 1);
+          const int R = row_of(min(part + parts * (j + u), rows - 1));
           v[p][u] = ld_cluster_f4(map_to_cta(o0 + (uint32_t)(R * kPartPitch + 4 * (lane & (D / 4 - 1))) * 4u, (uint32_t)(p * stride + offset)));
         }
       }
@@ -599,14 +640,14 @@ __device__ __forceinline__ void attn_merge_cluster(const DevParams& P, unsigned 
     }
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
-      const int R = part + parts * (j + u);
-      if (R >= rows) break;
+      if (part + parts * (j + u) >= rows) break;
+      const int R = row_of(part + parts * (j + u)), h = qr.head(P, R & 127), p = qr.position(P, R >> 7, R & 127);
       const float inv = 1.f / L[u];
       const __nv_bfloat162 a = __floats2bfloat162_rn(acc[u].x * inv, acc[u].y * inv), b = __floats2bfloat162_rn(acc[u].z * inv, acc[u].w * inv);
       if (lane < D / 4)
-        *reinterpret_cast<uint2*>(out + (long long)s * P.o_sb + (long long)h * P.o_sh + (long long)(r0 + R) * P.o_st + 4 * lane) =
+        *reinterpret_cast<uint2*>(out + (long long)s * P.o_sb + (long long)h * P.o_sh + (long long)p * P.o_st + 4 * lane) =
             make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
-      if (lse && lane == 0) lse[((long long)s * P.n_q + h) * P.chunk + r0 + R] = (M[u] + log2f(L[u])) * 0.6931471805599453f;
+      if (lse && lane == 0) lse[((long long)s * P.n_q + h) * P.chunk + p] = (M[u] + log2f(L[u])) * 0.6931471805599453f;
     }
   }
 }

@@ -38,11 +38,13 @@ struct DevParams {
   float* attn_partials;
   int32_t* attn_counters;
   int n_attn_counters;
-  // plan of the attention call at hand (set by the launcher): the row blocks [0, attn_split_rb) of every head are cut
+  // plan of the attention call at hand (set by the launcher): the row blocks [0, attn_split_rb) of every head group are cut
   // into attn_parts parts each, in a launch of their own after the one of the heavier row blocks above them, if any
   int rank_heads;      // (sequence, query head) pairs of the whole problem: the ranking kernel's slices go by them
   int attn_one_part;   // f32 attention: keep row blocks whole (a slice of a problem that has waves enough)
   int attn_row_blocks, attn_split_rb, attn_parts, attn_after_whole;
+  int attn_pack, attn_span;   // heads and chunk positions of a Q tile of 128 rows
+  int attn_qtiles;            // Q tiles of a CTA, 1 or 2
 };
 
 // B_s of one sequence: min(B_SA, T) or floor(frac*T + 0.5) in double.

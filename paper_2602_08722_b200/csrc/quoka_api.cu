@@ -153,6 +153,7 @@ static DevParams make_dev(const quoka_params* p, void* ws, const Workspace& w) {
   P.attn_partials = w.attn_partials; P.attn_counters = w.attn_counters; P.n_attn_counters = w.n_attn_counters;
   P.rank_heads = p->batch * p->n_q_heads;
   P.attn_one_part = 0; P.attn_row_blocks = 0; P.attn_split_rb = 0; P.attn_parts = 1; P.attn_after_whole = 0;
+  P.attn_pack = 1; P.attn_span = 128; P.attn_qtiles = 2;
   return P;
 }
 static DevParams make_dev(const quoka_params* p, void* ws) { return make_dev(p, ws, carve(p, ws)); }

@@ -13,20 +13,20 @@ quoka_status launch_score_keys_tc(const quoka_params* p, const DevParams& P, con
 // Grids that leave SMs idle, all the time or in their last wave: the key tiles of the lightest `split_rb` row blocks of
 // every head are cut into `parts` parts, one CTA each (split_rb = 0: none).
 // in_cluster: the parts of a row block are one cluster (and need no scratch)
-struct AttnPlan { int split_rb = 0, parts = 1; bool in_cluster = false; };
+// q_tiles: Q tiles of a CTA
+struct AttnPlan { int split_rb = 0, parts = 1; bool in_cluster = false; int q_tiles = 2; };
 AttnPlan attn_plan_sparse(const quoka_params* p, int budget_cap);
 AttnPlan attn_plan_dense(const quoka_params* p);
 // Scratch for the partial results
 size_t attn_split_partial_bytes(const quoka_params* p, const AttnPlan& plan);
 size_t attn_split_counter_bytes(const quoka_params* p, const AttnPlan& plan);
 bool attn_tc_supported(const quoka_params* p);
-// Whether the attention grid (256 chunk rows of a head per CTA) has fewer CTAs than the GPU has SMs.
+// Whether the attention grid (256 query rows per CTA) has fewer CTAs than the GPU has SMs.
 bool attn_below_a_wave(const quoka_params* p);
 quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                             const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                             bool after_selection, const AttnPlan& plan);
-// head_dim 128 with an even GQA ratio: the CTAs of two heads of a KV group work as a pair (cta_group::2)
-bool attn_tc_pair_applies(const DevParams& P);
+// head_dim 128: two CTAs with neighbouring positions of a KV group work as a pair (cta_group::2)
 quoka_status launch_attn_tc_pair(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                                  const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                                  bool after_selection, const AttnPlan& plan);
