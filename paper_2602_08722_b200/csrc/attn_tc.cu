@@ -162,6 +162,8 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     constexpr int RPT = GROUPS / kLoaderWarps;                // row groups per warp
     const int c16 = lane % PIECES;                            // this thread's piece of the row
     const int rsub = lane / PIECES;
+    static_assert(kLoaderWarps * ROWS_PER_INSTR % 8 == 0, "a thread's rows all have the same swizzle");
+    const uint32_t thread_dst = (uint32_t)((lw * ROWS_PER_INSTR + rsub) * 128 + ((c16 ^ (lw * ROWS_PER_INSTR + rsub)) << 4));
     const int32_t* idx = SPARSE ? k_idx + ((long long)s * P.n_kv + kv) * P.budget_cap : nullptr;
     uint32_t phase = 0;
     int slot = 0;
@@ -181,6 +183,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     static_assert(GROUPS % kLoaderWarps == 0 && RPT * ROWS_PER_INSTR % 32 == 0, "whole registers of rows");
     int rows[LIST_REGS], rr_of[LIST_REGS];
     uint32_t offs[LIST_REGS];
+    bool all_rows = false;
 #pragma unroll
     for (int k = 0; k < LIST_REGS; ++k) {
       const int pp = 32 * k + lane;
@@ -208,7 +211,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
       bool stop = false;
 #pragma unroll 1
       for (int kvi = 0; kvi < 2; ++kvi) {                     // the tile's K rows, then its V rows
-        if (!mbar_wait(&kv_empty[slot], phase ^ 1, wc)) { stop = true; break; }
+        if (!mbar_wait_done(&kv_empty[slot], phase ^ 1, wc)) { stop = true; break; }
         // A whole tile of consecutive rows (page-aligned in a paged cache) is fetched by the copy engine as 64-row
         // boxes: one thread issues them, the others only keep the barrier's arrival count.  Ragged tiles (rows past
         // the end must read as zeros, not as whatever the cache holds there) and listed rows take the copies below.
@@ -236,15 +239,24 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
           for (int k = 0; k < LIST_REGS; ++k) {
             if (!tr.from_list) rows[k] = rr_of[k] < tr.count ? tr.first + rr_of[k] : -1;
             offs[k] = kv_row_off16(P, table, st16, sb16, rows[k], tr.from_list, g.T);
+            all_rows = (k == 0 || all_rows) && offs[k] != kNoRow;
           }
+          all_rows = warp_all(all_rows);
         }
         const uint4* src_base = reinterpret_cast<const uint4*>(kvi ? vc : kc) + base16;
-        const uint32_t dst_tile = kv_base + slot * kTileBytes;
+        const uint32_t dst = kv_base + slot * kTileBytes + thread_dst;
+        if (all_rows) {                                           // no size to select
 #pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-          const uint32_t off = __shfl_sync(0xFFFFFFFFu, offs[(i * ROWS_PER_INSTR) / 32], (i * ROWS_PER_INSTR + rsub) & 31);
-          const int rr = (lw + i * kLoaderWarps) * ROWS_PER_INSTR + rsub;
-          cp_async_16(dst_tile + rr * 128 + ((c16 ^ (rr & 7)) << 4), src_base + (off == kNoRow ? 0u : off), off != kNoRow);
+          for (int i = 0; i < RPT; ++i) {
+            const uint32_t off = __shfl_sync(0xFFFFFFFFu, offs[(i * ROWS_PER_INSTR) / 32], (i * ROWS_PER_INSTR + rsub) & 31);
+            cp_async_16(dst + (uint32_t)(i * kLoaderWarps * ROWS_PER_INSTR * 128), src_base + off);
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < RPT; ++i) {
+            const uint32_t off = __shfl_sync(0xFFFFFFFFu, offs[(i * ROWS_PER_INSTR) / 32], (i * ROWS_PER_INSTR + rsub) & 31);
+            cp_async_16(dst + (uint32_t)(i * kLoaderWarps * ROWS_PER_INSTR * 128), src_base + (off == kNoRow ? 0u : off), off != kNoRow);
+          }
         }
         // this thread's share of the slot is signalled by the copy engine itself when the bytes have landed:
         // no wait in the loader, every slot of the ring can be in flight

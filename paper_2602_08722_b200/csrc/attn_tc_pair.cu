@@ -198,6 +198,10 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     // The warp's K rows of a tile are numbered p = 2 i + rsub (i = its i-th row group), its V rows p = 4 i + rsub; lane l
     // looks after K row p = l and V rows p = l, 32 + l: their row numbers (-1 past the end), for listed rows fetched one
     // tile ahead, and their offsets, worked out once per tile.  The thread that copies a row fetches its offset by shuffle.
+    static_assert(kPairLoaderWarps == 2, "rows 4 apart from one K row group of a warp to the next, 8 for V");
+    const int klr = lw * 2 + krsub, vlr = lw * 4 + vrsub;
+    const uint32_t k_dst = (uint32_t)((kc16 >> 3) * 8192 + klr * 128 + (((kc16 & 7) ^ klr) << 4));
+    const uint32_t v_dst = (uint32_t)(vlr * 128 + ((vc16 ^ vlr) << 4));
     int k_row = -1, v_row[2] = {-1, -1};
     uint32_t k_off = kNoRow, v_off[2] = {kNoRow, kNoRow};
     const int krr = krow0 + (lw + (lane >> 1) * kPairLoaderWarps) * 2 + (lane & 1);
@@ -219,7 +223,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
     auto item = [&](auto is_v_c, const TileRows& tr, bool first_list_tile) -> bool {
       constexpr bool V = decltype(is_v_c)::value;
       constexpr int RPI = V ? 4 : 2;                            // rows per warp instruction
-      if (!mbar_wait(&kv_empty[slot], phase ^ 1, wc)) return false;
+      if (!mbar_wait_done(&kv_empty[slot], phase ^ 1, wc)) return false;
       // A whole tile of consecutive rows (page-aligned in a paged cache) is fetched by the copy engine as two
       // 8 KB boxes: one thread issues them, the others only keep the barrier's arrival count.  Ragged tiles (rows
       // past the end must read as zeros) and listed rows take the copies below.
@@ -254,14 +258,14 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
           v_off[0] = row_off(v_row[0], tr.from_list);
           v_off[1] = row_off(v_row[1], tr.from_list);
         }
-        const int c16 = V ? vc16 : kc16, rsub = V ? vrsub : krsub;
         const uint4* src_base = reinterpret_cast<const uint4*>(V ? vc : kc) + (V ? vbase16 : kbase16);
-        const uint32_t dst_item = kv_base + (uint32_t)slot * kPairSlotBytes + (V ? 0u : (uint32_t)(c16 >> 3) * 8192u);
+        const uint32_t dst = kv_base + (uint32_t)slot * kPairSlotBytes + (V ? v_dst : k_dst);
+        // row (lw + i * warps) * RPI + rsub of the item: its swizzle is the thread's own, turned by 4 rows for odd i (K)
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
-          const uint32_t off = V ? __shfl_sync(0xFFFFFFFFu, v_off[i / 8], (i * 4 + rsub) & 31) : __shfl_sync(0xFFFFFFFFu, k_off, i * 2 + rsub);
-          const int lr = (lw + i * kPairLoaderWarps) * RPI + rsub;   // row of the item in shared memory
-          cp_async_16(dst_item + lr * 128 + (((c16 & 7) ^ (lr & 7)) << 4), src_base + (off == kNoRow ? 0u : off), off != kNoRow);
+          const uint32_t off = V ? __shfl_sync(0xFFFFFFFFu, v_off[i / 8], (i * 4 + vrsub) & 31) : __shfl_sync(0xFFFFFFFFu, k_off, i * 2 + krsub);
+          cp_async_16((V || (i & 1) == 0 ? dst : dst ^ 64u) + (uint32_t)(i * kPairLoaderWarps * RPI * 128),
+                      src_base + (off == kNoRow ? 0u : off), off != kNoRow);
         }
         // this thread's share of the slot is signalled by the copy engine itself when the bytes have landed
         cp_async_mbar_arrive_noinc(&kv_full[slot]);
