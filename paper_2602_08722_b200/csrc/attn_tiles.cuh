@@ -252,12 +252,8 @@ struct VisibleCols {
   __device__ __forceinline__ void advance() { lim += step; }
 };
 
-// Maximum of 32 score columns starting at col0; columns at and beyond `lim` are masked out (-inf: exp2 gives exactly 0).
-__device__ __forceinline__ float max32(uint32_t* v, bool masked, int col0, int lim) {
-  if (masked) {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) if (col0 + i >= lim) v[i] = 0xFF800000u;
-  }
+// Maximum of 32 score columns.
+__device__ __forceinline__ float max32(const uint32_t* v) {
   float m0 = __uint_as_float(v[0]), m1 = __uint_as_float(v[1]);
 #pragma unroll
   for (int i = 2; i < 30; i += 4) {
@@ -299,8 +295,15 @@ __device__ __forceinline__ bool attn_softmax_tile(uint32_t s_addr, uint32_t p_ad
       __syncwarp();
       if (lane == 0) s_read();
     }
-    mx = fmaxf(fmaxf(max32(v0, masked, 0, lim), max32(v0 + 32, masked, 32, lim)),
-               fmaxf(max32(v0 + 64, masked, 64, lim), max32(last, masked, 96, lim)));
+    if (masked) {                                          // one branch: four of them were 2 % of the kernel
+#pragma unroll
+      for (int i = 0; i < kHeld; ++i) if (i >= lim) v0[i] = 0xFF800000u;      // -inf: exp2 gives exactly 0
+      if (!APART) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) if (96 + i >= lim) last[i] = 0xFF800000u;
+      }
+    }
+    mx = fmaxf(fmaxf(max32(v0), max32(v0 + 32)), fmaxf(max32(v0 + 64), max32(last)));
   }
   const float m_tile = mx * scale_log2;
   // ---- lazy rescale of the accumulator: only when some row's maximum grew by more than the threshold
