@@ -379,7 +379,7 @@ static AttnShape attn_shape(const quoka_params* p, int q_tiles) {
   return a;
 }
 static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
-  constexpr double kPartCost = 6.0, kOneTile = 0.75;
+  constexpr double kPartCost = 6.0, kOneTile = 0.9;
   AttnPlan plan;
   if (p->dtype != QUOKA_BF16 || p->impl == QUOKA_IMPL_SIMT || p->chunk_len <= 1) return plan;
   const long long sms = device_sm_count();
@@ -392,7 +392,8 @@ static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
       if (a.jobs > sms) break;
       AttnPlan cand;
       cand.q_tiles = q_tiles;
-      // plus the chunk's own tiles, on average; in steps of two Q tiles
+      // plus the chunk's own tiles, on average; in steps of two Q tiles (one of a lone Q tile takes 2700 cycles, its own chain
+      // from scores to weights and back, one of two about 3000)
       const double step = q_tiles == 1 ? kOneTile : 1.0;
       const double t = tiles + 0.5 * (double)a.block / kKeyTile * (double)a.blocks;
       double best = step * t, cost = best;

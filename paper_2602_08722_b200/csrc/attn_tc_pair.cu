@@ -379,7 +379,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
   tc_fence_before();
   if constexpr (MODE == kPartsCluster) {
     cluster_sync_all();                                       // every part's result is in its shared memory
-    if (warp < 8) attn_merge_cluster<D>(P, smem, part_ml, warp, lane, 2, (int)rank, n_parts, blockIdx.y % n_parts, qr, s, out, lse);
+    attn_merge_cluster<D>(P, smem, part_ml, warp, kAttnThreads / 32, lane, 2, (int)rank, n_parts, blockIdx.y % n_parts, qr, s, out, lse);
   }
   cluster_sync_all();                                         // the other CTA's MMAs no longer read this CTA
   if (warp == kQkWarp) tmem_dealloc_pair(tmem_base, 512);

@@ -561,8 +561,7 @@ __device__ __forceinline__ void attn_split_epilogue(const DevParams& P, int job,
 
 // The same with the parts of a row block in one cluster: every part leaves its result in its own shared memory, and after a
 // cluster barrier each adds up an equal share of the rows, in part order, reading the others through distributed shared
-// memory.  The merge is bound by the latency of those reads, so a warp issues the reads of four rows of every part before it
-// uses any.  Against results through global memory, an arrival counter and a merge by the last part to arrive (five
+// memory.  Against results through global memory, an arrival counter and a merge by the last part to arrive (five
 // dependent L2 round trips) it is about 6 us shorter; `attn_plan` has the times.
 constexpr int kPartPitch = 132;                  // floats per row: 16 bytes off a multiple of the banks
 
@@ -586,72 +585,50 @@ __device__ __forceinline__ void attn_part_to_smem(unsigned char* smem, float* ml
   ml[x * 256 + 128 + row_in_tile] = have ? l_run : 0.f;
 }
 
-// One of 8 warps; the CTA of part p with this CTA's head has cluster rank p * stride + offset.  A warp takes kU rows at a
-// time, four elements of a row per lane.
+// One of n_warps warps; the CTA of part p with this CTA's rows has cluster rank p * stride + offset.  A row at a time, four
+// elements per lane, in a loop kept small: this code runs once per launch, and instructions have to be fetched too (four rows
+// side by side per warp, 10 KB of code, took 7.3 us for 32 rows of a CTA and four parts; this form 4.8: the reads of other
+// CTAs' shared memory, 50 KB at about 14 bytes per clock).
 template <int D>
-__device__ __forceinline__ void attn_merge_cluster(const DevParams& P, unsigned char* smem, float* ml, int warp, int lane, int stride,
-                                                   int offset, int parts, int part, const QRows& qr, int s,
+__device__ __forceinline__ void attn_merge_cluster(const DevParams& P, unsigned char* smem, float* ml, int warp, int n_warps, int lane,
+                                                   int stride, int offset, int parts, int part, const QRows& qr, int s,
                                                    __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
-  constexpr int kU = 4, kMaxParts = 4;
+  constexpr int kMaxParts = 4;
+  static_assert(D == 128, "four elements per lane");
   const uint32_t o0 = smem_u32(smem), ml0 = smem_u32(ml);
   const int rows_a = qr.count(P, 0), rows = rows_a + qr.count(P, 1);
-  const auto row_of = [&](int i) { return i < rows_a ? i : 128 + i - rows_a; };       // i-th row that exists -> tile * 128 + row
-  for (int j = warp * kU; part + parts * j < rows; j += 8 * kU) {
-    float m[kU], l[kU], wgt[kU], M[kU], L[kU];
-    float4 acc[kU];
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {                           // lane p holds part p's m and l
-      const int R = row_of(min(part + parts * (j + u), rows - 1)), x = R >> 7, lr = R & 127;
-      const uint32_t at = map_to_cta(ml0 + (uint32_t)(x * 256 + lr) * 4u, (uint32_t)(min(lane, parts - 1) * stride + offset));
-      m[u] = ld_cluster_f(at);
-      l[u] = ld_cluster_f(at + 512u);
-      acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+#pragma unroll 1
+  for (int i = part + parts * warp; i < rows; i += parts * n_warps) {
+    const int x = i < rows_a ? 0 : 1, lr = x ? i - rows_a : i;                  // i-th row that exists
+    const uint32_t at = map_to_cta(ml0 + (uint32_t)(x * 256 + lr) * 4u, (uint32_t)(min(lane, parts - 1) * stride + offset));
+    float m = ld_cluster_f(at), l = ld_cluster_f(at + 512u);                    // lane p: part p's
     // every part's elements before the first use of any (what a part without a result has there is not used)
-    float4 v[kMaxParts][kU];
+    float4 v[kMaxParts];
 #pragma unroll
     for (int p = 0; p < kMaxParts; ++p)
-      if (p < parts) {
+      v[p] = ld_cluster_f4(map_to_cta(o0 + (uint32_t)((x * 128 + lr) * kPartPitch + 4 * lane) * 4u, (uint32_t)(min(p, parts - 1) * stride + offset)));
+    if (lane >= parts) { m = -INFINITY; l = 0.f; }
+    float M = m;
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const int R = row_of(min(part + parts * (j + u), rows - 1));
-          v[p][u] = ld_cluster_f4(map_to_cta(o0 + (uint32_t)(R * kPartPitch + 4 * (lane & (D / 4 - 1))) * 4u, (uint32_t)(p * stride + offset)));
-        }
-      }
+    for (int o = 4; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
+    M = __shfl_sync(0xFFFFFFFFu, M, 0);
+    const float wgt = m == -INFINITY ? 0.f : ex2(m - M);
+    float L = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      if (lane >= parts) { m[u] = -INFINITY; l[u] = 0.f; }
-      M[u] = m[u];
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) M[u] = fmaxf(M[u], __shfl_xor_sync(0xFFFFFFFFu, M[u], o));
-      M[u] = __shfl_sync(0xFFFFFFFFu, M[u], 0);
-      wgt[u] = m[u] == -INFINITY ? 0.f : ex2(m[u] - M[u]);
-      L[u] = 0.f;
+    for (int p = 0; p < kMaxParts; ++p) {                                       // (lanes past the parts hold a weight of 0)
+      const float w = __shfl_sync(0xFFFFFFFFu, wgt, p);
+      const float4 o = w != 0.f ? v[p] : make_float4(0.f, 0.f, 0.f, 0.f);
+      L = fmaf(w, __shfl_sync(0xFFFFFFFFu, l, p), L);
+      acc.x = fmaf(w, o.x, acc.x); acc.y = fmaf(w, o.y, acc.y);
+      acc.z = fmaf(w, o.z, acc.z); acc.w = fmaf(w, o.w, acc.w);
     }
-#pragma unroll
-    for (int p = 0; p < kMaxParts; ++p) {
-      if (p < parts) {
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const float w = __shfl_sync(0xFFFFFFFFu, wgt[u], p);
-          const float4 o = w != 0.f ? v[p][u] : make_float4(0.f, 0.f, 0.f, 0.f);
-          L[u] = fmaf(w, __shfl_sync(0xFFFFFFFFu, l[u], p), L[u]);
-          acc[u].x = fmaf(w, o.x, acc[u].x); acc[u].y = fmaf(w, o.y, acc[u].y);
-          acc[u].z = fmaf(w, o.z, acc[u].z); acc[u].w = fmaf(w, o.w, acc[u].w);
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      if (part + parts * (j + u) >= rows) break;
-      const int R = row_of(part + parts * (j + u)), h = qr.head(P, R & 127), p = qr.position(P, R >> 7, R & 127);
-      const float inv = 1.f / L[u];
-      const __nv_bfloat162 a = __floats2bfloat162_rn(acc[u].x * inv, acc[u].y * inv), b = __floats2bfloat162_rn(acc[u].z * inv, acc[u].w * inv);
-      if (lane < D / 4)
-        *reinterpret_cast<uint2*>(out + (long long)s * P.o_sb + (long long)h * P.o_sh + (long long)p * P.o_st + 4 * lane) =
-            make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
-      if (lse && lane == 0) lse[((long long)s * P.n_q + h) * P.chunk + p] = (M[u] + log2f(L[u])) * 0.6931471805599453f;
-    }
+    const float inv = 1.f / L;
+    const __nv_bfloat162 a = __floats2bfloat162_rn(acc.x * inv, acc.y * inv), b = __floats2bfloat162_rn(acc.z * inv, acc.w * inv);
+    const int h = qr.head(P, lr), p = qr.position(P, x, lr);
+    *reinterpret_cast<uint2*>(out + (long long)s * P.o_sb + (long long)h * P.o_sh + (long long)p * P.o_st + 4 * lane) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    if (lse && lane == 0) lse[((long long)s * P.n_q + h) * P.chunk + p] = (M + log2f(L)) * 0.6931471805599453f;
   }
 }
 
