@@ -191,43 +191,46 @@ score_keys_tc_kernel(DevParams P, ScoreArgs A, const __grid_constant__ CUtensorM
       if (!waited) grid_dependency_wait();
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      TileWalk w; w.seek(P, lo, hi);
-      int stage = 0; uint32_t phase = 0, q_phase = 0; int head_cur = -1;
-      int slot = 0; uint32_t acc_phase = 0;
-      const uint32_t q_base = smem_u32(q_smem), k_base = smem_u32(k_smem);
-      for (; w.valid(); w.next(P)) {
-        const int head = w.s * P.n_kv + w.kv;
-        if (head != head_cur) {
-          if (head_cur >= 0) mma_commit(q_empty);     // arrives when every MMA on the old Qbar is done
-          if (!mbar_wait(q_full, q_phase, wc)) break;
-          q_phase ^= 1;
-          head_cur = head;
-        }
-        if (!mbar_wait(&full[stage], phase, wc)) break;
-        if (!mbar_wait(&acc_empty[slot], acc_phase ^ 1, wc)) break;
-        tc_fence_after();
-        for (int p = 0; p < A.n_parts; ++p) {
-          const int n_mma = (p == A.n_parts - 1) ? (A.n_pad - p * 256) : 256;
-          const uint32_t idesc = idesc_bf16_f32(128, n_mma, false, false);
-          const uint32_t d_tmem = tmem_base + (uint32_t)((A.n_parts == 1 ? slot : p) * 256);
+    // ------------------------------------------------------------------ MMA issuer (the whole warp, one lane issues)
+    TileWalk w; w.seek(P, lo, hi);
+    int stage = 0; uint32_t phase = 0, q_phase = 0; int head_cur = -1;
+    int slot = 0; uint32_t acc_phase = 0;
+    const bool leader = elect_one();
+    const uint32_t tmem = (uint32_t)warp_uniform((int)tmem_base);
+    const uint64_t desc_q = smem_desc_sw128(smem_u32(q_smem), 16, 1024), desc_k = smem_desc_sw128(smem_u32(k_smem), 16, 1024);
+    for (; w.valid(); w.next(P)) {
+      const int head = w.s * P.n_kv + w.kv;
+      if (head != head_cur) {
+        if (head_cur >= 0 && leader) mma_commit(q_empty);     // arrives when every MMA on the old Qbar is done
+        if (!warp_all(mbar_poll(q_full, q_phase, wc))) break;
+        q_phase ^= 1;
+        head_cur = head;
+      }
+      if (!warp_all(mbar_poll(&full[stage], phase, wc) && mbar_poll(&acc_empty[slot], acc_phase ^ 1, wc))) break;
+      tc_fence_after();
+      const uint64_t dk = desc_k + (uint64_t)((uint32_t)stage * (kStageBytes >> 4));
+      for (int p = 0; p < A.n_parts; ++p) {
+        const int n_mma = (p == A.n_parts - 1) ? (A.n_pad - p * 256) : 256;
+        const uint32_t idesc = idesc_bf16_f32(128, n_mma, false, false);
+        const uint32_t d_tmem = tmem + (uint32_t)((A.n_parts == 1 ? slot : p) * 256);
+        const uint64_t dq = desc_q + (uint64_t)((uint32_t)(p * A.box_rows * 128) >> 4);
 #pragma unroll
-          for (int h = 0; h < HALVES; ++h) {
+        for (int h = 0; h < HALVES; ++h) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              const uint64_t a_desc = smem_desc_sw128(k_base + stage * kStageBytes + h * kHalfBytes + kk * 32, 16, 1024);
-              const uint64_t b_desc = smem_desc_sw128(q_base + h * q_half_bytes + p * A.box_rows * 128 + kk * 32, 16, 1024);
-              mma_ss(d_tmem, a_desc, b_desc, idesc, (h | kk) ? 1u : 0u);
-            }
-          }
+          for (int kk = 0; kk < 4; ++kk)
+            if (leader)
+              mma_ss(d_tmem, dk + (uint64_t)((h * kHalfBytes + kk * 32) >> 4), dq + (uint64_t)((uint32_t)(h * q_half_bytes + kk * 32) >> 4),
+                     idesc, (h | kk) ? 1u : 0u);
         }
+      }
+      if (leader) {
         mma_commit(&empty[stage]);
         mma_commit(&acc_full[slot]);
-        if (++stage == A.stages) { stage = 0; phase ^= 1; }
-        if (++slot == slots) { slot = 0; acc_phase ^= 1; }
       }
+      if (++stage == A.stages) { stage = 0; phase ^= 1; }
+      if (++slot == slots) { slot = 0; acc_phase ^= 1; }
     }
+    __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue: one key per thread.
     // Two groups of four warps take alternate tiles (group g = accumulator slot g), because one tile's epilogue
