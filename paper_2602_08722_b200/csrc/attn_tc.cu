@@ -494,6 +494,11 @@ quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const A
   return cudaGetLastError() == cudaSuccess ? QUOKA_OK : QUOKA_ERR_CUDA;
 }
 
+// A call of fewer blocks of 256 positions of a head than SMs needs the scratch of its plan; a larger one may do without (the
+// row blocks then stay whole), also where its heads packed into tiles make fewer CTAs than SMs.
+bool attn_scratch_required(const quoka_params* p) {
+  return (long long)p->n_q_heads * p->batch * ((p->chunk_len + 255) / 256) < device_sm_count();
+}
 bool attn_below_a_wave(const quoka_params* p) { return attn_shape(p, 2).jobs < device_sm_count(); }
 
 bool attn_tc_supported(const quoka_params* p) {

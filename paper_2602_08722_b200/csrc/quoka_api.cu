@@ -79,7 +79,7 @@ static size_t attn_scratch_bytes(const quoka_params* p) {
 // only levels the last wave and may be missing: it does not grow with the chunk or the context (2048 queries of 32 heads at
 // 4096 rows have none, 1500 have 12 MiB), and a workspace made for the longest chunk serves the shorter ones.
 static size_t workspace_least(const quoka_params* p) {
-  return carve(p, nullptr).total + (attn_below_a_wave(p) ? attn_scratch_bytes(p) : 0);
+  return carve(p, nullptr).total + (attn_scratch_required(p) ? attn_scratch_bytes(p) : 0);
 }
 
 static quoka_status validate(const quoka_params* p) {

@@ -23,6 +23,7 @@ size_t attn_split_counter_bytes(const quoka_params* p, const AttnPlan& plan);
 bool attn_tc_supported(const quoka_params* p);
 // Whether the attention grid (256 query rows per CTA) has fewer CTAs than the GPU has SMs.
 bool attn_below_a_wave(const quoka_params* p);
+bool attn_scratch_required(const quoka_params* p);
 quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                             const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                             bool after_selection, const AttnPlan& plan);

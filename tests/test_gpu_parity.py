@@ -767,6 +767,7 @@ def test_attention_with_its_lightest_row_blocks_in_parts(n_q, n_kv, d, C, T, B):
 @pytest.mark.parametrize("n_q,n_kv,d,C,tail,T", [
     (32, 8, 128, 2048, 1500, 4096),       # no parts for the whole chunk, 12 MiB of them for the rest of the prompt
     (40, 8, 64, 2048, 1270, 8192),        # parts in both, more of them for the shorter chunk
+    (80, 10, 64, 2048, 260, 8192),        # 160 blocks of 256 positions, 90 CTAs of packed heads
 ])
 def test_a_workspace_made_for_the_longest_chunk_serves_the_shorter_ones(n_q, n_kv, d, C, tail, T):
     """The scratch of grids of a wave or more may be missing: what was sized for another chunk of the same prompt is accepted,
