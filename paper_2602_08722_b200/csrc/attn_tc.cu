@@ -340,23 +340,22 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
 // Split attention.  A grid of fewer CTAs than SMs (short chunks, few heads) leaves part of the GPU idle while
 // every CTA walks its whole key sequence; cutting each row block's tiles into parts, one CTA each, fills it.
 // The number of parts minimises  waves(parts) * (tiles / parts + 6):  a part costs about six tiles' time of
-// start-up, partial results and merge (the model fits the measured times of 1 to 5 parts on grids of 32 to 288 CTAs
-// within 3 %), parts keep at least six tiles, and a split has to promise 3 % to be taken.
+// start-up, partial results and merge, parts keep at least six tiles, and a split has to promise 3 % to be taken.
 // The pair kernel's parts merge in a cluster of 2 * parts CTAs where all of a grid's clusters are resident at once: the
-// device holds 33, 22 or 15 of 4, 6 or 8 CTAs of this shared memory, the limits leave one or two free (a second wave costs
-// more than any split gives: 16 clusters of eight took 38 us where the 14 that fit take 30).  A part then costs about one
-// tile on top of the walk against parts through memory, and four and a half against a whole row block (a sparse part's step
-// is slower than a whole row block's).  Sparse attention, whole or parts through memory / clusters: 32 heads, 128 queries
-// over 2396 listed rows 32.8 / 24.5 us, over 1024 22.0 / 17.2; 256 over 3600 42.9 / 38.0; 512 over 1966 41.6 / 36.4; 8 heads,
-// 256 queries over 1024 25.3 / 19.6, over 2048 35.7 / 23.9.  Below the line: 8 heads, 256 over 512 18.5 / 19.4; 32 heads,
-// 512 queries over 1024 in a whole prefill call 58.0 / 59.2.  Dense, 8 heads, 256 over 4096 37.0 / 30.4.
+// device holds 33, 22 or 15 of 4, 6 or 8 CTAs of this shared memory, the limits leave some free (a second wave costs
+// more than any split gives).  A part then costs about one tile on top of the walk against parts through memory, and six
+// against a whole row block.  Whole prefill calls, whole row blocks / parts through memory / in clusters: 32 heads of 8 KV heads, 128 queries
+// over 2396 listed rows 55.6 / 52.7 / 45.9 us, 256 over 3600 79.1 / 71.7 / 67.0; 8 heads of 2, 256 queries over 1024
+// 38.3 / 38.5 / 35.8, over 2048 50.6 / 48.4 / 39.7, dense over 4096 45.3 / 30.9 / 22.8.  Beyond the lines: 32 heads, 128
+// queries over 1024 36.5 / 36.7 / 37.9, 512 over 1966 (32 clusters) 59.3 / 64.6 / 62.3.
+// One Q tile per CTA instead of two: 32 heads, 64 queries over 2396 rows 61.0 -> 53.9 us, 512 over 1024 49.5 -> 46.1.
 // A grid of q full waves and a rest has its lightest row blocks, as many as the rest, cut instead: the whole ones then
 // end after about q waves and the parts level the end.  The model is the total work over the SMs plus a third of a part
-// for the uneven end, against q + 1 waves of average jobs; list-scheduling simulations agree with it within 4 %.  Dense
-// calls take 3 % promised, sparse ones 7 % and equal lengths (their parts run a quarter slower per tile than whole row
-// blocks, and a batch's budgets differ): 32 heads, without / with parts: 1536 queries at 64K, a quarter listed 508 / 420 us,
-// 4096 at 128K 1039 / 990, 3072 at 32K, half listed 789 / 746; 40 heads, 1536 at 32K, promised 4 %: 290 / 309; dense 1536 at
-// 32K 920 / 692, 2048 at 32K 942 / 908, 4096 at 128K 7412 / 6689.
+// for the uneven end, against q + 1 waves of average jobs; it is 3 to 15 % too low (parts run slower per tile than whole row
+// blocks, and at the power cap an idle SM's share goes to the others), so dense calls take 10 % promised, sparse ones 15 %
+// and equal lengths (a batch's budgets differ).  32 heads, without / with parts, and what the model says: 1536 queries at
+// 64K, a quarter listed 470 / 396 us (0.72), dense 1536 at 32K 829 / 649 (0.70), dense 4096 at 128K 7359 / 6670 (0.88);
+// beyond the line dense 2048 at 32K 860 / 916 (0.94), 40 heads, 1536 at 32K 209 / 220 (0.92).
 // Partial results above 128 MB are not written: such jobs have waves enough.
 // How the query rows of a call are laid out: see QRows.
 struct AttnShape {
@@ -406,8 +405,8 @@ static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
       if (a.ctas == 2) {
         for (int parts = 2; parts <= 4 && parts <= tiles / 2; ++parts) {
           cost = step * t / parts + 1.0;
-          const double limit = std::min(0.95 * best, 0.97 * step * t - 4.5);
-          if (a.jobs / 2 <= (parts == 2 ? 32 : parts == 3 ? 20 : 14) && cost < limit) {
+          const double limit = std::min(0.95 * best, 0.97 * step * t - 6.0);
+          if (a.jobs / 2 <= (parts == 2 ? 28 : parts == 3 ? 20 : 14) && cost < limit) {
             cand.split_rb = (int)a.blocks; cand.parts = parts; cand.in_cluster = true; best = cost / 0.95;
           }
         }
@@ -422,7 +421,7 @@ static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
   if (rest == 0 || (sparse && p->batch > 1)) return plan;
   const long long split = (rest + per_rb - 1) / per_rb;                      // row blocks to cut; block r has about (r + 1) * own of its own tiles
   const double t_all = tiles + 2 + 0.5 * own * n_rb, t_whole = tiles + 2 + 0.5 * own * (split + n_rb), t_split = tiles + 2 + 0.5 * own * split;
-  double best = (sparse ? 0.93 : 0.97) * (double)(q + 1) * t_all;
+  double best = (sparse ? 0.85 : 0.90) * (double)(q + 1) * t_all;
   for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
     const double t_part = t_split / parts + kPartCost;
     const double cost = ((double)(jobs - split * per_rb) * t_whole + (double)(split * per_rb * parts) * t_part) / (double)sms + 0.3 * t_part;
