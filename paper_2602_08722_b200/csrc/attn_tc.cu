@@ -339,12 +339,12 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
 // ---------------------------------------------------------------------------------------------- host
 // Split attention.  A grid of fewer CTAs than SMs (short chunks, few heads) leaves part of the GPU idle while
 // every CTA walks its whole key sequence; cutting each row block's tiles into parts, one CTA each, fills it.
-// The number of parts minimises  waves(parts) * (tiles / parts + 6):  a part costs about six tiles' time of
+// The number of parts minimises  waves(parts) * (tiles / parts + 10):  a part costs about ten tiles' time of
 // start-up, partial results and merge, parts keep at least six tiles, and a split has to promise 3 % to be taken.
 // The pair kernel's parts merge in a cluster of 2 * parts CTAs where all of a grid's clusters are resident at once: the
 // device holds 33, 22 or 15 of 4, 6 or 8 CTAs of this shared memory, the limits leave some free (a second wave costs
 // more than any split gives).  A part then costs about one tile on top of the walk against parts through memory, and six
-// against a whole row block.  Whole prefill calls, whole row blocks / parts through memory / in clusters: 32 heads of 8 KV heads, 128 queries
+// (one Q tile per CTA: four and a half) against a whole row block.  Whole prefill calls, whole row blocks / parts through memory / in clusters: 32 heads of 8 KV heads, 128 queries
 // over 2396 listed rows 55.6 / 52.7 / 45.9 us, 256 over 3600 79.1 / 71.7 / 67.0; 8 heads of 2, 256 queries over 1024
 // 38.3 / 38.5 / 35.8, over 2048 50.6 / 48.4 / 39.7, dense over 4096 45.3 / 30.9 / 22.8.  Beyond the lines: 32 heads, 128
 // queries over 1024 36.5 / 36.7 / 37.9, 512 over 1966 (32 clusters) 59.3 / 64.6 / 62.3.
@@ -378,7 +378,7 @@ static AttnShape attn_shape(const quoka_params* p, int q_tiles) {
   return a;
 }
 static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
-  constexpr double kPartCost = 6.0, kOneTile = 0.9;
+  constexpr double kPartCost = 6.0, kPartCostBelow = 10.0, kOneTile = 0.9;
   AttnPlan plan;
   if (p->dtype != QUOKA_BF16 || p->impl == QUOKA_IMPL_SIMT || p->chunk_len <= 1) return plan;
   const long long sms = device_sm_count();
@@ -398,14 +398,14 @@ static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
       double best = step * t, cost = best;
       for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
         const long long waves = (a.jobs * parts + sms - 1) / sms;
-        cost = (double)waves * (step * t / parts + kPartCost);
+        cost = (double)waves * (step * t / parts + kPartCostBelow);
         if (cost < 0.97 * best) { cand.split_rb = (int)a.blocks; cand.parts = parts; cand.in_cluster = false; best = cost; }
       }
       // the pair kernel's, in clusters
       if (a.ctas == 2) {
         for (int parts = 2; parts <= 4 && parts <= tiles / 2; ++parts) {
           cost = step * t / parts + 1.0;
-          const double limit = std::min(0.95 * best, 0.97 * step * t - 6.0);
+          const double limit = std::min(0.95 * best, 0.97 * step * t - (q_tiles == 1 ? 4.5 : 6.0));
           if (a.jobs / 2 <= (parts == 2 ? 28 : parts == 3 ? 20 : 14) && cost < limit) {
             cand.split_rb = (int)a.blocks; cand.parts = parts; cand.in_cluster = true; best = cost / 0.95;
           }
