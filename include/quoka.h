@@ -124,14 +124,15 @@ quoka_status quoka_kv_budget_cap(const quoka_params* p, int32_t* cap);
  * partial results of the split attention kernel (the keys of the lightest row
  * blocks, or of all, are cut into up to 8 parts, one CTA each, and added up in part
  * order: results are reproducible from run to run, and differ from the unsplit
- * kernel's in the last bits only).  It comes last and is sized for whichever of
- * quoka_prefill_chunk / quoka_sparse_attn and quoka_dense_chunk_attn needs more.
- * On grids of a wave or more (batch * n_Q * ceil(C / 256) no less than the number of
- * SMs) it is at most 128 MiB, mostly the dense call's (32 heads, C 2048, 32768 cached
- * rows: 65 MiB, nothing for the sparse call), and may be missing in part or
- * altogether: a call that does not find room for its own parts leaves the row blocks
- * whole.  So a workspace made for the longest chunk of a prompt serves the shorter
- * ones, although their size by this function may be larger. */
+ * kernel's in the last bits only).  It comes last, is sized for whichever of
+ * quoka_prefill_chunk / quoka_sparse_attn and quoka_dense_chunk_attn needs more, and
+ * may be missing in part or altogether: a call that does not find room for its own
+ * parts leaves the row blocks whole.  A workspace made for the longest chunk of a prompt
+ * therefore serves the shorter ones, and the size includes what these need to run as fast
+ * (dense calls over fewer than 16384 cached rows excepted): 32 heads over 8, C 2048,
+ * 32768 cached rows, a budget of 3932: 72 MiB, most of it for dense chunks of 800 to 900
+ * queries.  Where batch * n_Q * ceil(C / 256) is no less than the number of SMs, it is at
+ * most 128 MiB. */
 quoka_status quoka_workspace_size(const quoka_params* p, size_t* bytes);
 
 /* Alg. 1, "Query Sub-selection", then the normalisation and the mean over the G

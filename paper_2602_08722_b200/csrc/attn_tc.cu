@@ -356,7 +356,9 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
 // and equal lengths (a batch's budgets differ).  32 heads, without / with parts, and what the model says: 1536 queries at
 // 64K, a quarter listed 470 / 396 us (0.72), dense 1536 at 32K 829 / 649 (0.70), dense 4096 at 128K 7359 / 6670 (0.88);
 // beyond the line dense 2048 at 32K 860 / 916 (0.94), 40 heads, 1536 at 32K 209 / 220 (0.92).
-// Partial results above 128 MB are not written: such jobs have waves enough.
+// Partial results above 128 MiB are not written where a call has as many blocks of 256 positions of a head as there are SMs
+// (most such have waves enough; of those whose heads packed into tiles make fewer CTAs, eight parts of 127 CTAs and more,
+// which only dense calls over 94,000 rows and more would take, for a promised tenth).
 // How the query rows of a call are laid out: see QRows.
 struct AttnShape {
   int pack, span;                  // heads and chunk positions of a Q tile
@@ -384,6 +386,8 @@ static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
   const long long sms = device_sm_count();
   if (sms <= 0) return plan;
   const AttnShape two = attn_shape(p, 2);
+  // at least as many blocks of 256 positions of a head as SMs
+  const bool bounded = (long long)p->n_q_heads * p->batch * ((p->chunk_len + 255) / 256) >= sms;
   if (two.jobs < sms) {
     double best_of_all = 0;
     for (int q_tiles = 2; q_tiles >= 1; --q_tiles) {
@@ -399,7 +403,9 @@ static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
       for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
         const long long waves = (a.jobs * parts + sms - 1) / sms;
         cost = (double)waves * (step * t / parts + kPartCostBelow);
-        if (cost < 0.97 * best) { cand.split_rb = (int)a.blocks; cand.parts = parts; cand.in_cluster = false; best = cost; }
+        AttnPlan next = cand;
+        next.split_rb = (int)a.blocks; next.parts = parts;
+        if (cost < 0.97 * best && (!bounded || attn_split_partial_bytes(p, next) <= kMostAttnPartials)) { cand = next; best = cost; }
       }
       // the pair kernel's, in clusters
       if (a.ctas == 2) {
@@ -427,7 +433,7 @@ static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
     const double cost = ((double)(jobs - split * per_rb) * t_whole + (double)(split * per_rb * parts) * t_part) / (double)sms + 0.3 * t_part;
     AttnPlan cand;
     cand.split_rb = (int)split; cand.parts = parts;
-    if (cost < best && attn_split_partial_bytes(p, cand) <= ((size_t)128 << 20)) { best = cost; plan = cand; }
+    if (cost < best && attn_split_partial_bytes(p, cand) <= kMostAttnPartials) { best = cost; plan = cand; }
   }
   return plan;
 }
@@ -493,12 +499,10 @@ quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const A
   return cudaGetLastError() == cudaSuccess ? QUOKA_OK : QUOKA_ERR_CUDA;
 }
 
-// A call of fewer blocks of 256 positions of a head than SMs needs the scratch of its plan; a larger one may do without (the
-// row blocks then stay whole), also where its heads packed into tiles make fewer CTAs than SMs.
-bool attn_scratch_required(const quoka_params* p) {
-  return (long long)p->n_q_heads * p->batch * ((p->chunk_len + 255) / 256) < device_sm_count();
-}
 bool attn_below_a_wave(const quoka_params* p) { return attn_shape(p, 2).jobs < device_sm_count(); }
+// (the model's cost of a plan with parts is above q waves of average jobs, its line at most 0.9 (q + 1))
+bool attn_may_have_parts(const quoka_params* p) { return attn_shape(p, 2).jobs < 10ll * device_sm_count(); }
+int attn_least_block(const quoka_params* p) { return attn_shape(p, 1).block; }
 
 bool attn_tc_supported(const quoka_params* p) {
   if (p->dtype != QUOKA_BF16) return false;

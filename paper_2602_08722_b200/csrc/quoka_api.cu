@@ -1,5 +1,6 @@
 // Host side of the C ABI: argument validation, workspace carving, launch sequencing.
 // Nothing here allocates device memory or synchronises (except quoka_last_device_status).
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -66,20 +67,34 @@ static Workspace carve(const quoka_params* p, void* ws, size_t ws_bytes = 0, con
   return w;
 }
 
+static size_t plan_scratch_bytes(const quoka_params* p, const AttnPlan& plan) {
+  return align_up(attn_split_counter_bytes(p, plan)) + align_up(attn_split_partial_bytes(p, plan));
+}
 // The scratch of the larger of the two plans an attention call of this problem may follow.
 static size_t attn_scratch_bytes(const quoka_params* p) {
-  size_t bytes = 0;
-  for (const AttnPlan& plan : {attn_plan_sparse(p, budget_cap_of(p)), attn_plan_dense(p)}) {
-    const size_t b = align_up(attn_split_counter_bytes(p, plan)) + align_up(attn_split_partial_bytes(p, plan));
-    bytes = b > bytes ? b : bytes;
-  }
-  return bytes;
+  return std::max(plan_scratch_bytes(p, attn_plan_sparse(p, budget_cap_of(p))), plan_scratch_bytes(p, attn_plan_dense(p)));
 }
-// The least a call takes.  A grid below a wave needs its scratch (its parts are what fills the GPU); that of a larger grid
-// only levels the last wave and may be missing: it does not grow with the chunk or the context (2048 queries of 32 heads at
-// 4096 rows have none, 1500 have 12 MiB), and a workspace made for the longest chunk serves the shorter ones.
-static size_t workspace_least(const quoka_params* p) {
-  return carve(p, nullptr).total + (attn_scratch_required(p) ? attn_scratch_bytes(p) : 0);
+// What the shorter chunks of the same prompt take: the last chunk of a prompt comes with the workspace of its longest, and
+// parts are what fills the GPU there.  Dense calls count from 16384 cached rows on: over shorter caches parts are a matter of
+// some tens of microseconds; and no more than a grid of a wave or more may take.  A plan depends on the chunk's length
+// through the number of its smallest row blocks, and through the bound on its scratch, which holds from some length on; so both
+// ends of every such block are asked, until the grid is so large that no plan has parts.
+static size_t attn_scratch_of_shorter_chunks(const quoka_params* p) {
+  constexpr int kDenseFrom = 16384;
+  size_t bytes = 0;
+  const auto take = [&](const quoka_params* t, const AttnPlan& plan) {
+    if (attn_split_partial_bytes(t, plan) <= kMostAttnPartials) bytes = std::max(bytes, plan_scratch_bytes(t, plan));
+  };
+  quoka_params t = *p;
+  const int block = attn_least_block(p);
+  for (int first = 1;; first += block) {
+    for (int c : {first, first + block - 1}) {
+      t.chunk_len = c;
+      if (c >= p->chunk_len || !attn_may_have_parts(&t)) return bytes;
+      take(&t, attn_plan_sparse(&t, budget_cap_of(&t)));
+      if (p->max_ctx_len >= kDenseFrom) take(&t, attn_plan_dense(&t));
+    }
+  }
 }
 
 static quoka_status validate(const quoka_params* p) {
@@ -126,7 +141,7 @@ quoka_status check_prefill_args(const quoka_params* p, const void* q, const void
 
 static quoka_status check_ws(const quoka_params* p, void* ws, size_t ws_bytes) {
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0) return QUOKA_ERR_WORKSPACE;
-  if (ws_bytes < workspace_least(p)) return QUOKA_ERR_WORKSPACE;
+  if (ws_bytes < carve(p, nullptr).total) return QUOKA_ERR_WORKSPACE;       // the attention's scratch may be missing
   return QUOKA_OK;
 }
 
@@ -305,7 +320,7 @@ quoka_status quoka_workspace_size(const quoka_params* p, size_t* bytes) {
   if (!bytes) return QUOKA_ERR_INVALID_ARG;
   quoka_status st = validate(p);
   if (st != QUOKA_OK) return st;
-  *bytes = carve(p, nullptr).total + attn_scratch_bytes(p);
+  *bytes = carve(p, nullptr).total + std::max(attn_scratch_bytes(p), attn_scratch_of_shorter_chunks(p));
   return QUOKA_OK;
 }
 

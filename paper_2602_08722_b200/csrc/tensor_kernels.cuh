@@ -15,6 +15,7 @@ quoka_status launch_score_keys_tc(const quoka_params* p, const DevParams& P, con
 // in_cluster: the parts of a row block are one cluster (and need no scratch)
 // q_tiles: Q tiles of a CTA
 struct AttnPlan { int split_rb = 0, parts = 1; bool in_cluster = false; int q_tiles = 2; };
+constexpr size_t kMostAttnPartials = (size_t)128 << 20;     // what a grid of a wave or more may take, see attn_plan
 AttnPlan attn_plan_sparse(const quoka_params* p, int budget_cap);
 AttnPlan attn_plan_dense(const quoka_params* p);
 // Scratch for the partial results
@@ -23,7 +24,9 @@ size_t attn_split_counter_bytes(const quoka_params* p, const AttnPlan& plan);
 bool attn_tc_supported(const quoka_params* p);
 // Whether the attention grid (256 query rows per CTA) has fewer CTAs than the GPU has SMs.
 bool attn_below_a_wave(const quoka_params* p);
-bool attn_scratch_required(const quoka_params* p);
+// Whether it is small enough for a plan with parts; chunk positions of the smallest row block that a plan may use
+bool attn_may_have_parts(const quoka_params* p);
+int attn_least_block(const quoka_params* p);
 quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P, const void* q, const void* k, const void* v,
                             const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                             bool after_selection, const AttnPlan& plan);

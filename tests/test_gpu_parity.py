@@ -794,6 +794,38 @@ def test_a_workspace_made_for_the_longest_chunk_serves_the_shorter_ones(n_q, n_k
     assert e.value.status == api.ERR_WORKSPACE
 
 
+@pytest.mark.parametrize("n_q,n_kv,d,tail", [
+    (32, 8, 128, 2), (32, 8, 128, 64), (32, 8, 128, 512), (32, 8, 128, 896), (32, 4, 64, 64), (32, 4, 64, 900), (32, 32, 128, 300),
+])
+def test_the_end_of_a_prompt_runs_in_the_workspace_of_its_longest_chunk(n_q, n_kv, d, tail):
+    """A chunk far below a wave after chunks of 2048: accepted, and with the bits of a call that has its own workspace, that is
+    in as many parts.  Without any room for parts it is accepted too, and right."""
+    T, C = 32768, 2048
+    gp = problem(1350 + tail, n_q=n_q, n_kv=n_kv, d=d, T=T, C=tail, n_retain=64, kv_budget=3932)
+    full = GpuProblem(synth.make_chunk_inputs(0, 1, n_q, n_kv, d, 8, C, "bf16"), 64, kv_budget=3932)
+    full.p.max_ctx_len, full.p.kv_rows = T, T + C
+    plain = api.QuokaParams.from_buffer_copy(gp.p)
+    plain.impl = api.IMPL_SIMT                                  # (no parts: the intermediates alone)
+    heads, rows = stratified_rows(n_q, tail, 64, 5)
+    q, k, v = gp.oracle_inputs(0)[:3]
+    got = []
+    for n in (gp.ws.numel(), api.quoka_workspace_size(full.p), api.quoka_workspace_size(plain)):
+        guarded = torch.full((n + (1 << 20),), 0x5A, dtype=torch.uint8, device="cuda")
+        guarded[:256] = 0
+        ws = guarded[:n]
+        api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, gp.k_idx, gp.k_cnt, ws)
+        sparse = gp.out.clone()
+        api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, None, ws)
+        torch.cuda.synchronize()
+        got.append((sparse, gp.out.clone()))
+        assert (guarded[n:] == 0x5A).all() and api.quoka_last_device_status(ws) == 0
+    assert torch.equal(got[1][0], got[0][0]) and torch.equal(got[1][1], got[0][1])
+    idx = [gp.k_idx[0, h].cpu().numpy() for h in range(n_kv)]
+    for sparse, dense in got[1:]:
+        check_attention(f64(sparse[0])[heads, rows], O.sparse_attention_rows(q, k, v, T, idx, heads, rows), "bf16")
+        check_attention(f64(dense[0])[heads, rows], O.sparse_attention_rows(q, k, v, T, [np.arange(T)] * n_kv, heads, rows), "bf16")
+
+
 @pytest.mark.parametrize("n_q,n_kv,C,T,B", [
     (8, 2, 256, [4096], 2048),          # 4 clusters of eight CTAs
     (8, 4, 257, [2500, 40], 2000),      # a row block of one row; a list shorter than a tile: parts without a tile
