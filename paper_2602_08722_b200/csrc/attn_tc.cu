@@ -63,7 +63,7 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
   // (SPLIT: grid.y = row blocks times the parts a row block's key tiles are cut into)
   const int n_parts = SPLIT ? P.attn_parts : 1;
   const int rb = (SPLIT ? P.attn_split_rb : P.attn_row_blocks) - 1 - blockIdx.y / n_parts;
-  const QRows qr{hg * P.attn_pack, rb * P.attn_qtiles * P.attn_span};
+  const QRows qr(P, hg, rb, 0, 1);
   const int kv = qr.head0 / P.group;
   AttnGeom g = make_geom<SPARSE>(P, s, qr.p0, 1);
   // SPLIT: this CTA walks the tiles [t_lo, t_hi) of the row block's sequence only and leaves, per row, a partial

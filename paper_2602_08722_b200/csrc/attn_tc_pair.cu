@@ -72,7 +72,7 @@ attn_tc_pair_body(const DevParams& P, const CUtensorMap& tm_q, const CUtensorMap
   // grid.y = row blocks (heaviest first), times the parts a row block's key tiles are cut into (SPLIT)
   const int n_parts = SPLIT ? P.attn_parts : 1;
   const int rb = (SPLIT ? P.attn_split_rb : P.attn_row_blocks) - 1 - blockIdx.y / n_parts;
-  const QRows qr{hg * P.attn_pack, (rb * 2 + (int)rank) * P.attn_qtiles * P.attn_span};
+  const QRows qr(P, hg, rb, (int)rank, 2);
   const int kv = qr.head0 / P.group;
   AttnGeom g = make_geom<SPARSE>(P, s, rb * 2 * P.attn_qtiles * P.attn_span, 2);
   int t_lo = 0;

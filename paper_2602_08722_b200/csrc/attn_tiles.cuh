@@ -58,18 +58,23 @@ __device__ __forceinline__ int longest_first(const DevParams& P, int z) {
 // left over, seven at most, are zero.  Against 128 positions of one head each: a chunk of 777 with eight heads per KV head
 // takes 49 tiles instead of 56, one of 68 with three heads 2 instead of 3, the chunk's own tiles that a row block walks end
 // 32 positions after its first row and not 256 (four heads), and any number of heads per KV head makes pairs.
-// A row block is the Q tiles of one CTA (A, or A and B), or of both CTAs of a pair (A, B of the first, A, B of the second).
+// A row block is the Q tiles of one CTA (A, or A and B), or of both CTAs of a pair: A of the first, A of the second, then the
+// two Bs, so that a row block of no more positions than two tiles have walks one tile in each CTA.
 struct QRows {
   int head0;            // first head
   int p0;               // first chunk position of this CTA
+  int step;             // from its tile A to its tile B
+  // of the CTA `rank` of `ctas` of row block rb
+  __device__ __forceinline__ QRows(const DevParams& P, int hg, int rb, int rank, int ctas)
+      : head0(hg * P.attn_pack), p0((rb * P.attn_qtiles * ctas + rank) * P.attn_span), step(ctas * P.attn_span) {}
   __device__ __forceinline__ static int groups(const DevParams& P) { return P.n_q / P.attn_pack; }
   __device__ __forceinline__ int position(const DevParams& P, int x, int row_in_tile) const {
-    return p0 + x * P.attn_span + row_in_tile / P.attn_pack;
+    return p0 + x * step + row_in_tile / P.attn_pack;
   }
   __device__ __forceinline__ int head(const DevParams& P, int row_in_tile) const { return head0 + row_in_tile % P.attn_pack; }
   // rows of tile x that exist: the first ones
   __device__ __forceinline__ int count(const DevParams& P, int x) const {
-    return x < P.attn_qtiles ? P.attn_pack * max(0, min(P.attn_span, P.chunk - p0 - x * P.attn_span)) : 0;
+    return x < P.attn_qtiles ? P.attn_pack * max(0, min(P.attn_span, P.chunk - p0 - x * step)) : 0;
   }
 };
 
@@ -80,7 +85,7 @@ __device__ __forceinline__ void load_q_tiles(const DevParams& P, const QRows& qr
   mbar_arrive_expect_tx(q_full, P.attn_qtiles * (D / 64) * 128 * P.attn_pack * P.attn_span);
   for (int x = 0; x < P.attn_qtiles; ++x)
     for (int hh = 0; hh < D / 64; ++hh)
-      tma_load_5d(q_smem + (x * (D / 64) + hh) * 16384, tm_q, q_full, hh * 64, 0, qr.p0 + x * P.attn_span, qr.head0 / P.attn_pack, s);
+      tma_load_5d(q_smem + (x * (D / 64) + hh) * 16384, tm_q, q_full, hh * 64, 0, qr.p0 + x * qr.step, qr.head0 / P.attn_pack, s);
 }
 // The rows left over: by the calling threads, before the barrier that the issuing warps pass.
 template <int D>
@@ -120,16 +125,15 @@ __device__ __forceinline__ AttnGeom make_geom(const DevParams& P, int s, int p, 
   AttnGeom g;
   g.T = __ldg(P.ctx_len + s);
   g.C = P.chunk;
-  const int span = P.attn_span, per_cta = P.attn_qtiles * span;
+  const int span = ctas * P.attn_span;
   g.active_b = P.attn_qtiles == 2 && p + span < g.C;
-  // last positions of any A tile and of any tile
-  const int last = min(p + ctas * per_cta, g.C) - 1;
-  const int last_a = min(p + span + (ctas == 2 && p + per_cta < g.C ? per_cta : 0), g.C) - 1;
+  // last positions of any tile and of any A tile
+  const int last = min(p + P.attn_qtiles * span, g.C) - 1, last_a = min(p + span, g.C) - 1;
   g.cnt = 0;
   if (SPARSE) {
     g.n_chunk = last / kKeyTile + 1;
     g.lead = g.n_chunk - (p / kKeyTile + 1);
-    g.skip_a = g.active_b ? g.n_chunk - (last_a / kKeyTile + 1) : 0;       // 0 or 1: a Q tile spans at most 128 positions
+    g.skip_a = g.active_b ? g.n_chunk - (last_a / kKeyTile + 1) : 0;       // 0 or 1, for a pair up to 2: a Q tile spans at most 128 positions
     g.n_known = g.n_chunk;
     g.n_dense = 0;
     g.resolved = false;

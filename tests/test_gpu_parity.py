@@ -736,6 +736,36 @@ def test_q_tiles_that_walk_many_key_tiles(n_q, n_kv, d, C, T, B, paged):
     assert api.quoka_last_device_status(gp.ws) == 0
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_q,n_kv,C", [
+    (4, 4, 129), (4, 4, 256),           # one tile in each CTA of a pair, the second one's of one row and full
+    (4, 4, 257), (4, 4, 385),           # a third tile of one row, a fourth: the As begin two key tiles after the Bs
+    (4, 4, 512), (4, 4, 700),           # full row blocks; a last one without Bs
+    (4, 2, 64), (4, 2, 65), (4, 2, 193),
+    (12, 4, 85), (12, 4, 169),          # 42 positions per tile
+])
+def test_rows_of_a_pair_of_ctas(n_q, n_kv, C):
+    """Few query heads per KV head at head_dim 128, chunk lengths at the edges of a pair's tiles: sparse (staged and fused, the
+    same bits) and dense, every row and its log-sum-exp against the oracle."""
+    T = 1500
+    gp = problem(2100 + C, n_q=n_q, n_kv=n_kv, T=T, C=C, n_retain=16, kv_budget=300)
+    gp.run_staged()
+    check_chain(gp, attn_rows=400)
+    staged = gp.out.clone()
+    gp.out.zero_()
+    api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+    torch.cuda.synchronize()
+    assert torch.equal(gp.out, staged)
+    gp.out.zero_()
+    api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, gp.lse, gp.ws)
+    torch.cuda.synchronize()
+    q, k, v, t = gp.oracle_inputs(0)
+    dense, lse = O.dense_chunk_attention(q, k, v, t)
+    check_attention(f64(gp.out[0]), dense, "bf16")
+    assert np.abs(f64(gp.lse[0]) - lse).max() <= 2e-3
+    assert api.quoka_last_device_status(gp.ws) == 0
+
+
 @pytest.mark.parametrize("n_q,n_kv,d,C,T,B", [
     (32, 8, 128, 1300, 9000, 5000),     # pairs, 6 row blocks: the lightest in parts after the whole ones, ragged last block
     (24, 8, 64, 1800, 7000, 6000),      # one-CTA kernel, 8 row blocks
