@@ -126,8 +126,8 @@ quoka_status quoka_kv_budget_cap(const quoka_params* p, int32_t* cap);
  * order: results are reproducible from run to run, and differ from the unsplit
  * kernel's in the last bits only).  It comes last, is sized for whichever of
  * quoka_prefill_chunk / quoka_sparse_attn and quoka_dense_chunk_attn needs more, and
- * may be missing in part or altogether: a call that does not find room for its own
- * parts leaves the row blocks whole.  A workspace made for the longest chunk of a prompt
+ * may be missing in part or altogether: a call then cuts its row blocks into fewer parts,
+ * or leaves them whole.  A workspace made for the longest chunk of a prompt
  * therefore serves the shorter ones, and the size includes what these need to run as fast
  * (dense calls over fewer than 16384 cached rows excepted): 32 heads over 8, C 2048,
  * 32768 cached rows, a budget of 3932: 72 MiB, most of it for dense chunks of 800 to 900

@@ -3,8 +3,8 @@
 // or, without an index list, over every cached row (Eq. 2, dense chunk attention).  bf16 in, fp32
 // softmax and accumulation, P rounded to bf16 for the PV product.
 //
-// This file: the kernel for head_dim 64, and the plan and the launches of both (attn_tc_pair.cu has the one for head_dim
-// 128).  A CTA owns two Q tiles (A, B) of 128 rows, or one, chunk positions of all heads of a KV group, and walks the key
+// This file: the kernel whose row blocks are those of one CTA, and the plan and the launches of both (attn_tc_pair.cu has the
+// one of pairs, for head_dim 128).  A CTA owns two Q tiles (A, B) of 128 rows, or one, chunk positions of all heads of a KV group, and walks the key
 // tiles (128 keys) once for both.  Roles:
 //   warps 0-3 / 4-7  softmax of Q tile A / B: one thread per query row, S read from tensor memory,
 //                    running max / sum in registers, P written back to tensor memory, lazy rescale of
@@ -23,27 +23,32 @@
 // leave it 128.  Sixteen softmax warps with half a row each (96 registers) were slower: 121 us where these take 100
 // (777 queries of 32 heads over 5000 listed rows, head_dim 64, the whole call).
 #include <algorithm>
+#include <cmath>
 #include "attn_tiles.cuh"
 
 namespace quoka {
 
-constexpr int kSlots = 8;
+template <int D>
+constexpr int kSlotsOf = D == 64 ? 8 : 5;                    // of 16 KB, 32 KB
+template <int D>
+constexpr size_t kAttnSmem = 1024 + (size_t)(2 + kSlotsOf<D>) * (D / 64) * 16384 + 512;
 
-template <bool SPARSE, bool SPLIT>
+template <int D, bool SPARSE, bool SPLIT>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __nv_bfloat16* __restrict__ kc,
                const __nv_bfloat16* __restrict__ vc, const int32_t* __restrict__ k_idx,
                const int32_t* __restrict__ k_cnt, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
-  constexpr int D = 64;
-  constexpr uint32_t kTileBytes = 128 * 128;                 // one Q / K / V tile: 128 rows x 128 B
-  // tensor memory (see "order of the products"): S | S | S | O_A | O_B, P in place
-  constexpr int NBUF = 3;
-  constexpr uint32_t O_COL = NBUF * 128;                     // (Q tile B's O is 64 columns on)
+  constexpr int kSlots = kSlotsOf<D>, HALVES = D / 64;
+  constexpr uint32_t kHalfBytes = 128 * 128;                 // 128 rows x 128 B
+  constexpr uint32_t kTileBytes = HALVES * kHalfBytes;       // one Q / K / V tile
+  // tensor memory (see "order of the products"): S | S | S | O_A | O_B, head_dim 128: S | S | O_A | O_B; P in place
+  constexpr int NBUF = D == 64 ? 3 : 2;
+  constexpr uint32_t O_COL = NBUF * 128;                     // (Q tile B's O is D columns on)
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  unsigned char* q_smem = smem;                               // [2][128][128 B]
-  unsigned char* kv_smem = smem + 2 * kTileBytes;             // [kSlots][128][128 B]
+  unsigned char* q_smem = smem;                               // [2][HALVES][128][128 B]
+  unsigned char* kv_smem = smem + 2 * kTileBytes;             // [kSlots][HALVES][128][128 B]
   uint64_t* bars = reinterpret_cast<uint64_t*>(kv_smem + (size_t)kSlots * kTileBytes);
   uint64_t* kv_full = bars;                 // [kSlots]  the loader threads' cp.async arrivals
   uint64_t* kv_empty = bars + kSlots;       // [kSlots]  MMA commit
@@ -154,7 +159,8 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     }
   } else if (warp < 8 + kLoaderWarps) {
     // ================================================================== K / V row loaders (gather)
-    // One warp instruction copies four whole rows (eight lanes x 16 bytes cover a 128-byte row); the row groups of a tile are dealt round-robin to the loader warps.
+    // One warp instruction copies four whole rows (eight lanes x 16 bytes cover a 128-byte row; head_dim 128: two); the row
+    // groups of a tile are dealt round-robin to the loader warps.
     const int lw = warp - 8;
     constexpr int PIECES = D / 8;                             // 16-byte pieces per row (16 or 8)
     constexpr int ROWS_PER_INSTR = 32 / PIECES;               // 2 or 4
@@ -162,8 +168,13 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
     constexpr int RPT = GROUPS / kLoaderWarps;                // row groups per warp
     const int c16 = lane % PIECES;                            // this thread's piece of the row
     const int rsub = lane / PIECES;
-    static_assert(kLoaderWarps * ROWS_PER_INSTR % 8 == 0, "a thread's rows all have the same swizzle");
-    const uint32_t thread_dst = (uint32_t)((lw * ROWS_PER_INSTR + rsub) * 128 + ((c16 ^ (lw * ROWS_PER_INSTR + rsub)) << 4));
+    // a thread's rows are 8 apart and have the same swizzle, or 4 apart, and it is turned by 4 rows for every second one
+    static_assert(kLoaderWarps * ROWS_PER_INSTR == (HALVES == 1 ? 8 : 4), "rows of a thread");
+    const int lrow = lw * ROWS_PER_INSTR + rsub;
+    const uint32_t thread_dst = (uint32_t)((c16 >> 3) * kHalfBytes + lrow * 128 + (((c16 & 7) ^ lrow) << 4));
+    const auto row_dst = [](uint32_t dst, int i) {
+      return (HALVES == 1 || (i & 1) == 0 ? dst : dst ^ 64u) + (uint32_t)(i * kLoaderWarps * ROWS_PER_INSTR * 128);
+    };
     const int32_t* idx = SPARSE ? k_idx + ((long long)s * P.n_kv + kv) * P.budget_cap : nullptr;
     uint32_t phase = 0;
     int slot = 0;
@@ -225,7 +236,9 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
             for (int sub = 0; sub < 2; ++sub) {
               int c1 = tr.first + sub * 64, c3 = s;
               if (P.page_size != 0) { c1 = 0; c3 = __ldg(table + (tr.first >> 6) + sub); }
-              tma_load_4d(dst + sub * 64 * 128, tm, &kv_full[slot], 0, c1, kv, c3);
+#pragma unroll
+              for (int hh = 0; hh < HALVES; ++hh)
+                tma_load_4d(dst + hh * kHalfBytes + sub * 64 * 128, tm, &kv_full[slot], hh * 64, c1, kv, c3);
             }
           } else {
             mbar_arrive(&kv_full[slot]);
@@ -249,13 +262,13 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
 #pragma unroll
           for (int i = 0; i < RPT; ++i) {
             const uint32_t off = __shfl_sync(0xFFFFFFFFu, offs[(i * ROWS_PER_INSTR) / 32], (i * ROWS_PER_INSTR + rsub) & 31);
-            cp_async_16(dst + (uint32_t)(i * kLoaderWarps * ROWS_PER_INSTR * 128), src_base + off);
+            cp_async_16(row_dst(dst, i), src_base + off);
           }
         } else {
 #pragma unroll
           for (int i = 0; i < RPT; ++i) {
             const uint32_t off = __shfl_sync(0xFFFFFFFFu, offs[(i * ROWS_PER_INSTR) / 32], (i * ROWS_PER_INSTR + rsub) & 31);
-            cp_async_16(dst + (uint32_t)(i * kLoaderWarps * ROWS_PER_INSTR * 128), src_base + (off == kNoRow ? 0u : off), off != kNoRow);
+            cp_async_16(row_dst(dst, i), src_base + (off == kNoRow ? 0u : off), off != kNoRow);
           }
         }
         // this thread's share of the slot is signalled by the copy engine itself when the bytes have landed:
@@ -302,14 +315,18 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
               const uint64_t da = desc_q + (uint64_t)(x * (kTileBytes >> 4));
               const uint64_t db = desc_k + (uint64_t)((uint32_t)ks * (kTileBytes >> 4));
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                if (leader) mma_ss(tmem + buf * 128, da + (uint64_t)(kk * 32 >> 4), db + (uint64_t)(kk * 32 >> 4), idesc_qk, kk ? 1u : 0u);
+              for (int hh = 0; hh < HALVES; ++hh)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                  const uint64_t o = (uint64_t)((hh * kHalfBytes + kk * 32) >> 4);
+                  if (leader) mma_ss(tmem + buf * 128, da + o, db + o, idesc_qk, (hh | kk) ? 1u : 0u);
+                }
               if (leader) mma_commit(&s_full[buf]);
             },
             release);
     } else {
       const uint32_t idesc_pv = idesc_bf16_f32(128, D, false, true);
-      const uint64_t desc_v = smem_desc_sw128(kv_base, 16, 1024);            // MN-major rows (V tiles)
+      const uint64_t desc_v = smem_desc_sw128(kv_base, HALVES == 1 ? 16 : kHalfBytes, 1024);      // MN-major rows (V tiles)
       uint32_t p_phase = 0;
       attn_issue_pv<NBUF, kSlots>(
           g, t_lo, [&]() { resolve(g, k_cnt, s); uniform_geom(g); }, acquire,
@@ -337,113 +354,164 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
 }
 
 // ---------------------------------------------------------------------------------------------- host
-// Split attention.  A grid of fewer CTAs than SMs (short chunks, few heads) leaves part of the GPU idle while
-// every CTA walks its whole key sequence; cutting each row block's tiles into parts, one CTA each, fills it.
-// The number of parts minimises  waves(parts) * (tiles / parts + 10):  a part costs about ten tiles' time of
-// start-up, partial results and merge, parts keep at least six tiles, and a split has to promise 3 % to be taken.
-// The pair kernel's parts merge in a cluster of 2 * parts CTAs where all of a grid's clusters are resident at once: the
-// device holds 33, 22 or 15 of 4, 6 or 8 CTAs of this shared memory, the limits leave some free (a second wave costs
-// more than any split gives).  A part then costs about one tile on top of the walk against parts through memory, and six
-// (one Q tile per CTA: four and a half) against a whole row block.  Whole prefill calls, whole row blocks / parts through memory / in clusters: 32 heads of 8 KV heads, 128 queries
-// over 2396 listed rows 55.6 / 52.7 / 45.9 us, 256 over 3600 79.1 / 71.7 / 67.0; 8 heads of 2, 256 queries over 1024
-// 38.3 / 38.5 / 35.8, over 2048 50.6 / 48.4 / 39.7, dense over 4096 45.3 / 30.9 / 22.8.  Beyond the lines: 32 heads, 128
-// queries over 1024 36.5 / 36.7 / 37.9, 512 over 1966 (32 clusters) 59.3 / 64.6 / 62.3.
-// One Q tile per CTA instead of two: 32 heads, 64 queries over 2396 rows 61.0 -> 53.9 us, 512 over 1024 49.5 -> 46.1.
+// How an attention call is laid out on the GPU: the form of its row blocks, and parts of their key tiles.
+//
+// Forms: two Q tiles per CTA or one; at head_dim 128 a row block is that of a pair of CTAs or of one.  A pair's step (a key tile)
+// is the faster one per row, one CTA's row blocks are smaller: chunks of a few positions, or few heads per KV head, leave
+// a pair with CTAs or tiles without rows.
+// Parts: a grid of fewer CTAs than SMs (short chunks, few heads) leaves part of the GPU idle while every CTA walks its whole
+// key sequence; cutting each row block's tiles into parts, one CTA (pair) each, fills it.  Parts merge through memory, or,
+// a pair's, in a cluster of 2 * parts CTAs where all of a grid's clusters are resident at once: the device holds 33, 22 or 15
+// of 4, 6 or 8 CTAs of this shared memory, the limits leave some free (a second wave costs more than any split gives).
+//
+// The model, in microseconds: start and end of a CTA, its steps, and what parts cost on top; the parts of a sparse call start
+// only when the selection has ended, whole row blocks walk the chunk's own tiles under it (half of these count).  Measured with
+// one thing varied at a time, a step with one / two Q tiles: a pair 1.09 / 1.39 us (listed rows 1.25 / 1.45), one CTA at head_dim
+// 128 1.02 / 1.91 (1.41 / 1.93: it gathers whole rows of its own), at head_dim 64 1.02 / 1.38 (1.13 / 1.42); parts through memory
+// 9 us for two and 20 for eight, at head_dim 64 8 and 12; in a cluster 3 to 6.  Then moved, most by less than a tenth, to fit
+// whole calls: 284 of them, 1 to 8 sequences, 5 to 32 heads, chunks of 16 to 3238, 2 to 516 tiles, each with every form
+// and number of parts (5000 times).  The plan's choice takes 0.8 % more time than the best form in the geometric mean; pairs
+// only and the same cost of parts for both head dims took 2 % (25 % at most).  For instance, this choice / the one
+// before, us: dense, 8 heads of 8 KV heads, 1100 queries over 8192 rows 56 (one CTA, one tile, 2 parts) / 60 (pairs); 32 heads of 8,
+// 128 over 8192 38 / 45; 32 heads of 32, 64 over 32768 96 / 176; sparse, 8 heads of 8, 1100 queries, 983 of 8192 rows 48 (pairs,
+// one tile, whole) / 55 (two tiles, clusters of two parts).
+//
 // A grid of q full waves and a rest has its lightest row blocks, as many as the rest, cut instead: the whole ones then
 // end after about q waves and the parts level the end.  The model is the total work over the SMs plus a third of a part
 // for the uneven end, against q + 1 waves of average jobs; it is 3 to 15 % too low (parts run slower per tile than whole row
 // blocks, and at the power cap an idle SM's share goes to the others), so dense calls take 10 % promised, sparse ones 15 %
 // and equal lengths (a batch's budgets differ).  32 heads, without / with parts, and what the model says: 1536 queries at
 // 64K, a quarter listed 470 / 396 us (0.72), dense 1536 at 32K 829 / 649 (0.70), dense 4096 at 128K 7359 / 6670 (0.88);
-// beyond the line dense 2048 at 32K 860 / 916 (0.94), 40 heads, 1536 at 32K 209 / 220 (0.92).
+// beyond the line dense 2048 at 32K 860 / 916 (0.94), 40 heads, 1536 at 32K 209 / 220 (1.07).
 // Partial results above 128 MiB are not written where a call has as many blocks of 256 positions of a head as there are SMs
 // (most such have waves enough; of those whose heads packed into tiles make fewer CTAs, eight parts of 127 CTAs and more,
 // which only dense calls over 94,000 rows and more would take, for a promised tenth).
+
 // How the query rows of a call are laid out: see QRows.
 struct AttnShape {
-  int pack, span;                  // heads and chunk positions of a Q tile
-  int ctas, block;                 // CTAs and positions of a row block
+  int span, block;                 // chunk positions of a Q tile and of a row block
   long long blocks, per_rb, jobs;  // row blocks of a head group; CTAs of one row block of every head; CTAs
 };
-static AttnShape attn_shape(const quoka_params* p, int q_tiles) {
+static AttnShape attn_shape(const quoka_params* p, const AttnPlan& plan) {
   AttnShape a;
-  const int group = p->n_q_heads / p->n_kv_heads;
-  a.pack = 1;
-  for (int d = 2; d <= 32 && d <= group; ++d)
-    if (group % d == 0) a.pack = d;
-  a.span = kQTile / a.pack;
-  a.ctas = p->head_dim == 128 ? 2 : 1;
-  a.block = q_tiles * a.ctas * a.span;
+  a.span = kQTile / plan.pack;
+  a.block = plan.q_tiles * plan.ctas * a.span;
   a.blocks = (p->chunk_len + a.block - 1) / a.block;
-  a.per_rb = (long long)(p->n_q_heads / a.pack) * a.ctas * p->batch;
+  a.per_rb = (long long)(p->n_q_heads / plan.pack) * plan.ctas * p->batch;
   a.jobs = a.per_rb * a.blocks;
   return a;
 }
-static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse) {
-  constexpr double kPartCost = 6.0, kPartCostBelow = 10.0, kOneTile = 0.9;
+// Whole row blocks of two Q tiles per CTA (head_dim 128: of a pair of CTAs), `pack` heads to a tile.
+static AttnPlan attn_whole(const quoka_params* p, int pack) {
   AttnPlan plan;
-  if (p->dtype != QUOKA_BF16 || p->impl == QUOKA_IMPL_SIMT || p->chunk_len <= 1) return plan;
-  const long long sms = device_sm_count();
-  if (sms <= 0) return plan;
-  const AttnShape two = attn_shape(p, 2);
+  plan.ctas = p->head_dim == 128 ? 2 : 1;
+  plan.pack = pack;
+  return plan;
+}
+static int attn_largest_pack(const quoka_params* p) {
+  const int group = p->n_q_heads / p->n_kv_heads;
+  int pack = std::min(group, 32);
+  while (group % pack != 0) --pack;
+  return pack;
+}
+static double attn_step_us(const quoka_params* p, int q_tiles, int ctas, bool sparse) {
+  static constexpr double us[3][2][2] = {{{1.02, 1.13}, {1.38, 1.42}},     // head_dim 64: one Q tile, two; dense, listed
+                                         {{0.95, 1.35}, {2.00, 2.05}},     // head_dim 128, one CTA
+                                         {{1.09, 1.25}, {1.35, 1.30}}};    // and a pair
+  return us[p->head_dim == 64 ? 0 : ctas][q_tiles - 1][sparse ? 1 : 0];
+}
+// The plan for `pack` heads to a tile over `tiles` key tiles besides the chunk's own, with no more scratch than `room`;
+// *model_us: what the model says.
+static AttnPlan attn_plan_of(const quoka_params* p, int pack, int tiles, bool sparse, size_t room, long long sms, double* model_us) {
+  constexpr double kStart[3] = {6.0, 9.0, 9.5}, kStartTwoOfPair = 11.5;                // head_dim 64, 128, a pair
+  constexpr double kParts128 = 5.2, kPart128 = 1.6, kParts64 = 5.5, kPart64 = 1.0, kCluster = 3.8, kSparseParts = 3.0, kOwn = 0.5;
+  const bool wide = p->head_dim == 128;
+  AttnPlan plan = attn_whole(p, pack);
+  const AttnShape two = attn_shape(p, plan);
+  const auto own = [](long long positions) { return (double)((positions + kKeyTile - 1) / kKeyTile); };
   // at least as many blocks of 256 positions of a head as SMs
   const bool bounded = (long long)p->n_q_heads * p->batch * ((p->chunk_len + 255) / 256) >= sms;
-  if (two.jobs < sms) {
-    double best_of_all = 0;
+  double best = 1e30;
+  for (int ctas = wide ? 2 : 1; ctas >= 1; --ctas) {
     for (int q_tiles = 2; q_tiles >= 1; --q_tiles) {
-      const AttnShape a = attn_shape(p, q_tiles);
-      if (a.jobs > sms) break;
-      AttnPlan cand;
-      cand.q_tiles = q_tiles;
-      // plus the chunk's own tiles, on average; in steps of two Q tiles (one of a lone Q tile takes 2700 cycles, its own chain
-      // from scores to weights and back, one of two about 3000)
-      const double step = q_tiles == 1 ? kOneTile : 1.0;
-      const double t = tiles + 0.5 * (double)a.block / kKeyTile * (double)a.blocks;
-      double best = step * t, cost = best;
-      for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
-        const long long waves = (a.jobs * parts + sms - 1) / sms;
-        cost = (double)waves * (step * t / parts + kPartCostBelow);
-        AttnPlan next = cand;
-        next.split_rb = (int)a.blocks; next.parts = parts;
-        if (cost < 0.97 * best && (!bounded || attn_split_partial_bytes(p, next) <= kMostAttnPartials)) { cand = next; best = cost; }
+      AttnPlan form = attn_whole(p, pack);
+      form.q_tiles = q_tiles; form.ctas = ctas;
+      const AttnShape a = attn_shape(p, form);
+      // the last row block, which may have no second tiles, and the one before it
+      const double step = attn_step_us(p, q_tiles, ctas, sparse);
+      const long long before = (a.blocks - 1) * a.block;
+      const double step_last = p->chunk_len - before <= ctas * a.span ? attn_step_us(p, 1, ctas, sparse) : step;
+      const auto walk = [&](double w) {
+        return std::max(step_last * (tiles + w * own(p->chunk_len)), before > 0 ? step * (tiles + w * own(before)) : 0.0);
+      };
+      const double start = ctas == 2 && q_tiles == 2 ? kStartTwoOfPair : kStart[wide ? ctas : 0];
+      const double w = sparse ? kOwn : 1.0, x = (double)a.jobs / (double)sms;
+      // (CTAs of a grid of waves do not start in step: between the number of waves and the mean)
+      const double mean = step * (tiles + 0.5 * w * (own(p->chunk_len) + (double)a.block / kKeyTile));
+      const double whole = a.jobs <= sms ? start + walk(w) : 0.5 * (x + std::ceil(x)) * (start + mean);
+      // what lies further from the calls that the model was fitted to has to promise some percent: one CTA in the place of a pair,
+      // parts through memory, more than a wave; in grids of a wave and more every other form
+      const double sure = (wide && ctas == 1 ? 1.04 : 1.0) * (a.jobs > sms ? 1.02 : 1.0);
+      const auto consider = [&](double us, int parts, bool in_cluster) {
+        AttnPlan next = form;
+        next.parts = parts; next.in_cluster = in_cluster;
+        next.split_rb = parts > 1 ? (int)a.blocks : 0;
+        us *= parts > 1 && !in_cluster ? 1.02 * sure : sure;
+        if (best < 1e30 && (us >= (two.jobs >= sms ? 0.97 : 1.0) * best || a.blocks * parts > 65535)) return;
+        if (attn_plan_scratch_bytes(p, next) > room || (bounded && attn_split_partial_bytes(p, next) > kMostAttnPartials)) return;
+        best = us;
+        plan = next;
+      };
+      consider(whole, 1, false);
+      if (a.jobs > sms) continue;
+      const double rest = start + (sparse ? kSparseParts : 0.0), t = walk(1.0);
+      for (int parts = 2; parts <= 8 && 2 * parts <= tiles + 1; ++parts) {
+        const double waves = (double)(((int)a.jobs * parts - 1) / (int)sms + 1);
+        consider(rest + waves * (t / parts + (wide ? kParts128 + kPart128 * parts : kParts64 + kPart64 * parts)), parts, false);
+        if (ctas == 2 && parts <= 4 && a.jobs / 2 <= (parts == 2 ? 28 : parts == 3 ? 20 : 14))
+          consider(rest + t / parts + kCluster, parts, true);
       }
-      // the pair kernel's, in clusters
-      if (a.ctas == 2) {
-        for (int parts = 2; parts <= 4 && parts <= tiles / 2; ++parts) {
-          cost = step * t / parts + 1.0;
-          const double limit = std::min(0.95 * best, 0.97 * step * t - (q_tiles == 1 ? 4.5 : 6.0));
-          if (a.jobs / 2 <= (parts == 2 ? 28 : parts == 3 ? 20 : 14) && cost < limit) {
-            cand.split_rb = (int)a.blocks; cand.parts = parts; cand.in_cluster = true; best = cost / 0.95;
-          }
-        }
-      }
-      if (q_tiles == 2 || best < best_of_all) { plan = cand; best_of_all = best; }
     }
-    return plan;
   }
+  *model_us = best;
   const long long n_rb = two.blocks, per_rb = two.per_rb, jobs = two.jobs;
-  const double own = (double)two.block / kKeyTile;                           // the chunk's own tiles grow by this per row block
   const long long q = jobs / sms, rest = jobs % sms;
-  if (rest == 0 || (sparse && p->batch > 1)) return plan;
-  const long long split = (rest + per_rb - 1) / per_rb;                      // row blocks to cut; block r has about (r + 1) * own of its own tiles
-  const double t_all = tiles + 2 + 0.5 * own * n_rb, t_whole = tiles + 2 + 0.5 * own * (split + n_rb), t_split = tiles + 2 + 0.5 * own * split;
-  double best = (sparse ? 0.85 : 0.90) * (double)(q + 1) * t_all;
-  for (int parts = 2; parts <= 8 && parts <= tiles / 6; ++parts) {
+  if (jobs < sms || rest == 0 || (sparse && p->batch > 1) || plan.q_tiles != 2 || plan.ctas != (wide ? 2 : 1)) return plan;
+  constexpr double kPartCost = 6.0;
+  const double own_step = (double)two.block / kKeyTile;                      // the chunk's own tiles grow by this per row block
+  const long long split = (rest + per_rb - 1) / per_rb;                      // row blocks to cut; block r has about (r + 1) * own_step of its own tiles
+  const double t_all = tiles + 3 + 0.5 * own_step * n_rb, t_whole = tiles + 3 + 0.5 * own_step * (split + n_rb), t_split = tiles + 3 + 0.5 * own_step * split;
+  double least = (sparse ? 0.85 : 0.90) * (double)(q + 1) * t_all;
+  for (int parts = 2; parts <= 8 && parts <= (tiles + 1) / 6; ++parts) {
     const double t_part = t_split / parts + kPartCost;
     const double cost = ((double)(jobs - split * per_rb) * t_whole + (double)(split * per_rb * parts) * t_part) / (double)sms + 0.3 * t_part;
-    AttnPlan cand;
+    AttnPlan cand = attn_whole(p, pack);
     cand.split_rb = (int)split; cand.parts = parts;
-    if (cost < best && attn_split_partial_bytes(p, cand) <= kMostAttnPartials) { best = cost; plan = cand; }
+    if (cost < least && attn_split_partial_bytes(p, cand) <= kMostAttnPartials && attn_plan_scratch_bytes(p, cand) <= room) {
+      least = cost;
+      plan = cand;
+      *model_us = std::min(*model_us, kStartTwoOfPair + attn_step_us(p, 2, plan.ctas, sparse) * cost / 0.9);
+    }
   }
   return plan;
 }
-AttnPlan attn_plan_sparse(const quoka_params* p, int budget_cap) { return attn_plan(p, (budget_cap + kKeyTile - 1) / kKeyTile + 1, true); }
-AttnPlan attn_plan_dense(const quoka_params* p) { return attn_plan(p, (p->max_ctx_len + kKeyTile - 1) / kKeyTile + 1, false); }
-static size_t attn_split_jobs(const quoka_params* p, const AttnPlan& plan) { return (size_t)attn_shape(p, plan.q_tiles).per_rb * plan.split_rb; }
+static AttnPlan attn_plan(const quoka_params* p, int tiles, bool sparse, size_t room) {
+  const int pack = attn_largest_pack(p);
+  const long long sms = device_sm_count();
+  if (p->dtype != QUOKA_BF16 || p->impl == QUOKA_IMPL_SIMT || p->chunk_len <= 1 || sms <= 0) return attn_whole(p, pack);
+  double us;
+  return attn_plan_of(p, pack, tiles, sparse, room, sms, &us);
+}
+AttnPlan attn_plan_sparse(const quoka_params* p, int budget_cap, size_t room) { return attn_plan(p, (budget_cap + kKeyTile - 1) / kKeyTile, true, room); }
+AttnPlan attn_plan_dense(const quoka_params* p, size_t room) { return attn_plan(p, (p->max_ctx_len + kKeyTile - 1) / kKeyTile, false, room); }
+static size_t attn_split_jobs(const quoka_params* p, const AttnPlan& plan) { return (size_t)attn_shape(p, plan).per_rb * plan.split_rb; }
 size_t attn_split_partial_bytes(const quoka_params* p, const AttnPlan& plan) {
   return plan.in_cluster ? 0 : attn_split_jobs(p, plan) * plan.parts * 2 * kSplitTileFloats * sizeof(float);
 }
 size_t attn_split_counter_bytes(const quoka_params* p, const AttnPlan& plan) { return plan.in_cluster ? 0 : attn_split_jobs(p, plan) * 8 * sizeof(int32_t); }
+size_t attn_plan_scratch_bytes(const quoka_params* p, const AttnPlan& plan) {
+  return (attn_split_counter_bytes(p, plan) + 255) / 256 * 256 + (attn_split_partial_bytes(p, plan) + 255) / 256 * 256;
+}
 
 // The launches of an attention call: the whole row blocks, then the ones in parts.
 //
@@ -460,7 +528,7 @@ quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const A
                               void* out, float* lse, cudaStream_t st, bool after_selection) {
   const bool sparse = k_idx != nullptr, split = plan.split_rb > 0 && (P.attn_partials || plan.in_cluster);
   DevParams PP = P;
-  const AttnShape shape = attn_shape(p, plan.q_tiles);
+  const AttnShape shape = attn_shape(p, plan);
   PP.attn_row_blocks = (int)shape.blocks;
   PP.attn_split_rb = split ? plan.split_rb : 0;
   PP.attn_parts = split ? plan.parts : 1;
@@ -490,7 +558,7 @@ quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const A
       attr[cfg.numAttrs].val.clusterDim.y = (unsigned)PP.attn_parts;
       attr[cfg.numAttrs++].val.clusterDim.z = 1;
     }
-    log_launch(name, cfg.gridDim, cfg.blockDim, smem, cluster, early);
+    log_launch(name, cfg.gridDim, cfg.blockDim, smem, parts && plan.in_cluster ? cluster * PP.attn_parts : cluster, early);
     if (cudaLaunchKernelEx(&cfg, kernel, PP, tm_q, tm_k, tm_v, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, k_idx, k_cnt,
                            (__nv_bfloat16*)out, lse) != cudaSuccess)
       return QUOKA_ERR_CUDA;
@@ -499,10 +567,14 @@ quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const A
   return cudaGetLastError() == cudaSuccess ? QUOKA_OK : QUOKA_ERR_CUDA;
 }
 
-bool attn_below_a_wave(const quoka_params* p) { return attn_shape(p, 2).jobs < device_sm_count(); }
-// (the model's cost of a plan with parts is above q waves of average jobs, its line at most 0.9 (q + 1))
-bool attn_may_have_parts(const quoka_params* p) { return attn_shape(p, 2).jobs < 10ll * device_sm_count(); }
-int attn_least_block(const quoka_params* p) { return attn_shape(p, 1).block; }
+static AttnShape attn_usual_shape(const quoka_params* p) { return attn_shape(p, attn_whole(p, attn_largest_pack(p))); }
+bool attn_below_a_wave(const quoka_params* p) { return attn_usual_shape(p).jobs < device_sm_count(); }
+// (above a wave the cost of a plan with parts is more than q waves of average jobs, its line at most 0.9 (q + 1))
+bool attn_may_have_parts(const quoka_params* p) { return attn_usual_shape(p).jobs < 10ll * device_sm_count(); }
+int attn_same_plan_up_to(const quoka_params* p, int chunk) {
+  const int span = kQTile / attn_largest_pack(p);
+  return std::min((chunk + span - 1) / span * span, (chunk + kKeyTile - 1) / kKeyTile * kKeyTile);
+}
 
 bool attn_tc_supported(const quoka_params* p) {
   if (p->dtype != QUOKA_BF16) return false;
@@ -519,25 +591,26 @@ bool encode_q_tensor_map(CUtensorMap* out, const DevParams& P, const void* q) {
   return encode_tensor_map_bf16(out, q, 5, dims, strides, box);
 }
 
+template <int D>
 static AttnKernel pick_attn_tc(bool sparse, bool parts, bool) {
-  if (parts) return sparse ? attn_tc_kernel<true, true> : attn_tc_kernel<false, true>;
-  return sparse ? attn_tc_kernel<true, false> : attn_tc_kernel<false, false>;
+  if (parts) return sparse ? attn_tc_kernel<D, true, true> : attn_tc_kernel<D, false, true>;
+  return sparse ? attn_tc_kernel<D, true, false> : attn_tc_kernel<D, false, false>;
 }
 
 quoka_status launch_attn_tc(const quoka_params* p, const DevParams& P0, const void* q, const void* k, const void* v,
                             const int32_t* k_idx, const int32_t* k_cnt, void* out, float* lse, cudaStream_t st,
                             bool after_selection, const AttnPlan& plan) {
   DevParams P = P0;
-  const AttnShape shape = attn_shape(p, plan.q_tiles);
-  P.attn_pack = shape.pack;
-  P.attn_span = shape.span;
+  P.attn_pack = plan.pack;
+  P.attn_span = attn_shape(p, plan).span;
   P.attn_qtiles = plan.q_tiles;
-  if (shape.ctas == 2) return launch_attn_tc_pair(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection, plan);
+  if (plan.ctas == 2) return launch_attn_tc_pair(p, P, q, k, v, k_idx, k_cnt, out, lse, st, after_selection, plan);
   CUtensorMap tm_q, tm_k, tm_v;
   if (!encode_q_tensor_map(&tm_q, P, q)) return QUOKA_ERR_CUDA;
   if (!encode_kv_tensor_map(&tm_k, p, k, 64) || !encode_kv_tensor_map(&tm_v, p, v, 64)) return QUOKA_ERR_CUDA;
-  const size_t smem = 1024 + (2 + kSlots) * 16384 + 512;
-  return launch_attn_plan(p, P, plan, pick_attn_tc, "attn_tc", /*cluster=*/1, smem, tm_q, tm_k, tm_v, k, v, k_idx, k_cnt, out, lse, st, after_selection);
+  const bool wide = P.d == 128;
+  return launch_attn_plan(p, P, plan, wide ? pick_attn_tc<128> : pick_attn_tc<64>, "attn_tc", /*cluster=*/1,
+                          wide ? kAttnSmem<128> : kAttnSmem<64>, tm_q, tm_k, tm_v, k, v, k_idx, k_cnt, out, lse, st, after_selection);
 }
 
 }  // namespace quoka

@@ -92,7 +92,7 @@ template <int D>
 __device__ __forceinline__ void zero_spare_q_rows(const DevParams& P, unsigned char* q_smem, int thread, int threads) {
   const int used = P.attn_pack * P.attn_span, spare = (128 - used) * 8;      // 16-byte pieces of a half tile
   if (spare == 0) return;
-  for (int i = thread; i < 2 * (D / 64) * spare; i += threads)
+  for (int i = thread; i < P.attn_qtiles * (D / 64) * spare; i += threads)
     reinterpret_cast<uint4*>(q_smem + (i / spare) * 16384 + used * 128)[i % spare] = make_uint4(0, 0, 0, 0);
   fence_proxy_async_smem();
 }

@@ -37,8 +37,7 @@ static int budget_cap_of(const quoka_params* p) {
 }
 
 // The buffers of a call in a workspace of ws_bytes.  The scratch of `plan` (partial results and arrival counters of row
-// blocks in parts that merge through memory), where the plan has any, comes last and only if there is room for it: the
-// attention leaves the row blocks whole without it.
+// blocks in parts that merge through memory), where the plan has any, comes last.
 static Workspace carve(const quoka_params* p, void* ws, size_t ws_bytes = 0, const AttnPlan* plan = nullptr) {
   Workspace w{};
   const size_t es = p->dtype == QUOKA_BF16 ? 2 : 4;
@@ -67,34 +66,32 @@ static Workspace carve(const quoka_params* p, void* ws, size_t ws_bytes = 0, con
   return w;
 }
 
-static size_t plan_scratch_bytes(const quoka_params* p, const AttnPlan& plan) {
-  return align_up(attn_split_counter_bytes(p, plan)) + align_up(attn_split_partial_bytes(p, plan));
+// What a workspace of ws_bytes has left for the scratch of a plan.
+static size_t attn_room(const quoka_params* p, size_t ws_bytes) {
+  const size_t least = carve(p, nullptr).total;
+  return ws_bytes > least ? ws_bytes - least : 0;
 }
 // The scratch of the larger of the two plans an attention call of this problem may follow.
 static size_t attn_scratch_bytes(const quoka_params* p) {
-  return std::max(plan_scratch_bytes(p, attn_plan_sparse(p, budget_cap_of(p))), plan_scratch_bytes(p, attn_plan_dense(p)));
+  return std::max(attn_plan_scratch_bytes(p, attn_plan_sparse(p, budget_cap_of(p))), attn_plan_scratch_bytes(p, attn_plan_dense(p)));
 }
 // What the shorter chunks of the same prompt take: the last chunk of a prompt comes with the workspace of its longest, and
 // parts are what fills the GPU there.  Dense calls count from 16384 cached rows on: over shorter caches parts are a matter of
-// some tens of microseconds; and no more than a grid of a wave or more may take.  A plan depends on the chunk's length
-// through the number of its smallest row blocks, and through the bound on its scratch, which holds from some length on; so both
-// ends of every such block are asked, until the grid is so large that no plan has parts.
+// some tens of microseconds; and no more than a grid of a wave or more may take.  Chunk lengths of one plan
+// are asked once, until the grid is so large that no plan has parts.
 static size_t attn_scratch_of_shorter_chunks(const quoka_params* p) {
   constexpr int kDenseFrom = 16384;
   size_t bytes = 0;
   const auto take = [&](const quoka_params* t, const AttnPlan& plan) {
-    if (attn_split_partial_bytes(t, plan) <= kMostAttnPartials) bytes = std::max(bytes, plan_scratch_bytes(t, plan));
+    if (attn_split_partial_bytes(t, plan) <= kMostAttnPartials) bytes = std::max(bytes, attn_plan_scratch_bytes(t, plan));
   };
   quoka_params t = *p;
-  const int block = attn_least_block(p);
-  for (int first = 1;; first += block) {
-    for (int c : {first, first + block - 1}) {
-      t.chunk_len = c;
-      if (c >= p->chunk_len || !attn_may_have_parts(&t)) return bytes;
-      take(&t, attn_plan_sparse(&t, budget_cap_of(&t)));
-      if (p->max_ctx_len >= kDenseFrom) take(&t, attn_plan_dense(&t));
-    }
+  for (t.chunk_len = attn_same_plan_up_to(p, 1); t.chunk_len < p->chunk_len && attn_may_have_parts(&t);
+       t.chunk_len = attn_same_plan_up_to(p, t.chunk_len + 1)) {
+    take(&t, attn_plan_sparse(&t, budget_cap_of(&t)));
+    if (p->max_ctx_len >= kDenseFrom) take(&t, attn_plan_dense(&t));
   }
+  return bytes;
 }
 
 static quoka_status validate(const quoka_params* p) {
@@ -298,7 +295,7 @@ static quoka_status run_prefill(const quoka_params* p, const DevParams& P, const
 // room for the split attention's scratch, among them).
 quoka_status prefill_chunk_impl(const quoka_params* p, const void* q, const void* k_cache, const void* v_cache, void* out,
                                 int32_t* k_idx_out, int32_t* k_cnt_out, void* ws, size_t ws_bytes, void* stream) {
-  const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p));
+  const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p), attn_room(p, ws_bytes));
   const Workspace w = carve(p, ws, ws_bytes, &plan);
   return run_prefill(p, make_dev(p, ws, w), w, plan, q, k_cache, v_cache, out,
                      k_idx_out ? k_idx_out : w.k_idx, k_cnt_out ? k_cnt_out : w.k_cnt, static_cast<cudaStream_t>(stream));
@@ -372,7 +369,7 @@ quoka_status quoka_sparse_attn(const quoka_params* p, const void* q, const void*
   if (!q || !k_cache || !v_cache || !k_idx || !k_cnt || !out) return QUOKA_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k_cache) || !aligned16(v_cache) || !aligned16(out)) return QUOKA_ERR_INVALID_ARG;
   if ((st = check_ws(p, ws, ws_bytes)) != QUOKA_OK) return st;
-  const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p));
+  const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p), attn_room(p, ws_bytes));
   return run_attn(p, make_dev(p, ws, carve(p, ws, ws_bytes, &plan)), q, k_cache, v_cache, k_idx, k_cnt, out, lse,
                   static_cast<cudaStream_t>(stream), plan);
 }
@@ -384,7 +381,7 @@ quoka_status quoka_dense_chunk_attn(const quoka_params* p, const void* q, const 
   if (!q || !k_cache || !v_cache || !out) return QUOKA_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k_cache) || !aligned16(v_cache) || !aligned16(out)) return QUOKA_ERR_INVALID_ARG;
   if ((st = check_ws(p, ws, ws_bytes)) != QUOKA_OK) return st;
-  const AttnPlan plan = attn_plan_dense(p);
+  const AttnPlan plan = attn_plan_dense(p, attn_room(p, ws_bytes));
   return run_attn(p, make_dev(p, ws, carve(p, ws, ws_bytes, &plan)), q, k_cache, v_cache, nullptr, nullptr, out, lse,
                   static_cast<cudaStream_t>(stream), plan);
 }
@@ -462,7 +459,7 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
   // 811, of 4 / 4 791; queries, keys and values of four equal slices one after another 805.
   int n_slices = 1, slice[kHostSlices] = {p->n_kv_heads, 0, 0};
   const size_t q_bytes = (size_t)p->batch * p->n_q_heads * head_bytes;
-  const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p));
+  const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p), attn_room(p, ws_bytes));
   const bool below = attn_below_a_wave(p), whole_below = plan.split_rb > 0 || p->dtype != QUOKA_BF16;
   const int n_kv = p->n_kv_heads;
   if (!p->k_inv_norm && !(below && whole_below) && q_bytes >= ((size_t)8 << 20) && n_kv > 1) {

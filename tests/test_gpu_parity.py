@@ -1,4 +1,9 @@
 """Parity of the CUDA path (through the C ABI) with the CPU oracle on the same seeded inputs."""
+import os
+import re
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -882,6 +887,85 @@ def test_attention_parts_in_a_cluster(n_q, n_kv, C, T, B):
         dense, lse = O.dense_chunk_attention(q, k, v, t)
         check_attention(f64(gp.out[s]), dense, "bf16")
         assert np.abs(f64(gp.lse[s]) - lse).max() <= 2e-3
+
+
+# n_q, n_kv, C, T, B, call; kernel, CTAs of a cluster, grid of its launch on 148 SMs
+FORMS = [
+    (16, 16, 1030, 600, 300, "dense", "attn_tc", 1, (16, 9, 1)),         # one CTA, one Q tile, whole; the last one of six rows
+    (16, 16, 1030, 600, 300, "sparse", "attn_tc", 1, (16, 9, 1)),
+    (8, 8, 1030, 3000, 1500, "dense", "attn_tc", 1, (8, 18, 1)),         # in two parts
+    (128, 128, 200, 600, 300, "sparse", "attn_tc", 1, (128, 1, 1)),      # two Q tiles, whole
+    (32, 32, 200, 8000, 6000, "sparse", "attn_tc", 1, (32, 4, 1)),       # in four parts
+    (37, 1, 40, 3000, 3000, "sparse", "attn_tc", 1, (37, 4, 1)),         # the list is the identity
+    (32, 32, 100, 3000, 1500, "dense", "attn_tc", 1, (32, 4, 1)),
+    (74, 2, 64, 1000, 120, "dense", "attn_tc", 1, (74, 1, 1)),           # a pair's second CTA would be idle
+    (32, 32, 633, 1500, 700, "sparse", "attn_tc_pair", 2, (64, 2, 1)),   # pairs, two Q tiles each, whole
+    (4, 4, 64, 1500, 700, "sparse", "attn_tc_pair", 2, (8, 1, 1)),       # one
+    (32, 8, 400, 3000, 3000, "sparse", "attn_tc_pair", 2, (16, 8, 1)),   # two parts through memory
+    (24, 24, 40, 3000, 1500, "sparse", "attn_tc_pair", 4, (48, 2, 1)),   # 24 clusters of four, one Q tile
+    (24, 24, 64, 1500, 700, "dense", "attn_tc_pair", 4, (48, 2, 1)),
+    (32, 8, 257, 3000, 3000, "sparse", "attn_tc_pair", 4, (16, 6, 1)),   # and two
+    (32, 8, 300, 3000, 1500, "dense", "attn_tc_pair", 4, (16, 6, 1)),
+    (8, 8, 257, 3000, 1500, "sparse", "attn_tc_pair", 6, (16, 6, 1)),    # 16 clusters of six
+    (8, 8, 300, 3000, 3000, "sparse", "attn_tc_pair", 8, (16, 4, 1)),    # 8 of eight
+]
+
+
+@pytest.mark.gpu
+def test_attention_forms_are_the_ones_meant():
+    """The launches of the calls in FORMS, by the library's launch log."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the plan goes by the number of SMs")
+    code = """
+import sys, torch
+from paper_2602_08722_b200 import api
+from tests.test_gpu_parity import FORMS
+for n_q, n_kv, C, T, B, call, *_ in FORMS:
+    q = torch.zeros(1, n_q, C, 128, dtype=torch.bfloat16, device="cuda")
+    k = torch.zeros(1, n_kv, T + C, 128, dtype=torch.bfloat16, device="cuda")
+    p = api.make_params(q, k, q.clone(), torch.full((1,), T, dtype=torch.int32, device="cuda"), n_retain=16, kv_budget=B, max_ctx_len=T)
+    ws, out = api.alloc_workspace(p), torch.empty_like(q)
+    print("form", file=sys.stderr, flush=True)
+    if call == "dense":
+        api.quoka_dense_chunk_attn(p, q, k, k, out, None, ws)
+    else:
+        api.quoka_prefill_chunk(p, q, k, k, out, None, None, ws)
+    torch.cuda.synchronize()
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    run = subprocess.run([sys.executable, "-c", code], cwd=root, env=dict(os.environ, QUOKA_LOG="1"), capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stderr[-2000:]
+    logs = run.stderr.split("form\n")[1:]
+    assert len(logs) == len(FORMS)
+    for form, log in zip(FORMS, logs):
+        got = re.findall(r"\] (attn\w+) +grid \((\d+),(\d+),(\d+)\).* cluster (\d+)", log)
+        assert [(g[0], int(g[4]), (int(g[1]), int(g[2]), int(g[3]))) for g in got] == [form[6:]], (form, log)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_q,n_kv,C,T,B,call", [f[:6] for f in FORMS])
+def test_attention_forms(n_q, n_kv, C, T, B, call):
+    """Every form of row block and of parts at head_dim 128: two calls over one workspace with the same bits, against the oracle."""
+    gp = problem(2200 + C, n_q=n_q, n_kv=n_kv, T=T, C=C, n_retain=16, kv_budget=B)
+    heads, rows = stratified_rows(n_q, C, 400, 5)
+    if call == "sparse":
+        gp.run_staged()
+        check_chain(gp, attn_rows=400)
+    got = gp.out.clone()
+    for rep in range(2):
+        gp.out.zero_()
+        if call == "sparse":
+            api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+        else:
+            api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, gp.lse, gp.ws)
+        torch.cuda.synchronize()
+        if call == "dense" and rep == 0:
+            q, k, v, t = gp.oracle_inputs(0)
+            want = O.sparse_attention_rows(q, k, v, t, [np.arange(t)] * n_kv, heads, rows)
+            check_attention(f64(gp.out[0])[heads, rows], want, "bf16")
+            got = gp.out.clone()
+        assert torch.equal(gp.out, got)
+    assert api.quoka_last_device_status(gp.ws) == 0
 
 
 @pytest.mark.parametrize("n_q,C,n_retain,d,dtype", [
