@@ -408,10 +408,14 @@ static AttnPlan attn_whole(const quoka_params* p, int pack) {
   plan.pack = pack;
   return plan;
 }
+// Heads that may share a Q tile: divisors of the group whose row blocks the grid's second dimension holds (32 heads to a tile
+// at head_dim 64: chunks of 524280 positions; one head: of 16.7 million).
+static bool attn_pack_fits(const quoka_params* p, int pack) {
+  return p->n_q_heads / p->n_kv_heads % pack == 0 && (pack == 1 || attn_shape(p, attn_whole(p, pack)).blocks <= 65535);
+}
 static int attn_largest_pack(const quoka_params* p) {
-  const int group = p->n_q_heads / p->n_kv_heads;
-  int pack = std::min(group, 32);
-  while (group % pack != 0) --pack;
+  int pack = std::min(p->n_q_heads / p->n_kv_heads, 32);
+  while (pack > 1 && !attn_pack_fits(p, pack)) --pack;
   return pack;
 }
 static double attn_step_us(const quoka_params* p, int q_tiles, int ctas, bool sparse) {

@@ -968,6 +968,25 @@ def test_attention_forms(n_q, n_kv, C, T, B, call):
     assert api.quoka_last_device_status(gp.ws) == 0
 
 
+@pytest.mark.gpu
+def test_a_dense_chunk_of_more_row_blocks_than_a_grid_dimension_holds():
+    """32 heads to a tile would make 65537 row blocks of 8 positions: sampled rows against a softmax in 64 bits."""
+    C, n_q, d = 65536 * 8 + 3, 32, 64
+    g = torch.Generator("cuda").manual_seed(3)
+    q = torch.randn(1, n_q, C, d, dtype=torch.bfloat16, device="cuda", generator=g)
+    k, v = (torch.randn(1, 1, C, d, dtype=torch.bfloat16, device="cuda", generator=g) for _ in range(2))
+    out, ctx = torch.zeros_like(q), torch.zeros(1, dtype=torch.int32, device="cuda")
+    p = api.make_params(q, k, out, ctx, n_retain=C, kv_budget=64, max_ctx_len=0)
+    ws = api.alloc_workspace(p)
+    api.quoka_dense_chunk_attn(p, q, k, v, out, None, ws)
+    torch.cuda.synchronize()
+    assert api.quoka_last_device_status(ws) == 0
+    for h, r in ((0, 0), (31, 200), (5, 70001), (17, C // 2), (0, C - 4), (31, C - 3), (9, C - 1)):
+        w = torch.softmax(k[0, 0, :r + 1].double() @ q[0, h, r].double() / d ** 0.5, 0)
+        want = (w[:, None] * v[0, 0, :r + 1].double()).sum(0)
+        check_attention(f64(out[0, h, r])[None], f64(want)[None], "bf16")
+
+
 @pytest.mark.parametrize("n_q,C,n_retain,d,dtype", [
     (4, 2, 1, 128, "bf16"),             # one row per CTA
     (4, 65, 64, 64, "f32"),             # 33 rows: a block of one row
