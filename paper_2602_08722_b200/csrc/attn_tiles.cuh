@@ -53,11 +53,11 @@ __device__ __forceinline__ int longest_first(const DevParams& P, int z) {
 }
 
 // The query rows of a Q tile: `pack` heads of one KV group at `span` consecutive chunk positions, position by position, so
-// that the heads of a group share every key tile and a tile's rows end at nearly the same causal limit.  A KV group's heads
-// all go into one tile where they are up to 32 (else its largest divisor does): 128 / pack positions each, the rows that are
-// left over, seven at most, are zero.  Against 128 positions of one head each: a chunk of 777 with eight heads per KV head
+// that the heads of a group share every key tile and a tile's rows end at nearly the same causal limit; 128 / pack positions
+// each, the rows that are left over (two for three heads, three for five, eight for ten) are zero.  `attn_plan` says how many
+// heads, as a rule all of a KV group.  Against 128 positions of one head each: a chunk of 777 with eight heads per KV head
 // takes 49 tiles instead of 56, one of 68 with three heads 2 instead of 3, the chunk's own tiles that a row block walks end
-// 32 positions after its first row and not 256 (four heads), and any number of heads per KV head makes pairs.
+// 32 positions after its first row and not 256 (four heads).
 // A row block is the Q tiles of one CTA (A, or A and B), or of both CTAs of a pair: A of the first, A of the second, then the
 // two Bs, so that a row block of no more positions than two tiles have walks one tile in each CTA.
 struct QRows {

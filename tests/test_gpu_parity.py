@@ -969,6 +969,36 @@ def test_attention_forms(n_q, n_kv, C, T, B, call):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("n_q,n_kv,C", [
+    (32, 2, 70), (32, 2, 301),          # 16 heads to a tile, 8 positions
+    (26, 1, 40), (26, 2, 300),          # 26: 4 positions and 24 rows left over, or 13: 9 and 11
+    (64, 2, 33), (40, 1, 130),          # 32; 20 or 8
+    (37, 1, 20), (37, 1, 200),          # a prime above 32: one head to a tile
+    (19, 1, 90), (28, 1, 610),          # one or 19; 14, 7 or 4
+])
+def test_many_heads_per_kv_head(n_q, n_kv, C, d):
+    """Groups of 13 to 40 heads: sparse (staged and fused, the same bits) and dense, sampled rows against the oracle."""
+    T = 2300
+    gp = problem(2300 + C, n_q=n_q, n_kv=n_kv, d=d, T=T, C=C, n_retain=24, kv_budget=900)
+    gp.run_staged()
+    check_chain(gp, attn_rows=300)
+    staged = gp.out.clone()
+    gp.out.zero_()
+    api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+    torch.cuda.synchronize()
+    assert torch.equal(gp.out, staged)
+    gp.out.zero_()
+    api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, gp.lse, gp.ws)
+    torch.cuda.synchronize()
+    q, k, v, t = gp.oracle_inputs(0)
+    heads, rows = stratified_rows(n_q, C, 300, 5)
+    want = O.sparse_attention_rows(q, k, v, t, [np.arange(t)] * n_kv, heads, rows)
+    check_attention(f64(gp.out[0])[heads, rows], want, "bf16")
+    assert api.quoka_last_device_status(gp.ws) == 0
+
+
+@pytest.mark.gpu
 def test_a_dense_chunk_of_more_row_blocks_than_a_grid_dimension_holds():
     """32 heads to a tile would make 65537 row blocks of 8 positions: sampled rows against a softmax in 64 bits."""
     C, n_q, d = 65536 * 8 + 3, 32, 64
