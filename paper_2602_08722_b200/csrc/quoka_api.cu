@@ -454,17 +454,22 @@ quoka_status quoka_prefill_chunk_host(const quoka_params* p, const int32_t* ctx_
   // 523 / 571 us whole, 481 / 484 in halves, 483 / 528 in slices as below; f32, whose kernels are the longer part, 954 whole, 1572
   // in slices).
   // What bounds it: the host link, and on it the number of copies: one that starts while the other direction is busy costs
-  // about 17 us.  So all keys and values first, then the queries in three pieces, the first the smallest.  32 query / 8 KV
-  // heads, 2048 queries at 32K (25.2 MB in: 500 us alone, 16.8 MB out): slices of 2, 3 and 3 KV groups 745 us, of 2 / 2 / 2 / 2
-  // 811, of 4 / 4 791; queries, keys and values of four equal slices one after another 805.
+  // about 17 us; and behind the last copy in, the last slice's kernels and its copy out.  So all keys and values first, then the
+  // queries in three pieces, the last no larger than the others, or in two where 16 MiB and more do not come in.  32 query / 8 KV
+  // heads, 2048 queries at 32K (25.2 MB in: 500 us alone, 16.8 MB out), a pass alone and one of many: slices of 3, 3 and 2 KV groups
+  // 724 / 722 us, of 2, 3 and 3 738 / 757, of 3, 2 and 3 758 / 756, of 4, 2 and 2 780, of 4 / 4 793, of 2 / 2 / 2 / 2 811; copies out
+  // only when the last copy in is through 797; 4096 at 16K 1386 (3, 3, 2), 1399, 1460.  16 / 4 heads, 2048 (8 MiB) 467 in halves, 490
+  // to 530 in three; 24 / 3 (12 MiB) 620 (2, 1), 666 (1, 1, 1); 32 / 4 700 (2, 1, 1), 715 (2, 2); 32 / 16 at 8K 870 to 890 whichever
+  // the thirds, 915 (4, 6, 6).
   int n_slices = 1, slice[kHostSlices] = {p->n_kv_heads, 0, 0};
   const size_t q_bytes = (size_t)p->batch * p->n_q_heads * head_bytes;
   const AttnPlan plan = attn_plan_sparse(p, budget_cap_of(p), attn_room(p, ws_bytes));
   const bool below = attn_below_a_wave(p), whole_below = plan.split_rb > 0 || p->dtype != QUOKA_BF16;
   const int n_kv = p->n_kv_heads;
   if (!p->k_inv_norm && !(below && whole_below) && q_bytes >= ((size_t)8 << 20) && n_kv > 1) {
-    slice[0] = below ? n_kv / 2 : (n_kv / 4 > 0 ? n_kv / 4 : 1);
-    slice[1] = below || n_kv == 2 ? n_kv - slice[0] : (n_kv - slice[0]) / 2;
+    const bool two = below || q_bytes < ((size_t)16 << 20);
+    slice[0] = below ? n_kv / 2 : two ? (n_kv + 1) / 2 : (n_kv + 2) / 3;
+    slice[1] = two ? n_kv - slice[0] : (n_kv - slice[0] + 1) / 2;
     slice[2] = n_kv - slice[0] - slice[1];
     n_slices = slice[2] > 0 ? 3 : 2;
   }
