@@ -76,7 +76,7 @@ def test_gqa_ratios(G, impl):
 
 @pytest.mark.parametrize("n_q,n_kv", [(12, 2), (10, 5), (14, 7), (9, 3), (5, 5)])
 def test_gqa_ratios_that_are_not_powers_of_two(n_q, n_kv):
-    # 6 and 2 query heads per KV head run as CTA pairs (with 5 or 7 KV heads), 3 and 1 in the one-CTA kernel
+    # clusters of pairs in three or four parts, tiles of 126 (six and three heads) and 128 rows
     gp = problem(960, batch=2, n_q=n_q, n_kv=n_kv, T=[4100, 200], C=129, n_retain=16, kv_budget=0, budget_frac=0.9)
     gp.run_staged()
     check_chain(gp)
@@ -716,7 +716,7 @@ def test_decode_scoring_units(T, d, dtype, group, cached_norms, paged):
     (32, 4, 64, 777, 6000, 1500, False),    # P in place, three S buffers; the last row block has one Q tile, of nine rows
     (32, 4, 64, 384, 3000, 2999, True),     # and of 128
     (32, 8, 128, 633, 6000, 1500, True),    # pairs: one S buffer, P apart
-    (32, 32, 128, 640, 2500, 700, False),   # the same in the one-CTA kernel
+    (32, 32, 128, 640, 2500, 700, False),   # the same with one head per tile
 ])
 def test_q_tiles_that_walk_many_key_tiles(n_q, n_kv, d, C, T, B, paged):
     """Row blocks of two Q tiles and of one over dozens of key tiles: the buffers of scores and weights go round many times.
@@ -772,8 +772,8 @@ def test_rows_of_a_pair_of_ctas(n_q, n_kv, C):
 
 
 @pytest.mark.parametrize("n_q,n_kv,d,C,T,B", [
-    (32, 8, 128, 1300, 9000, 5000),     # pairs, 6 row blocks: the lightest in parts after the whole ones, ragged last block
-    (24, 8, 64, 1800, 7000, 6000),      # one-CTA kernel, 8 row blocks
+    (32, 8, 128, 1300, 9000, 5000),     # pairs, 11 row blocks: the lightest in parts after the whole ones, ragged last block
+    (24, 8, 64, 1800, 7000, 6000),      # one-CTA kernel, 22 row blocks
     (32, 8, 128, 1281, 6000, 6000),     # the budget covers the cache: the list is the identity
 ])
 def test_attention_with_its_lightest_row_blocks_in_parts(n_q, n_kv, d, C, T, B):
@@ -866,7 +866,7 @@ def test_the_end_of_a_prompt_runs_in_the_workspace_of_its_longest_chunk(n_q, n_k
     (8, 4, 257, [2500, 40], 2000),      # a row block of one row; a list shorter than a tile: parts without a tile
     (32, 8, 130, [3000], 1500),         # 16 clusters of six
     (32, 8, 2, [1030], 1024),           # two query rows
-    (32, 8, 400, [3000], 3000),         # 32 clusters of four, the list is the identity
+    (32, 8, 400, [3000], 3000),         # two parts through memory, the list is the identity; dense: one CTA, whole
     (2, 1, 64, [1100], 1025),           # one cluster
 ])
 def test_attention_parts_in_a_cluster(n_q, n_kv, C, T, B):
@@ -1137,6 +1137,40 @@ def test_f32_values_of_later_rows_do_not_reach_earlier_ones(T, C, B, n_q, n_kv, 
         assert not torch.isfinite(got[1][:, :, row:, d // 3]).any()
 
 
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+@pytest.mark.parametrize("T,C,B,n_q,n_kv,d", [
+    (3000, 700, 1500, 4, 4, 128),       # row blocks of up to four key tiles: pairs in clusters
+    (3000, 400, 3000, 32, 8, 128),      # pairs in parts through memory; dense: one CTA, whole
+    (3000, 1030, 1500, 8, 8, 128),      # dense: one CTA in parts through memory
+    (1500, 900, 200, 16, 16, 128),      # whole pairs
+    (2500, 600, 2300, 8, 8, 64),        # head_dim 64: parts
+    (700, 1300, 100, 16, 16, 64),       # and whole
+])
+def test_bf16_values_of_later_tiles_do_not_reach_earlier_rows(T, C, B, n_q, n_kv, d, bad):
+    """A value that is not finite leaves the bits of all rows that end in an earlier key tile (a tile that a row does not see
+    adds 0 * inf to it until its first own tile wipes the sum), and reaches the rows that attend it."""
+    gp = problem(970 + T, n_q=n_q, n_kv=n_kv, d=d, T=T, C=C, n_retain=16, kv_budget=B)
+    row = C // 2 + 77
+    for call in ("sparse", "dense"):
+        got = []
+        for broken in (False, True):
+            keep = gp.v[:, :, T + row, d // 3].clone()
+            if broken:
+                gp.v[:, :, T + row, d // 3] = bad
+            if call == "sparse":
+                api.quoka_prefill_chunk(gp.p, gp.q, gp.k, gp.v, gp.out, None, None, gp.ws)
+            else:
+                api.quoka_dense_chunk_attn(gp.p, gp.q, gp.k, gp.v, gp.out, None, gp.ws)
+            torch.cuda.synchronize()
+            got.append(gp.out.clone())
+            gp.v[:, :, T + row, d // 3] = keep
+        first = T if call == "dense" else 0                      # where a tile of the walk begins
+        end = (first + row) // 128 * 128 - first
+        assert end > 0 and torch.isfinite(got[0]).all()
+        assert torch.equal(got[1][:, :, :end], got[0][:, :, :end])
+        assert not torch.isfinite(got[1][:, :, row:, d // 3]).any()
+
+
 @pytest.mark.parametrize("mode", ["cosine", "dot"])
 @pytest.mark.parametrize("T,n_kv", [(513, 3), (8193, 8), (16385, 8), (16385, 33), (20011, 73), (32768, 14), (32769, 15)])
 def test_select_keys_every_cluster_width(T, n_kv, mode):
@@ -1356,9 +1390,10 @@ def test_split_attention_dense_against_the_oracle(T, C):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("d,n_q,n_kv", [(64, 8, 2), (128, 4, 4), (128, 6, 2)])
+@pytest.mark.parametrize("d,n_q,n_kv", [(64, 8, 2), (64, 4, 4), (64, 6, 2), (128, 4, 4), (128, 6, 2)])
 def test_split_attention_in_the_one_cta_kernel(d, n_q, n_kv):
-    # head_dim 64, one query head per KV head, an odd GQA ratio: the shapes the CTA-pair kernel does not take
+    # head_dim 64 with four, one and three query heads per KV head: parts of one Q tile.  At head_dim 128 these are clusters
+    # of pairs; FORMS has the one-CTA kernel's parts
     gp = problem(33, batch=2, n_q=n_q, n_kv=n_kv, d=d, T=[4100, 300], C=200, n_retain=16, kv_budget=0, budget_frac=0.9)
     gp.run_staged()
     check_chain(gp)
@@ -1399,9 +1434,9 @@ def test_f32_rows_that_one_key_dominates_keep_the_thousands_of_small_weights():
 @pytest.mark.gpu
 @pytest.mark.parametrize("n_q,n_kv,d,T,C,frac,paged,fac", [
     (8, 2, 128, 4100, 300, 0.9, False, 6.0),       # CTA pairs, split into parts
-    (4, 4, 128, 3000, 257, 0.5, True, 8.0),        # one-CTA kernel (one query head per KV head), paged
+    (4, 4, 128, 3000, 257, 0.5, True, 8.0),        # one query head per KV head, paged
     (8, 2, 64, 2500, 200, 0.9, False, 6.0),        # head_dim 64
-    (32, 8, 128, 3000, 512, 0.3, False, 5.0)])     # two row blocks per head, unsplit
+    (32, 8, 128, 3000, 512, 0.3, False, 5.0)])     # row blocks of one Q tile per CTA, unsplit
 def test_logits_far_beyond_the_lazy_rescale_threshold(n_q, n_kv, d, T, C, frac, paged, fac):
     """The tensor-core kernels move the reference point of their exponentials (and rescale the accumulator in
     tensor memory) only when a row's maximum outgrows it by 2^32.  Unit-variance inputs never get there, so here
