@@ -379,10 +379,12 @@ __device__ __forceinline__ bool attn_softmax_tile(uint32_t s_addr, uint32_t p_ad
 // key tile; items run A0 B0 A1 B1 ... (a Q tile that does not take part in a key tile has no item there).  S has NBUF
 // tensor-memory buffers, used in turn; the QK^T of item i + NBUF waits until item i's is free, and nothing else orders it
 // against PV.
-//   head_dim 128: O takes 256 of the 512 columns, one S and two P (one per Q tile) the rest: S is free when item i's scores
+//   head_dim 128, pairs: O takes 256 of the 512 columns, one S and two P (one per Q tile) the rest: S is free when item i's scores
 //     have been READ, the next QK^T then runs under item i's exponentials.
 //   head_dim 64: O takes 128 columns, three S the rest, P in place: free when item i's weights have been multiplied, which
 //     is an item and a half before its next scores are wanted.
+//   head_dim 128, one CTA: O takes 256 columns, two S the rest, P in place: with two Q tiles a tile's next QK^T waits for its own
+//     products (1.91 us a step where a pair takes 1.39), with one it has both buffers (1.02).
 // So a softmax warp finds its next scores ready, or nearly, when it is done with a tile.  Two warps because a wait on a
 // barrier that is complete already costs 75 to 100 cycles and there are five to a pair of products, which take 1024: one
 // warp for both left the tensor core idle for 45 % of a step (3650 cycles at head_dim 128).  Products of two warps
