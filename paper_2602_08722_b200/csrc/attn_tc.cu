@@ -378,11 +378,15 @@ attn_tc_kernel(DevParams P, const __grid_constant__ CUtensorMap tm_q, const __gr
 //
 // A grid of q full waves and a rest has its lightest row blocks, as many as the rest, cut instead: the whole ones then
 // end after about q waves and the parts level the end.  The model is the total work over the SMs plus a third of a part
-// for the uneven end, against q + 1 waves of average jobs; it is 3 to 15 % too low (parts run slower per tile than whole row
-// blocks, and at the power cap an idle SM's share goes to the others), so dense calls take 10 % promised, sparse ones 15 %
-// and equal lengths (a batch's budgets differ).  32 heads, without / with parts, and what the model says: 1536 queries at
-// 64K, a quarter listed 470 / 396 us (0.72), dense 1536 at 32K 829 / 649 (0.70), dense 4096 at 128K 7359 / 6670 (0.88);
-// beyond the line dense 2048 at 32K 860 / 916 (0.94), 40 heads, 1536 at 32K 209 / 220 (1.07).
+// for the uneven end, against q + 1 waves of average jobs.  48 calls without / with parts, in turns over the same buffers: what
+// the model puts below 0.92 of the whole row blocks (sparse) and 0.94 (dense) gains 1 to 11 %,
+// around the line some gain 5 % and some lose 7, above it nearly all lose 4 to 10.  32 heads, us, and the model: sparse, 3700 queries
+// over 8192 of 65536 rows 621 / 561 (0.82), 1550 over 3932 of 32768 165 / 154 (0.86), 2900 over 8192 415 / 404 (0.91), 4096 over
+// 15729 of 131072 1132 / 1086 (0.91), 1700 over 3932 168 / 182 (0.925), 3072 over 16384 828 / 784 (0.93), 1850 over 8192 270 / 287 (0.95), 2000
+// over 8192 276 / 297 (1.01); head_dim 64 3800 over 3932 304 / 284 (0.85), 1850 over 8192 243 / 228 (0.91), 2000 over 8192 246 / 260 (0.99);
+// dense, 1850 over 16384 411 / 392 (0.91), 3000 over 32768 1444 / 1331 (0.91), 2048 over 32768 967 / 914 (0.94), 1850 over 8192 217 / 241
+// (0.95), 2150 over 32768 945 / 1002 (1.00); head_dim 64 2000 over 32768 746 / 682 (0.92), 3050 over 8192 331 / 344 (0.95).  Sparse
+// calls of a batch stay whole (their budgets differ).
 // Partial results above 128 MiB are not written where a call has as many blocks of 256 positions of a head as there are SMs
 // (most such have waves enough; of those whose heads packed into tiles make fewer CTAs, eight parts of 127 CTAs and more,
 // which only dense calls over 94,000 rows and more would take, for a promised tenth).
@@ -485,7 +489,7 @@ static AttnPlan attn_plan_of(const quoka_params* p, int pack, int tiles, bool sp
   const double own_step = (double)two.block / kKeyTile;                      // the chunk's own tiles grow by this per row block
   const long long split = (rest + per_rb - 1) / per_rb;                      // row blocks to cut; block r has about (r + 1) * own_step of its own tiles
   const double t_all = tiles + 3 + 0.5 * own_step * n_rb, t_whole = tiles + 3 + 0.5 * own_step * (split + n_rb), t_split = tiles + 3 + 0.5 * own_step * split;
-  double least = (sparse ? 0.85 : 0.90) * (double)(q + 1) * t_all;
+  double least = (sparse ? 0.92 : 0.94) * (double)(q + 1) * t_all;
   for (int parts = 2; parts <= 8 && parts <= (tiles + 1) / 6; ++parts) {
     const double t_part = t_split / parts + kPartCost;
     const double cost = ((double)(jobs - split * per_rb) * t_whole + (double)(split * per_rb * parts) * t_part) / (double)sms + 0.3 * t_part;
@@ -586,8 +590,8 @@ quoka_status launch_attn_plan(const quoka_params* p, const DevParams& P, const A
 
 static AttnShape attn_usual_shape(const quoka_params* p) { return attn_shape(p, attn_whole(p, attn_largest_pack(p))); }
 bool attn_below_a_wave(const quoka_params* p) { return attn_usual_shape(p).jobs < device_sm_count(); }
-// (above a wave the cost of a plan with parts is more than q waves of average jobs, its line at most 0.9 (q + 1))
-bool attn_may_have_parts(const quoka_params* p) { return attn_usual_shape(p).jobs < 10ll * device_sm_count(); }
+// (above a wave the cost of a plan with parts is more than q waves of average jobs, its line at most 0.94 (q + 1): none from q = 16 on)
+bool attn_may_have_parts(const quoka_params* p) { return attn_usual_shape(p).jobs < 17ll * device_sm_count(); }
 int attn_same_plan_up_to(const quoka_params* p, int chunk) {
   int last = (chunk + kKeyTile - 1) / kKeyTile * kKeyTile;
   for (int pack = attn_largest_pack(p); pack >= 1; --pack) {
